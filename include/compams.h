@@ -404,6 +404,21 @@ int compams_blocksign_sweep_static(const float* grads, float* x_state, const flo
                                    uint32_t* sign_bits, int32_t n, int64_t d, int32_t deferred, void* cuda_stream);
 int compams_blocksign_sweep_static_limits(int64_t* max_workers, int64_t* max_tiles);
 
+/*
+ * compams_collect - gathers one worker's gradient, held as one tensor per parameter as a backward pass leaves it,
+ * into that worker's packed row of the [n, d] gradient buffer that compams_step takes.
+ *
+ *   row          device; [d] fp32, 4-byte aligned; coordinates offsets[0] ... offsets[count] - 1 are written.
+ *   tensors      host; count DEVICE pointers, tensor k packed fp32 of offsets[k + 1] - offsets[k] elements, 4-byte
+ *                aligned; null: the tensor has no gradient, its coordinates become 0. Read only.
+ *   offsets      host; count + 1 entries, offsets[0] >= 0, strictly increasing. Both arrays are read during the call.
+ *   count        number of tensors, at least 1.
+ *   cuda_stream  a cudaStream_t passed as void* (null = default stream); one kernel for up to 160 tensors is enqueued
+ *                there and the call returns without synchronising.
+ * Errors: INVALID_ARG (null or misaligned pointer, offsets not increasing), CUDA.
+ */
+int compams_collect(float* row, const float* const* tensors, const int64_t* offsets, int32_t count, void* cuda_stream);
+
 /* Static strings (never null). */
 const char* compams_error_string(int status);
 const char* compams_kernel_name(int32_t kernel);

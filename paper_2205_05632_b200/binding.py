@@ -117,6 +117,8 @@ def load_library() -> ctypes.CDLL:
     L.compams_blocksign_sweep_static.argtypes = [c.c_void_p] * 5 + [c.c_int32, c.c_int64, c.c_int32, c.c_void_p]
     L.compams_blocksign_sweep_static_limits.restype = c.c_int
     L.compams_blocksign_sweep_static_limits.argtypes = [c.POINTER(c.c_int64), c.POINTER(c.c_int64)]
+    L.compams_collect.restype = c.c_int
+    L.compams_collect.argtypes = [c.c_void_p, c.POINTER(c.c_void_p), c.POINTER(c.c_int64), c.c_int32, c.c_void_p]
     L.compams_error_string.restype = c.c_char_p
     L.compams_error_string.argtypes = [c.c_int]
     L.compams_kernel_name.restype = c.c_char_p

@@ -15,12 +15,13 @@ torch is used for the model and its autograd; the optimizer step itself runs in 
 """
 from __future__ import annotations
 
+import ctypes
 from typing import Iterable, List
 
 import numpy as np
 import torch
 
-from .binding import RANDK, TOPK, CompAMS, CompAMSError
+from .binding import RANDK, TOPK, CompAMS, CompAMSError, _check, load_library
 
 
 class CompAMSOptimizer:
@@ -43,6 +44,9 @@ class CompAMSOptimizer:
             self.theta[lo:hi].copy_(p.data.reshape(-1))
             p.data = self.theta[lo:hi].view(p.shape)
         self.G = torch.zeros(self.n, self.d, dtype=torch.float32, device=dev)
+        # collect(): the tensors' places in a row, and room for their gradients' addresses
+        self._places = (ctypes.c_int64 * len(self.offsets))(*self.offsets.tolist())
+        self._addresses = (ctypes.c_void_p * len(self.params))()
         blocks = np.array([0, self.d], dtype=np.int64) if whole_vector else self.offsets
         with torch.cuda.device(dev):
             self.opt = CompAMS(self.n, self.d, blocks, compressor, k_ratio, lr, beta1, beta2, eps)
@@ -53,13 +57,17 @@ class CompAMSOptimizer:
         """Row `worker` of G <- the gradients accumulated since the last collect(); they are cleared."""
         if not 0 <= worker < self.n:
             raise CompAMSError("worker %d outside [0, %d)" % (worker, self.n))
-        row = self.G[worker]
-        for p, lo, hi in zip(self.params, self.offsets[:-1], self.offsets[1:]):
-            if p.grad is None:
-                row[lo:hi].zero_()
-            else:
-                row[lo:hi].copy_(p.grad.reshape(-1))
-                p.grad = None
+        # one kernel for all tensors; a gradient that is not packed (channels-last, an expanded view) is packed first
+        grads = [p.grad for p in self.params]
+        grads = [g if g is None or g.is_contiguous() else g.contiguous() for g in grads]
+        self._addresses[:] = [None if g is None else g.data_ptr() for g in grads]
+        dev = self.G.device
+        with torch.cuda.device(dev):
+            stream = torch.cuda.current_stream(dev).cuda_stream
+            _check(load_library().compams_collect(self.G.data_ptr() + 4 * self.d * worker, self._addresses, self._places,
+                                                  len(grads), stream), "compams_collect")
+        for p in self.params:
+            p.grad = None
 
     def step(self) -> None:
         self.opt.step(self.G, self.theta)
