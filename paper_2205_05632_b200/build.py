@@ -9,7 +9,7 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libcompams.so")
 SOURCES = ["api.cu", "dense.cu", "blocksign.cu", "topk.cu", "randk.cu", "noalloc.cu", "collect.cu"]
-HEADERS = ["common.cuh", "context.h", "scatter.cuh", os.path.join("..", "..", "include", "compams.h")]
+HEADERS = ["common.cuh", "context.h", "scatter.cuh", "select.cuh", "predict.cuh", os.path.join("..", "..", "include", "compams.h")]
 
 # -fmad=false: no fused multiply-add anywhere, so each fp32 operation of the update rounds on its own.
 NVCC_FLAGS = [

@@ -82,6 +82,65 @@ int64_t kept_per_block(double k_ratio, int64_t d_b) {
     return k;
 }
 
+#ifndef SEL_CMAX
+#define SEL_CMAX 16
+#endif
+#ifndef SEL_PER
+#define SEL_PER 4
+#endif
+#ifndef SEL_LONG
+#define SEL_LONG 4096
+#endif
+constexpr int64_t kClusterMax = (int64_t)1 << 21;  // coordinates per CTA that a cluster goes through itself
+constexpr int64_t kListless = (int64_t)1 << 18;    // ... of a block that never has a list
+
+// Decides which kernels select from which blocks, and with how many CTAs.
+int group_segments(compams_context* c, const std::vector<SegInfo>& segs) {
+    c->tk.cluster_max = (int32_t)kClusterMax;
+    c->select_groups.clear();
+    c->dense_kernel = false;
+    c->seg_always_dense.assign(segs.size(), false);
+    if (c->randk) return COMPAMS_OK;
+    auto add = [&](std::vector<compams_context::SegGroup>& groups, std::vector<int32_t> list, int cluster) -> int {
+        if (list.empty()) return COMPAMS_OK;
+        // longest first (their CTAs differ in length by the lists' lengths)
+        std::stable_sort(list.begin(), list.end(), [&](int32_t a, int32_t b) { return segs[(size_t)a].cap > segs[(size_t)b].cap; });
+        compams_context::SegGroup g;
+        RC(dev_upload(c, &g.segs, list));
+        g.count = (int)list.size();
+        g.cluster = cluster;
+        groups.push_back(g);
+        return COMPAMS_OK;
+    };
+    // Long candidate lists get a cluster of CTAs each while there are too few of them to fill the GPU with one CTA per
+    // list; the others one CTA.
+    std::vector<int32_t> few, many;  // blocks for one CTA, for a cluster of them
+    auto expected = [&](const SegInfo& si) { return (int64_t)si.kb + si.kb / 4; };
+    for (size_t s = 0; s < segs.size(); ++s) (expected(segs[s]) < SEL_LONG ? few : many).push_back((int32_t)s);
+    int cluster = 1;
+    while (cluster < SEL_CMAX && (int64_t)many.size() * c->n * cluster * 2 <= SEL_PER * (int64_t)c->num_sms) cluster *= 2;
+    if (cluster == 1) {
+        few.insert(few.end(), many.begin(), many.end());
+        many.clear();
+    }
+    for (std::vector<int32_t>* l : {&few, &many}) {
+        const int64_t ctas = l == &few ? 1 : cluster;
+        std::vector<int32_t> listed;
+        for (int32_t s : *l) {
+            if (segs[(size_t)s].len > kClusterMax * ctas) c->dense_kernel = true;
+            if (segs[(size_t)s].cap || segs[(size_t)s].len <= kListless * ctas) {
+                listed.push_back(s);
+            } else {  // always the dense passes
+                c->seg_always_dense[(size_t)s] = true;
+                c->dense_kernel = true;
+            }
+        }
+        *l = listed;
+    }
+    RC(add(c->select_groups, many, cluster));
+    return add(c->select_groups, few, 1);
+}
+
 // Cuts the listed blocks into tiles of kTile coordinates and uploads the tile and segment tables.
 // For Top-k (`topk` true) every listed block also gets its message slots and candidate capacity.
 int build_tiles(compams_context* c, const std::vector<int32_t>& blocks, bool topk) {
@@ -108,9 +167,10 @@ int build_tiles(compams_context* c, const std::vector<int32_t>& blocks, bool top
             const int64_t kb = c->seg_off[(size_t)b + 1] - c->seg_off[(size_t)b];
             si.slot0 = c->seg_off[(size_t)b];
             si.kb = (uint32_t)kb;
-            // the candidate path pays off for sparse selections only: at most 1/32 of the block kept
-            int64_t cap = (!c->randk && kb * 32 <= len) ? 8 * kb + 1024 : 0;
-            if (cap > len) cap = len;
+            // the candidate path pays off for sparse selections only: at most 1/9 of the block kept
+            int64_t cap = (!c->randk && kb * 9 <= len) ? 8 * kb + 1024 : 0;
+            if (cap) cap = std::min(cap, len <= 65536 ? len : len / 4 + kb);
+            cap = (cap + 1) & ~(int64_t)1;  // lists are read in 128-bit pairs
             si.cap = (uint32_t)cap;
             si.cand_off = cand_total;
             cand_total += cap;
@@ -148,41 +208,9 @@ int build_tiles(compams_context* c, const std::vector<int32_t>& blocks, bool top
         c->segp.tile0[segs.size()] = (int32_t)tiles.size();
     }
     c->tk.cand_total = cand_total;
-    c->seg_cap_host.clear();
-    for (const SegInfo& si : segs) c->seg_cap_host.push_back(si.cap);
+    c->many_candidates = 4 * cand_total > c->d;  // more than d / 32 kept (a list has room for 8 k_b)
     if (topk) {
-        // Short candidate lists get one CTA each; a long one is cut into slices that many CTAs work on
-        // (two kernels that meet through a global histogram). Slices finish one list sooner, but with
-        // many long lists (layer-wise selection over many workers) one CTA per list has the higher
-        // throughput.
-        size_t n_long = 0;
-        for (const SegInfo& si : segs) n_long += si.cap > (uint32_t)kSelectSingleMax ? 1 : 0;
-        const uint32_t single_max = (n_long * (size_t)c->n >= 64) ? (1u << 20) : (uint32_t)kSelectSingleMax;
-        std::vector<int32_t> small_l, big_l;
-        for (size_t s = 0; s < segs.size(); ++s) {
-            if (segs[s].cap == 0) continue;  // never predicts: always the dense passes, no select needed
-            (segs[s].cap <= single_max ? small_l : big_l).push_back((int32_t)s);
-        }
-        // one-CTA lists are worked on longest first (their CTAs differ in length by the lists' lengths)
-        std::stable_sort(small_l.begin(), small_l.end(),
-                         [&](int32_t a, int32_t b) { return segs[(size_t)a].cap > segs[(size_t)b].cap; });
-        RC(dev_upload(c, &c->sel_small, small_l));
-        RC(dev_upload(c, &c->sel_big, big_l));
-        c->n_sel_small = (int)small_l.size();
-        c->n_sel_big = (int)big_l.size();
-        if (c->n_sel_big > 0) {
-            // enough slices for about four CTAs per SM over all long lists, and short enough (about
-            // 12 K of the expected 2.5 k_b candidates each) that a slice is a few dozen loads per thread
-            const int64_t lists = (int64_t)c->n * c->n_sel_big;
-            int64_t parts = (4 * (int64_t)c->num_sms + lists - 1) / lists;
-            int64_t kb_max = 0;
-            for (int32_t sg : big_l) kb_max = std::max<int64_t>(kb_max, segs[(size_t)sg].kb);
-            parts = std::max<int64_t>(parts, (5 * kb_max / 2 + 12287) / 12288);
-            c->sel_parts = (int)(parts < 1 ? 1 : parts > 1024 ? 1024 : parts);
-            RC(dev_alloc(c, &c->tk.sel_hist, (size_t)lists * kSelBins));
-            RC(dev_alloc(c, &c->tk.sel_ticket, (size_t)lists * 2));
-            RC(dev_alloc(c, &c->tk.sel_surv, (size_t)lists * kSurvCapBig, false));
-        }
+        RC(group_segments(c, segs));
     }
     return COMPAMS_OK;
 }
@@ -249,13 +277,15 @@ int init_context(compams_context* c, const int64_t* block_offsets) {
             init.tau_prev = kNoPrediction;
             std::vector<SegState> seg0((size_t)n * (size_t)c->tab.nseg, init);
             uint32_t never = 0;
-            for (uint32_t cap : c->seg_cap_host) never += cap ? 0u : 1u;
-            for (size_t k = 0; k < seg0.size(); ++k)
-                seg0[k].fallback = c->seg_cap_host[k % (size_t)c->tab.nseg] ? 0u : 1u;
+            for (size_t k = 0; k < seg0.size(); ++k) {
+                seg0[k].fallback = c->seg_always_dense[k % (size_t)c->tab.nseg] ? 1u : 0u;
+                never += seg0[k].fallback;
+            }
             RC(dev_upload(c, &t.seg, seg0));
             c->seg_init_host = seg0;
-            c->dense_count_init = never * (uint32_t)n;
-            std::vector<uint32_t> dc(1, never * (uint32_t)n);
+            c->dense_count_init = never;
+            c->deliver = !c->randk && n == c->n_total && never == 0;
+            std::vector<uint32_t> dc(1, never);
             RC(dev_upload(c, &t.dense_count, dc));
         }
         RC(dev_alloc(c, &t.tile_ties, c->randk ? 1 : (size_t)n * (size_t)c->tab.ntiles));
@@ -373,8 +403,8 @@ int compress_device(compams_context* c, const void* grads) {
     if (c->tk.nsmall > 0) RC(run_kernel(c, COMPAMS_K_TOPK_SMALL, [&] { return launch_topk_small(c, grads); }));
     if (c->tab.ntiles > 0) {
         RC(run_kernel(c, COMPAMS_K_TOPK_SWEEP, [&] { return launch_topk_sweep(c, grads); }));
-        RC(run_kernel(c, COMPAMS_K_TOPK_SELECT, [&] { return launch_topk_select(c); }));
-        RC(run_kernel(c, COMPAMS_K_TOPK_DENSE, [&] { return launch_topk_dense(c); }));
+        if (!c->select_groups.empty()) RC(run_kernel(c, COMPAMS_K_TOPK_SELECT, [&] { return launch_topk_select(c); }));
+        if (c->dense_kernel) RC(run_kernel(c, COMPAMS_K_TOPK_DENSE, [&] { return launch_topk_dense(c); }));
         c->e_mask_pending = true;
     }
     return COMPAMS_OK;
@@ -385,9 +415,9 @@ int apply_device(compams_context* c, float* theta) {
     if (c->compressor == COMPAMS_BLOCKSIGN) {
         return run_kernel(c, COMPAMS_K_BS_APPLY, [&] { return launch_bs_apply(c, theta); });
     }
-    // (a Random-k step with every worker in this handle has delivered its messages already)
-    if (!(c->randk && c->n == c->n_total))
-        RC(run_kernel(c, COMPAMS_K_TOPK_SCATTER, [&] { return launch_topk_scatter(c, !c->randk); }));
+    // (with every worker in this handle Random-k and most selections have delivered their messages already)
+    if (!(c->deliver || (c->randk && c->n == c->n_total)))
+        RC(run_kernel(c, COMPAMS_K_TOPK_SCATTER, [&] { return launch_topk_scatter(c); }));
     RC(run_kernel(c, COMPAMS_K_AMSGRAD, [&] { return launch_amsgrad(c, theta); }));
     return COMPAMS_OK;
 }

@@ -23,14 +23,11 @@ constexpr int kMaxTimed = 4096;    // event pairs kept for per-kernel timing
 constexpr int64_t kMaxD = ((int64_t)1 << 31) - 4 * kTile;  // largest d: tile coordinates are 32-bit and overshoot a block's end
 
 constexpr uint32_t kNoPrediction = 0xffffffffu;  // tau_hat value that no key reaches
-constexpr int kTileCand = 1024;          // candidates one tile can stage in shared memory
-constexpr int kSurvCap = 1536;           // threshold-bin candidates a select can rank in shared memory
-constexpr int kSurvCapBig = 65536;       // threshold-bin candidates of a long list (kept in global memory)
-constexpr int kSurvSmem = 4096;          // ... of which this many fit the finishing CTA's shared memory
-constexpr int kRankMax = 256;            // ... and up to this many are ranked pair by pair
+constexpr int kWarpCand = 128;           // candidates a warp of the sweep can stage in shared memory
+constexpr int kWarpCandMany = 256;       // ... where more than 1/32 of the coordinates are kept
+constexpr int kSurvCap = 2048;           // threshold-bin entries a select can rank in shared memory
 constexpr int kSelBins = 4096;           // bins of the candidate select's first histogram
 constexpr int64_t kChainMaxElems = COMPAMS_CHAIN_MAX;  // n d up to which a step's kernels are chained
-constexpr int kSelectSingleMax = 98304;  // candidate capacity up to which one CTA handles a segment
 
 // Per (worker, large block) Top-k selection state.
 struct SegState {
@@ -45,11 +42,9 @@ struct SegState {
     uint32_t prefix;      // high key bits decided so far
     uint32_t k_rem;       // entries still to take among the keys that match the prefix
     uint32_t tau;         // threshold key (after the last pass)
-    uint32_t ties_total;  // number of keys equal to tau
     uint32_t ties_take;   // how many of them belong to the kept set
-    uint32_t need_order;  // 1 when ties_take < ties_total: the lowest indices must be chosen
+    uint32_t need_order;  // 1 when not all keys equal to tau are kept: the lowest indices must be chosen
     uint32_t emit_count;  // message slots handed out so far
-    uint32_t sel_ready;   // multi-CTA select: the threshold bin has been found, the emit kernel may run
     uint32_t boost;       // the candidate margin is doubled this many times (raised when a list came up short)
     uint32_t streak;      // selections decided inside the list since the margin last changed
     uint32_t hold;        // a doubling is taken back after 32 << hold such selections in a row
@@ -92,11 +87,9 @@ struct TopkBuffers {
     SegState* seg;             // [n * nseg]
     uint32_t* tile_ties;       // [n, ntiles]
     uint2* cand;               // [n, cand_total] (coordinate, bits of x) pairs collected by the sweep
-    int64_t cand_total;        // candidate slots per worker
+    int64_t cand_total;        // candidate slots per worker (even: lists are read in 128-bit pairs)
+    int32_t cluster_max;       // coordinates per CTA up to which a select's cluster goes through the block itself
     uint32_t* dense_count;     // [1] segments currently marked for the dense passes
-    uint32_t* sel_hist;        // [n * long lists, kSelBins] histogram a long list's slices add into
-    uint32_t* sel_ticket;      // [n * long lists, 2] slices arrived; threshold-bin candidates appended
-    uint2* sel_surv;           // [n * long lists, kSurvCapBig] threshold-bin candidates of a long list
     double* acc;               // [d] binary64 accumulator, used only by entries that overflow their bucket
     uint32_t* thr;             // [n * nseg] bits of the magnitude from which on the segment's last selection kept
                                // everything: E still holds x at those elements; their e is 0
@@ -135,7 +128,7 @@ struct compams_context {
 
     std::vector<int64_t> off;      // host copy of the block offsets
     std::vector<int64_t> seg_off;  // host prefix sums of k_b (Top-k)
-    std::vector<uint32_t> seg_cap_host;  // candidate capacity of every tiled block (Top-k)
+    std::vector<bool> seg_always_dense;  // tiled blocks that only the dense passes select from (Top-k)
     int64_t K = 0;
     int64_t W = 0;
 
@@ -143,10 +136,16 @@ struct compams_context {
     compams::SegParams segp{};  // kernel-argument copy of the tiled blocks (nseg = 0: not usable)
     compams::BsBuffers bs{};
     compams::TopkBuffers tk{};
-    int32_t* sel_small = nullptr;  // tiled blocks whose candidate lists one CTA selects from
-    int32_t* sel_big = nullptr;    // tiled blocks whose candidate lists are cut into slices over many CTAs
-    int n_sel_small = 0, n_sel_big = 0;
-    int sel_parts = 1;  // slices a long candidate list is cut into
+    struct SegGroup {  // blocks whose selection is launched together
+        int32_t* segs = nullptr;
+        int count = 0;
+        int cluster = 1;    // CTAs per (worker, block)
+        bool wide = false;  // CTAs of 1024 threads
+    };
+    std::vector<SegGroup> select_groups;  // Top-k: blocks swept tile by tile, then selected from their candidate lists
+    bool many_candidates = false;  // Top-k: the lists hold more than 1/32 of the coordinates
+    bool dense_kernel = false;  // some blocks are too long for a cluster to go through: the dense passes are launched every step
+    bool deliver = false;       // the selection hands the kept entries to the server itself (no topk_scatter)
     std::vector<compams::SegState> seg_init_host;  // Top-k: the segments' state before the first step (set_state restores it)
     uint32_t dense_count_init = 0;
     uint64_t steps_done = 0;
@@ -201,7 +200,7 @@ cudaError_t launch_topk_sweep(compams_context* c, const void* grads);
 cudaError_t launch_topk_select(compams_context* c);
 cudaError_t launch_topk_dense(compams_context* c);
 cudaError_t launch_topk_materialize(compams_context* c);
-cudaError_t launch_topk_scatter(compams_context* c, bool close);
+cudaError_t launch_topk_scatter(compams_context* c);
 cudaError_t launch_randk_emit(compams_context* c, bool deliver);
 cudaError_t launch_amsgrad(compams_context* c, float* theta);
 

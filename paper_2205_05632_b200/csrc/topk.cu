@@ -33,12 +33,10 @@
 //   whoever reads E next - the next sweep, or topk_materialize - treats them as 0. Where a selection cuts through
 //   a group of equal magnitudes (some kept, some not), it zeroes the few kept ones in E itself and leaves the
 //   next larger magnitude.
-#include <cooperative_groups.h>
-
 #include "context.h"
+#include "predict.cuh"
 #include "scatter.cuh"
-
-namespace cg = cooperative_groups;
+#include "select.cuh"
 
 namespace compams {
 
@@ -81,16 +79,46 @@ __device__ __forceinline__ void load_x_tile(const float* __restrict__ e, int len
 // "Nothing kept": as a float this pattern is a NaN, which no magnitude reaches.
 constexpr uint32_t kNothingKept = 0xffffffffu;
 
+// A warp's candidates on their way to the list. MANY: of blocks that keep so many entries that most of a warp's
+// elements would meet in the shared counter, so the slots come from ballots and the count stays in a register.
+template <bool MANY>
+struct Stage {
+    static constexpr uint32_t kCap = MANY ? kWarpCandMany : kWarpCand;
+    uint2* stage;
+    uint32_t* staged;  // !MANY: the warp's counter in shared memory
+    uint32_t* g_cnt;
+    uint2* g_out;
+    uint32_t cap, count;
+    __device__ __forceinline__ void put(uint32_t slot, uint32_t coord, float x) {
+        const uint2 cv = make_uint2(coord, __float_as_uint(x));
+        if (slot < kCap) {
+            stage[slot] = cv;
+        } else {  // a stretch dense with candidates: the staging buffer is full, append directly
+            const uint32_t p = atomicAdd(g_cnt, 1u);
+            if (p < cap) g_out[p] = cv;
+        }
+    }
+    // Called by the whole warp.
+    __device__ __forceinline__ void add(bool is, uint32_t coord, float x) {
+        if constexpr (MANY) {
+            const unsigned m = __ballot_sync(0xffffffffu, is);
+            if (is) put(count + (uint32_t)__popc(m & ((1u << (threadIdx.x & 31)) - 1u)), coord, x);
+            count += (uint32_t)__popc(m);
+        } else {
+            if (is) put(atomicAdd(staged, 1u), coord, x);
+        }
+    }
+};
+
 // One tile of the sweep. The tile starts at r0 (relative to the block), which is the block's tile
 // boundary shifted down to a 128-byte line of G and E: r0 may be negative and the tile may reach
 // past the block; such coordinates are skipped.
 // `kept_from`: elements of E whose magnitude is at or above it were kept by the last step's selection and still
 // hold x; their e is 0 (one float comparison: the key order is the order of |x|).
-template <bool FULL, typename GT>
+template <bool FULL, typename GT, bool MANY>
 __device__ __forceinline__ void topk_sweep_tile(const GT* __restrict__ g, float* __restrict__ e, int len, int r0,
                                                 int warp, int lane, uint32_t tau_hat, uint32_t coord0,
-                                                uint2* sh_cand, uint32_t* sh_cnt, uint32_t* g_cnt, uint2* g_out,
-                                                uint32_t cap, float kept_from) {
+                                                Stage<MANY>& stage, float kept_from) {
     const int cg_ = align_class(g + r0), ce = align_class(e + r0);
     constexpr int NB = 2;  // iterations whose loads are in flight together
 #pragma unroll
@@ -124,16 +152,7 @@ __device__ __forceinline__ void topk_sweep_tile(const GT* __restrict__ g, float*
                 const float eo = lane_elem(ev[u], k);
                 const float ek = fabsf(eo) >= kept_from ? 0.0f : eo;
                 xs[k] = __fadd_rn(lane_elem(gv[u], k), ek);  // the corrected-gradient step: x = g + e
-                if ((FULL || (unsigned)(r + k) < (unsigned)len) && mag_key(xs[k]) >= tau_hat) {
-                    const uint2 cv = make_uint2(coord0 + (uint32_t)(r + k), __float_as_uint(xs[k]));
-                    const uint32_t slot = atomicAdd(sh_cnt, 1u);
-                    if (slot < (uint32_t)kTileCand) {
-                        sh_cand[slot] = cv;
-                    } else {  // a tile dense with candidates: the staging buffer is full, append directly
-                        const uint32_t p = atomicAdd(g_cnt, 1u);
-                        if (p < cap) g_out[p] = cv;
-                    }
-                }
+                stage.add((FULL || (unsigned)(r + k) < (unsigned)len) && mag_key(xs[k]) >= tau_hat, coord0 + (uint32_t)(r + k), xs[k]);
             }
             if (FULL || (r >= 0 && r + 3 < len)) {
                 store4(e + r, ce, make_float4(xs[0], xs[1], xs[2], xs[3]));
@@ -150,10 +169,10 @@ __device__ __forceinline__ void topk_sweep_tile(const GT* __restrict__ g, float*
 // lane and iteration, so that the gradient load is 128 bits wide like the loads and stores of E (with 4
 // coordinates per lane the 64-bit gradient loads leave too few bytes in flight). A warp's 1024 coordinates are
 // 4 chunks of 256; the next chunk's loads are in flight while one is worked on.
+template <bool MANY>
 __device__ __forceinline__ void topk_sweep_tile_bf16x8(const bf16_bits* __restrict__ g, float* __restrict__ e, int r0,
                                                        int warp, int lane, uint32_t tau_hat, uint32_t coord0,
-                                                       uint2* sh_cand, uint32_t* sh_cnt, uint32_t* g_cnt, uint2* g_out,
-                                                       uint32_t cap, float kept_from) {
+                                                       Stage<MANY>& stage, float kept_from) {
     constexpr int NC = kWarpSpan / 256;
     const int rw = r0 + warp * kWarpSpan;
     uint4 gbuf[2];
@@ -183,16 +202,7 @@ __device__ __forceinline__ void topk_sweep_tile_bf16x8(const bf16_bits* __restri
                 const float eo = lane_elem(ev[h], k);
                 const float ek = fabsf(eo) >= kept_from ? 0.0f : eo;
                 xs[k] = __fadd_rn(gk, ek);  // the corrected-gradient step: x = g + e
-                if (mag_key(xs[k]) >= tau_hat) {
-                    const uint2 cv = make_uint2(coord0 + (uint32_t)(r + h * 4 + k), __float_as_uint(xs[k]));
-                    const uint32_t slot = atomicAdd(sh_cnt, 1u);
-                    if (slot < (uint32_t)kTileCand) {
-                        sh_cand[slot] = cv;
-                    } else {  // a tile dense with candidates: the staging buffer is full, append directly
-                        const uint32_t p = atomicAdd(g_cnt, 1u);
-                        if (p < cap) g_out[p] = cv;
-                    }
-                }
+                stage.add(mag_key(xs[k]) >= tau_hat, coord0 + (uint32_t)(r + h * 4 + k), xs[k]);
             }
             *reinterpret_cast<float4*>(e + r + h * 4) = make_float4(xs[0], xs[1], xs[2], xs[3]);
         }
@@ -205,13 +215,15 @@ __device__ __forceinline__ void topk_sweep_tile_bf16x8(const bf16_bits* __restri
 #ifndef COMPAMS_BF16_TOPK_SWEEP_CTAS
 #define COMPAMS_BF16_TOPK_SWEEP_CTAS 5
 #endif
-template <typename GT>
-__global__ void __launch_bounds__(kThreads, sizeof(GT) == 2 ? COMPAMS_BF16_TOPK_SWEEP_CTAS : 6) topk_sweep_kernel(Tables t, TopkBuffers b, const GT* __restrict__ G,
+template <typename GT, bool MANY>
+__global__ void __launch_bounds__(kThreads, sizeof(GT) == 2 || MANY ? COMPAMS_BF16_TOPK_SWEEP_CTAS : 6) topk_sweep_kernel(Tables t, TopkBuffers b, const GT* __restrict__ G,
                                                                  const __grid_constant__ SegParams sp_) {
     dependency_wait();   // launched as a programmatic dependent while n d <= kChainMaxElems: the kernel before must be done
     allow_dependents();  // ... and the next one may move in behind this one's last wave
-    __shared__ uint2 sh_cand[kTileCand];
-    __shared__ uint32_t sh_cnt, sh_base;
+    // every warp stages the candidates of its 1024 coordinates by itself: in the list they then lie together, and the
+    // selection's warps meet few server buckets at a time
+    __shared__ uint2 sh_stage[kWarps][Stage<MANY>::kCap];
+    __shared__ uint32_t sh_staged[kWarps], sh_base;
     const TileInfo ti = sp_.nseg ? find_tile(sp_, blockIdx.x) : load_tile(t.tiles, blockIdx.x);
     const int i = blockIdx.y;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -221,8 +233,9 @@ __global__ void __launch_bounds__(kThreads, sizeof(GT) == 2 ? COMPAMS_BF16_TOPK_
     const SegInfo* si = t.segs + ti.seg;
     const uint32_t cap = si->cap;
     uint2* out = b.cand + (size_t)i * (size_t)b.cand_total + (size_t)si->cand_off;
-    if (threadIdx.x == 0) sh_cnt = 0u;
-    __syncthreads();
+    Stage<MANY> stage{sh_stage[warp], &sh_staged[warp], &st->cand_count, out, cap, 0u};
+    if (lane == 0) sh_staged[warp] = 0u;
+    __syncwarp();
     const int64_t row0 = (int64_t)i * t.d + ti.o;
     const GT* g = G + row0;
     float* e = b.E + row0;
@@ -234,696 +247,129 @@ __global__ void __launch_bounds__(kThreads, sizeof(GT) == 2 ? COMPAMS_BF16_TOPK_
         wide = whole && ((reinterpret_cast<uintptr_t>(g + r0s) | reinterpret_cast<uintptr_t>(e + r0s)) & 15u) == 0;
     if (wide) {
         if constexpr (sizeof(GT) == 2)
-            topk_sweep_tile_bf16x8(g, e, r0s, warp, lane, tau_hat, (uint32_t)ti.o, sh_cand, &sh_cnt, &st->cand_count, out,
-                                   cap, kept_from);
+            topk_sweep_tile_bf16x8(g, e, r0s, warp, lane, tau_hat, (uint32_t)ti.o, stage, kept_from);
     } else if (whole)
-        topk_sweep_tile<true>(g, e, ti.len, r0s, warp, lane, tau_hat, (uint32_t)ti.o, sh_cand, &sh_cnt,
-                              &st->cand_count, out, cap, kept_from);
+        topk_sweep_tile<true>(g, e, ti.len, r0s, warp, lane, tau_hat, (uint32_t)ti.o, stage, kept_from);
     else
-        topk_sweep_tile<false>(g, e, ti.len, r0s, warp, lane, tau_hat, (uint32_t)ti.o, sh_cand, &sh_cnt,
-                               &st->cand_count, out, cap, kept_from);
+        topk_sweep_tile<false>(g, e, ti.len, r0s, warp, lane, tau_hat, (uint32_t)ti.o, stage, kept_from);
+    if (MANY && lane == 0) sh_staged[warp] = stage.count;
     __syncthreads();
-    const uint32_t cnt = sh_cnt;
-    if (cnt == 0u) return;
-    const uint32_t stored = cnt < (uint32_t)kTileCand ? cnt : (uint32_t)kTileCand;
-    if (threadIdx.x == 0) sh_base = atomicAdd(&st->cand_count, stored);
+    uint32_t before = 0, total = 0, mine = 0;
+#pragma unroll
+    for (int w = 0; w < kWarps; ++w) {
+        const uint32_t k = sh_staged[w] < Stage<MANY>::kCap ? sh_staged[w] : Stage<MANY>::kCap;
+        if (w < warp) before += k;
+        if (w == warp) mine = k;
+        total += k;
+    }
+    if (total == 0u) return;
+    if (threadIdx.x == 0) sh_base = atomicAdd(&st->cand_count, total);
     __syncthreads();
-    const uint32_t base = sh_base;
-    for (uint32_t k = threadIdx.x; k < stored; k += kThreads)
-        if (base + k < cap) out[base + k] = sh_cand[k];
+    const uint32_t base = sh_base + before;
+    for (uint32_t k = lane; k < mine; k += 32)
+        if (base + k < cap) out[base + k] = sh_stage[warp][k];
 }
 
 // ------------------------------------------------------------------------------------------
 // select: exact Top-k inside the candidate list
 
-// Prediction for the next step's sweep, from this step's threshold key `tau` and the bin edge
-// `edge` at or above which about the wanted number of candidates (want_candidates) lay: the threshold keeps rising while the error
-// accumulators fill, so tau_hat follows half of the last rise. `sel_shift` sizes the bins of the
-// next select so that the expected threshold lands near the middle of its 4096 bins.
-__device__ __forceinline__ void predict_next(SegState* st, uint32_t tau, uint32_t edge, bool enabled) {
-    const uint32_t prev = st->tau_prev;
-    uint32_t rise = 0;
-    if (prev != kNoPrediction && tau > prev) rise = (tau - prev) >> 1;
-    if (edge > tau) edge = tau;
-    uint32_t next = edge + rise;
-    if (next >= 0x7f800000u) next = edge;
-    const uint32_t tau_pred = tau + rise;
-    uint32_t span = tau_pred > next ? tau_pred - next : 1u;
-    // ... but never so fine that the bins end close above the prediction: they cover at least a quarter of a
-    // binade (values up to about 19 % above tau_hat), so a threshold that lands higher than predicted - gradients
-    // that alternate between two levels do that - is still found inside the list
-    if (span < (1u << 19)) span = 1u << 19;
-    st->sel_shift = 32u - (uint32_t)__clz(span >> 11);  // smallest S with span >> S < 2048
-    st->tau_hat = enabled ? next : kNoPrediction;
-    st->tau_prev = tau;
-}
-
-// How many candidates the next step's predicted threshold should let through for a segment that keeps kb: the
-// count of keys above a fixed threshold moves by about sqrt(kb) from one step to the next (eight of those are
-// allowed for), plus a quarter of kb for drift of the gradient scale. A segment whose list came up short gets
-// its margin doubled (`boost` times, at most three); the doubling is taken back one step at a time after enough
-// selections in a row were decided inside the list (margin_held). Long lists thus carry about 1.26 kb entries, short ones
-// (kb = 50: 170) proportionally more.
-__device__ __forceinline__ uint32_t want_candidates(uint32_t kb, uint32_t boost) {
-    const uint32_t margin = ((kb >> 2) + (uint32_t)(8.0f * sqrtf((float)kb)) + 32u) << (boost < 3u ? boost : 3u);
-    const uint32_t most = 4u * kb + 512u;  // half the list's capacity
-    return kb + (margin < most - kb ? margin : most - kb);
-}
-// Taking a doubling back is a probe: if the smaller margin comes up short (a dense-pass step, which costs several
-// ordinary steps), the margin was needed, and the next probe waits twice as long (32, 64, ... 32768 selections). A
-// probe that holds for a whole waiting time halves the wait again. Gradients that alternate between two levels
-// need the first doubling for good: with a fixed wait of 32 every 33rd step ran the dense passes (n = 32,
-// d = 2^27: 9.1 -> 9.6 ms per step on average).
-constexpr uint32_t kHoldMax = 10u;
-__device__ __forceinline__ void margin_came_up_short(SegState* st) {
-    if (st->boost < 3u) ++st->boost;
-    if (st->probing && st->hold < kHoldMax) ++st->hold;
-    st->probing = 0u;
-    st->streak = 0u;
-}
-__device__ __forceinline__ void margin_held(SegState* st) {
-    if (++st->streak >= (32u << st->hold)) {
-        st->streak = 0u;
-        if (st->probing && st->hold) --st->hold;
-        st->probing = 0u;
-        if (st->boost) {
-            --st->boost;
-            st->probing = 1u;
-        }
-    }
-}
-
-// After a selection decided inside its list of c candidates: a list that held by less than a quarter of its margin
-// was a near miss and is treated like a list that came up short, only without the dense passes (thresholds that
-// swing from step to step announce themselves this way: d = 2^24, n = 8, two alternating batches: 1.01 k_b
-// candidates a dozen steps before 0.94 k_b).
-__device__ __forceinline__ void margin_after_selection(SegState* st, uint32_t kb, uint32_t c) {
-    if (c - kb < (want_candidates(kb, st->boost) - kb) >> 2) margin_came_up_short(st);
-    else margin_held(st);
-}
-
-constexpr int kSelUnroll = 4;   // candidate loads in flight per thread while scanning a list
-// One CTA per short list, 2048 threads to the SM at 32 registers. 1024 threads per list keep enough loads in flight
-// to finish one list soonest (few lists: d = 2^20, n = 8: step 0.051 ms against 0.058 with 512); with more lists
-// than the GPU holds CTAs, 512 threads per list and twice as many lists in flight get through them sooner
-// (ResNet-50 shapes layer-wise, n = 32, 1696 lists: select 0.121 -> 0.111 ms; with 256: 0.178).
-constexpr int kSelThreads = 1024;
-constexpr int kSelThreadsMany = 512;
-
-// Adds the `pred` lanes of a warp to a shared counter with one atomic; returns this lane's slot.
-__device__ __forceinline__ uint32_t warp_slot(bool pred, uint32_t* counter, int lane) {
-    const unsigned m = __ballot_sync(0xffffffffu, pred);
-    uint32_t base = 0;
-    if (m) {
-        const int leader = __ffs(m) - 1;
-        if (lane == leader) base = atomicAdd(counter, (uint32_t)__popc(m));
-        base = __shfl_sync(0xffffffffu, base, leader);
-    }
-    return base + (uint32_t)__popc(m & ((1u << lane) - 1u));
-}
-
-// A histogram of nb bins scanned from its top bin down: every thread owns nb / kThreads
-// consecutive bins (from the top) and learns how many entries lie above and inside its bins.
-struct BinScan {
-    uint32_t incl, excl;
-};
-template <int NT>
-__device__ __forceinline__ BinScan scan_from_top(const uint32_t* hm, int nb, uint32_t* scratch, uint32_t* total) {
-    const int per = nb / NT > 0 ? nb / NT : 1;
-    uint32_t sum = 0;
-    for (int j = 0; j < per; ++j) {
-        const int bin = nb - 1 - ((int)threadIdx.x * per + j);
-        if (bin >= 0) sum += hm[bin];
-    }
-    BinScan r;
-    r.incl = block_inclusive_scan<NT / 32>(sum, scratch, total);
-    r.excl = r.incl - sum;
-    return r;
-}
-// The thread whose bins hold the `target`-th entry from the top writes
-// sh_out[0] = bin, sh_out[1] = entries above the bin, sh_out[2] = entries in the bin.
-template <int NT>
-__device__ __forceinline__ void locate(const uint32_t* hm, int nb, const BinScan& sc, uint32_t target, uint32_t* sh_out) {
-    if (sc.excl < target && target <= sc.incl) {
-        const int per = nb / NT > 0 ? nb / NT : 1;
-        uint32_t running = sc.excl;
-        for (int j = 0; j < per; ++j) {
-            const int bin = nb - 1 - ((int)threadIdx.x * per + j);
-            const uint32_t cj = bin >= 0 ? hm[bin] : 0u;
-            if (running < target && target <= running + cj) {
-                sh_out[0] = (uint32_t)bin;
-                sh_out[1] = running;
-                sh_out[2] = cj;
-            }
-            running += cj;
-        }
-    }
-}
-
-__device__ __forceinline__ uint32_t offset_digit(uint32_t xbits, uint32_t tau_hat, int S) {
-    const uint32_t dg = ((xbits & 0x7fffffffu) - tau_hat) >> S;  // every candidate has key >= tau_hat
-    return dg < (uint32_t)(kSelBins - 1) ? dg : (uint32_t)(kSelBins - 1);
-}
+// One cluster per (worker, block) decides the selection inside the candidate list (see select.cuh) and closes the
+// segment. A list that cannot decide: the cluster goes through the block itself, or, where the block is too long for
+// its few CTAs, leaves it to the dense passes of the whole GPU. Lists come longest first, every worker's copy of one
+// block side by side: the clusters that take longest start first and the last wave holds the shortest.
+#ifndef SEL_NT
+#define SEL_NT 512
+#endif
+#ifndef SEL_CTAS
+#define SEL_CTAS 2
+#endif
+constexpr int kSelThreads = SEL_NT;
 
 template <int NT>
-__global__ void __launch_bounds__(NT, 2048 / NT) topk_select_kernel(Tables t, TopkBuffers b, const int32_t* __restrict__ seg_list,
-                                                               int nlist) {
-    dependency_wait();   // launched as a programmatic dependent while n d <= kChainMaxElems: the kernel before must be done
-    allow_dependents();  // ... and the next one may move in behind this one's last wave
-    __shared__ uint32_t local[kSelBins];  // histogram of the list
-    __shared__ uint2 surv[kSurvCap];
-    __shared__ uint32_t scratch[NT / 32];
-    __shared__ uint32_t sh_bin[3], sh_edge[3], sh_base, sh_wcnt, sh_scnt;
-    const int lane = threadIdx.x & 31;
-    // the lists come longest first, every worker's copy of one block side by side: the CTAs that take longest
-    // start first and the last wave holds the shortest lists
-    const int i = (int)(blockIdx.x % (unsigned)t.n);
-    const int seg = seg_list[blockIdx.x / (unsigned)t.n];
-    const size_t sg = (size_t)i * t.nseg + seg;
-    const SegInfo* si = t.segs + seg;
-    SegState* st = b.seg + sg;
-    const uint32_t kb = si->kb, cap = si->cap;
-    const uint32_t c = st->cand_count;
-    const uint32_t tau_hat = st->tau_hat;
-    const int S = (int)st->sel_shift;
-    if (!(tau_hat != kNoPrediction && c >= kb && c <= cap)) {
-        if (threadIdx.x == 0) {
-            st->fallback = 1u;
-            atomicAdd(b.dense_count, 1u);
-            if (tau_hat != kNoPrediction) atomicAdd(b.status + (c < kb ? 3 : 4), 1u);  // too few / too many candidates
-            if (tau_hat != kNoPrediction && c < kb) margin_came_up_short(st);
-        }
-        return;
-    }
-    const uint2* list = b.cand + (size_t)i * (size_t)b.cand_total + (size_t)si->cand_off;
-    const uint32_t lo = 0u, hi = c;
-    auto digit0 = [&](uint32_t xbits) -> uint32_t { return offset_digit(xbits, tau_hat, S); };
-
-    // ---- pass 0: histogram of the key offsets above tau_hat in bins of 2^S; the last bin is open-ended
-    for (int k = threadIdx.x; k < kSelBins; k += NT) local[k] = 0u;
-    if (threadIdx.x == 0) sh_scnt = 0u;
-    __syncthreads();
-    for (uint32_t p0 = lo; p0 < hi; p0 += kSelUnroll * NT) {
-        uint32_t y[kSelUnroll];
-#pragma unroll
-        for (int u = 0; u < kSelUnroll; ++u) {
-            const uint32_t p = p0 + u * NT + threadIdx.x;
-            y[u] = p < hi ? list[p].y : 0xffffffffu;  // no candidate has this pattern (NaN)
-        }
-#pragma unroll
-        for (int u = 0; u < kSelUnroll; ++u) {
-            const bool valid = y[u] != 0xffffffffu;
-            const uint32_t dg = valid ? digit0(y[u]) : 0u;
-            // the open-ended last bin collects every far-above-threshold candidate: one atomic per warp
-            const bool far = valid && dg == (uint32_t)(kSelBins - 1);
-            const unsigned m = __ballot_sync(0xffffffffu, far);
-            if (m && lane == __ffs(m) - 1) atomicAdd(&local[kSelBins - 1], (uint32_t)__popc(m));
-            if (valid && !far) atomicAdd(&local[dg], 1u);
-        }
-    }
-    __syncthreads();
-    uint32_t total;
-    {
-        const BinScan sc = scan_from_top<NT>(local, kSelBins, scratch, &total);
-        const uint32_t want = want_candidates(kb, st->boost);
-        if (threadIdx.x == 0) sh_edge[0] = 0xffffffffu;  // "fewer than `want` candidates"
-        __syncthreads();
-        locate<NT>(local, kSelBins, sc, kb, sh_bin);
-        locate<NT>(local, kSelBins, sc, want, sh_edge);
-    }
-    __syncthreads();
-    const uint32_t b0 = sh_bin[0];
-    uint32_t k_rem = kb - sh_bin[1];
-    const uint32_t c0 = sh_bin[2];
-    const uint32_t edge_bin = sh_edge[0];
-    const bool take_all0 = (c0 == k_rem);
-    // the number of winners, from the histogram
-    uint32_t mine = 0;
-    for (int k = threadIdx.x; k < kSelBins; k += NT)
-        if ((uint32_t)k > b0 || (take_all0 && (uint32_t)k == b0)) mine += local[k];
-    uint32_t my_winners;
-    block_inclusive_scan<NT / 32>(mine, scratch, &my_winners);
-    __syncthreads();
-    if (b0 == (uint32_t)(kSelBins - 1) && !take_all0) {
-        // the threshold lies in the open-ended bin: the prediction was far off, let the dense passes decide
-        if (threadIdx.x == 0) {
-            st->fallback = 1u;
-            atomicAdd(b.dense_count, 1u);
-            atomicAdd(b.status + 5, 1u);
-        }
-        return;
-    }
-
-    // ---- second scan of the list: winners to the message, threshold-bin candidates to shared memory
-    const size_t slot0 = (size_t)i * (size_t)b.K + (size_t)si->slot0;
-    uint2* surv0 = &surv[0];
-    uint32_t* scnt0 = &sh_scnt;
+__device__ __forceinline__ void start_select(SelectShared<NT>& sh) {
+    clear_hist<NT>(sh);
     if (threadIdx.x == 0) {
-        sh_base = my_winners ? atomicAdd(&st->emit_count, my_winners) : 0u;
-        sh_wcnt = 0u;
+        sh.winners = 0u;
+        sh.slots = 0u;
+        sh.nsurv = 0u;
+        sh.listed = 0u;
     }
     __syncthreads();
-    for (uint32_t p0 = lo; p0 < hi; p0 += kSelUnroll * NT) {
-        uint2 cvs[kSelUnroll];
-#pragma unroll
-        for (int u = 0; u < kSelUnroll; ++u) {
-            const uint32_t p = p0 + u * NT + threadIdx.x;
-            cvs[u] = p < hi ? list[p] : make_uint2(0u, 0xffffffffu);
+}
+
+// What a selection starts from, requested in one go.
+struct SelectState {
+    uint32_t c, tau_hat, boost;
+    int S;
+};
+__device__ __forceinline__ SelectState load_state(const SegState* st) {
+    SelectState s;
+    s.c = st->cand_count;
+    s.tau_hat = st->tau_hat;
+    s.S = (int)st->sel_shift;
+    s.boost = st->boost;
+    return s;
+}
+
+// Called by all threads of the cluster; CTAs that have nothing to do return early.
+template <int NT>
+__device__ __forceinline__ void select_segment(SelectShared<NT>& sh, const Tables& t, const TopkBuffers& b, const SegInfo& si, int i,
+                                               int seg, const SelectState& s, bool deliver) {
+    const size_t sg = (size_t)i * t.nseg + seg;
+    SegState* st = b.seg + sg;
+    const cg::cluster_group cluster = cg::this_cluster();
+    Group grp{cluster.num_blocks(), cluster.block_rank()};
+    const bool first = grp.rank == 0 && threadIdx.x == 0;
+    SelectJob job;
+    job.idx = b.idx + (size_t)i * (size_t)b.K + (size_t)si.slot0;
+    job.val = b.val + (size_t)i * (size_t)b.K + (size_t)si.slot0;
+    job.erow = b.E + (size_t)i * (size_t)t.d;
+    job.kb = si.kb;
+    job.cap = si.cap;
+    job.deliver = deliver;
+    // the same decision in every CTA of the cluster: nobody writes these words before all have read them
+    int why = s.c < si.kb ? 3 : 4;
+    if (s.tau_hat != kNoPrediction && s.c >= si.kb && s.c <= si.cap) {
+        if (s.c <= (uint32_t)(ListSlice::kU * NT) && grp.size > 1) {  // a short list: barriers of the cluster would cost
+            if (grp.rank) return;                                    // more than the other CTAs save
+            grp.size = 1;
         }
-#pragma unroll
-        for (int u = 0; u < kSelUnroll; ++u) {
-            const uint2 cv = cvs[u];
-            const bool valid = cv.y != 0xffffffffu;
-            const uint32_t dg = valid ? digit0(cv.y) : 0u;
-            const bool win = valid && (dg > b0 || (take_all0 && dg == b0));
-            const bool keep = valid && !take_all0 && dg == b0;
-            const uint32_t wpos = sh_base + warp_slot(win, &sh_wcnt, lane);
-            if (win) {
-                if (wpos < kb) {
-                    b.idx[slot0 + wpos] = (int32_t)cv.x;
-                    b.val[slot0 + wpos] = __uint_as_float(cv.y);
-                } else {
-                    atomicOr(b.status, 1u);
-                }
-            }
-            if (__any_sync(0xffffffffu, keep)) {  // rare: only the threshold bin's candidates
-                const uint32_t spos = warp_slot(keep, scnt0, lane);
-                if (keep && spos < (uint32_t)kSurvCap) surv0[spos] = cv;
-            }
-        }
-    }
-    // threshold key of this step (a lower bound if every candidate of the threshold bin is kept)
-    const unsigned long long tau_wide = (unsigned long long)tau_hat + ((unsigned long long)b0 << S);
-    uint32_t tau = tau_wide < 0x7f7fffffull ? (uint32_t)tau_wide : 0x7f7fffffu;
-    // the magnitude from which on everything was kept. With the whole threshold bin kept that is the bin's lower
-    // edge; otherwise the kept candidates of the bin are zeroed in E right here and the next key above the
-    // threshold is left
-    uint32_t kept_from = tau_wide < 0xffffffffull ? (uint32_t)tau_wide : kNothingKept;
-    float* erow = b.E + (size_t)i * (size_t)t.d;
-    if (!take_all0) {
-        __syncthreads();
-        const uint32_t nsurv = sh_scnt;
-        if (nsurv > (uint32_t)kSurvCap) {
-            // too many candidates share the threshold bin (heavily duplicated values): dense passes
-            if (threadIdx.x == 0) {
-                st->fallback = 1u;
-                atomicAdd(b.dense_count, 1u);
-                atomicAdd(b.status + 6, 1u);
-            }
+        const uint2* list = b.cand + (size_t)i * (size_t)b.cand_total + (size_t)si.cand_off;
+        if (select_from_list<NT>(grp, b, job, sh, st, b.thr + sg, list, s.c, s.tau_hat, s.S, s.boost, &why)) {
+            // the first CTA's shared memory stays until all have read from it (CTAs that have returned count as arrived)
+            if (cluster.num_blocks() > 1) cg::this_cluster().sync();
             return;
         }
-        // ---- the survivors are ordered by (key, lower index first): survivor q is kept when fewer
-        // than k_rem survivors beat it
-        const uint32_t lowmask = S ? ((1u << S) - 1u) : 0u;
-        auto comp_of = [&](const uint2& cv) -> unsigned long long {
-            const uint32_t o = (cv.y & 0x7fffffffu) - tau_hat;
-            return ((unsigned long long)(o & lowmask) << 32) | (unsigned long long)(0xffffffffu - cv.x);
-        };
-        for (uint32_t q0 = 0; q0 < nsurv; q0 += NT) {  // uniform trip count: the loop holds barriers
-            const uint32_t q = q0 + threadIdx.x;
-            bool kept = false;
-            uint2 cv = make_uint2(0u, 0u);
-            if (q < nsurv) {
-                cv = surv[q];
-                const unsigned long long mine_c = comp_of(cv);
-                uint32_t beaten = 0;
-                for (uint32_t p = 0; p < nsurv; ++p) beaten += (comp_of(surv[p]) > mine_c) ? 1u : 0u;
-                kept = beaten < k_rem;
-                if (beaten == k_rem - 1u) sh_edge[1] = (cv.y & 0x7fffffffu);  // the k-th largest key overall
-            }
-            uint32_t tot3;
-            const uint32_t incl = block_inclusive_scan<NT / 32>(kept ? 1u : 0u, scratch, &tot3);
-            if (threadIdx.x == 0) sh_base = tot3 ? atomicAdd(&st->emit_count, tot3) : 0u;
-            __syncthreads();
-            if (kept) {
-                const uint32_t pos = sh_base + incl - 1u;
-                if (pos < kb) {
-                    b.idx[slot0 + pos] = (int32_t)cv.x;
-                    b.val[slot0 + pos] = __uint_as_float(cv.y);
-                } else {
-                    atomicOr(b.status, 1u);
-                }
-                erow[cv.x] = 0.0f;  // the residual of a kept coordinate: e = x - x
-            }
-            __syncthreads();
-        }
-        tau = sh_edge[1];
-        kept_from = tau + 1u;
     }
-    if (threadIdx.x == 0) {
-        b.thr[sg] = kept_from;
-        uint32_t edge;
-        if (edge_bin != 0xffffffffu) {
-            const unsigned long long ew = (unsigned long long)tau_hat + ((unsigned long long)edge_bin << S);
-            edge = ew < 0x7f7fffffull ? (uint32_t)ew : 0x7f7fffffu;
-        } else {
-            // fewer candidates than wanted: reach further down next time, by half the distance to the threshold
-            const uint32_t gap = ((tau - tau_hat) >> 1) + (1u << 16);
-            edge = tau_hat > gap ? tau_hat - gap : 0u;
-        }
-        predict_next(st, tau, edge, true);
-        margin_after_selection(st, kb, c);
-        st->fallback = 0u;
-        atomicAdd(b.status + 2, 1u);  // selections decided inside their candidate list
+    if (first && s.tau_hat != kNoPrediction && si.cap) atomicAdd(b.status + why, 1u);
+    if ((int64_t)si.len <= (int64_t)b.cluster_max * cluster.num_blocks()) {
+        grp.sync();  // the state has been read by all
+        if (first && s.tau_hat != kNoPrediction && s.c < si.kb) margin_came_up_short(st);
+        select_from_block<NT>(grp, b, job, sh, st, b.thr + sg, job.erow + si.o, (uint32_t)si.len, (uint32_t)si.o, si.cap != 0u, s.boost);
+        if (cluster.num_blocks() > 1) cg::this_cluster().sync();
+        return;
+    }
+    if (first) {
+        st->fallback = 1u;
+        atomicAdd(b.dense_count, 1u);
+        if (s.tau_hat != kNoPrediction && s.c < si.kb) margin_came_up_short(st);
     }
 }
 
-// ------------------------------------------------------------------------------------------
-// select for a few long lists (whole-vector selection): every list is cut into `parts` slices and
-// two kernels of ordinary CTAs work on all slices at once. The slices of a list meet through a
-// histogram in global memory and "the last slice to arrive does the serial part" tickets; nobody
-// waits for anybody.
-//   topk_selhist  slice histograms of the key offsets above tau_hat, added into the list's global
-//                 histogram; the last slice finds the threshold bin and the next tau_hat's bin edge
-//   topk_selemit  winners above the threshold bin go to the message, the bin's candidates to the
-//                 list's survivor buffer; the last slice ranks the survivors, emits the best and predicts
-
-__global__ void __launch_bounds__(kThreads) topk_selhist_kernel(Tables t, TopkBuffers b, const int32_t* __restrict__ seg_list,
-                                                                int nlist, int parts) {
+template <int NT>
+__global__ void __launch_bounds__(NT, SEL_CTAS) topk_select_kernel(const __grid_constant__ Tables t,
+                                                                   const __grid_constant__ TopkBuffers b,
+                                                                   const int32_t* __restrict__ seg_list, int deliver) {
+    __shared__ SelectShared<NT> sh;
+    const unsigned item = blockIdx.x / cg::this_cluster().num_blocks();
+    const int i = (int)(item % (unsigned)t.n);
+    const int seg = seg_list[item / (unsigned)t.n];  // the block tables are never written by a kernel
+    const SegInfo si = t.segs[seg];
+    start_select<NT>(sh);
     dependency_wait();   // launched as a programmatic dependent while n d <= kChainMaxElems: the kernel before must be done
     allow_dependents();  // ... and the next one may move in behind this one's last wave
-    __shared__ uint32_t local[kSelBins];
-    __shared__ uint32_t scratch[kWarps];
-    __shared__ uint32_t sh_bin[3], sh_edge[3];
-    __shared__ int is_last;
-    const int lane = threadIdx.x & 31;
-    const int part = blockIdx.x % parts;
-    const size_t item = blockIdx.x / parts;  // (worker, list)
-    const int i = (int)(item / (size_t)nlist);
-    const int seg = seg_list[item % (size_t)nlist];
-    const size_t sg = (size_t)i * t.nseg + seg;
-    const SegInfo* si = t.segs + seg;
-    SegState* st = b.seg + sg;
-    const uint32_t kb = si->kb, cap = si->cap;
-    const uint32_t c = st->cand_count;
-    const uint32_t tau_hat = st->tau_hat;
-    const int S = (int)st->sel_shift;
-    // the same decision in every slice of the list: nobody writes these words in this kernel
-    if (!(tau_hat != kNoPrediction && c >= kb && c <= cap)) {
-        if (part == 0 && threadIdx.x == 0) {
-            st->fallback = 1u;
-            atomicAdd(b.dense_count, 1u);
-            if (tau_hat != kNoPrediction) atomicAdd(b.status + (c < kb ? 3 : 4), 1u);  // too few / too many candidates
-            if (tau_hat != kNoPrediction && c < kb) margin_came_up_short(st);
-        }
-        return;
-    }
-    const uint2* list = b.cand + (size_t)i * (size_t)b.cand_total + (size_t)si->cand_off;
-    const uint32_t per = (c + parts - 1) / parts;
-    const uint32_t lo = (uint32_t)part * per < c ? (uint32_t)part * per : c;
-    const uint32_t hi = (lo + per < c) ? lo + per : c;
-    for (int k = threadIdx.x; k < kSelBins; k += kThreads) local[k] = 0u;
-    __syncthreads();
-    for (uint32_t p0 = lo; p0 < hi; p0 += kSelUnroll * kThreads) {
-        uint32_t y[kSelUnroll];
-#pragma unroll
-        for (int u = 0; u < kSelUnroll; ++u) {
-            const uint32_t p = p0 + u * kThreads + threadIdx.x;
-            y[u] = p < hi ? list[p].y : 0xffffffffu;  // no candidate has this pattern (NaN)
-        }
-#pragma unroll
-        for (int u = 0; u < kSelUnroll; ++u) {
-            const bool valid = y[u] != 0xffffffffu;
-            const uint32_t dg = valid ? offset_digit(y[u], tau_hat, S) : 0u;
-            // the open-ended last bin collects every far-above-threshold candidate: one atomic per warp
-            const bool far = valid && dg == (uint32_t)(kSelBins - 1);
-            const unsigned m = __ballot_sync(0xffffffffu, far);
-            if (m && lane == __ffs(m) - 1) atomicAdd(&local[kSelBins - 1], (uint32_t)__popc(m));
-            if (valid && !far) atomicAdd(&local[dg], 1u);
-        }
-    }
-    __syncthreads();
-    uint32_t* gh = b.sel_hist + item * kSelBins;
-    for (int k = threadIdx.x; k < kSelBins; k += kThreads) {
-        const uint32_t v = local[k];
-        if (v) atomicAdd(gh + k, v);
-    }
-    __threadfence();
-    __syncthreads();
-    if (threadIdx.x == 0) is_last = (atomicAdd(b.sel_ticket + 2 * item, 1u) == (uint32_t)(parts - 1));
-    __syncthreads();
-    if (!is_last) return;
-    __threadfence();
-    // ---- the last slice: the list's histogram is complete
-    for (int k = threadIdx.x; k < kSelBins; k += kThreads) {
-        local[k] = __ldcg(gh + k);
-        gh[k] = 0u;  // clean for the next step
-    }
-    __syncthreads();
-    uint32_t total;
-    const BinScan sc = scan_from_top<kThreads>(local, kSelBins, scratch, &total);
-    const uint32_t want = want_candidates(kb, st->boost);
-    if (threadIdx.x == 0) sh_edge[0] = 0xffffffffu;  // "fewer than `want` candidates"
-    __syncthreads();
-    locate<kThreads>(local, kSelBins, sc, kb, sh_bin);
-    locate<kThreads>(local, kSelBins, sc, want, sh_edge);
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        b.sel_ticket[2 * item] = 0u;
-        const uint32_t b0 = sh_bin[0], k_rem = kb - sh_bin[1];
-        const bool take_all0 = (sh_bin[2] == k_rem);
-        if (b0 == (uint32_t)(kSelBins - 1) && !take_all0) {
-            // the threshold lies in the open-ended bin: the prediction was far off, let the dense passes decide
-            st->fallback = 1u;
-            atomicAdd(b.dense_count, 1u);
-            atomicAdd(b.status + 5, 1u);
-        } else {
-            st->prefix = b0;  // the dense passes' fields are free while the candidate path owns the segment
-            st->k_rem = k_rem;
-            st->ties_total = take_all0 ? 1u : 0u;
-            st->edge = sh_edge[0];
-            st->sel_ready = 1u;
-        }
-    }
-}
-
-__global__ void __launch_bounds__(kThreads) topk_selemit_kernel(Tables t, TopkBuffers b, const int32_t* __restrict__ seg_list,
-                                                                int nlist, int parts) {
-    dependency_wait();   // launched as a programmatic dependent while n d <= kChainMaxElems: the kernel before must be done
-    allow_dependents();  // ... and the next one may move in behind this one's last wave
-    __shared__ uint2 surv[kSurvSmem];
-    __shared__ uint32_t sh_hist[kThreads];
-    __shared__ uint32_t scratch[kWarps];
-    __shared__ uint32_t sh_base, sh_wcnt, sh_tau;
-    __shared__ int is_last;
-    const int lane = threadIdx.x & 31;
-    const int part = blockIdx.x % parts;
-    const size_t item = blockIdx.x / parts;
-    const int i = (int)(item / (size_t)nlist);
-    const int seg = seg_list[item % (size_t)nlist];
-    const size_t sg = (size_t)i * t.nseg + seg;
-    const SegInfo* si = t.segs + seg;
-    SegState* st = b.seg + sg;
-    if (st->sel_ready == 0u) return;  // not decided by the candidate path (same word for every slice)
-    const uint32_t kb = si->kb;
-    const uint32_t c = st->cand_count;
-    const uint32_t tau_hat = st->tau_hat;
-    const int S = (int)st->sel_shift;
-    const uint32_t b0 = st->prefix, k_rem = st->k_rem, edge_bin = st->edge;
-    const bool take_all0 = st->ties_total != 0u;
-    const uint2* list = b.cand + (size_t)i * (size_t)b.cand_total + (size_t)si->cand_off;
-    const uint32_t per = (c + parts - 1) / parts;
-    const uint32_t lo = (uint32_t)part * per < c ? (uint32_t)part * per : c;
-    const uint32_t hi = (lo + per < c) ? lo + per : c;
-    const size_t slot0 = (size_t)i * (size_t)b.K + (size_t)si->slot0;
-    uint2* gsurv = b.sel_surv + item * kSurvCapBig;
-    uint32_t* gscnt = b.sel_ticket + 2 * item + 1;  // survivors appended so far (second word of the pair)
-
-    // one pass over the slice, a chunk of kSelUnroll candidates per thread at a time: the chunk's winners are
-    // counted (a scan over the CTA), get one contiguous range of message slots with a single atomic, and are
-    // written there
-    for (uint32_t p0 = lo; p0 < hi; p0 += kSelUnroll * kThreads) {  // uniform trip count: the loop holds barriers
-        uint2 cvs[kSelUnroll];
-#pragma unroll
-        for (int u = 0; u < kSelUnroll; ++u) {
-            const uint32_t p = p0 + u * kThreads + threadIdx.x;
-            cvs[u] = p < hi ? list[p] : make_uint2(0u, 0xffffffffu);
-        }
-        uint32_t winmask = 0, keepmask = 0;
-#pragma unroll
-        for (int u = 0; u < kSelUnroll; ++u) {
-            const bool valid = cvs[u].y != 0xffffffffu;
-            const uint32_t dg = valid ? offset_digit(cvs[u].y, tau_hat, S) : 0u;
-            if (valid && (dg > b0 || (take_all0 && dg == b0))) winmask |= 1u << u;
-            if (valid && !take_all0 && dg == b0) keepmask |= 1u << u;
-        }
-        const uint32_t mine = (uint32_t)__popc(winmask);
-        uint32_t chunk_winners;
-        const uint32_t incl = block_inclusive_scan(mine, scratch, &chunk_winners);
-        if (threadIdx.x == 0) sh_base = chunk_winners ? atomicAdd(&st->emit_count, chunk_winners) : 0u;
-        __syncthreads();
-        uint32_t wpos = sh_base + incl - mine;
-#pragma unroll
-        for (int u = 0; u < kSelUnroll; ++u) {
-            if ((winmask >> u) & 1u) {
-                if (wpos < kb) {
-                    b.idx[slot0 + wpos] = (int32_t)cvs[u].x;
-                    b.val[slot0 + wpos] = __uint_as_float(cvs[u].y);
-                } else {
-                    atomicOr(b.status, 1u);
-                }
-                ++wpos;
-            }
-            const bool keep = (keepmask >> u) & 1u;
-            if (__any_sync(0xffffffffu, keep)) {  // rare: only the threshold bin's candidates
-                const uint32_t spos = warp_slot(keep, gscnt, lane);
-                if (keep && spos < (uint32_t)kSurvCapBig) gsurv[spos] = cvs[u];
-            }
-        }
-    }
-    __threadfence();
-    __syncthreads();
-    if (threadIdx.x == 0) is_last = (atomicAdd(b.sel_ticket + 2 * item, 1u) == (uint32_t)(parts - 1));
-    __syncthreads();
-    if (!is_last) return;
-    __threadfence();
-    // ---- the last slice finishes the list
-    const uint32_t nsurv = take_all0 ? 0u : __ldcg(gscnt);
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        b.sel_ticket[2 * item] = 0u;
-        b.sel_ticket[2 * item + 1] = 0u;
-        st->sel_ready = 0u;
-    }
-    if (nsurv > (uint32_t)kSurvCapBig) {
-        // too many candidates share the threshold bin (heavily duplicated values): dense passes
-        if (threadIdx.x == 0) {
-            st->fallback = 1u;
-            atomicAdd(b.dense_count, 1u);
-            atomicAdd(b.status + 6, 1u);
-        }
-        return;
-    }
-    const unsigned long long tau_wide = (unsigned long long)tau_hat + ((unsigned long long)b0 << S);
-    uint32_t tau = tau_wide < 0x7f7fffffull ? (uint32_t)tau_wide : 0x7f7fffffu;
-    // the magnitude from which on everything was kept. With the whole threshold bin kept that is the bin's lower
-    // edge; otherwise the kept candidates of the bin are zeroed in E right here and the next key above the
-    // threshold is left
-    uint32_t kept_from = tau_wide < 0xffffffffull ? (uint32_t)tau_wide : kNothingKept;
-    float* erow = b.E + (size_t)i * (size_t)t.d;
-    if (!take_all0 && nsurv > (uint32_t)kRankMax) {
-        // Too many candidates in the threshold bin to rank pair by pair. They differ in the low S key
-        // bits and the index; the k_rem-th largest of these (low bits, lower index first) composites
-        // is found digit by digit, 8 bits at a time from the top, with a 256-bin histogram over the
-        // candidates that match the digits found so far. The composites sit in shared memory when
-        // they fit, otherwise every pass reads the candidates again.
-        static_assert(kThreads == 256, "one histogram bin per thread");
-        unsigned long long* comp = reinterpret_cast<unsigned long long*>(surv);
-        uint32_t* hist = sh_hist;
-        const uint32_t lowmask = S ? ((1u << S) - 1u) : 0u;
-        auto comp_of = [&](const uint2& cv) -> unsigned long long {
-            const uint32_t o = (cv.y & 0x7fffffffu) - tau_hat;
-            return ((unsigned long long)(o & lowmask) << 32) | (unsigned long long)(0xffffffffu - cv.x);
-        };
-        const bool in_smem = nsurv <= (uint32_t)kSurvSmem;
-        if (in_smem)
-            for (uint32_t q = threadIdx.x; q < nsurv; q += kThreads) comp[q] = comp_of(__ldcg(gsurv + q));
-        unsigned long long prefix = 0ull;  // digits found so far, right-aligned
-        uint32_t need = k_rem;             // rank still to be located among the candidates matching `prefix`
-        const int top = ((S + 32 + 7) / 8 - 1) * 8;
-        for (int shift = top; shift >= 0; shift -= 8) {
-            __syncthreads();
-            hist[threadIdx.x] = 0u;
-            __syncthreads();
-            for (uint32_t q = threadIdx.x; q < nsurv; q += kThreads) {
-                const unsigned long long cq = in_smem ? comp[q] : comp_of(__ldcg(gsurv + q));
-                const bool match = (shift + 8 >= 64) || ((cq >> (shift + 8)) == prefix);
-                if (match) atomicAdd(&hist[(uint32_t)(cq >> shift) & 255u], 1u);
-            }
-            __syncthreads();
-            // thread t looks at digit 255 - t: `incl` candidates have this digit or a larger one
-            const uint32_t hv = hist[255 - threadIdx.x];
-            uint32_t tot;
-            const uint32_t incl = block_inclusive_scan(hv, scratch, &tot);
-            if (incl - hv < need && need <= incl) {
-                sh_base = 255u - threadIdx.x;
-                sh_wcnt = incl - hv;
-            }
-            __syncthreads();
-            prefix = (prefix << 8) | (unsigned long long)sh_base;
-            need -= sh_wcnt;
-        }
-        // `prefix` is now the composite of the k_rem-th largest candidate (composites are distinct)
-        const unsigned long long thr = prefix;
-        tau = tau_hat + (uint32_t)(((unsigned long long)b0 << S) | (thr >> 32));
-        kept_from = tau + 1u;
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            sh_base = atomicAdd(&st->emit_count, k_rem);
-            sh_wcnt = 0u;
-        }
-        __syncthreads();
-        for (uint32_t q = threadIdx.x; q < nsurv; q += kThreads) {
-            const uint2 cv = __ldcg(gsurv + q);
-            if (comp_of(cv) >= thr) {
-                const uint32_t pos = sh_base + atomicAdd(&sh_wcnt, 1u);
-                if (pos < kb) {
-                    b.idx[slot0 + pos] = (int32_t)cv.x;
-                    b.val[slot0 + pos] = __uint_as_float(cv.y);
-                } else {
-                    atomicOr(b.status, 1u);
-                }
-                erow[cv.x] = 0.0f;  // the residual of a kept coordinate: e = x - x
-            }
-        }
-        __syncthreads();
-        if (threadIdx.x == 0 && sh_wcnt != k_rem) atomicOr(b.status, 1u);
-    } else if (!take_all0) {
-        for (uint32_t q = threadIdx.x; q < nsurv; q += kThreads) surv[q] = __ldcg(gsurv + q);
-        __syncthreads();
-        // survivor q is kept when fewer than k_rem survivors beat it in (key, lower index first) order
-        const uint32_t lowmask = S ? ((1u << S) - 1u) : 0u;
-        auto comp_of = [&](const uint2& cv) -> unsigned long long {
-            const uint32_t o = (cv.y & 0x7fffffffu) - tau_hat;
-            return ((unsigned long long)(o & lowmask) << 32) | (unsigned long long)(0xffffffffu - cv.x);
-        };
-        for (uint32_t q0 = 0; q0 < nsurv; q0 += kThreads) {  // uniform trip count: the loop holds barriers
-            const uint32_t q = q0 + threadIdx.x;
-            bool kept = false;
-            uint2 cv = make_uint2(0u, 0u);
-            if (q < nsurv) {
-                cv = surv[q];
-                const unsigned long long mine_c = comp_of(cv);
-                uint32_t beaten = 0;
-                for (uint32_t p = 0; p < nsurv; ++p) beaten += (comp_of(surv[p]) > mine_c) ? 1u : 0u;
-                kept = beaten < k_rem;
-                if (beaten == k_rem - 1u) sh_tau = (cv.y & 0x7fffffffu);  // the k-th largest key overall
-            }
-            uint32_t tot3;
-            const uint32_t incl = block_inclusive_scan(kept ? 1u : 0u, scratch, &tot3);
-            if (threadIdx.x == 0) sh_base = tot3 ? atomicAdd(&st->emit_count, tot3) : 0u;
-            __syncthreads();
-            if (kept) {
-                const uint32_t pos = sh_base + incl - 1u;
-                if (pos < kb) {
-                    b.idx[slot0 + pos] = (int32_t)cv.x;
-                    b.val[slot0 + pos] = __uint_as_float(cv.y);
-                } else {
-                    atomicOr(b.status, 1u);
-                }
-                erow[cv.x] = 0.0f;  // the residual of a kept coordinate: e = x - x
-            }
-            __syncthreads();
-        }
-        tau = sh_tau;
-        kept_from = tau + 1u;
-    }
-    if (threadIdx.x == 0) {
-        b.thr[sg] = kept_from;
-        uint32_t edge;
-        if (edge_bin != 0xffffffffu) {
-            const unsigned long long ew = (unsigned long long)tau_hat + ((unsigned long long)edge_bin << S);
-            edge = ew < 0x7f7fffffull ? (uint32_t)ew : 0x7f7fffffu;
-        } else {
-            // fewer candidates than wanted: reach further down next time, by half the distance to the threshold
-            const uint32_t gap = ((tau - tau_hat) >> 1) + (1u << 16);
-            edge = tau_hat > gap ? tau_hat - gap : 0u;
-        }
-        predict_next(st, tau, edge, true);
-        margin_after_selection(st, kb, c);
-        st->fallback = 0u;
-        atomicAdd(b.status + 2, 1u);  // selections decided inside their candidate list
-    }
+    const SelectState s = load_state(b.seg + (size_t)i * t.nseg + seg);
+    select_segment<NT>(sh, t, b, si, i, seg, s, deliver != 0);
 }
 
 // ------------------------------------------------------------------------------------------
@@ -1010,7 +456,6 @@ __device__ __forceinline__ void dense_find(const Tables& t, const TopkBuffers& b
                     // the ties zeroes in E the ones it takes and everything from the next key up counts as kept
                     b.thr[sg] = (nk < cnt[j]) ? np + 1u : np;
                     st->tau = np;
-                    st->ties_total = cnt[j];
                     st->ties_take = nk;
                     st->need_order = (nk < cnt[j]) ? 1u : 0u;
                     // prediction for the next step's sweep (blocks without a candidate buffer never predict)
@@ -1023,7 +468,7 @@ __device__ __forceinline__ void dense_find(const Tables& t, const TopkBuffers& b
     if (PASS == 1) {
         // the highest pass-1 bin edge at or above which at least the wanted number of candidates lie (0 if there
         // are fewer); a candidate path that gave up may have handed out message slots: start over
-        const uint32_t want = want_candidates(kb, st->boost);
+        const uint32_t want = want_candidates(kb, st->boost, si->cap);
         if (threadIdx.x == 0) {
             st->emit_count = 0u;
             if (total < want) st->edge = 0u;
@@ -1045,7 +490,7 @@ __device__ __forceinline__ void dense_find(const Tables& t, const TopkBuffers& b
         // back to the dense passes step after step. When the wanted number is reached inside the threshold's own
         // pass-1 bin, this pass places the edge 1024 times finer; when that bin and the bins above hold fewer than
         // wanted, the edge is extrapolated below the bin's lower edge (see there).
-        const uint32_t want = want_candidates(kb, st->boost);
+        const uint32_t want = want_candidates(kb, st->boost, si->cap);
         const uint32_t above = kb - k_rem;     // keys in the pass-1 bins above the threshold's
         const uint32_t want2 = want - above;   // want > kb > above
         if (excl < want2 && want2 <= incl) {
@@ -1075,7 +520,7 @@ __device__ __forceinline__ void dense_find(const Tables& t, const TopkBuffers& b
 }
 
 __device__ __forceinline__ void dense_collect(const Tables& t, const TopkBuffers& b, uint32_t* scratch,
-                                              uint32_t* sh_base_p) {
+                                              uint32_t* sh_base_p, bool deliver) {
     uint32_t& sh_base = *sh_base_p;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int64_t total = (int64_t)t.n * t.ntiles;
@@ -1129,6 +574,7 @@ __device__ __forceinline__ void dense_collect(const Tables& t, const TopkBuffers
                         if (pos < kb) {
                             b.idx[slot0 + pos] = (int32_t)(ti.o + r + k);
                             b.val[slot0 + pos] = x;
+                            if (deliver) scatter_one(b, (int32_t)(ti.o + r + k), __float_as_uint(x));
                         } else {
                             atomicOr(b.status, 1u);
                         }
@@ -1145,7 +591,7 @@ __device__ __forceinline__ void dense_collect(const Tables& t, const TopkBuffers
 // tile. The ties land in the message slots after the `emit_count` winners; the count itself is
 // checked (with the ties added) when the step is closed.
 __device__ __forceinline__ void dense_ties(const Tables& t, const TopkBuffers& b, size_t sg, uint32_t* scratch,
-                                           uint32_t* sh_c, uint32_t* sh_excl) {
+                                           uint32_t* sh_c, uint32_t* sh_excl, bool deliver) {
     const int i = (int)(sg / (size_t)t.nseg);
     const SegInfo* si = t.segs + (sg % (size_t)t.nseg);
     const SegState* st = b.seg + sg;
@@ -1193,6 +639,7 @@ __device__ __forceinline__ void dense_ties(const Tables& t, const TopkBuffers& b
                 if (pos < kb) {
                     b.idx[slot0 + pos] = (int32_t)(o + r);
                     b.val[slot0 + pos] = e[r];
+                    if (deliver) scatter_one(b, (int32_t)(o + r), __float_as_uint(e[r]));
                 }
                 e[r] = 0.0f;  // the residual of a kept coordinate: e = x - x (this thread alone reads and writes e[r])
                 ++rank;
@@ -1205,29 +652,28 @@ __device__ __forceinline__ void dense_ties(const Tables& t, const TopkBuffers& b
     if (threadIdx.x == 0 && taken < want) atomicOr(b.status, 1u);
 }
 
-// Closes the step for one large-block segment: exactly k_b entries must have been emitted; the counters go
-// back to their resting values.
+// Closes the step for a segment that the dense passes decided: exactly k_b entries must have been emitted; the
+// counters go back to their resting values.
 __device__ __forceinline__ void close_segment(const TopkBuffers& b, const SegInfo* si, SegState* st) {
-    const bool dense = st->fallback != 0u;
-    const uint32_t ties = (dense && st->need_order) ? st->ties_take : 0u;
+    const uint32_t ties = st->need_order ? st->ties_take : 0u;
     if (st->emit_count + ties != si->kb) atomicOr(b.status, 1u);
-    if (dense) atomicAdd(b.status + 1, 1u);              // selections decided by the dense passes
-    if (dense && si->cap) atomicSub(b.dense_count, 1u);  // back to the number of blocks that never predict
+    atomicAdd(b.status + 1, 1u);                // selections decided by passes over the block
+    if (si->cap) atomicSub(b.dense_count, 1u);  // back to the number of blocks that are always selected here
     st->emit_count = 0u;
     st->cand_count = 0u;
-    st->fallback = si->cap ? 0u : 1u;  // blocks without a candidate buffer always take the dense passes
+    st->fallback = si->cap ? 0u : 1u;  // a block without a list that came here always does
     st->need_order = 0u;
 }
 
 // All dense passes in one cooperative launch: the grid is resident as a whole and the passes are
 // separated by grid-wide barriers. When no segment is marked every CTA returns at once, so in the
 // steady state the dense path costs one empty launch per step.
-__global__ void __launch_bounds__(kThreads) topk_dense_kernel(Tables t, TopkBuffers b) {
+__global__ void __launch_bounds__(kThreads) topk_dense_kernel(Tables t, TopkBuffers b, int deliver) {
     __shared__ uint32_t sh[kBins1];
     __shared__ uint32_t scratch[kWarps];
     __shared__ uint32_t sh_c[kThreads], sh_excl[kThreads];
     __shared__ uint32_t sh_base;
-    // the same word for every CTA; it only changes when the step is closed, in a later kernel
+    // the same word for every CTA; it only changes after the last barrier
     if (*b.dense_count == 0u) return;
     cg::grid_group grid = cg::this_grid();
     const size_t nsg = (size_t)t.n * (size_t)t.nseg;
@@ -1252,11 +698,12 @@ __global__ void __launch_bounds__(kThreads) topk_dense_kernel(Tables t, TopkBuff
         __syncthreads();
     }
     grid.sync();
-    dense_collect(t, b, scratch, &sh_base);
+    dense_collect(t, b, scratch, &sh_base, deliver != 0);
     grid.sync();
     for (size_t sg = blockIdx.x; sg < nsg; sg += gridDim.x) {
-        dense_ties(t, b, sg, scratch, sh_c, sh_excl);
+        dense_ties(t, b, sg, scratch, sh_c, sh_excl, deliver != 0);
         __syncthreads();
+        if (threadIdx.x == 0 && b.seg[sg].fallback) close_segment(b, t.segs + (sg % (size_t)t.nseg), b.seg + sg);
     }
 }
 
@@ -1264,7 +711,7 @@ __global__ void __launch_bounds__(kThreads) topk_dense_kernel(Tables t, TopkBuff
 // small blocks: the whole selection inside one CTA's shared memory
 
 template <typename GT>
-__global__ void __launch_bounds__(kThreads) topk_small_kernel(Tables t, TopkBuffers b, const GT* __restrict__ G) {
+__global__ void __launch_bounds__(kThreads) topk_small_kernel(Tables t, TopkBuffers b, const GT* __restrict__ G, int deliver) {
     __shared__ uint32_t xs[kSmallMax];
     __shared__ uint32_t hist[256];
     __shared__ uint32_t scratch[kWarps];
@@ -1343,6 +790,7 @@ __global__ void __launch_bounds__(kThreads) topk_small_kernel(Tables t, TopkBuff
             if (pos < kb) {
                 b.idx[slot0 + pos] = (int32_t)(o + r);
                 b.val[slot0 + pos] = __uint_as_float(xs[r]);
+                if (deliver) scatter_one(b, (int32_t)(o + r), xs[r]);
             }
             ++pos;
         }
@@ -1355,13 +803,13 @@ __global__ void __launch_bounds__(kThreads) topk_small_kernel(Tables t, TopkBuff
 // ------------------------------------------------------------------------------------------
 // scatter: the kept (index, value) pairs of the messages are handed to the server grouped by coordinate range.
 
-// All messages at once: `count` pairs of every worker the server averages over. The first n * nseg threads also
-// close the step for one large-block segment each when `close` is set (Top-k; Random-k has no selection to close).
-__global__ void __launch_bounds__(kThreads) topk_scatter_kernel(Tables t, TopkBuffers b, int64_t count, int close) {
+// All messages at once: `count` pairs of every worker the server averages over. For the messages that the selection did
+// not deliver itself: those of a sharded job, and of handles whose blocks keep so many entries that the dense passes
+// select them (their CTAs append entry by entry; here the lanes of a warp that meet in a bucket share one atomic).
+__global__ void __launch_bounds__(kThreads) topk_scatter_kernel(TopkBuffers b, int64_t count) {
     dependency_wait();
     allow_dependents();
     const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (close && p < (int64_t)t.n * t.nseg) close_segment(b, t.segs + (p % t.nseg), b.seg + p);
     const bool valid = p < count;
     int32_t j = 0;
     uint32_t xbits = 0;
@@ -1398,58 +846,47 @@ static TopkBuffers own_rows(const compams_context* c) {
 cudaError_t launch_topk_small(compams_context* c, const void* grads) {
     dim3 grid((unsigned)c->tk.nsmall, (unsigned)c->n);
     if (c->grad_bf16)
-        topk_small_kernel<bf16_bits><<<grid, kThreads, 0, c->stream>>>(c->tab, own_rows(c), (const bf16_bits*)grads);
+        topk_small_kernel<bf16_bits><<<grid, kThreads, 0, c->stream>>>(c->tab, own_rows(c), (const bf16_bits*)grads,
+                                                                    c->deliver ? 1 : 0);
     else
-        topk_small_kernel<float><<<grid, kThreads, 0, c->stream>>>(c->tab, own_rows(c), (const float*)grads);
+        topk_small_kernel<float><<<grid, kThreads, 0, c->stream>>>(c->tab, own_rows(c), (const float*)grads, c->deliver ? 1 : 0);
+    return counted(c, cudaGetLastError());
+}
+
+template <typename GT>
+static cudaError_t launch_sweep_typed(compams_context* c, const GT* grads) {
+    const dim3 grid((unsigned)c->tab.ntiles, (unsigned)c->n);
+    void (*kernel)(Tables, TopkBuffers, const GT*, const SegParams) =
+        c->many_candidates ? topk_sweep_kernel<GT, true> : topk_sweep_kernel<GT, false>;
+    if (c->chain) return counted(c, launch_after(kernel, grid, dim3(kThreads), c->stream, c->tab, own_rows(c), grads, c->segp));
+    kernel<<<grid, kThreads, 0, c->stream>>>(c->tab, own_rows(c), grads, c->segp);
     return counted(c, cudaGetLastError());
 }
 
 cudaError_t launch_topk_sweep(compams_context* c, const void* grads) {
-    dim3 grid((unsigned)c->tab.ntiles, (unsigned)c->n);
-    if (c->chain) {
-        if (c->grad_bf16)
-            return counted(c, launch_after(topk_sweep_kernel<bf16_bits>, grid, dim3(kThreads), c->stream, c->tab, own_rows(c),
-                                (const bf16_bits*)grads, c->segp));
-        return counted(c, launch_after(topk_sweep_kernel<float>, grid, dim3(kThreads), c->stream, c->tab, own_rows(c),
-                            (const float*)grads, c->segp));
-    }
-    if (c->grad_bf16)
-        topk_sweep_kernel<bf16_bits><<<grid, kThreads, 0, c->stream>>>(c->tab, own_rows(c), (const bf16_bits*)grads,
-                                                                       c->segp);
-    else
-        topk_sweep_kernel<float><<<grid, kThreads, 0, c->stream>>>(c->tab, own_rows(c), (const float*)grads, c->segp);
-    return counted(c, cudaGetLastError());
+    return c->grad_bf16 ? launch_sweep_typed(c, (const bf16_bits*)grads) : launch_sweep_typed(c, (const float*)grads);
 }
 
 // While n d <= kChainMaxElems the kernels of a step are launched as programmatic dependents of one another (each
 // waits for its predecessor before its first global access): the launch latency and the prologue of a
 // kernel then overlap the tail of the one before, which is most of what such a step costs.
-template <typename... KArgs, typename... Args>
-static cudaError_t launch_chained(compams_context* c, void (*kernel)(KArgs...), dim3 grid, dim3 block, Args... args) {
-    if (c->chain) return counted(c, launch_after(kernel, grid, block, c->stream, args...));
-    kernel<<<grid, block, 0, c->stream>>>(static_cast<KArgs>(args)...);
-    return counted(c, cudaGetLastError());
+
+// Clusters of more than 8 CTAs have to be asked for, once per kernel and device.
+template <typename K>
+static cudaError_t allow_large_cluster(K* kernel, int cluster) {
+    return cluster > 8 ? cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) : cudaSuccess;
 }
 
 cudaError_t launch_topk_select(compams_context* c) {
-    cudaError_t e = cudaSuccess;
-    const TopkBuffers b = own_rows(c);
-    if (c->n_sel_small > 0) {
-        const int64_t lists = (int64_t)c->n * c->n_sel_small;
-        if (lists >= 4 * (int64_t)c->num_sms)
-            e = launch_chained(c, topk_select_kernel<kSelThreadsMany>, dim3((unsigned)lists), dim3(kSelThreadsMany), c->tab, b,
-                               (const int32_t*)c->sel_small, c->n_sel_small);
-        else
-            e = launch_chained(c, topk_select_kernel<kSelThreads>, dim3((unsigned)lists), dim3(kSelThreads), c->tab, b,
-                               (const int32_t*)c->sel_small, c->n_sel_small);
+    for (const compams_context::SegGroup& g : c->select_groups) {
+        const dim3 grid((unsigned)((int64_t)c->n * g.count * g.cluster));
+        cudaError_t e = allow_large_cluster(topk_select_kernel<kSelThreads>, g.cluster);
+        if (e != cudaSuccess) return e;
+        e = counted(c, launch_cluster(topk_select_kernel<kSelThreads>, grid, dim3(kSelThreads), g.cluster, c->chain, c->stream, c->tab,
+                                      own_rows(c), (const int32_t*)g.segs, c->deliver ? 1 : 0));
+        if (e != cudaSuccess) return e;
     }
-    if (e != cudaSuccess || c->n_sel_big == 0) return e;
-    const dim3 grid((unsigned)((int64_t)c->n * c->n_sel_big * c->sel_parts));
-    e = launch_chained(c, topk_selhist_kernel, grid, dim3(kThreads), c->tab, b, (const int32_t*)c->sel_big, c->n_sel_big,
-                       c->sel_parts);
-    if (e != cudaSuccess) return e;
-    return launch_chained(c, topk_selemit_kernel, grid, dim3(kThreads), c->tab, b, (const int32_t*)c->sel_big,
-                          c->n_sel_big, c->sel_parts);
+    return cudaSuccess;
 }
 
 cudaError_t launch_topk_dense(compams_context* c) {
@@ -1461,7 +898,8 @@ cudaError_t launch_topk_dense(compams_context* c) {
         c->dense_grid = per_sm * c->num_sms;  // every CTA resident at once, as a cooperative launch requires
     }
     TopkBuffers b = own_rows(c);
-    void* args[] = {(void*)&c->tab, (void*)&b};
+    int deliver = c->deliver ? 1 : 0;
+    void* args[] = {(void*)&c->tab, (void*)&b, (void*)&deliver};
     return counted(c, cudaLaunchCooperativeKernel((const void*)topk_dense_kernel, dim3((unsigned)c->dense_grid),
                                                   dim3(kThreads), args, 0, c->stream));
 }
@@ -1472,15 +910,14 @@ cudaError_t launch_topk_materialize(compams_context* c) {
     return counted(c, cudaGetLastError());
 }
 
-cudaError_t launch_topk_scatter(compams_context* c, bool close) {
-    // one thread per message entry of every worker (>= n * nseg: every block keeps at least one entry)
+cudaError_t launch_topk_scatter(compams_context* c) {
+    // one thread per message entry of every worker
     const int64_t count = (int64_t)c->n_total * c->K;
     const unsigned grid = (unsigned)((count + kThreads - 1) / kThreads);
     // (a sharded handle's exchange sits in front of this kernel: a plain launch waits for it)
     if (c->chain && c->n == c->n_total)
-        return counted(c, launch_after(topk_scatter_kernel, dim3(grid), dim3(kThreads), c->stream, c->tab, c->tk, count,
-                                       close ? 1 : 0));
-    topk_scatter_kernel<<<grid, kThreads, 0, c->stream>>>(c->tab, c->tk, count, close ? 1 : 0);
+        return counted(c, launch_after(topk_scatter_kernel, dim3(grid), dim3(kThreads), c->stream, c->tk, count));
+    topk_scatter_kernel<<<grid, kThreads, 0, c->stream>>>(c->tk, count);
     return counted(c, cudaGetLastError());
 }
 
