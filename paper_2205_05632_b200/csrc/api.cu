@@ -86,7 +86,7 @@ int64_t kept_per_block(double k_ratio, int64_t d_b) {
 #define SEL_CMAX 16
 #endif
 #ifndef SEL_PER
-#define SEL_PER 4
+#define SEL_PER 1
 #endif
 #ifndef SEL_LONG
 #define SEL_LONG 4096
@@ -94,24 +94,18 @@ int64_t kept_per_block(double k_ratio, int64_t d_b) {
 constexpr int64_t kClusterMax = (int64_t)1 << 21;  // coordinates per CTA that a cluster goes through itself
 constexpr int64_t kListless = (int64_t)1 << 18;    // ... of a block that never has a list
 
+#ifndef DEFER_MIN
+#define DEFER_MIN 8
+#endif
+
 // Decides which kernels select from which blocks, and with how many CTAs.
 int group_segments(compams_context* c, const std::vector<SegInfo>& segs) {
     c->tk.cluster_max = (int32_t)kClusterMax;
-    c->select_groups.clear();
+    c->sel_long = c->sel_short = c->sel_parts = 0;
+    c->sel_cluster = 1;
     c->dense_kernel = false;
     c->seg_always_dense.assign(segs.size(), false);
     if (c->randk) return COMPAMS_OK;
-    auto add = [&](std::vector<compams_context::SegGroup>& groups, std::vector<int32_t> list, int cluster) -> int {
-        if (list.empty()) return COMPAMS_OK;
-        // longest first (their CTAs differ in length by the lists' lengths)
-        std::stable_sort(list.begin(), list.end(), [&](int32_t a, int32_t b) { return segs[(size_t)a].cap > segs[(size_t)b].cap; });
-        compams_context::SegGroup g;
-        RC(dev_upload(c, &g.segs, list));
-        g.count = (int)list.size();
-        g.cluster = cluster;
-        groups.push_back(g);
-        return COMPAMS_OK;
-    };
     // Long candidate lists get a cluster of CTAs each while there are too few of them to fill the GPU with one CTA per
     // list; the others one CTA.
     std::vector<int32_t> few, many;  // blocks for one CTA, for a cluster of them
@@ -119,10 +113,7 @@ int group_segments(compams_context* c, const std::vector<SegInfo>& segs) {
     for (size_t s = 0; s < segs.size(); ++s) (expected(segs[s]) < SEL_LONG ? few : many).push_back((int32_t)s);
     int cluster = 1;
     while (cluster < SEL_CMAX && (int64_t)many.size() * c->n * cluster * 2 <= SEL_PER * (int64_t)c->num_sms) cluster *= 2;
-    if (cluster == 1) {
-        few.insert(few.end(), many.begin(), many.end());
-        many.clear();
-    }
+    int64_t entries = 0;
     for (std::vector<int32_t>* l : {&few, &many}) {
         const int64_t ctas = l == &few ? 1 : cluster;
         std::vector<int32_t> listed;
@@ -130,15 +121,28 @@ int group_segments(compams_context* c, const std::vector<SegInfo>& segs) {
             if (segs[(size_t)s].len > kClusterMax * ctas) c->dense_kernel = true;
             if (segs[(size_t)s].cap || segs[(size_t)s].len <= kListless * ctas) {
                 listed.push_back(s);
+                if (l == &many && segs[(size_t)s].cap) entries = std::max(entries, expected(segs[(size_t)s]));
             } else {  // always the dense passes
                 c->seg_always_dense[(size_t)s] = true;
                 c->dense_kernel = true;
             }
         }
+        // longest first (their CTAs differ in length by the lists' lengths)
+        std::stable_sort(listed.begin(), listed.end(), [&](int32_t a, int32_t b) { return segs[(size_t)a].cap > segs[(size_t)b].cap; });
         *l = listed;
     }
-    RC(add(c->select_groups, many, cluster));
-    return add(c->select_groups, few, 1);
+    c->sel_long = (int)many.size();
+    c->sel_short = (int)few.size();
+    c->sel_cluster = cluster;
+    // lists that their clusters would have to go through in many rounds are emitted by a kernel of its own
+    if (c->sel_long && entries >= (int64_t)DEFER_MIN * cluster * 4096) {
+        const int64_t lists = (int64_t)c->n * c->sel_long;
+        c->sel_parts = (int)((entries + 2047) / 2048);
+        RC(dev_alloc(c, &c->tk.sel_ticket, (size_t)lists * 2));
+        RC(dev_alloc(c, &c->tk.sel_surv, (size_t)lists * kSurvCap, false));
+    }
+    many.insert(many.end(), few.begin(), few.end());
+    return dev_upload(c, &c->sel_segs, many);
 }
 
 // Cuts the listed blocks into tiles of kTile coordinates and uploads the tile and segment tables.
@@ -403,7 +407,7 @@ int compress_device(compams_context* c, const void* grads) {
     if (c->tk.nsmall > 0) RC(run_kernel(c, COMPAMS_K_TOPK_SMALL, [&] { return launch_topk_small(c, grads); }));
     if (c->tab.ntiles > 0) {
         RC(run_kernel(c, COMPAMS_K_TOPK_SWEEP, [&] { return launch_topk_sweep(c, grads); }));
-        if (!c->select_groups.empty()) RC(run_kernel(c, COMPAMS_K_TOPK_SELECT, [&] { return launch_topk_select(c); }));
+        if (c->sel_long + c->sel_short > 0) RC(run_kernel(c, COMPAMS_K_TOPK_SELECT, [&] { return launch_topk_select(c); }));
         if (c->dense_kernel) RC(run_kernel(c, COMPAMS_K_TOPK_DENSE, [&] { return launch_topk_dense(c); }));
         c->e_mask_pending = true;
     }

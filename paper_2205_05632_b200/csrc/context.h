@@ -45,6 +45,8 @@ struct SegState {
     uint32_t ties_take;   // how many of them belong to the kept set
     uint32_t need_order;  // 1 when not all keys equal to tau are kept: the lowest indices must be chosen
     uint32_t emit_count;  // message slots handed out so far
+    uint32_t emit_n;      // entries of a long list that is still to be emitted (0: none)
+    uint32_t emit_from;   // ... keys from here on are kept
     uint32_t boost;       // the candidate margin is doubled this many times (raised when a list came up short)
     uint32_t streak;      // selections decided inside the list since the margin last changed
     uint32_t hold;        // a doubling is taken back after 32 << hold such selections in a row
@@ -90,6 +92,8 @@ struct TopkBuffers {
     int64_t cand_total;        // candidate slots per worker (even: lists are read in 128-bit pairs)
     int32_t cluster_max;       // coordinates per CTA up to which a select's cluster goes through the block itself
     uint32_t* dense_count;     // [1] segments currently marked for the dense passes
+    uint32_t* sel_ticket;      // [n * long lists, 2] threshold-bin entries collected; parts of the emission done
+    uint2* sel_surv;           // [n * long lists, kSurvCap] threshold-bin entries of a long list
     double* acc;               // [d] binary64 accumulator, used only by entries that overflow their bucket
     uint32_t* thr;             // [n * nseg] bits of the magnitude from which on the segment's last selection kept
                                // everything: E still holds x at those elements; their e is 0
@@ -136,13 +140,10 @@ struct compams_context {
     compams::SegParams segp{};  // kernel-argument copy of the tiled blocks (nseg = 0: not usable)
     compams::BsBuffers bs{};
     compams::TopkBuffers tk{};
-    struct SegGroup {  // blocks whose selection is launched together
-        int32_t* segs = nullptr;
-        int count = 0;
-        int cluster = 1;    // CTAs per (worker, block)
-        bool wide = false;  // CTAs of 1024 threads
-    };
-    std::vector<SegGroup> select_groups;  // Top-k: blocks swept tile by tile, then selected from their candidate lists
+    int32_t* sel_segs = nullptr;  // Top-k: the tiled blocks with a selection kernel: sel_long, then sel_short of them
+    int sel_long = 0, sel_short = 0;
+    int sel_cluster = 1;          // CTAs per (worker, long block)
+    int sel_parts = 0;            // CTAs that emit a long list in a kernel of its own (0: the cluster emits it)
     bool many_candidates = false;  // Top-k: the lists hold more than 1/32 of the coordinates
     bool dense_kernel = false;  // some blocks are too long for a cluster to go through: the dense passes are launched every step
     bool deliver = false;       // the selection hands the kept entries to the server itself (no topk_scatter)

@@ -158,6 +158,7 @@ struct SelectJob {
     float* erow;   // the worker's row of E
     uint32_t kb, cap;
     bool deliver;  // kept pairs also go to the server's buckets
+    bool defer;    // the entries are emitted by a kernel of their own
 };
 
 // One kept pair in message slot `pos`.
@@ -170,11 +171,11 @@ __device__ __forceinline__ void put_pair(const TopkBuffers& b, const SelectJob& 
     }
 }
 
-// Emits U entries per thread, the whole warp together: keys from `win_from` up go to the message, those in
-// [bin_from, win_from) to the first CTA's survivors.
-template <int NT, int U>
-__device__ __forceinline__ void emit(const TopkBuffers& b, const SelectJob& job, SelectShared<NT>& sh, uint2* surv, uint32_t* nsurv,
-                                     const uint2* all, uint32_t win_from, uint32_t bin_from) {
+// Emits U entries per thread, the whole warp together: keys from `win_from` up go to the message, at `base` + slots
+// taken from `*taken`; those in [bin_from, win_from) to the survivors.
+template <int U>
+__device__ __forceinline__ void emit(const TopkBuffers& b, const SelectJob& job, uint32_t base, uint32_t* taken, uint2* surv,
+                                     uint32_t* nsurv, const uint2* all, uint32_t win_from, uint32_t bin_from) {
     const int lane = threadIdx.x & 31;
     uint2 cv[U];
     bool win[U];
@@ -196,7 +197,7 @@ __device__ __forceinline__ void emit(const TopkBuffers& b, const SelectJob& job,
     }
     if (warp_wins == 0u) return;
     uint32_t slot = 0;
-    if (lane == 0) slot = sh.base + atomicAdd(&sh.winners, warp_wins);
+    if (lane == 0) slot = base + atomicAdd(taken, warp_wins);
     slot = __shfl_sync(0xffffffffu, slot, 0);
 #pragma unroll
     for (int u = 0; u < U; ++u)
@@ -204,27 +205,21 @@ __device__ __forceinline__ void emit(const TopkBuffers& b, const SelectJob& job,
     if (job.deliver) scatter_runs<U>(b, win, cv);
 }
 
-// The k_rem best of the threshold bin's entries, larger key first, then lower index; an entry's rank is its slot
-// after the winners. Returns true in the one thread that holds the last one kept, with its key in *tau.
-template <int NT>
-__device__ __forceinline__ bool rank_survivors(const Group& grp, const TopkBuffers& b, const SelectJob& job, SelectShared<NT>& sh,
-                                               uint32_t nsurv, uint32_t k_rem, uint32_t* tau) {
-    const unsigned C = grp.size, rank = grp.rank;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    if (rank) {
-        const uint2* src = grp.of(sh.surv, 0);
-        for (uint32_t q = threadIdx.x; q < nsurv; q += NT) sh.surv[q] = src[q];
-        __syncthreads();
-    }
+// The k_rem best of the threshold bin's entries surv[0 .. nsurv), larger key first, then lower index; an entry's rank is
+// its slot after the winners. Warp w of W takes the entries w, w + W, ... Returns true in the one thread that holds the
+// last one kept, with its key in *tau.
+__device__ __forceinline__ bool rank_survivors(const TopkBuffers& b, const SelectJob& job, const uint2* surv, uint32_t nsurv,
+                                               uint32_t k_rem, uint32_t w, uint32_t W, uint32_t* tau) {
+    const int lane = threadIdx.x & 31;
     auto order = [](const uint2& cv) -> unsigned long long {
         return ((unsigned long long)(cv.y & 0x7fffffffu) << 32) | (unsigned long long)(0xffffffffu - cv.x);
     };
     bool last = false;
-    for (uint32_t q = (uint32_t)warp * C + rank; q < nsurv; q += C * (NT / 32)) {
-        const uint2 cv = sh.surv[q];
+    for (uint32_t q = w; q < nsurv; q += W) {
+        const uint2 cv = surv[q];
         const unsigned long long mine = order(cv);
         uint32_t beaten = 0;
-        for (uint32_t p = lane; p < nsurv; p += 32) beaten += order(sh.surv[p]) > mine ? 1u : 0u;
+        for (uint32_t p = lane; p < nsurv; p += 32) beaten += order(surv[p]) > mine ? 1u : 0u;
         beaten = __reduce_add_sync(0xffffffffu, beaten);
         if (lane == 0 && beaten < k_rem) {
             put_pair(b, job, job.kb - k_rem + beaten, cv.x, cv.y);
@@ -239,24 +234,20 @@ __device__ __forceinline__ bool rank_survivors(const Group& grp, const TopkBuffe
     return last;
 }
 
-// A slice of a candidate list: (coordinate, bits) pairs in any order, read two at a time (lists are 16-byte aligned),
-// from the L2: other CTAs of the cluster may have written them.
+// A slice of a candidate list: (coordinate, bits) pairs in any order, but those of one coordinate range mostly together.
+// Every warp reads 32 kU consecutive ones, from the L2: other CTAs of the cluster may have written them.
 struct ListSlice {
     static constexpr int kU = 8;
     static constexpr bool kOrdered = false;
     const uint2* list;
-    uint32_t lo, hi;  // lo is even
+    uint32_t lo, hi;
     template <int NT>
     __device__ __forceinline__ void load(uint32_t p0, uint2 (&cv)[kU]) const {
+        const uint32_t first = p0 + (threadIdx.x >> 5) * (32 * kU) + (threadIdx.x & 31);
 #pragma unroll
-        for (int u = 0; u < kU / 2; ++u) {
-            const uint32_t p = p0 + 2 * (u * NT + threadIdx.x);
-            cv[2 * u] = cv[2 * u + 1] = make_uint2(0u, kNoCandidate);
-            if (p < hi) {
-                const uint4 v = __ldcg(reinterpret_cast<const uint4*>(list + p));
-                cv[2 * u] = make_uint2(v.x, v.y);
-                if (p + 1 < hi) cv[2 * u + 1] = make_uint2(v.z, v.w);
-            }
+        for (int u = 0; u < kU; ++u) {
+            const uint32_t p = first + u * 32;
+            cv[u] = p < hi ? __ldcg(list + p) : make_uint2(0u, kNoCandidate);
         }
     }
 };
@@ -281,6 +272,7 @@ struct BlockSlice {
 // when the whole bin was kept), the key that about the wanted number of entries reach (reached = false: fewer do).
 struct Selected {
     uint32_t kept_from, tau, edge;
+    uint32_t k_rem;  // deferred emission: entries to take from the bin [tau, kept_from), 0: keys from tau = kept_from on
     bool reached;
     bool closer;  // this thread closes the segment's state
     int why;      // not decided: 5 the threshold lies beyond the histogram's range, 6 too many equal keys
@@ -374,20 +366,27 @@ __device__ __forceinline__ bool select_slices(const Group& grp, const TopkBuffer
         locate_bins<NT>(grp, sh, edge_need, 0u);
         out.edge += sh.bin[0] << s;
     }
+    const unsigned long long beyond = (unsigned long long)from + (1ull << S);
+    const uint32_t win_from = take_all ? from : beyond < 0x7f800000ull ? (uint32_t)beyond : 0x7f800000u;
+    if (job.defer) {
+        out.kept_from = win_from;
+        out.tau = from;
+        out.k_rem = take_all ? 0u : k_rem;
+        out.closer = rank == 0 && threadIdx.x == 0;
+        return true;
+    }
     __syncthreads();
     if (threadIdx.x == 0) {
         sh.base = my_wins ? atomicAdd(grp.of(&sh.slots, 0), my_wins) : 0u;
         sh.winners = 0u;
     }
     __syncthreads();
-    const unsigned long long beyond = (unsigned long long)from + (1ull << S);
-    const uint32_t win_from = take_all ? from : beyond < 0x7f800000ull ? (uint32_t)beyond : 0x7f800000u;
     uint2* surv = grp.of(sh.surv, 0);
     uint32_t* nsurv = grp.of(&sh.nsurv, 0);
     for (uint32_t p0 = sl.lo; p0 < sl.hi; p0 += U * NT) {
         if (!kHold || p0 != sl.lo) sl.template load<NT>(p0, held);
 #pragma unroll
-        for (int h = 0; h < U; h += 4) emit<NT, 4>(b, job, sh, surv, nsurv, held + h, win_from, by_index ? win_from : from);
+        for (int h = 0; h < U; h += 4) emit<4>(b, job, sh.base, &sh.winners, surv, nsurv, held + h, win_from, by_index ? win_from : from);
     }
     if (by_index && threadIdx.x < C) grp.of(sh.range, threadIdx.x)[rank] = my_ties;
     grp.sync();  // all winners have their slots, the first CTA has all survivors, everyone the counts of ties
@@ -413,7 +412,14 @@ __device__ __forceinline__ bool select_slices(const Group& grp, const TopkBuffer
             }
         }
     }
-    if (!take_all && !by_index) out.closer = rank_survivors<NT>(grp, b, job, sh, c0, k_rem, &out.tau);
+    if (!take_all && !by_index) {
+        if (rank) {
+            const uint2* src = grp.of(sh.surv, 0);
+            for (uint32_t q = threadIdx.x; q < c0; q += NT) sh.surv[q] = src[q];
+            __syncthreads();
+        }
+        out.closer = rank_survivors(b, job, sh.surv, c0, k_rem, (threadIdx.x >> 5) * C + rank, C * (NT / 32), &out.tau);
+    }
     // with the whole bin kept, everything from its lower edge on; otherwise the kept entries of the bin have been zeroed
     // in E and the next key above the k-th largest is left
     out.kept_from = take_all ? from : out.tau + 1u;
@@ -421,12 +427,28 @@ __device__ __forceinline__ bool select_slices(const Group& grp, const TopkBuffer
     return true;
 }
 
+// A list of c candidates above tau_hat has decided: leaves what the next step needs. `edge`: see Selected (kNoBin: not
+// reached).
+__device__ __forceinline__ void close_list(const TopkBuffers& b, const SelectJob& job, SegState* st, uint32_t* thr,
+                                           uint32_t kept_from, uint32_t tau, uint32_t edge, uint32_t c, uint32_t tau_hat) {
+    *thr = kept_from;
+    if (edge == kNoBin) {
+        // fewer candidates than wanted: reach further down next time, by half the distance to the threshold
+        const uint32_t gap = ((tau - tau_hat) >> 1) + (1u << 16);
+        edge = tau_hat > gap ? tau_hat - gap : 0u;
+    }
+    predict_next(st, tau, edge, true);
+    margin_after_selection(st, job.kb, c, job.cap);
+    st->cand_count = 0u;
+    atomicAdd(b.status + 2, 1u);  // selections decided inside their candidate list
+}
+
 // From a candidate list of c entries (k_b <= c) whose keys all reach tau_hat.
 template <int NT>
 __device__ __forceinline__ bool select_from_list(const Group& grp, const TopkBuffers& b, const SelectJob& job, SelectShared<NT>& sh,
                                                  SegState* st, uint32_t* thr, const uint2* list, uint32_t c, uint32_t tau_hat, int S,
                                                  uint32_t boost, int* why) {
-    const uint32_t per = ((c + grp.size - 1) / grp.size + 1u) & ~1u;
+    const uint32_t per = (c + grp.size - 1) / grp.size;
     ListSlice sl;
     sl.list = list;
     sl.lo = grp.rank * per < c ? grp.rank * per : c;
@@ -437,16 +459,18 @@ __device__ __forceinline__ bool select_from_list(const Group& grp, const TopkBuf
         return false;
     }
     if (s.closer) {
-        *thr = s.kept_from;
-        if (!s.reached) {
-            // fewer candidates than wanted: reach further down next time, by half the distance to the threshold
-            const uint32_t gap = ((s.tau - tau_hat) >> 1) + (1u << 16);
-            s.edge = tau_hat > gap ? tau_hat - gap : 0u;
+        const uint32_t edge = s.reached ? s.edge : kNoBin;
+        if (job.defer) {
+            st->emit_n = c;
+            st->emit_from = s.kept_from;
+            st->prefix = s.tau;  // (the dense passes' fields are free while the list decides)
+            st->k_rem = s.k_rem;
+            st->edge = edge;
+            st->emit_count = 0u;
+            st->cand_count = 0u;
+        } else {
+            close_list(b, job, st, thr, s.kept_from, s.tau, edge, c, tau_hat);
         }
-        predict_next(st, s.tau, s.edge, true);
-        margin_after_selection(st, job.kb, c, job.cap);
-        st->cand_count = 0u;
-        atomicAdd(b.status + 2, 1u);  // selections decided inside their candidate list
     }
     return true;
 }

@@ -311,15 +311,7 @@ __device__ __forceinline__ SelectState load_state(const SegState* st) {
     return s;
 }
 
-// Called by all threads of the cluster; CTAs that have nothing to do return early.
-template <int NT>
-__device__ __forceinline__ void select_segment(SelectShared<NT>& sh, const Tables& t, const TopkBuffers& b, const SegInfo& si, int i,
-                                               int seg, const SelectState& s, bool deliver) {
-    const size_t sg = (size_t)i * t.nseg + seg;
-    SegState* st = b.seg + sg;
-    const cg::cluster_group cluster = cg::this_cluster();
-    Group grp{cluster.num_blocks(), cluster.block_rank()};
-    const bool first = grp.rank == 0 && threadIdx.x == 0;
+__device__ __forceinline__ SelectJob select_job(const Tables& t, const TopkBuffers& b, const SegInfo& si, int i, bool deliver) {
     SelectJob job;
     job.idx = b.idx + (size_t)i * (size_t)b.K + (size_t)si.slot0;
     job.val = b.val + (size_t)i * (size_t)b.K + (size_t)si.slot0;
@@ -327,26 +319,42 @@ __device__ __forceinline__ void select_segment(SelectShared<NT>& sh, const Table
     job.kb = si.kb;
     job.cap = si.cap;
     job.deliver = deliver;
-    // the same decision in every CTA of the cluster: nobody writes these words before all have read them
+    job.defer = false;
+    return job;
+}
+
+// Called by all threads of the group; CTAs that have nothing to do return early.
+template <int NT>
+__device__ __forceinline__ void select_segment(Group grp, SelectShared<NT>& sh, const Tables& t, const TopkBuffers& b,
+                                               const SegInfo& si, int i, int seg, const SelectState& s, bool deliver, bool defer) {
+    const size_t sg = (size_t)i * t.nseg + seg;
+    SegState* st = b.seg + sg;
+    const unsigned ctas = grp.size;
+    const bool first = grp.rank == 0 && threadIdx.x == 0;
+    SelectJob job = select_job(t, b, si, i, deliver);
+    // the same decision in every CTA of the group: nobody writes these words before all have read them
     int why = s.c < si.kb ? 3 : 4;
     if (s.tau_hat != kNoPrediction && s.c >= si.kb && s.c <= si.cap) {
-        if (s.c <= (uint32_t)(ListSlice::kU * NT) && grp.size > 1) {  // a short list: barriers of the cluster would cost
-            if (grp.rank) return;                                    // more than the other CTAs save
+        if (s.c <= (uint32_t)(ListSlice::kU * NT) && ctas > 1) {  // a short list: barriers of the cluster would cost more
+            if (grp.rank) return;                                  // than the other CTAs save
             grp.size = 1;
+        } else {
+            job.defer = defer;
         }
         const uint2* list = b.cand + (size_t)i * (size_t)b.cand_total + (size_t)si.cand_off;
         if (select_from_list<NT>(grp, b, job, sh, st, b.thr + sg, list, s.c, s.tau_hat, s.S, s.boost, &why)) {
             // the first CTA's shared memory stays until all have read from it (CTAs that have returned count as arrived)
-            if (cluster.num_blocks() > 1) cg::this_cluster().sync();
+            if (ctas > 1) cg::this_cluster().sync();
             return;
         }
+        job.defer = false;
     }
     if (first && s.tau_hat != kNoPrediction && si.cap) atomicAdd(b.status + why, 1u);
-    if ((int64_t)si.len <= (int64_t)b.cluster_max * cluster.num_blocks()) {
+    if ((int64_t)si.len <= (int64_t)b.cluster_max * ctas) {
         grp.sync();  // the state has been read by all
         if (first && s.tau_hat != kNoPrediction && s.c < si.kb) margin_came_up_short(st);
         select_from_block<NT>(grp, b, job, sh, st, b.thr + sg, job.erow + si.o, (uint32_t)si.len, (uint32_t)si.o, si.cap != 0u, s.boost);
-        if (cluster.num_blocks() > 1) cg::this_cluster().sync();
+        if (ctas > 1) cg::this_cluster().sync();
         return;
     }
     if (first) {
@@ -356,20 +364,126 @@ __device__ __forceinline__ void select_segment(SelectShared<NT>& sh, const Table
     }
 }
 
+// seg_list: `nlong` blocks that a cluster selects from, then `nshort` that one CTA does; a cluster's CTAs take as many
+// of the latter as they are. `defer`: the long lists' entries are emitted by topk_emit.
 template <int NT>
 __global__ void __launch_bounds__(NT, SEL_CTAS) topk_select_kernel(const __grid_constant__ Tables t,
                                                                    const __grid_constant__ TopkBuffers b,
-                                                                   const int32_t* __restrict__ seg_list, int deliver) {
+                                                                   const int32_t* __restrict__ seg_list, int nlong, int nshort,
+                                                                   int deliver, int defer) {
     __shared__ SelectShared<NT> sh;
-    const unsigned item = blockIdx.x / cg::this_cluster().num_blocks();
+    Group grp{cg::this_cluster().num_blocks(), cg::this_cluster().block_rank()};
+    unsigned item = blockIdx.x / grp.size;
+    const unsigned longs = (unsigned)(t.n * nlong);
+    const int32_t* segs = seg_list;
+    const bool alone = item >= longs;
+    if (alone) {
+        item = (item - longs) * grp.size + grp.rank;
+        segs += nlong;
+        grp = Group{1u, 0u};
+    }
     const int i = (int)(item % (unsigned)t.n);
-    const int seg = seg_list[item / (unsigned)t.n];  // the block tables are never written by a kernel
+    const unsigned q = item / (unsigned)t.n;
+    const bool idle = alone && q >= (unsigned)nshort;
+    const int seg = segs[idle ? 0u : q];  // the block tables are never written by a kernel
     const SegInfo si = t.segs[seg];
     start_select<NT>(sh);
     dependency_wait();   // launched as a programmatic dependent while n d <= kChainMaxElems: the kernel before must be done
     allow_dependents();  // ... and the next one may move in behind this one's last wave
+    if (idle) return;
     const SelectState s = load_state(b.seg + (size_t)i * t.nseg + seg);
-    select_segment<NT>(sh, t, b, si, i, seg, s, deliver != 0);
+    select_segment<NT>(grp, sh, t, b, si, i, seg, s, deliver != 0, defer != 0 && !alone);
+}
+
+// Emission of long lists that topk_select has found the threshold of: `parts` CTAs stream through each list, the winners
+// take message slots warp by warp, the threshold bin's entries are collected, and the CTA that comes last ranks them
+// and closes the segment. Bound by memory: 8 bytes read per candidate, 8 written per message entry and 8 per delivery.
+__global__ void __launch_bounds__(kThreads) topk_emit_kernel(const __grid_constant__ Tables t, const __grid_constant__ TopkBuffers b,
+                                                             const int32_t* __restrict__ seg_list, int nlong, int parts,
+                                                             int deliver) {
+    __shared__ uint2 surv[kSurvCap], few[kSurvCap];
+    __shared__ uint32_t hist[kThreads], scratch[kWarps], sh_bin[2], sh_above, sh_in;
+    __shared__ int is_last;
+    // all lists' first parts first: the workers' entries of one coordinate range then reach its bucket close in time
+    const unsigned lists = (unsigned)(t.n * nlong), item = blockIdx.x % lists, part = blockIdx.x / lists;
+    const int i = (int)(item % (unsigned)t.n);
+    const int seg = seg_list[item / (unsigned)t.n];
+    const SegInfo si = t.segs[seg];
+    const SelectJob job = select_job(t, b, si, i, deliver != 0);
+    dependency_wait();
+    allow_dependents();
+    const size_t sg = (size_t)i * t.nseg + seg;
+    SegState* st = b.seg + sg;
+    const uint32_t c = st->emit_n;
+    if (c == 0u) return;  // decided otherwise (the same word for every part: it changes when the last one is done)
+    const uint32_t win_from = st->emit_from, bin_from = st->prefix;
+    uint2* gsurv = b.sel_surv + (size_t)item * kSurvCap;
+    uint32_t* nsurv = b.sel_ticket + 2 * item;
+    ListSlice sl;
+    sl.list = b.cand + (size_t)i * (size_t)b.cand_total + (size_t)si.cand_off;
+    sl.lo = 0u;
+    sl.hi = c;
+    for (uint32_t p0 = part * (ListSlice::kU * kThreads); p0 < c; p0 += (uint32_t)parts * (ListSlice::kU * kThreads)) {
+        uint2 cv[ListSlice::kU];
+        sl.load<kThreads>(p0, cv);
+#pragma unroll
+        for (int h = 0; h < ListSlice::kU; h += 4)
+            emit<4>(b, job, 0u, &st->emit_count, gsurv, nsurv, cv + h, win_from, bin_from);
+    }
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) is_last = atomicAdd(nsurv + 1, 1u) == (uint32_t)(parts - 1);
+    __syncthreads();
+    if (!is_last) return;
+    __threadfence();
+    uint32_t k_rem = st->k_rem, count = k_rem ? __ldcg(nsurv) : 0u;
+    const uint32_t wins = job.kb - k_rem;
+    for (uint32_t q = threadIdx.x; q < count; q += kThreads) surv[q] = __ldcg(gsurv + q);
+    if (threadIdx.x == 0) sh_bin[0] = sh_bin[1] = sh_above = sh_in = 0u;
+    hist[threadIdx.x] = 0u;
+    __syncthreads();
+    const uint2* last = surv;
+    if (count > 64u) {
+        // too many for one CTA to rank one against the other: a histogram of 256 bins leaves the few that share a bin
+        static_assert(kThreads == 256, "one histogram bin per thread");
+        const uint32_t width = win_from - bin_from;
+        const int s = width > 256u ? 24 - __clz(width - 1u) : 0;
+        for (uint32_t q = threadIdx.x; q < count; q += kThreads) atomicAdd(&hist[((surv[q].y & 0x7fffffffu) - bin_from) >> s], 1u);
+        __syncthreads();
+        const uint32_t in = hist[255 - threadIdx.x];  // from the top bin down
+        uint32_t total;
+        const uint32_t incl = block_inclusive_scan(in, scratch, &total);
+        if (incl - in < k_rem && k_rem <= incl) {
+            sh_bin[0] = 255u - threadIdx.x;
+            sh_bin[1] = incl - in;
+        }
+        __syncthreads();
+        for (uint32_t q = threadIdx.x; q < count; q += kThreads) {
+            const uint2 cv = surv[q];
+            const uint32_t dg = ((cv.y & 0x7fffffffu) - bin_from) >> s;
+            if (dg > sh_bin[0]) {
+                put_pair(b, job, wins + atomicAdd(&sh_above, 1u), cv.x, cv.y);
+                if (job.deliver) scatter_one(b, (int32_t)cv.x, cv.y);
+                job.erow[cv.x] = 0.0f;  // the residual of a kept coordinate: e = x - x
+            } else if (dg == sh_bin[0]) {
+                few[atomicAdd(&sh_in, 1u)] = cv;
+            }
+        }
+        __syncthreads();
+        k_rem -= sh_bin[1];
+        count = sh_in;
+        last = few;
+    }
+    uint32_t tau = bin_from;
+    bool closer = threadIdx.x == 0 && wins == job.kb;
+    if (wins != job.kb) closer = rank_survivors(b, job, last, count, k_rem, threadIdx.x >> 5, kWarps, &tau);
+    if (closer) {
+        if (__ldcg(&st->emit_count) != wins) atomicOr(b.status, 1u);
+        st->emit_n = 0u;
+        nsurv[0] = 0u;
+        nsurv[1] = 0u;
+        close_list(b, job, st, b.thr + sg, wins != job.kb ? tau + 1u : win_from, tau, st->edge, c, st->tau_hat);
+    }
 }
 
 // ------------------------------------------------------------------------------------------
@@ -878,15 +992,19 @@ static cudaError_t allow_large_cluster(K* kernel, int cluster) {
 }
 
 cudaError_t launch_topk_select(compams_context* c) {
-    for (const compams_context::SegGroup& g : c->select_groups) {
-        const dim3 grid((unsigned)((int64_t)c->n * g.count * g.cluster));
-        cudaError_t e = allow_large_cluster(topk_select_kernel<kSelThreads>, g.cluster);
-        if (e != cudaSuccess) return e;
-        e = counted(c, launch_cluster(topk_select_kernel<kSelThreads>, grid, dim3(kSelThreads), g.cluster, c->chain, c->stream, c->tab,
-                                      own_rows(c), (const int32_t*)g.segs, c->deliver ? 1 : 0));
-        if (e != cudaSuccess) return e;
-    }
-    return cudaSuccess;
+    const int64_t clusters = (int64_t)c->n * c->sel_long + ((int64_t)c->n * c->sel_short + c->sel_cluster - 1) / c->sel_cluster;
+    cudaError_t e = allow_large_cluster(topk_select_kernel<kSelThreads>, c->sel_cluster);
+    if (e != cudaSuccess) return e;
+    e = counted(c, launch_cluster(topk_select_kernel<kSelThreads>, dim3((unsigned)(clusters * c->sel_cluster)), dim3(kSelThreads),
+                                  c->sel_cluster, c->chain, c->stream, c->tab, own_rows(c), (const int32_t*)c->sel_segs, c->sel_long,
+                                  c->sel_short, c->deliver ? 1 : 0, c->sel_parts ? 1 : 0));
+    if (e != cudaSuccess || !c->sel_parts) return e;
+    const dim3 grid((unsigned)((int64_t)c->n * c->sel_long * c->sel_parts));
+    if (c->chain)
+        return counted(c, launch_after(topk_emit_kernel, grid, dim3(kThreads), c->stream, c->tab, own_rows(c),
+                                       (const int32_t*)c->sel_segs, c->sel_long, c->sel_parts, c->deliver ? 1 : 0));
+    topk_emit_kernel<<<grid, kThreads, 0, c->stream>>>(c->tab, own_rows(c), c->sel_segs, c->sel_long, c->sel_parts, c->deliver ? 1 : 0);
+    return counted(c, cudaGetLastError());
 }
 
 cudaError_t launch_topk_dense(compams_context* c) {
