@@ -82,21 +82,8 @@ int64_t kept_per_block(double k_ratio, int64_t d_b) {
     return k;
 }
 
-#ifndef SEL_CMAX
-#define SEL_CMAX 16
-#endif
-#ifndef SEL_PER
-#define SEL_PER 1
-#endif
-#ifndef SEL_LONG
-#define SEL_LONG 4096
-#endif
 constexpr int64_t kClusterMax = (int64_t)1 << 21;  // coordinates per CTA that a cluster goes through itself
 constexpr int64_t kListless = (int64_t)1 << 18;    // ... of a block that never has a list
-
-#ifndef DEFER_MIN
-#define DEFER_MIN 8
-#endif
 
 // Decides which kernels select from which blocks, and with how many CTAs.
 int group_segments(compams_context* c, const std::vector<SegInfo>& segs) {
@@ -106,13 +93,37 @@ int group_segments(compams_context* c, const std::vector<SegInfo>& segs) {
     c->dense_kernel = false;
     c->seg_always_dense.assign(segs.size(), false);
     if (c->randk) return COMPAMS_OK;
-    // Long candidate lists get a cluster of CTAs each while there are too few of them to fill the GPU with one CTA per
-    // list; the others one CTA.
-    std::vector<int32_t> few, many;  // blocks for one CTA, for a cluster of them
+    // Long candidate lists get a cluster of CTAs each, the others one CTA. Which are long, and how many CTAs they get, is
+    // what makes the estimate of the kernel's time least: the longest CTA, or all CTAs over 1.5 per SM. In entries, a CTA
+    // costs its share and about a round of 4096 for its fixed latencies, half a round more for the cluster's barriers.
+    // More than one cluster of 16 per 16 SMs does not fit the GPCs at once (ResNet-18 shapes whole, n = 16, 1 %, bfloat16:
+    // 394 us with 16 CTAs per list, 377 with 8), more than two CTAs per SM wait for others.
     auto expected = [&](const SegInfo& si) { return (int64_t)si.kb + si.kb / 4; };
-    for (size_t s = 0; s < segs.size(); ++s) (expected(segs[s]) < SEL_LONG ? few : many).push_back((int32_t)s);
     int cluster = 1;
-    while (cluster < SEL_CMAX && (int64_t)many.size() * c->n * cluster * 2 <= SEL_PER * (int64_t)c->num_sms) cluster *= 2;
+    int64_t from = INT64_MAX;  // lists are long from here on
+    double best = 1e300;
+    for (int c16 = 1; c16 <= 16; c16 *= 2) {
+        for (int64_t th = 4096; th <= ((int64_t)1 << 20); th *= 2) {
+            double longest = 0.0, total = 0.0;
+            int64_t longs = 0;
+            for (const SegInfo& si : segs) {
+                const bool is_long = c16 > 1 && expected(si) >= th;
+                const double cost = is_long ? (double)expected(si) / c16 + 6144.0 : (double)expected(si) + 4096.0;
+                longest = std::max(longest, cost);
+                total += cost * (is_long ? c16 : 1) * c->n;
+                longs += is_long ? c->n : 0;
+            }
+            if (longs * c16 > (c16 == 16 ? 1 : 2) * (int64_t)c->num_sms) continue;
+            const double cost = std::max(longest, total / (1.5 * c->num_sms));
+            if (cost < 0.98 * best) {
+                best = cost;
+                cluster = longs ? c16 : 1;
+                from = longs ? th : INT64_MAX;
+            }
+        }
+    }
+    std::vector<int32_t> few, many;  // blocks for one CTA, for a cluster of them
+    for (size_t s = 0; s < segs.size(); ++s) (expected(segs[s]) < from ? few : many).push_back((int32_t)s);
     int64_t entries = 0;
     for (std::vector<int32_t>* l : {&few, &many}) {
         const int64_t ctas = l == &few ? 1 : cluster;
@@ -134,8 +145,10 @@ int group_segments(compams_context* c, const std::vector<SegInfo>& segs) {
     c->sel_long = (int)many.size();
     c->sel_short = (int)few.size();
     c->sel_cluster = cluster;
-    // lists that their clusters would have to go through in many rounds are emitted by a kernel of its own
-    if (c->sel_long && entries >= (int64_t)DEFER_MIN * cluster * 4096) {
+    // Lists that their clusters would have to go through in many rounds are emitted by a kernel of its own: from three
+    // rounds on where the clusters leave SMs idle (n = 2, d = 4.4 M, 7.85 % kept: 119 us by the cluster, 95 by topk_emit), from eight
+    // where they do not (ResNet-18 shapes whole, n = 16, 1 %: 4.3 rounds, 386 against 398 us)
+    if (c->sel_long && entries >= (cluster == 16 ? 3 : 8) * (int64_t)cluster * 4096) {
         const int64_t lists = (int64_t)c->n * c->sel_long;
         c->sel_parts = (int)((entries + 2047) / 2048);
         RC(dev_alloc(c, &c->tk.sel_ticket, (size_t)lists * 2));

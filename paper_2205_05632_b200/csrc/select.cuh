@@ -286,17 +286,20 @@ __device__ __forceinline__ bool select_slices(const Group& grp, const TopkBuffer
                                               const Slice& sl, uint32_t from, int S, bool open, uint32_t want, bool refine_edge,
                                               Selected& out) {
     constexpr int U = Slice::kU;
-    constexpr bool kHold = !Slice::kOrdered;  // the first round's entries stay in registers for the emission
+    constexpr bool kHold = !Slice::kOrdered;  // a slice of one round stays in registers from the count to the emission
     const unsigned C = grp.size, rank = grp.rank;
     const int lane = threadIdx.x & 31;
     uint2 held[U];
-    if constexpr (kHold) sl.template load<NT>(sl.lo, held);
+    const bool one_round = sl.hi - sl.lo <= (uint32_t)(U * NT);
+    if (kHold && one_round) sl.template load<NT>(sl.lo, held);
     auto count = [&](uint32_t base, int s, uint32_t width, bool clip) {  // entries with keys in [base, base + width)
+        if (kHold && !one_round) sl.template load<NT>(sl.lo, held);
         for (uint32_t p0 = sl.lo; p0 < sl.hi; p0 += U * NT) {
             uint2 cv[U];
-            if (kHold && p0 == sl.lo) {
+            if constexpr (kHold) {  // the next round is requested before this one is worked on
 #pragma unroll
                 for (int u = 0; u < U; ++u) cv[u] = held[u];
+                if (p0 + U * NT < sl.hi) sl.template load<NT>(p0 + U * NT, held);
             } else {
                 sl.template load<NT>(p0, cv);
             }
@@ -384,7 +387,7 @@ __device__ __forceinline__ bool select_slices(const Group& grp, const TopkBuffer
     uint2* surv = grp.of(sh.surv, 0);
     uint32_t* nsurv = grp.of(&sh.nsurv, 0);
     for (uint32_t p0 = sl.lo; p0 < sl.hi; p0 += U * NT) {
-        if (!kHold || p0 != sl.lo) sl.template load<NT>(p0, held);
+        if (!kHold || !one_round) sl.template load<NT>(p0, held);
 #pragma unroll
         for (int h = 0; h < U; h += 4) emit<4>(b, job, sh.base, &sh.winners, surv, nsurv, held + h, win_from, by_index ? win_from : from);
     }
