@@ -235,7 +235,7 @@ __device__ __forceinline__ bool rank_survivors(const TopkBuffers& b, const Selec
 }
 
 // A slice of a candidate list: (coordinate, bits) pairs in any order, but those of one coordinate range mostly together.
-// Every warp reads 32 kU consecutive ones, from the L2: other CTAs of the cluster may have written them.
+// A warp reads 32 consecutive ones at a time, all warps take part in a short list.
 struct ListSlice {
     static constexpr int kU = 8;
     static constexpr bool kOrdered = false;
@@ -243,10 +243,9 @@ struct ListSlice {
     uint32_t lo, hi;
     template <int NT>
     __device__ __forceinline__ void load(uint32_t p0, uint2 (&cv)[kU]) const {
-        const uint32_t first = p0 + (threadIdx.x >> 5) * (32 * kU) + (threadIdx.x & 31);
 #pragma unroll
         for (int u = 0; u < kU; ++u) {
-            const uint32_t p = first + u * 32;
+            const uint32_t p = p0 + u * NT + threadIdx.x;
             cv[u] = p < hi ? __ldcg(list + p) : make_uint2(0u, kNoCandidate);
         }
     }
