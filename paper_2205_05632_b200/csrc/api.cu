@@ -82,8 +82,26 @@ int64_t kept_per_block(double k_ratio, int64_t d_b) {
     return k;
 }
 
+constexpr int64_t kPlanSms = 148;              // SMs that the choices below count on (a plan is made without a device)
+constexpr int64_t kFusedRound = 8192;          // coordinates one CTA of the fused sweep and selection has in flight
+constexpr int64_t kListlessFused = 2048;       // blocks up to this size are always selected from directly there
 constexpr int64_t kClusterMax = (int64_t)1 << 21;  // coordinates per CTA that a cluster goes through itself
 constexpr int64_t kListless = (int64_t)1 << 18;    // ... of a block that never has a list
+
+// CTAs per long block when sweep and selection are one kernel, 0 when they are not. It pays where no CTA needs more than
+// one round of loads for its share and no two share an SM: n = 4, d = 65,536 15.9 -> 15.3 us, n = 3, d = 111,947 in 78
+// blocks 24.2 -> 18.4; but n = 1, d = 2^20 (16 CTAs, eight rounds) 25.7 -> 38.7, n = 32, d = 65,536 (256 CTAs) 17.8 -> 21.3.
+int fused_cluster(const compams_context* c) {
+    int64_t longest = 0, longs = 0, shorts = 0;
+    for (int32_t b = 0; b < c->M; ++b) {
+        const int64_t len = c->off[(size_t)b + 1] - c->off[(size_t)b];
+        longest = std::max(longest, len);
+        (len > kFusedRound ? longs : shorts) += c->n;
+    }
+    int64_t cluster = 1;
+    while (cluster * kFusedRound < longest) cluster *= 2;
+    return cluster <= 16 && longs * cluster <= kPlanSms && shorts <= 2 * kPlanSms ? (int)cluster : 0;
+}
 
 // Decides which kernels select from which blocks, and with how many CTAs.
 int group_segments(compams_context* c, const std::vector<SegInfo>& segs) {
@@ -93,6 +111,17 @@ int group_segments(compams_context* c, const std::vector<SegInfo>& segs) {
     c->dense_kernel = false;
     c->seg_always_dense.assign(segs.size(), false);
     if (c->randk) return COMPAMS_OK;
+    if (c->fused) {
+        std::vector<int32_t> one, several;
+        for (size_t s = 0; s < segs.size(); ++s) (segs[s].len <= kFusedRound ? one : several).push_back((int32_t)s);
+        c->sel_cluster = fused_cluster(c);
+        std::stable_sort(several.begin(), several.end(), [&](int32_t a, int32_t b) { return segs[(size_t)a].len > segs[(size_t)b].len; });
+        c->tk.cluster_max = INT32_MAX;  // the dense passes are never launched
+        c->sel_long = (int)several.size();
+        c->sel_short = (int)one.size();
+        several.insert(several.end(), one.begin(), one.end());
+        return dev_upload(c, &c->sel_segs, several);
+    }
     // Long candidate lists get a cluster of CTAs each, the others one CTA. Which are long, and how many CTAs they get, is
     // what makes the estimate of the kernel's time least: the longest CTA, or all CTAs over 1.5 per SM. In entries, a CTA
     // costs its share and about a round of 4096 for its fixed latencies, half a round more for the cluster's barriers.
@@ -113,8 +142,8 @@ int group_segments(compams_context* c, const std::vector<SegInfo>& segs) {
                 total += cost * (is_long ? c16 : 1) * c->n;
                 longs += is_long ? c->n : 0;
             }
-            if (longs * c16 > (c16 == 16 ? 1 : 2) * (int64_t)c->num_sms) continue;
-            const double cost = std::max(longest, total / (1.5 * c->num_sms));
+            if (longs * c16 > (c16 == 16 ? 1 : 2) * kPlanSms) continue;
+            const double cost = std::max(longest, total / (1.5 * kPlanSms));
             if (cost < 0.98 * best) {
                 best = cost;
                 cluster = longs ? c16 : 1;
@@ -186,6 +215,7 @@ int build_tiles(compams_context* c, const std::vector<int32_t>& blocks, bool top
             si.kb = (uint32_t)kb;
             // the candidate path pays off for sparse selections only: at most 1/9 of the block kept
             int64_t cap = (!c->randk && kb * 9 <= len) ? 8 * kb + 1024 : 0;
+            if (c->fused && len <= kListlessFused) cap = 0;
             if (cap) cap = std::min(cap, len <= 65536 ? len : len / 4 + kb);
             cap = (cap + 1) & ~(int64_t)1;  // lists are read in 128-bit pairs
             si.cap = (uint32_t)cap;
@@ -270,10 +300,11 @@ int init_context(compams_context* c, const int64_t* block_offsets) {
     } else if (c->sparse()) {
         RC(dev_alloc(c, &c->E, (size_t)n * (size_t)d));
         RC(dev_upload(c, &c->d_seg_off, c->seg_off));
+        c->fused = !c->randk && fused_cluster(c) > 0;
         std::vector<int32_t> small, large;
         // (Random-k has no selection: every block is tiled for the sweep, none goes to the shared-memory select)
         for (int32_t b = 0; b < M; ++b)
-            ((!c->randk && c->off[b + 1] - c->off[b] <= kSmallMax) ? small : large).push_back(b);
+            ((!c->randk && !c->fused && c->off[b + 1] - c->off[b] <= kSmallMax) ? small : large).push_back(b);
         RC(build_tiles(c, large, true));
         TopkBuffers& t = c->tk;
         t.E = c->E;
@@ -417,9 +448,14 @@ int compress_device(compams_context* c, const void* grads) {
         RC(run_kernel(c, COMPAMS_K_RANDK_EMIT, [&] { return launch_randk_emit(c, c->n == c->n_total); }));
         return COMPAMS_OK;
     }
+    if (c->fused) {
+        RC(run_kernel(c, COMPAMS_K_TOPK_SELECT, [&] { return launch_topk_fused(c, grads); }));
+        c->e_mask_pending = true;
+        return COMPAMS_OK;
+    }
+    if (c->tab.ntiles > 0) RC(run_kernel(c, COMPAMS_K_TOPK_SWEEP, [&] { return launch_topk_sweep(c, grads); }));
     if (c->tk.nsmall > 0) RC(run_kernel(c, COMPAMS_K_TOPK_SMALL, [&] { return launch_topk_small(c, grads); }));
     if (c->tab.ntiles > 0) {
-        RC(run_kernel(c, COMPAMS_K_TOPK_SWEEP, [&] { return launch_topk_sweep(c, grads); }));
         if (c->sel_long + c->sel_short > 0) RC(run_kernel(c, COMPAMS_K_TOPK_SELECT, [&] { return launch_topk_select(c); }));
         if (c->dense_kernel) RC(run_kernel(c, COMPAMS_K_TOPK_DENSE, [&] { return launch_topk_dense(c); }));
         c->e_mask_pending = true;

@@ -109,6 +109,9 @@ __device__ __forceinline__ int align_class(const bf16_bits* p) { return (int)((r
 __device__ __forceinline__ float widen(bf16_bits h) { return __uint_as_float((uint32_t)h << 16); }
 __device__ __forceinline__ float load1_stream(const float* p) { return __ldg(p); }
 __device__ __forceinline__ float load1_stream(const bf16_bits* p) { return widen(__ldg(p)); }
+// One element from the L2, for kernels that may start beside the one before them.
+__device__ __forceinline__ float load1_l2(const float* p) { return __ldcg(p); }
+__device__ __forceinline__ float load1_l2(const bf16_bits* p) { return widen(__ldcg(p)); }
 __device__ __forceinline__ float4 load4_stream(const bf16_bits* p, int cls) {
     uint32_t lo, hi;
     if (cls == 0) {

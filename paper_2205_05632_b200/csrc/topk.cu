@@ -395,6 +395,125 @@ __global__ void __launch_bounds__(NT, SEL_CTAS) topk_select_kernel(const __grid_
     select_segment<NT>(grp, sh, t, b, si, i, seg, s, deliver != 0, defer != 0 && !alone);
 }
 
+// Sweep and selection in one kernel, for problems so small that launches and latency are what a step costs: a cluster, or one CTA, takes one (worker, block), forms x = g + e, lists the candidates and selects
+// among them; blocks without a list are selected from directly. A warp takes 512 coordinates at a time, all loads of such
+// a stretch in flight together, and its candidates get their places with one atomic.
+constexpr int kSpan = 512;
+
+template <bool FULL, typename GT>
+__device__ __forceinline__ void fused_span(const GT* __restrict__ g, float* __restrict__ e, int len, int r0, int lane, uint32_t tau_hat,
+                                           float kept_from, uint32_t coord0, uint32_t* listed, uint2* out, uint32_t cap) {
+    constexpr int NI = kSpan / 128;
+    const int cg_ = align_class(g + r0), ce = align_class(e + r0);
+    float4 gv[NI], x[NI];
+#pragma unroll
+    for (int u = 0; u < NI; ++u) {
+        const int r = r0 + u * 128 + lane * 4;
+        if (FULL || (r >= 0 && r + 3 < len)) {
+            gv[u] = load4_stream(g + r, cg_);
+            x[u] = load4(e + r, ce);
+        } else {
+            float gt[4], et[4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const bool live = (unsigned)(r + k) < (unsigned)len;
+                gt[k] = live ? load1_stream(g + r + k) : 0.0f;
+                et[k] = live ? e[r + k] : 0.0f;
+            }
+            gv[u] = make_float4(gt[0], gt[1], gt[2], gt[3]);
+            x[u] = make_float4(et[0], et[1], et[2], et[3]);
+        }
+    }
+    // coordinates kept in the last step still hold x in E: their e is 0 (Algorithm 2, the residual update)
+    auto corrected = [&](float gk, float eo) { return __fadd_rn(gk, fabsf(eo) >= kept_from ? 0.0f : eo); };
+    auto is = [&](int u, int k) {
+        const int r = r0 + u * 128 + lane * 4 + k;
+        return (FULL || (unsigned)r < (unsigned)len) && mag_key(lane_elem(x[u], k)) >= tau_hat;
+    };
+    uint32_t total = 0;
+#pragma unroll
+    for (int u = 0; u < NI; ++u) {
+        const int r = r0 + u * 128 + lane * 4;
+        x[u] = make_float4(corrected(gv[u].x, x[u].x), corrected(gv[u].y, x[u].y), corrected(gv[u].z, x[u].z),
+                           corrected(gv[u].w, x[u].w));  // the corrected-gradient step: x = g + e
+        if (FULL || (r >= 0 && r + 3 < len)) {
+            store4(e + r, ce, x[u]);
+        } else {
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+                if ((unsigned)(r + k) < (unsigned)len) e[r + k] = lane_elem(x[u], k);
+        }
+#pragma unroll
+        for (int k = 0; k < 4; ++k) total += (uint32_t)__popc(__ballot_sync(0xffffffffu, is(u, k)));
+    }
+    if (total == 0u) return;
+    uint32_t base = 0;
+    if (lane == 0) base = atomicAdd(listed, total);
+    base = __shfl_sync(0xffffffffu, base, 0);
+#pragma unroll
+    for (int u = 0; u < NI; ++u) {
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const bool c = is(u, k);
+            const unsigned m = __ballot_sync(0xffffffffu, c);
+            const uint32_t p = base + (uint32_t)__popc(m & ((1u << lane) - 1u));
+            if (c && p < cap) out[p] = make_uint2(coord0 + (uint32_t)(r0 + u * 128 + lane * 4 + k), __float_as_uint(lane_elem(x[u], k)));
+            base += (uint32_t)__popc(m);
+        }
+    }
+}
+
+template <typename GT>
+__global__ void __launch_bounds__(kSelThreads, SEL_CTAS) topk_fused_kernel(const __grid_constant__ Tables t,
+                                                                           const __grid_constant__ TopkBuffers b,
+                                                                           const GT* __restrict__ G,
+                                                                           const int32_t* __restrict__ seg_list, int nlong, int nshort,
+                                                                           int deliver) {
+    constexpr int NT = kSelThreads;
+    __shared__ SelectShared<NT> sh;
+    Group grp{cg::this_cluster().num_blocks(), cg::this_cluster().block_rank()};
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    unsigned item = blockIdx.x / grp.size;
+    const unsigned longs = (unsigned)(t.n * nlong);
+    const int32_t* segs = seg_list;
+    const bool alone = item >= longs;
+    if (alone) {
+        item = (item - longs) * grp.size + grp.rank;
+        segs += nlong;
+        grp = Group{1u, 0u};
+    }
+    const int i = (int)(item % (unsigned)t.n);
+    const unsigned q = item / (unsigned)t.n;
+    const bool idle = alone && q >= (unsigned)nshort;
+    const int seg = segs[idle ? 0u : q];  // the block tables are never written by a kernel
+    const SegInfo si = t.segs[seg];
+    const size_t sg = (size_t)i * t.nseg + seg;
+    start_select<NT>(sh);
+    dependency_wait();
+    allow_dependents();
+    if (idle) return;
+    SelectState s = load_state(b.seg + sg);
+    const float kept_from = __uint_as_float(b.use_thr ? b.thr[sg] : kNothingKept);
+    const int64_t row0 = (int64_t)i * t.d + si.o;
+    const GT* g = G + row0;
+    float* e = b.E + row0;
+    uint2* out = b.cand + (size_t)i * (size_t)b.cand_total + (size_t)si.cand_off;
+    grp.sync();  // the first CTA's counter is clear
+    uint32_t* listed = grp.of(&sh.listed, 0);
+    const int shift = (int)(row0 & 31);  // stretches start on 128-byte lines of G and E, as the sweep's tiles do
+    const int spans = (si.len + shift + kSpan - 1) / kSpan;
+    for (int u = warp * (int)grp.size + (int)grp.rank; u < spans; u += (int)grp.size * (NT / 32)) {
+        const int r0 = u * kSpan - shift;
+        if (r0 >= 0 && r0 + kSpan <= si.len)
+            fused_span<true>(g, e, si.len, r0, lane, s.tau_hat, kept_from, (uint32_t)si.o, listed, out, si.cap);
+        else
+            fused_span<false>(g, e, si.len, r0, lane, s.tau_hat, kept_from, (uint32_t)si.o, listed, out, si.cap);
+    }
+    grp.sync();  // the list and x are complete
+    s.c = *listed;
+    select_segment<NT>(grp, sh, t, b, si, i, seg, s, deliver != 0, false);
+}
+
 // Emission of long lists that topk_select has found the threshold of: `parts` CTAs stream through each list, the winners
 // take message slots warp by warp, the threshold bin's entries are collected, and the CTA that comes last ranks them
 // and closes the segment. Bound by memory: 8 bytes read per candidate, 8 written per message entry and 8 per delivery.
@@ -825,11 +944,16 @@ __global__ void __launch_bounds__(kThreads) topk_dense_kernel(Tables t, TopkBuff
 // small blocks: the whole selection inside one CTA's shared memory
 
 template <typename GT>
-__global__ void __launch_bounds__(kThreads) topk_small_kernel(Tables t, TopkBuffers b, const GT* __restrict__ G, int deliver) {
+__global__ void __launch_bounds__(kThreads) topk_small_kernel(Tables t, TopkBuffers b, const GT* __restrict__ G, int deliver,
+                                                              int after_sweep) {
     __shared__ uint32_t xs[kSmallMax];
     __shared__ uint32_t hist[256];
     __shared__ uint32_t scratch[kWarps];
     __shared__ uint32_t sh_prefix, sh_krem, sh_cnt, sh_rlast;
+    // Shares no block with the sweep before it: its CTAs move in behind the sweep's last wave, which has ordered itself
+    // after everything earlier on the stream, and wait for the sweep only at their end, for the sake of the kernel after.
+    if (!after_sweep) dependency_wait();
+    allow_dependents();
     const int blk = b.small_blk[blockIdx.x];
     const int i = blockIdx.y;
     const int64_t o = t.off[blk];
@@ -837,7 +961,7 @@ __global__ void __launch_bounds__(kThreads) topk_small_kernel(Tables t, TopkBuff
     const uint32_t kb = (uint32_t)(b.seg_off[blk + 1] - b.seg_off[blk]);
     const GT* g = G + (size_t)i * (size_t)t.d + (size_t)o;
     float* e = b.E + (size_t)i * (size_t)t.d + (size_t)o;
-    for (int r = threadIdx.x; r < len; r += kThreads) xs[r] = __float_as_uint(__fadd_rn(load1_stream(g + r), e[r]));
+    for (int r = threadIdx.x; r < len; r += kThreads) xs[r] = __float_as_uint(__fadd_rn(load1_l2(g + r), __ldcg(e + r)));
 
     // radix select over the 31-bit key: digits of 8, 8, 8 and 7 bits from the top
     uint32_t prefix = 0, k_rem = kb;
@@ -912,6 +1036,7 @@ __global__ void __launch_bounds__(kThreads) topk_small_kernel(Tables t, TopkBuff
     if (threadIdx.x == 0 && total != kb) atomicOr(b.status, 1u);
     // Algorithm 2, the residual update: e = x - g~ (0 where kept, x elsewhere)
     for (int r = threadIdx.x; r < len; r += kThreads) e[r] = kept(r) ? 0.0f : __uint_as_float(xs[r]);
+    if (after_sweep) dependency_wait();
 }
 
 // ------------------------------------------------------------------------------------------
@@ -957,14 +1082,15 @@ static TopkBuffers own_rows(const compams_context* c) {
     return b;
 }
 
+template <typename GT>
+static cudaError_t launch_small_typed(compams_context* c, const GT* grads) {
+    const dim3 grid((unsigned)c->tk.nsmall, (unsigned)c->n);
+    return counted(c, launch_after(topk_small_kernel<GT>, grid, dim3(kThreads), c->stream, c->tab, own_rows(c), grads,
+                                   c->deliver ? 1 : 0, c->tab.ntiles > 0 ? 1 : 0));
+}
+
 cudaError_t launch_topk_small(compams_context* c, const void* grads) {
-    dim3 grid((unsigned)c->tk.nsmall, (unsigned)c->n);
-    if (c->grad_bf16)
-        topk_small_kernel<bf16_bits><<<grid, kThreads, 0, c->stream>>>(c->tab, own_rows(c), (const bf16_bits*)grads,
-                                                                    c->deliver ? 1 : 0);
-    else
-        topk_small_kernel<float><<<grid, kThreads, 0, c->stream>>>(c->tab, own_rows(c), (const float*)grads, c->deliver ? 1 : 0);
-    return counted(c, cudaGetLastError());
+    return c->grad_bf16 ? launch_small_typed(c, (const bf16_bits*)grads) : launch_small_typed(c, (const float*)grads);
 }
 
 template <typename GT>
@@ -1005,6 +1131,20 @@ cudaError_t launch_topk_select(compams_context* c) {
                                        (const int32_t*)c->sel_segs, c->sel_long, c->sel_parts, c->deliver ? 1 : 0));
     topk_emit_kernel<<<grid, kThreads, 0, c->stream>>>(c->tab, own_rows(c), c->sel_segs, c->sel_long, c->sel_parts, c->deliver ? 1 : 0);
     return counted(c, cudaGetLastError());
+}
+
+template <typename GT>
+static cudaError_t launch_fused_typed(compams_context* c, const GT* grads) {
+    const int64_t clusters = (int64_t)c->n * c->sel_long + ((int64_t)c->n * c->sel_short + c->sel_cluster - 1) / c->sel_cluster;
+    const cudaError_t e = allow_large_cluster(topk_fused_kernel<GT>, c->sel_cluster);
+    if (e != cudaSuccess) return e;
+    return counted(c, launch_cluster(topk_fused_kernel<GT>, dim3((unsigned)(clusters * c->sel_cluster)), dim3(kSelThreads), c->sel_cluster,
+                                     true, c->stream, c->tab, own_rows(c), grads, (const int32_t*)c->sel_segs, c->sel_long, c->sel_short,
+                                     c->deliver ? 1 : 0));
+}
+
+cudaError_t launch_topk_fused(compams_context* c, const void* grads) {
+    return c->grad_bf16 ? launch_fused_typed(c, (const bf16_bits*)grads) : launch_fused_typed(c, (const float*)grads);
 }
 
 cudaError_t launch_topk_dense(compams_context* c) {
