@@ -85,7 +85,10 @@ int64_t kept_per_block(double k_ratio, int64_t d_b) {
 constexpr int64_t kPlanSms = 148;              // SMs that the choices below count on (a plan is made without a device)
 constexpr int64_t kFusedRound = 8192;          // coordinates one CTA of the fused sweep and selection has in flight
 constexpr int64_t kListlessFused = 2048;       // blocks up to this size are always selected from directly there
-constexpr int64_t kClusterMax = (int64_t)1 << 21;  // coordinates per CTA that a cluster goes through itself
+// Coordinates per CTA up to which a cluster goes through a block itself when the list cannot decide. Beyond, the dense
+// passes of the whole GPU are launched every step to stand by: about 4 us, which only matters to short steps (a CTA gets through
+// about 2^16 coordinates in 30 us per pass, and needs five).
+constexpr int64_t kClusterMax = (int64_t)1 << 21, kClusterMaxLongStep = (int64_t)1 << 17;
 constexpr int64_t kListless = (int64_t)1 << 18;    // ... of a block that never has a list
 
 // CTAs per long block when sweep and selection are one kernel, 0 when they are not. It pays where no CTA needs more than
@@ -105,7 +108,8 @@ int fused_cluster(const compams_context* c) {
 
 // Decides which kernels select from which blocks, and with how many CTAs.
 int group_segments(compams_context* c, const std::vector<SegInfo>& segs) {
-    c->tk.cluster_max = (int32_t)kClusterMax;
+    const int64_t cluster_max = (int64_t)c->n * c->tab.d <= kChainMaxElems ? kClusterMax : kClusterMaxLongStep;
+    c->tk.cluster_max = (int32_t)cluster_max;
     c->sel_long = c->sel_short = c->sel_parts = 0;
     c->sel_cluster = 1;
     c->dense_kernel = false;
@@ -158,8 +162,8 @@ int group_segments(compams_context* c, const std::vector<SegInfo>& segs) {
         const int64_t ctas = l == &few ? 1 : cluster;
         std::vector<int32_t> listed;
         for (int32_t s : *l) {
-            if (segs[(size_t)s].len > kClusterMax * ctas) c->dense_kernel = true;
-            if (segs[(size_t)s].cap || segs[(size_t)s].len <= kListless * ctas) {
+            if (segs[(size_t)s].len > cluster_max * ctas) c->dense_kernel = true;
+            if (segs[(size_t)s].cap || segs[(size_t)s].len <= std::min(kListless, cluster_max) * ctas) {
                 listed.push_back(s);
                 if (l == &many && segs[(size_t)s].cap) entries = std::max(entries, expected(segs[(size_t)s]));
             } else {  // always the dense passes

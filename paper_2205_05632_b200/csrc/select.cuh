@@ -251,18 +251,30 @@ struct ListSlice {
     }
 };
 
-// A stretch of the block itself, in index order.
+// A stretch of the block itself, in index order. Positions count from the 16-byte boundary at or before the block's first
+// element, `skip` elements earlier, so that a thread reads 4 consecutive ones at once; lo is a multiple of 4.
 struct BlockSlice {
-    static constexpr int kU = 4;
+    static constexpr int kU = 16;
     static constexpr bool kOrdered = true;
     const float* x;
-    uint32_t lo, hi, coord0;
+    uint32_t lo, hi, skip, coord0;  // coord0: coordinate of position 0
+    __device__ __forceinline__ uint32_t bits(uint32_t r) const {
+        return r >= skip && r < hi ? __float_as_uint(__ldcg(x + r)) : kNoCandidate;
+    }
     template <int NT>
-    __device__ __forceinline__ void load(uint32_t r0, uint2 (&cv)[kU]) const {
+    __device__ __forceinline__ void load(uint32_t p0, uint2 (&cv)[kU]) const {
 #pragma unroll
-        for (int u = 0; u < kU; ++u) {
-            const uint32_t r = r0 + u * NT + threadIdx.x;
-            cv[u] = r < hi ? make_uint2(coord0 + r, __float_as_uint(__ldcg(x + r))) : make_uint2(0u, kNoCandidate);
+        for (int u = 0; u < kU; u += 4) {
+            const uint32_t r = p0 + u * NT + threadIdx.x * 4;
+            float4 v;
+            if (r >= skip && r + 3 < hi) {
+                v = __ldcg(reinterpret_cast<const float4*>(x + r));
+            } else {
+                v = make_float4(__uint_as_float(bits(r)), __uint_as_float(bits(r + 1)), __uint_as_float(bits(r + 2)),
+                                __uint_as_float(bits(r + 3)));
+            }
+#pragma unroll
+            for (int k = 0; k < 4; ++k) cv[u + k] = make_uint2(coord0 + r + k, __float_as_uint(lane_elem(v, k)));
         }
     }
 };
@@ -401,8 +413,8 @@ __device__ __forceinline__ bool select_slices(const Group& grp, const TopkBuffer
             for (unsigned q = 0; q < rank; ++q) before += sh.range[q];
             for (uint32_t r0 = sl.lo; r0 < sl.hi && before < k_rem; r0 += NT) {
                 const uint32_t r = r0 + threadIdx.x;
-                const uint32_t xb = r < sl.hi ? __float_as_uint(__ldcg(sl.x + r)) : kNoCandidate;
-                const bool tie = r < sl.hi && (xb & 0x7fffffffu) == from;
+                const uint32_t xb = sl.bits(r);
+                const bool tie = xb != kNoCandidate && (xb & 0x7fffffffu) == from;
                 uint32_t total;
                 const uint32_t pos = before + scan_cta<NT>(tie ? 1u : 0u, sh.warp_sum, &total) - 1u;
                 if (tie && pos < k_rem) {
@@ -484,10 +496,12 @@ template <int NT>
 __device__ __noinline__ void select_from_block(Group grp, const TopkBuffers& b, SelectJob job, SelectShared<NT>& sh, SegState* st,
                                                uint32_t* thr, const float* x, uint32_t len, uint32_t coord0, bool predicts,
                                                uint32_t boost) {
-    const uint32_t per = (len + grp.size - 1) / grp.size;
     BlockSlice sl;
-    sl.x = x;
-    sl.coord0 = coord0;
+    sl.skip = (uint32_t)align_class(x);
+    sl.x = x - sl.skip;
+    sl.coord0 = coord0 - sl.skip;
+    len += sl.skip;
+    const uint32_t per = ((len + grp.size - 1) / grp.size + 3u) & ~3u;
     sl.lo = grp.rank * per < len ? grp.rank * per : len;
     sl.hi = sl.lo + per < len ? sl.lo + per : len;
     if (threadIdx.x == 0) sh.winners = 0u;
