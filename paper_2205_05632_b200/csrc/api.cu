@@ -387,6 +387,7 @@ int init_context(compams_context* c, const int64_t* block_offsets) {
         RC(dev_alloc(c, &s.tile_sum, (size_t)n * (size_t)c->tab.ntiles));
         RC(dev_alloc(c, &s.edge, (size_t)n * (size_t)c->tab.ntiles));
         s.gbar = nullptr;  // set by compams_record_average
+        s.status = c->status;
         s.m = c->m;
         s.v = c->v;
         s.vhat = c->vhat;

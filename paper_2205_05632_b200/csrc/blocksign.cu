@@ -279,171 +279,181 @@ __global__ void __launch_bounds__(kThreads) bs_materialize_kernel(Tables t, floa
     }
 }
 
-constexpr int kApplyChunk = 32;  // workers whose sign words are staged (and transposed) at a time: one per lane
-#ifndef COMPAMS_APPLY_TABLES_FROM
-#define COMPAMS_APPLY_TABLES_FROM 20
+#ifndef APPLY_CTAS
+#define APPLY_CTAS 4
 #endif
-constexpr int kApplyTablesFrom = COMPAMS_APPLY_TABLES_FROM;  // workers from which the table form of bs_apply is used
+constexpr int kApplyChunk = 16;         // workers whose sign words and scales are staged at a time
+constexpr int kApplySpan = 8 * kThreads;  // coordinates per CTA of bs_apply
 
-// Transposes four 32 x 32 bit matrices held across a warp: on entry lane i holds x[q] = row i of matrix q
-// (bit c = element (i, c)); on return lane c holds column c (bit i = element (i, c)). Five rounds of the
-// usual block swap: in round j a lane exchanges with lane ^ j the half of its bits whose position differs
-// from its own index in bit j. Shifting the partner's word by +-j and keeping only the positions that
-// change is a rotation followed by a bitwise select.
-__device__ __forceinline__ void transpose32x4(uint32_t (&x)[4], int lane) {
-#pragma unroll
-    for (int j = 16; j >= 1; j >>= 1) {
-        const uint32_t m = j == 16 ? 0x0000ffffu : j == 8 ? 0x00ff00ffu : j == 4 ? 0x0f0f0f0fu : j == 2 ? 0x33333333u : 0x55555555u;
-        const bool up = (lane & j) != 0;
-        const uint32_t keep = up ? ~m : m;          // positions whose bit j equals the lane's stay
-        const uint32_t rot = up ? 32u - j : (uint32_t)j;  // the partner's bits move down (up) by j
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            const uint32_t y = __shfl_xor_sync(0xffffffffu, x[q], j);
-            x[q] = (x[q] & keep) | (__funnelshift_l(y, y, rot) & ~keep);
-        }
-    }
+// Transposes an 8 x 8 bit matrix whose rows are the bytes of lo (rows 0-3) and hi (rows 4-7): afterwards bit i of byte k
+// is what bit k of byte i was. Three rounds of the usual block swap.
+__device__ __forceinline__ void transpose8(uint32_t& lo, uint32_t& hi) {
+    uint32_t t;
+    t = (lo ^ (lo >> 7)) & 0x00aa00aau;
+    lo ^= t ^ (t << 7);
+    t = (hi ^ (hi >> 7)) & 0x00aa00aau;
+    hi ^= t ^ (t << 7);
+    t = (lo ^ (lo >> 14)) & 0x0000ccccu;
+    lo ^= t ^ (t << 14);
+    t = (hi ^ (hi >> 14)) & 0x0000ccccu;
+    hi ^= t ^ (t << 14);
+    t = (lo & 0x0f0f0f0fu) | ((hi << 4) & 0xf0f0f0f0u);
+    hi = ((lo >> 4) & 0x0f0f0f0fu) | (hi & 0xf0f0f0f0u);
+    lo = t;
 }
 
-// Server side of Block-Sign (Algorithm 2, the server's average and update): one CTA per 1024 consecutive
-// coordinates of a block, one float4 group per thread. The tile's block comes from the constant bank, so the
-// sign words, the scales and the optimizer state are all requested at once.
+// Shared memory of one bs_apply CTA.
+struct ApplyShared {
+    float state[4][kApplySpan + 4];  // m, v, vhat, theta of the CTA's coordinates, from a 16-byte boundary on
+    union {
+        struct {
+            uint32_t bits[kApplyChunk][kApplySpan / 32];  // [worker][word]
+            double eight[kApplyChunk / 8][256];           // subset sums of 8 workers' scales
+            double four[kApplyChunk / 4][16];             // ... of 4 workers'
+        } sum;
+        float gbar[kApplySpan + 4];
+    };
+    uint64_t arrived;  // mbarrier: the state is there
+};
+
+// Server side of Block-Sign (Algorithm 2, the server's average and update): one CTA per 2048 consecutive coordinates of a
+// block. The tile's block comes from the constant bank, and the optimizer state is on its way to shared memory (four bulk
+// copies) before the kernel in front is done.
 //
-// Per coordinate the sum over workers of +-s_i is (sum of all s_i) - 2 (sum of the s_i whose bit is set).
-// TABLES = false (few workers): one predicated binary64 add per worker and coordinate.
-// TABLES = true: the second sum depends only on the coordinate's pattern of sign bits over the workers, and all
-// 1024 coordinates of the CTA share the workers' scales: for every 4 workers a 16-entry table holds the sum of
-// each subset of their scales (exact in binary64 wherever the plain sum is), and a coordinate adds one table entry
-// per 4 workers instead of testing one bit per worker. The patterns come from transposing the sign words in the
-// warp: lane i reads worker i's four words of the warp's 128 coordinates, transpose32x4 turns them into one word
-// per coordinate, and 16 shuffles hand every lane the patterns of its own 4 coordinates. Up to 32 workers per
-// round. The kernel is bound by instruction issue: the fixed cost of the transposition (36 shuffles per round)
-// pays from about two dozen workers up (n = 32, d = 2^27: step 9.23 -> 8.87 ms; n = 16: no change; n = 8: 3 %
-// slower, hence the two forms).
-template <bool TABLES, bool RECORD>
-__global__ void __launch_bounds__(kThreads, 5) bs_apply_kernel(Tables t, BsBuffers b, float* __restrict__ theta,
-                                                               HyperParams hp,
+// Per coordinate the sum over workers of +-s_i is (sum of all s_i) - 2 (sum of the s_i whose bit is set). The second sum
+// depends only on the coordinate's pattern of sign bits, and all coordinates of the CTA share the workers' scales: for
+// every 8 workers a 256-entry table holds the sum of each subset of their scales (exact in binary64 wherever the plain
+// sum is), and a coordinate adds one entry per 8 workers. A thread's 8 coordinates are one byte of each worker's sign
+// words, so the patterns of 8 workers come from transposing 8 bytes in registers. The averages pass through shared memory,
+// and the update runs over groups of 4 coordinates that start on 16-byte boundaries, whatever the block's offset.
+template <bool RECORD>
+__global__ void __launch_bounds__(kThreads, APPLY_CTAS) bs_apply_kernel(const __grid_constant__ Tables t, const __grid_constant__ BsBuffers b,
+                                                               float* __restrict__ theta, const __grid_constant__ HyperParams hp,
                                                                const __grid_constant__ SegParams sp_) {
-    __shared__ uint32_t sh_bits[kApplyChunk][33];        // [worker][word], rows padded against bank conflicts
-    __shared__ double sh_tab[kApplyChunk / 4][16];       // TABLES: [group of 4 workers][subset] sum of the subset's
-                                                         // scales; else: the workers' scales
-    const int tile = blockIdx.x >> 3;
+    __shared__ __align__(128) ApplyShared sh;
+    const int tile = blockIdx.x / (kTile / kApplySpan);
     const TileInfo ti = sp_.nseg ? find_tile(sp_, tile) : load_tile(t.tiles, tile);
     const int blk = ti.blk;
     const int len = ti.len;
-    const int rs = ti.r0 + (int)(blockIdx.x & 7) * kWarpSpan;  // first coordinate of this CTA, relative to the block
+    const int rs = ti.r0 + (int)(blockIdx.x % (kTile / kApplySpan)) * kApplySpan;  // first coordinate, relative to the block
     if (rs >= len) return;
-    const int r = rs + (int)threadIdx.x * 4;
-    const int64_t o = ti.o;
-    float* gbar = b.gbar + o;
-    float* m = b.m + o;
-    float* v = b.v + o;
-    float* vh = b.vhat + o;
-    float* th = theta + o;
-    const int cls = align_class(m);  // all five vectors are 16-byte aligned at coordinate 0
-    const bool full = r + 3 < len;
-    float4 mm = make_float4(0.f, 0.f, 0.f, 0.f), vv = mm, hh = mm, tt = mm;
-    if (full) {
-        mm = load4(m + r, cls);
-        vv = load4(v + r, cls);
-        hh = load4(vh + r, cls);
-        tt = load4(th + r, cls);
+    const int count = len - rs < kApplySpan ? len - rs : kApplySpan;
+    // coordinates j0 .. j1 - 1; positions in shared memory count from the 16-byte boundary g0 (all four vectors are
+    // 16-byte aligned at coordinate 0); whole groups of 4 lie in [lo, hi)
+    const int64_t j0 = ti.o + rs, g0 = j0 & ~(int64_t)3;
+    const int skip = (int)(j0 - g0), end = skip + count;
+    const int lo = skip ? 4 : 0, hi = end & ~3;
+    float* const vec[4] = {b.m, b.v, b.vhat, theta};
+    const uint32_t bar = (uint32_t)__cvta_generic_to_shared(&sh.arrived);
+    if (threadIdx.x == 0) {
+        const uint32_t bytes = hi > lo ? (uint32_t)(hi - lo) * 4u : 0u;
+        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar) : "memory");
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(4u * bytes) : "memory");
+        if (bytes) {
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+                asm volatile("cp.async.bulk.shared::cta.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
+                                 (uint32_t)__cvta_generic_to_shared(&sh.state[q][lo])),
+                             "l"(vec[q] + g0 + lo), "r"(bytes), "r"(bar)
+                             : "memory");
+        }
     }
-    dependency_wait();  // the state above was last written a step ago; sign words and scales are this step's
+    dependency_wait();  // the state was last written a step ago; sign words and scales are this step's
     const size_t wbase = (size_t)(sp_.nseg ? (int64_t)sp_.wofs[ti.seg] : b.word_off[blk]) + (size_t)(rs >> 5);
-    const int lane = threadIdx.x & 31, wr = threadIdx.x >> 5;  // warp wr owns coordinates 128 wr ... of the CTA's 1024
-    const bool word_live = rs + lane * 32 < len;
-    double a0 = 0.0, a1 = 0.0, a2 = 0.0, a3 = 0.0, all = 0.0;
+    const int lane = threadIdx.x & 31, wr = threadIdx.x >> 5;
+    const int words = (len - rs + 31) >> 5;  // sign words of this CTA's coordinates (possibly more than it has)
+    double a[8] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0}, all = 0.0;
     for (int i0 = 0; i0 < t.n; i0 += kApplyChunk) {
         const int nc = (t.n - i0 < kApplyChunk) ? t.n - i0 : kApplyChunk;
+        const int ng = (nc + 7) >> 3;  // groups of 8 workers in this round; absent workers have sign + and scale 0
+        if (i0) __syncthreads();
+#pragma unroll
+        for (int c = wr; c < kApplyChunk; c += kWarps) {
+            const uint32_t* src = b.bits + (size_t)(i0 + c) * (size_t)b.W + wbase;
+            sh.sum.bits[c][lane] = c < nc && lane < words ? __ldg(src + lane) : 0u;
+            sh.sum.bits[c][lane + 32] = c < nc && lane + 32 < words ? __ldg(src + lane + 32) : 0u;
+        }
+        if (threadIdx.x < kApplyChunk * 4) {  // one table entry per thread: the scales of the subset's members
+            const int q = threadIdx.x >> 4, sub = threadIdx.x & 15;
+            double e = 0.0;
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+                if (((sub >> j) & 1) && q * 4 + j < nc) e += (double)b.scales_cur[(size_t)(i0 + q * 4 + j) * t.M + blk];
+            sh.sum.four[q][sub] = e;
+        }
         __syncthreads();
-        // warp wr stages the words of workers wr, wr + 8, ...: 32 consecutive words each, one per lane
-        for (int c = wr; c < nc; c += kWarps)
-            sh_bits[c][lane] = word_live ? __ldg(b.bits + (size_t)(i0 + c) * (size_t)b.W + wbase + lane) : 0u;
-        if constexpr (TABLES) {
-            const int ng = (nc + 3) >> 2;  // groups of 4 workers in this round
-            if (threadIdx.x < ng * 16) {   // one table entry per thread: the scales of the subset's members
-                const int gq = threadIdx.x >> 4, sub = threadIdx.x & 15;
-                double e = 0.0;
 #pragma unroll
-                for (int j = 0; j < 4; ++j)
-                    if (((sub >> j) & 1) && gq * 4 + j < nc)
-                        e += (double)b.scales_cur[(size_t)(i0 + gq * 4 + j) * t.M + blk];
-                sh_tab[gq][sub] = e;
-            }
-            __syncthreads();
-            // lane i: worker i's words of this warp's coordinates -> lane c: the workers' bits of coordinate 32 q + c
-            uint32_t x[4];
+        for (int g = 0; g < kApplyChunk / 8; ++g)
+            if (g < ng) sh.sum.eight[g][threadIdx.x] = sh.sum.four[2 * g][threadIdx.x & 15] + sh.sum.four[2 * g + 1][threadIdx.x >> 4];
+        __syncthreads();
 #pragma unroll
-            for (int q = 0; q < 4; ++q) x[q] = lane < nc ? sh_bits[lane][wr * 4 + q] : 0u;
-            transpose32x4(x, lane);
-            // this thread's coordinates 4 lane + k lie in word q = lane / 8 at bit 4 (lane % 8) + k: their patterns
-            // sit in lane 4 (lane % 8) + k, matrix lane / 8 (a trip through shared memory instead of these 16
-            // shuffles was slower)
-            uint4 pat = make_uint4(0u, 0u, 0u, 0u);
+        for (int g = 0; g < kApplyChunk / 8; ++g) {
+            if (g < ng) {  // the same for every thread of the CTA
+                uint32_t x[8];
 #pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                const uint32_t y0 = __shfl_sync(0xffffffffu, x[q], (lane & 7) * 4 + 0);
-                const uint32_t y1 = __shfl_sync(0xffffffffu, x[q], (lane & 7) * 4 + 1);
-                const uint32_t y2 = __shfl_sync(0xffffffffu, x[q], (lane & 7) * 4 + 2);
-                const uint32_t y3 = __shfl_sync(0xffffffffu, x[q], (lane & 7) * 4 + 3);
-                if ((lane >> 3) == q) pat = make_uint4(y0, y1, y2, y3);
-            }
+                for (int j = 0; j < 8; ++j) x[j] = reinterpret_cast<const unsigned char*>(sh.sum.bits[g * 8 + j])[threadIdx.x];
+                uint32_t p0 = __byte_perm(__byte_perm(x[0], x[1], 0x0040), __byte_perm(x[2], x[3], 0x0040), 0x5410);
+                uint32_t p1 = __byte_perm(__byte_perm(x[4], x[5], 0x0040), __byte_perm(x[6], x[7], 0x0040), 0x5410);
+                transpose8(p0, p1);
+                all += sh.sum.eight[g][255];
 #pragma unroll
-            for (int gq = 0; gq < kApplyChunk / 4; ++gq) {
-                if (gq < ng) {  // the same for every thread of the CTA
-                    all += sh_tab[gq][15];
-                    a0 += sh_tab[gq][(pat.x >> (4 * gq)) & 15u];
-                    a1 += sh_tab[gq][(pat.y >> (4 * gq)) & 15u];
-                    a2 += sh_tab[gq][(pat.z >> (4 * gq)) & 15u];
-                    a3 += sh_tab[gq][(pat.w >> (4 * gq)) & 15u];
+                for (int k = 0; k < 4; ++k) {
+                    a[k] += sh.sum.eight[g][(p0 >> (8 * k)) & 255u];
+                    a[4 + k] += sh.sum.eight[g][(p1 >> (8 * k)) & 255u];
                 }
-            }
-        } else {
-            double* sh_s = &sh_tab[0][0];
-            if (threadIdx.x < nc) sh_s[threadIdx.x] = (double)b.scales_cur[(size_t)(i0 + threadIdx.x) * t.M + blk];
-            __syncthreads();
-            const int wsel = threadIdx.x >> 3, nsh = (threadIdx.x & 7) * 4;  // this thread's word and its nibble in it
-#pragma unroll 4
-            for (int c = 0; c < nc; ++c) {
-                const double sc = sh_s[c];
-                const uint32_t nib = sh_bits[c][wsel] >> nsh;
-                all += sc;
-                if (nib & 1u) a0 += sc;
-                if (nib & 2u) a1 += sc;
-                if (nib & 4u) a2 += sc;
-                if (nib & 8u) a3 += sc;
             }
         }
     }
-    a0 = all - (a0 + a0);
-    a1 = all - (a1 + a1);
-    a2 = all - (a2 + a2);
-    a3 = all - (a3 + a3);
-    if (r >= len) return;
-    const float gb[4] = {mean_from_acc(a0, hp), mean_from_acc(a1, hp), mean_from_acc(a2, hp),
-                         mean_from_acc(a3, hp)};
-    if (full) {
-        amsgrad_update(gb[0], mm.x, vv.x, hh.x, tt.x, hp);
-        amsgrad_update(gb[1], mm.y, vv.y, hh.y, tt.y, hp);
-        amsgrad_update(gb[2], mm.z, vv.z, hh.z, tt.z, hp);
-        amsgrad_update(gb[3], mm.w, vv.w, hh.w, tt.w, hp);
-        if constexpr (RECORD) store4(gbar + r, cls, make_float4(gb[0], gb[1], gb[2], gb[3]));
-        store4(m + r, cls, mm);
-        store4(v + r, cls, vv);
-        store4(vh + r, cls, hh);
-        store4(th + r, cls, tt);
-    } else {
+    __syncthreads();  // the tables make room for the averages
+    {
+        float gb[8];
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            if (r + k < len) {
-                float m1 = m[r + k], v1 = v[r + k], h1 = vh[r + k], t1 = th[r + k];
-                amsgrad_update(gb[k], m1, v1, h1, t1, hp);
-                if constexpr (RECORD) gbar[r + k] = gb[k];
-                m[r + k] = m1;
-                v[r + k] = v1;
-                vh[r + k] = h1;
-                th[r + k] = t1;
+        for (int k = 0; k < 8; ++k) gb[k] = mean_from_acc(all - (a[k] + a[k]), hp);
+        const int p = skip + (int)threadIdx.x * 8;
+        if (skip == 0) {
+            *reinterpret_cast<float4*>(sh.gbar + p) = make_float4(gb[0], gb[1], gb[2], gb[3]);
+            *reinterpret_cast<float4*>(sh.gbar + p + 4) = make_float4(gb[4], gb[5], gb[6], gb[7]);
+        } else {
+#pragma unroll
+            for (int k = 0; k < 8; ++k) sh.gbar[p + k] = gb[k];
+        }
+    }
+    __syncthreads();
+    uint32_t there = 0;
+    for (int tries = 0; tries < (1 << 16) && !there; ++tries)
+        asm volatile("{\n.reg .pred p;\nmbarrier.try_wait.parity.shared::cta.b64 p, [%1], 0;\nselp.u32 %0, 1, 0, p;\n}"
+                     : "=r"(there)
+                     : "r"(bar)
+                     : "memory");
+    if (!there) {  // cannot happen: the copies are this CTA's own
+        atomicOr(b.status, 4u);
+        return;
+    }
+    for (int p = (int)threadIdx.x * 4; p < end; p += kThreads * 4) {
+        if (p >= lo && p < hi) {
+            float4 mm = *reinterpret_cast<const float4*>(&sh.state[0][p]), vv = *reinterpret_cast<const float4*>(&sh.state[1][p]);
+            float4 hh = *reinterpret_cast<const float4*>(&sh.state[2][p]), tt = *reinterpret_cast<const float4*>(&sh.state[3][p]);
+            const float4 gb = *reinterpret_cast<const float4*>(sh.gbar + p);
+            amsgrad_update(gb.x, mm.x, vv.x, hh.x, tt.x, hp);
+            amsgrad_update(gb.y, mm.y, vv.y, hh.y, tt.y, hp);
+            amsgrad_update(gb.z, mm.z, vv.z, hh.z, tt.z, hp);
+            amsgrad_update(gb.w, mm.w, vv.w, hh.w, tt.w, hp);
+            if constexpr (RECORD) *reinterpret_cast<float4*>(b.gbar + g0 + p) = gb;
+            *reinterpret_cast<float4*>(vec[0] + g0 + p) = mm;
+            *reinterpret_cast<float4*>(vec[1] + g0 + p) = vv;
+            *reinterpret_cast<float4*>(vec[2] + g0 + p) = hh;
+            *reinterpret_cast<float4*>(vec[3] + g0 + p) = tt;
+        } else {  // the group that this block's first or last coordinates share with a neighbour
+            for (int k = p < skip ? skip : p; k < p + 4 && k < end; ++k) {
+                const int64_t j = g0 + k;
+                float m1 = b.m[j], v1 = b.v[j], h1 = b.vhat[j], t1 = theta[j];
+                amsgrad_update(sh.gbar[k], m1, v1, h1, t1, hp);
+                if constexpr (RECORD) b.gbar[j] = sh.gbar[k];
+                b.m[j] = m1;
+                b.v[j] = v1;
+                b.vhat[j] = h1;
+                theta[j] = t1;
             }
         }
     }
@@ -490,13 +500,10 @@ cudaError_t launch_bs_apply(compams_context* c, float* theta) {
     b.scales_cur = c->scales[c->scales_cur];
     Tables t = c->tab;
     t.n = c->n_total;  // the average runs over every worker's message
-    const dim3 grid((unsigned)c->tab.ntiles * kWarps);
-    const bool tables = c->n_total >= kApplyTablesFrom;
-    // four builds: the inner sum by tables or worker by worker; gbar stored or not (a run-time branch around the
-    // store slowed the kernel by a tenth)
-    void (*kernel)(Tables, BsBuffers, float*, HyperParams, const SegParams) =
-        tables ? (b.gbar ? bs_apply_kernel<true, true> : bs_apply_kernel<true, false>)
-               : (b.gbar ? bs_apply_kernel<false, true> : bs_apply_kernel<false, false>);
+    const dim3 grid((unsigned)(c->tab.ntiles * (kTile / kApplySpan)));
+    // two builds: gbar stored or not (a run-time branch around the store slowed the kernel by a tenth)
+    void (*kernel)(const Tables, const BsBuffers, float*, const HyperParams, const SegParams) =
+        b.gbar ? bs_apply_kernel<true> : bs_apply_kernel<false>;
     if (c->n == c->n_total) return counted(c, launch_after(kernel, grid, dim3(kThreads), c->stream, t, b, theta, c->hp, c->segp));
     // sharded workers: the other workers' messages were written by the caller's exchange, which is
     // ordered on the stream like any kernel; a plain launch waits for it

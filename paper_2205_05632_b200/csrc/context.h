@@ -75,6 +75,7 @@ struct BsBuffers {
     double* tile_sum;         // [n, ntiles]
     uint2* edge;              // [n, ntiles] a tile's share of the sign words it has in common with its neighbours
     float *gbar, *m, *v, *vhat;
+    uint32_t* status;
 };
 
 struct TopkBuffers {
