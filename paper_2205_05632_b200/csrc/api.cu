@@ -197,6 +197,7 @@ int build_tiles(compams_context* c, const std::vector<int32_t>& blocks, bool top
     std::vector<TileInfo> tiles;
     std::vector<SegInfo> segs;
     int64_t cand_total = 0;
+    c->bs_max_tiles = 0;
     for (size_t s = 0; s < blocks.size(); ++s) {
         const int32_t b = blocks[s];
         const int64_t len = c->off[b + 1] - c->off[b];
@@ -213,6 +214,7 @@ int build_tiles(compams_context* c, const std::vector<int32_t>& blocks, bool top
         si.blk = b;
         si.tile0 = (int32_t)tiles.size();
         si.ntile_b = (int32_t)nt;
+        c->bs_max_tiles = std::max(c->bs_max_tiles, (int)si.ntile_b);
         if (topk) {
             const int64_t kb = c->seg_off[(size_t)b + 1] - c->seg_off[(size_t)b];
             si.slot0 = c->seg_off[(size_t)b];
@@ -439,7 +441,7 @@ int compress_device(compams_context* c, const void* grads) {
         c->scales_cur ^= 1;
         RC(run_kernel(c, COMPAMS_K_BS_SWEEP, [&] { return launch_bs_sweep(c, grads); }));
         c->e_is_x = true;
-        RC(run_kernel(c, COMPAMS_K_BS_SCALES, [&] { return launch_bs_scales(c); }));
+        if (!bs_apply_adds_up(c)) RC(run_kernel(c, COMPAMS_K_BS_SCALES, [&] { return launch_bs_scales(c); }));
         return COMPAMS_OK;
     }
     // a selection leaves x in E at the coordinates it keeps, and the pair that delimits them; their e is zeroed

@@ -221,6 +221,19 @@ __global__ void __launch_bounds__(kThreads, sizeof(GT) == 2 ? COMPAMS_BF16_SWEEP
     }
 }
 
+// Sum of a block's tile sums by one warp, in an order fixed by the tile count (result in lane 0). bs_scales and bs_apply
+// add up blocks of at most kWarpTiles tiles this way, so that it does not matter which of them does.
+constexpr int kWarpTiles = 256;
+__device__ __forceinline__ double tile_sums_by_warp(const double* ts, int nt, int lane) {
+    double part = 0.0;
+    for (int k = lane; k < nt; k += 32) part += ts[k];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) part += __shfl_down_sync(0xffffffffu, part, o);
+    return part;
+}
+// One division in binary64, one rounding to fp32.
+__device__ __forceinline__ float scale_of(double sum, int len) { return __double2float_rn(sum / (double)len); }
+
 // One CTA per (worker, block): scale = ||x_B||_1 / d_B from the tile sums (Definition 2). Built for 256 threads
 // (many blocks of a few tiles) and for 1024 with four tile sums requested at a time (a whole-vector block has
 // thousands of tiles and only n CTAs to add them: 256 threads took 33 us at d = 2^26, n = 8, most of it waiting
@@ -236,7 +249,7 @@ __global__ void __launch_bounds__(NT) bs_scales_kernel(Tables t, BsBuffers b) {
     const double* ts = b.tile_sum + (size_t)i * t.ntiles + si->tile0;
     const int nt = si->ntile_b;
     double part = 0.0;
-    int k = threadIdx.x;
+    int k = nt > kWarpTiles ? (int)threadIdx.x : nt;
     for (; k + 3 * NT < nt; k += 4 * NT) {
         const double s0 = ts[k], s1 = ts[k + NT], s2 = ts[k + 2 * NT], s3 = ts[k + 3 * NT];
         part += s0;
@@ -256,9 +269,14 @@ __global__ void __launch_bounds__(NT) bs_scales_kernel(Tables t, BsBuffers b) {
             if (q < wb) words[q] = ed[j].y | (j + 1 < nt ? ed[j + 1].x : 0u);
         }
     }
-    const double S = block_sum_double<NT / 32>(part, red);
-    // one division in binary64, one rounding to fp32
-    if (threadIdx.x == 0) b.scales_cur[(size_t)i * t.M + blk] = __double2float_rn(S / (double)si->len);
+    double S;
+    if (nt > kWarpTiles) {
+        S = block_sum_double<NT / 32>(part, red);
+    } else {
+        if (threadIdx.x >= 32) return;
+        S = tile_sums_by_warp(ts, nt, threadIdx.x);
+    }
+    if (threadIdx.x == 0) b.scales_cur[(size_t)i * t.M + blk] = scale_of(S, si->len);
 }
 
 // E holds x; turn it into e = x - sign(x) * s in place (Algorithm 2, the residual update).
@@ -279,11 +297,7 @@ __global__ void __launch_bounds__(kThreads) bs_materialize_kernel(Tables t, floa
     }
 }
 
-#ifndef APPLY_CTAS
-#define APPLY_CTAS 4
-#endif
 constexpr int kApplyChunk = 16;         // workers whose sign words and scales are staged at a time
-constexpr int kApplySpan = 8 * kThreads;  // coordinates per CTA of bs_apply
 
 // Transposes an 8 x 8 bit matrix whose rows are the bytes of lo (rows 0-3) and hi (rows 4-7): afterwards bit i of byte k
 // is what bit k of byte i was. Three rounds of the usual block swap.
@@ -302,6 +316,8 @@ __device__ __forceinline__ void transpose8(uint32_t& lo, uint32_t& hi) {
     lo = t;
 }
 
+constexpr int kApplySpan = 8 * kThreads;  // coordinates per CTA of bs_apply
+
 // Shared memory of one bs_apply CTA.
 struct ApplyShared {
     float state[4][kApplySpan + 4];  // m, v, vhat, theta of the CTA's coordinates, from a 16-byte boundary on
@@ -310,6 +326,7 @@ struct ApplyShared {
             uint32_t bits[kApplyChunk][kApplySpan / 32];  // [worker][word]
             double eight[kApplyChunk / 8][256];           // subset sums of 8 workers' scales
             double four[kApplyChunk / 4][16];             // ... of 4 workers'
+            double scale[kApplyChunk];
         } sum;
         float gbar[kApplySpan + 4];
     };
@@ -326,8 +343,17 @@ struct ApplyShared {
 // sum is), and a coordinate adds one entry per 8 workers. A thread's 8 coordinates are one byte of each worker's sign
 // words, so the patterns of 8 workers come from transposing 8 bytes in registers. The averages pass through shared memory,
 // and the update runs over groups of 4 coordinates that start on 16-byte boundaries, whatever the block's offset.
-template <bool RECORD>
-__global__ void __launch_bounds__(kThreads, APPLY_CTAS) bs_apply_kernel(const __grid_constant__ Tables t, const __grid_constant__ BsBuffers b,
+//
+// Bound by memory from here on (32 B per coordinate and the sign bits); before, with one predicated binary64 add per worker
+// and coordinate, or 16-entry tables and a transposition across the warp, by instruction issue (786 instructions per 4
+// coordinates at n = 16, half of them the sum), and with blocks off the 16-byte grid by 32-bit accesses: steps of ResNet-18
+// shapes, n = 16 427 -> 404 us; d = 6.6 M in 7 ragged blocks, n = 4 105 -> 96; 8 of 32 workers, ResNet-50 shapes 649 -> 623.
+// Tried: 8 consecutive coordinates per thread in the update too, by 256-bit accesses from registers (417 us on the first,
+// 142 on the second), three and five CTAs per SM, CTAs of 64 and 128 threads for small vectors (slower than 256).
+// OWN: the tile sums have not been added up by bs_scales (small blocks, all workers in this handle): every CTA adds up
+// its block's, and completes the sign words that its tile has in common with the next.
+template <bool RECORD, bool OWN>
+__global__ void __launch_bounds__(kThreads, 4) bs_apply_kernel(const __grid_constant__ Tables t, const __grid_constant__ BsBuffers b,
                                                                float* __restrict__ theta, const __grid_constant__ HyperParams hp,
                                                                const __grid_constant__ SegParams sp_) {
     __shared__ __align__(128) ApplyShared sh;
@@ -363,6 +389,7 @@ __global__ void __launch_bounds__(kThreads, APPLY_CTAS) bs_apply_kernel(const __
     const size_t wbase = (size_t)(sp_.nseg ? (int64_t)sp_.wofs[ti.seg] : b.word_off[blk]) + (size_t)(rs >> 5);
     const int lane = threadIdx.x & 31, wr = threadIdx.x >> 5;
     const int words = (len - rs + 31) >> 5;  // sign words of this CTA's coordinates (possibly more than it has)
+    const int edge_word = rs + kApplySpan == ti.r0 + kTile ? kApplySpan / 32 - 1 : -1;
     double a[8] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0}, all = 0.0;
     for (int i0 = 0; i0 < t.n; i0 += kApplyChunk) {
         const int nc = (t.n - i0 < kApplyChunk) ? t.n - i0 : kApplyChunk;
@@ -370,16 +397,41 @@ __global__ void __launch_bounds__(kThreads, APPLY_CTAS) bs_apply_kernel(const __
         if (i0) __syncthreads();
 #pragma unroll
         for (int c = wr; c < kApplyChunk; c += kWarps) {
-            const uint32_t* src = b.bits + (size_t)(i0 + c) * (size_t)b.W + wbase;
-            sh.sum.bits[c][lane] = c < nc && lane < words ? __ldg(src + lane) : 0u;
-            sh.sum.bits[c][lane + 32] = c < nc && lane + 32 < words ? __ldg(src + lane + 32) : 0u;
+            uint32_t* src = b.bits + (size_t)(i0 + c) * (size_t)b.W + wbase;
+#pragma unroll
+            for (int w = lane; w < kApplySpan / 32; w += 32) {
+                uint32_t word = 0u;
+                if (c < nc && w < words) {
+                    if (OWN && w == edge_word) {  // the word in common with the next tile: one share from each
+                        const uint2* ed = b.edge + (size_t)(i0 + c) * t.ntiles + tile;
+                        word = ed[0].y | (tile + 1 < ti.tile0 + ti.ntile_b ? ed[1].x : 0u);
+                        src[w] = word;
+                    } else {
+                        word = src[w];
+                    }
+                }
+                sh.sum.bits[c][w] = word;
+            }
         }
+        if (OWN) {
+            for (int c = wr; c < nc; c += kWarps) {
+                const double s = tile_sums_by_warp(b.tile_sum + (size_t)(i0 + c) * t.ntiles + ti.tile0, ti.ntile_b, lane);
+                if (lane == 0) {
+                    const float f = scale_of(s, len);
+                    sh.sum.scale[c] = (double)f;
+                    if (rs == 0) b.scales_cur[(size_t)(i0 + c) * t.M + blk] = f;
+                }
+            }
+        } else if (threadIdx.x < nc) {
+            sh.sum.scale[threadIdx.x] = (double)b.scales_cur[(size_t)(i0 + threadIdx.x) * t.M + blk];
+        }
+        __syncthreads();
         if (threadIdx.x < kApplyChunk * 4) {  // one table entry per thread: the scales of the subset's members
             const int q = threadIdx.x >> 4, sub = threadIdx.x & 15;
             double e = 0.0;
 #pragma unroll
             for (int j = 0; j < 4; ++j)
-                if (((sub >> j) & 1) && q * 4 + j < nc) e += (double)b.scales_cur[(size_t)(i0 + q * 4 + j) * t.M + blk];
+                if (((sub >> j) & 1) && q * 4 + j < nc) e += sh.sum.scale[q * 4 + j];
             sh.sum.four[q][sub] = e;
         }
         __syncthreads();
@@ -488,6 +540,14 @@ cudaError_t launch_bs_sweep(compams_context* c, const void* grads) {
     return counted(c, cudaGetLastError());
 }
 
+// Whether bs_apply adds up the tile sums itself, and bs_scales is not launched: n = 4, d = 65,536 10.8 -> 9.7 us, n = 8,
+// d = 2^20 29.3 -> 27.5. Not before an exchange (the messages have to be complete), not for larger blocks, of which every
+// CTA would read more sums than its share of the rest, nor for many workers (n = 24, d = 3.3 M in 90 blocks: 194.4 us
+// with bs_scales, 198.3 without: a warp adds up one worker after the other).
+bool bs_apply_adds_up(const compams_context* c) {
+    return c->n == c->n_total && c->n <= 2 * kWarps && c->bs_max_tiles <= kWarpTiles && (int64_t)c->bs_max_tiles * c->n <= 1024;
+}
+
 cudaError_t launch_bs_scales(compams_context* c) {
     dim3 grid((unsigned)c->M, (unsigned)c->n);
     if (c->tab.ntiles > 256 * (int64_t)c->M)  // on average more than 256 tiles to a block
@@ -500,10 +560,12 @@ cudaError_t launch_bs_apply(compams_context* c, float* theta) {
     b.scales_cur = c->scales[c->scales_cur];
     Tables t = c->tab;
     t.n = c->n_total;  // the average runs over every worker's message
+    const bool own = bs_apply_adds_up(c);
     const dim3 grid((unsigned)(c->tab.ntiles * (kTile / kApplySpan)));
-    // two builds: gbar stored or not (a run-time branch around the store slowed the kernel by a tenth)
+    // (gbar stored or not is a template parameter: a run-time branch around the store slowed the kernel by a tenth)
     void (*kernel)(const Tables, const BsBuffers, float*, const HyperParams, const SegParams) =
-        b.gbar ? bs_apply_kernel<true> : bs_apply_kernel<false>;
+        own ? (b.gbar ? bs_apply_kernel<true, true> : bs_apply_kernel<false, true>)
+            : (b.gbar ? bs_apply_kernel<true, false> : bs_apply_kernel<false, false>);
     if (c->n == c->n_total) return counted(c, launch_after(kernel, grid, dim3(kThreads), c->stream, t, b, theta, c->hp, c->segp));
     // sharded workers: the other workers' messages were written by the caller's exchange, which is
     // ordered on the stream like any kernel; a plain launch waits for it

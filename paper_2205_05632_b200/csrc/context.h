@@ -156,6 +156,7 @@ struct compams_context {
     int dense_grid = 0;  // CTAs of the cooperative dense-pass kernel (0: not yet sized)
     float* scales[2] = {nullptr, nullptr};
     int scales_cur = 0;
+    int bs_max_tiles = 0;     // Block-Sign: tiles of the longest block
     bool e_is_x = false;  // Block-Sign: E holds the corrected gradient x of the last step, not e
     bool compressed = false;  // compams_compress has run and its compams_apply has not: the step is half done
 
@@ -195,6 +196,7 @@ inline cudaError_t counted(compams_context* c, cudaError_t e) {
 // Each launcher enqueues its kernel(s) on ctx->stream and returns the launch status.
 cudaError_t launch_dense_mean_amsgrad(compams_context* c, const void* grads, float* theta);
 cudaError_t launch_bs_sweep(compams_context* c, const void* grads);
+bool bs_apply_adds_up(const compams_context* c);
 cudaError_t launch_bs_scales(compams_context* c);
 cudaError_t launch_bs_apply(compams_context* c, float* theta);
 cudaError_t launch_bs_materialize(compams_context* c);
