@@ -87,7 +87,7 @@ enum compams_kernel {
     COMPAMS_K_TOPK_DENSE = 5,         /* Top-k dense passes (one cooperative launch): radix histograms over x,
                                          threshold search, emission, lowest-index ties                        */
     COMPAMS_K_TOPK_MATERIALIZE = 6,   /* Top-k: zero e at the coordinates kept in the last step when E is read   */
-    COMPAMS_K_RANDK_EMIT = 7,         /* Random-k: every message slot computes its drawn coordinate and fetches x there */
+    COMPAMS_K_RANDK_EMIT = 7,         /* Random-k: marks the drawn coordinates, then the sweep that takes their x */
     /* 8: reserved (never returned, never timed) */
     COMPAMS_K_TOPK_SCATTER = 9,       /* Top-k: closes the step per segment; sparse scatter-accumulate         */
     COMPAMS_K_AMSGRAD = 10,           /* Top-k: AMSGrad update from the accumulated average                   */

@@ -345,6 +345,14 @@ int init_context(compams_context* c, const int64_t* block_offsets) {
         RC(dev_alloc(c, &t.tile_ties, c->randk ? 1 : (size_t)n * (size_t)c->tab.ntiles));
         RC(dev_alloc(c, &t.cand, (size_t)n * (size_t)t.cand_total, false));
         RC(dev_alloc(c, &t.acc, (size_t)d));
+        if (c->randk) {
+            // workers whose map fits 64 MB of the L2 together, at least one
+            constexpr int64_t kMapBits = (int64_t)64 * 8 * 1024 * 1024;
+            c->randk_group = (int32_t)std::min<int64_t>(n, std::max<int64_t>(1, kMapBits / d));
+            c->randk_words = ((int64_t)c->randk_group * d + 31) / 32 + 1;
+            RC(dev_alloc(c, &t.map, (size_t)c->randk_words));
+            RC(dev_alloc(c, &t.slots, (size_t)n * (size_t)c->tab.nseg));
+        }
         {
             std::vector<uint32_t> none((size_t)n * (size_t)std::max(c->tab.nseg, 1), 0xffffffffu);
             RC(dev_upload(c, &t.thr, none));
@@ -448,11 +456,9 @@ int compress_device(compams_context* c, const void* grads) {
     // when E is next read (by the next sweep, or by topk_materialize when the caller asks for E)
     c->tk.use_thr = c->e_mask_pending ? 1 : 0;
     if (c->randk) {
-        // no selection: the sweep leaves x in E, then every message slot fetches the x of its drawn coordinate and
-        // zeroes it; with all workers in this handle the pairs go to the server in the same kernel, otherwise
-        // compams_apply delivers the exchanged messages
-        RC(run_kernel(c, COMPAMS_K_TOPK_SWEEP, [&] { return launch_topk_sweep(c, grads); }));
-        RC(run_kernel(c, COMPAMS_K_RANDK_EMIT, [&] { return launch_randk_emit(c, c->n == c->n_total); }));
+        // no selection: the drawn coordinates are marked, and the sweep takes them; with all workers in this handle the
+        // pairs go to the server in the same kernel, otherwise compams_apply delivers the exchanged messages
+        RC(run_kernel(c, COMPAMS_K_RANDK_EMIT, [&] { return launch_randk(c, grads, c->n == c->n_total); }));
         return COMPAMS_OK;
     }
     if (c->fused) {

@@ -95,6 +95,8 @@ struct TopkBuffers {
     uint32_t* dense_count;     // [1] segments currently marked for the dense passes
     uint32_t* sel_ticket;      // [n * long lists, 2] threshold-bin entries collected; parts of the emission done
     uint2* sel_surv;           // [n * long lists, kSurvCap] threshold-bin entries of a long list
+    uint32_t* map;             // Random-k: a bit per element of a group of workers, set where it is drawn
+    uint32_t* slots;           // Random-k: [n * nseg] message slots handed out this step
     double* acc;               // [d] binary64 accumulator, used only by entries that overflow their bucket
     uint32_t* thr;             // [n * nseg] bits of the magnitude from which on the segment's last selection kept
                                // everything: E still holds x at those elements; their e is 0
@@ -146,6 +148,8 @@ struct compams_context {
     int sel_cluster = 1;          // CTAs per (worker, long block)
     bool fused = false;           // Top-k: every block is swept and selected from by one kernel (small n d)
     int sel_parts = 0;            // CTAs that emit a long list in a kernel of its own (0: the cluster emits it)
+    int32_t randk_group = 1;       // Random-k: workers whose elements share the map at a time
+    int64_t randk_words = 0;       // ... its words
     bool many_candidates = false;  // Top-k: the lists hold more than 1/32 of the coordinates
     bool dense_kernel = false;  // some blocks are too long for a cluster to go through: the dense passes are launched every step
     bool deliver = false;       // the selection hands the kept entries to the server itself (no topk_scatter)
@@ -207,7 +211,7 @@ cudaError_t launch_topk_fused(compams_context* c, const void* grads);
 cudaError_t launch_topk_dense(compams_context* c);
 cudaError_t launch_topk_materialize(compams_context* c);
 cudaError_t launch_topk_scatter(compams_context* c);
-cudaError_t launch_randk_emit(compams_context* c, bool deliver);
+cudaError_t launch_randk(compams_context* c, const void* grads, bool deliver);
 cudaError_t launch_amsgrad(compams_context* c, float* theta);
 
 }  // namespace compams

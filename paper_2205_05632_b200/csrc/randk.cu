@@ -8,9 +8,14 @@
 // halves of the first three words of one Philox4x64-10 block (Salmon, Moraes, Dror, Shaw, SC 2011) at counter
 // (0, 0, b, i) under key (seed, t); the round function is the 32-bit finalizer of MurmurHash3 applied to
 // (right half xor round key). Being the image of k_b distinct inputs under a bijection, the set has exactly k_b
-// members and needs no selection pass: the sweep is the Top-k sweep without candidates (x = g + e written over
-// E), then one thread per message slot computes its coordinate, fetches x there, zeroes it (the residual of a
-// kept coordinate) and hands the pair to the server.
+// members and needs no selection. Two kernels per group of workers: randk_mark, one thread per message slot, computes the
+// slot's coordinate and sets its bit in a map of the group's elements; randk_sweep forms x = g + e, and where the bit is
+// set x goes to the message and to the server and 0 to E (the residual of a kept coordinate), x to E elsewhere.
+//
+// The map is what makes the drawn coordinates meet their x in index order: it is small enough for the L2 (64 MB: hence the
+// groups), where setting a bit costs a fraction of a visit to DRAM. (A sweep that left x in E, and one atomic exchange per
+// slot that fetched it from there and zeroed it, was bound by the rate of scattered accesses, 16 to 18 G per second: step on
+// ResNet-18 shapes, n = 16, 1 % 481 -> 415 us, n = 8, d = 2^26, 10 % 4086 -> 2397.)
 #include "context.h"
 #include "scatter.cuh"
 
@@ -85,6 +90,8 @@ struct Drawn {
     int32_t il;  // worker within the handle
     int64_t q;   // slot within the worker's message row
     int32_t j;   // the drawn coordinate
+    int32_t blk; // its block
+    uint32_t r;  // the slot within the block's
 };
 
 // A CTA covers kThreads consecutive message slots of one worker; every thread computes the coordinate of its
@@ -99,7 +106,8 @@ __device__ __forceinline__ Drawn randk_draw(const Tables& t, const TopkBuffers& 
     dr.il = (int32_t)(blockIdx.x / per_worker);
     dr.q = (int64_t)(blockIdx.x % per_worker) * kThreads + tid;
     dr.valid = dr.q < b.K;
-    dr.j = 0;
+    dr.j = dr.blk = 0;
+    dr.r = 0;
     int64_t o = 0;
     uint32_t len = 1, r = 0;
     if (dr.valid) {
@@ -108,9 +116,10 @@ __device__ __forceinline__ Drawn randk_draw(const Tables& t, const TopkBuffers& 
             const int mid = (lo + hi + 1) >> 1;
             if (__ldg(b.seg_off + mid) <= dr.q) lo = mid; else hi = mid - 1;
         }
+        dr.blk = lo;
         o = __ldg(t.off + lo);
         len = (uint32_t)(__ldg(t.off + lo + 1) - o);
-        r = (uint32_t)(dr.q - __ldg(b.seg_off + lo));
+        dr.r = r = (uint32_t)(dr.q - __ldg(b.seg_off + lo));
         if (tid == 0 || r == 0) {
             const RoundKeys rk = randk_round_keys(seed, step, (uint64_t)(row0 + dr.il), (uint64_t)lo);
 #pragma unroll
@@ -125,35 +134,264 @@ __device__ __forceinline__ Drawn randk_draw(const Tables& t, const TopkBuffers& 
     return dr;
 }
 
-// Worker il keeps coordinate j in message slot q: x goes to the message, its residual is zero.
-__device__ __forceinline__ uint32_t randk_take(const Tables& t, const TopkBuffers& b, int32_t row0, int32_t il, int64_t q,
-                                               int32_t j) {
-    // the sweep left x = g + e there; the residual of a kept coordinate is e = x - x = 0. One exchange at the L2
-    // fetches the one and leaves the other (a load followed by a store to the same scattered word made this
-    // kernel six times slower).
-    uint32_t* ex = reinterpret_cast<uint32_t*>(b.E + (size_t)il * (size_t)t.d + (size_t)j);
-    const uint32_t xbits = atomicExch(ex, 0u);
-    const size_t slot = (size_t)(row0 + il) * (size_t)b.K + (size_t)q;
-    b.idx[slot] = j;
-    b.val[slot] = __uint_as_float(xbits);
-    return xbits;
-}
-
-// One thread per message slot draws its coordinate and takes it.
-__global__ void __launch_bounds__(kThreads) randk_emit_kernel(Tables t, TopkBuffers b, int32_t row0, uint64_t seed,
-                                                              uint64_t step, int deliver) {
+// Bit f - origin of the map stands for element f of the flat [n, d] buffers; origin is a multiple of 32, so that the map's
+// words are the 128-byte lines of E.
+__global__ void __launch_bounds__(kThreads) randk_mark_kernel(const __grid_constant__ Tables t, const __grid_constant__ TopkBuffers b,
+                                                              int32_t row0, int32_t i0, int64_t origin, uint64_t seed, uint64_t step) {
     __shared__ uint32_t keys[kThreads][6];
-    const Drawn dr = randk_draw(t, b, row0, seed, step, keys);
-    uint32_t xbits = 0;
-    if (dr.valid) xbits = randk_take(t, b, row0, dr.il, dr.q, dr.j);
-    if (deliver) scatter_warp(b, dr.valid, dr.j, xbits);
+    dependency_wait();
+    allow_dependents();
+    const Drawn dr = randk_draw(t, b, row0 + i0, seed, step, keys);
+    if (!dr.valid) return;
+    if (dr.r == 0u) b.slots[(size_t)(i0 + dr.il) * t.nseg + dr.blk] = 0u;  // every block is tiled: segment = block
+    const int64_t f = (int64_t)(i0 + dr.il) * t.d + dr.j - origin;
+    atomicOr(b.map + (f >> 5), 1u << (f & 31));
 }
 
-cudaError_t launch_randk_emit(compams_context* c, bool deliver) {
+// A warp's drawn coordinates while it streams: lane l's word of the map for the warp's l-th 32 coordinates, the number of
+// drawn ones before it, and room for their x in index order.
+// (kRoom of them: the loads in flight need the rest of the SM's memory, 4 KB per warp slowed the kernel by a quarter; an x
+// that finds no room stays in E and is fetched from there).
+template <int kRoom>
+struct Drawing {
+    uint32_t word, before;
+    float* x;
+};
+// Element `bit` of the 32 that `word` and `before` describe: a drawn one leaves its x, and its residual is 0.
+template <int kRoom>
+__device__ __forceinline__ float take_drawn(const Drawing<kRoom>& dr, uint32_t word, uint32_t before, int bit, float x) {
+    if (!((word >> bit) & 1u)) return x;
+    const uint32_t p = before + (uint32_t)__popc(word & ((1u << bit) - 1u));
+    if (p >= (uint32_t)kRoom) return x;
+    dr.x[p] = x;
+    return 0.0f;  // Algorithm 2, the residual update: e = x - x
+}
+
+// One warp's 1024 consecutive coordinates from rw on (relative to the block; at a block's ends some lie outside it): the
+// residual of x = g + e written over E. The next iteration's loads are in flight while one is worked on.
+template <bool FULL, typename GT, int kRoom>
+__device__ __forceinline__ void randk_sweep_span(const GT* __restrict__ g, float* __restrict__ e, int len, int rw, int lane,
+                                                 const Drawing<kRoom>& dr) {
+    const int cg = align_class(g + rw), ce = align_class(e + rw);
+    float4 gv[2], ev[2];
+    auto load = [&](int it) {
+        const int r = rw + it * 128 + lane * 4;
+        if (FULL || (r >= 0 && r + 3 < len)) {
+            gv[it & 1] = load4_stream(g + r, cg);
+            ev[it & 1] = load4(e + r, ce);
+        } else {
+            float gt[4], et[4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const bool live = (unsigned)(r + k) < (unsigned)len;
+                gt[k] = live ? load1_stream(g + r + k) : 0.0f;
+                et[k] = live ? e[r + k] : 0.0f;
+            }
+            gv[it & 1] = make_float4(gt[0], gt[1], gt[2], gt[3]);
+            ev[it & 1] = make_float4(et[0], et[1], et[2], et[3]);
+        }
+    };
+    load(0);
+#pragma unroll
+    for (int it = 0; it < kIters; ++it) {
+        if (it + 1 < kIters) load(it + 1);
+        const int r = rw + it * 128 + lane * 4, src = it * 4 + (lane >> 3), bit = (lane & 7) * 4;
+        const uint32_t word = __shfl_sync(0xffffffffu, dr.word, src), before = __shfl_sync(0xffffffffu, dr.before, src);
+        const float4 a = gv[it & 1], b = ev[it & 1];
+        // the corrected-gradient step of Algorithm 2
+        float4 x = make_float4(__fadd_rn(a.x, b.x), __fadd_rn(a.y, b.y), __fadd_rn(a.z, b.z), __fadd_rn(a.w, b.w));
+        if ((word >> bit) & 15u) {
+            x.x = take_drawn(dr, word, before, bit, x.x);
+            x.y = take_drawn(dr, word, before, bit + 1, x.y);
+            x.z = take_drawn(dr, word, before, bit + 2, x.z);
+            x.w = take_drawn(dr, word, before, bit + 3, x.w);
+        }
+        if (FULL || (r >= 0 && r + 3 < len)) {
+            store4(e + r, ce, x);
+        } else {
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+                if ((unsigned)(r + k) < (unsigned)len) e[r + k] = lane_elem(x, k);
+        }
+    }
+}
+
+// The same for bfloat16 gradients where whole spans start on 16-byte boundaries of G and E: 8 coordinates per lane and
+// iteration, so that the gradient load is 128 bits wide too.
+template <int kRoom>
+__device__ __forceinline__ void randk_sweep_span_bf16x8(const bf16_bits* __restrict__ g, float* __restrict__ e, int rw, int lane,
+                                                        const Drawing<kRoom>& dr) {
+    constexpr int NC = kWarpSpan / 256;
+    uint4 gv[2];
+    float4 ev[2][2];
+    auto load = [&](int c) {
+        const int r = rw + c * 256 + lane * 8;
+        gv[c & 1] = __ldg(reinterpret_cast<const uint4*>(g + r));
+        ev[c & 1][0] = *reinterpret_cast<const float4*>(e + r);
+        ev[c & 1][1] = *reinterpret_cast<const float4*>(e + r + 4);
+    };
+    load(0);
+#pragma unroll
+    for (int c = 0; c < NC; ++c) {
+        if (c + 1 < NC) load(c + 1);
+        const int r = rw + c * 256 + lane * 8, src = c * 8 + (lane >> 2), bit = (lane & 3) * 8;
+        const uint32_t word = __shfl_sync(0xffffffffu, dr.word, src), before = __shfl_sync(0xffffffffu, dr.before, src);
+        const uint32_t w[4] = {gv[c & 1].x, gv[c & 1].y, gv[c & 1].z, gv[c & 1].w};
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const float4 b = ev[c & 1][h];
+            float4 x = make_float4(__fadd_rn(__uint_as_float(w[2 * h] << 16), b.x), __fadd_rn(__uint_as_float(w[2 * h] & 0xffff0000u), b.y),
+                                   __fadd_rn(__uint_as_float(w[2 * h + 1] << 16), b.z),
+                                   __fadd_rn(__uint_as_float(w[2 * h + 1] & 0xffff0000u), b.w));
+            if ((word >> (bit + 4 * h)) & 15u) {
+                x.x = take_drawn(dr, word, before, bit + 4 * h, x.x);
+                x.y = take_drawn(dr, word, before, bit + 4 * h + 1, x.y);
+                x.z = take_drawn(dr, word, before, bit + 4 * h + 2, x.z);
+                x.w = take_drawn(dr, word, before, bit + 4 * h + 3, x.w);
+            }
+            *reinterpret_cast<float4*>(e + r + h * 4) = x;
+        }
+    }
+}
+
+// Sum of x over the lanes below this one; *total: over all lanes.
+__device__ __forceinline__ uint32_t warp_exclusive_sum(uint32_t x, int lane, uint32_t* total) {
+    uint32_t s = x;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xffffffffu, s, o);
+        if (lane >= o) s += y;
+    }
+    *total = __shfl_sync(0xffffffffu, s, 31);
+    return s - x;
+}
+
+// Grid: tiles x workers of the group. Tiles are shifted to 128-byte lines of G and E as in the Top-k sweep. A warp knows
+// from the map how many of its 1024 coordinates are drawn, and asks for their message and bucket slots before it starts on
+// g and e; their x wait in shared memory until they do, and every lane then delivers the drawn ones of its 32. The span's
+// lines are asked into the L2 before the map is looked at, which lets four CTAs per SM (64 registers) do better than six
+// (ResNet-18 shapes 415 us, five 425, six 452; without the prefetch and six 460).
+template <typename GT, int kRoom>
+__global__ void __launch_bounds__(kThreads, 4) randk_sweep_kernel(
+    const __grid_constant__ Tables t, const __grid_constant__ TopkBuffers b, const GT* __restrict__ G, int32_t i0, int64_t origin,
+    int64_t words, int deliver, const __grid_constant__ SegParams sp_) {
+    __shared__ float sh_x[kWarps][kRoom];
+    __shared__ uint32_t sh_count[kWarps], sh_base;
+    dependency_wait();
+    allow_dependents();
+    const TileInfo ti = sp_.nseg ? find_tile(sp_, blockIdx.x) : load_tile(t.tiles, blockIdx.x);
+    const int i = i0 + (int)blockIdx.y;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int64_t row0 = (int64_t)i * t.d + ti.o;
+    const int rw = ti.r0 - (int)(row0 & 31) + warp * kWarpSpan;
+    const GT* g = G + row0;
+    float* e = b.E + row0;
+    const bool whole = rw >= 0 && rw + kWarpSpan <= ti.len;
+    if (whole) {  // on their way to the L2 while the map is looked at: one line of E per lane, one of g for as many
+        asm volatile("prefetch.global.L2 [%0];" ::"l"(e + rw + lane * 32));
+        asm volatile("prefetch.global.L2 [%0];" ::"l"(g + rw + lane * 32));
+    }
+    // lane l: the map's word of the warp's l-th 32 coordinates, of which `own` are the block's; the word goes back to 0
+    const int64_t q = ((row0 + rw - origin) >> 5) + lane;
+    const int w0 = rw + lane * 32;
+    uint32_t own = 0xffffffffu;
+    if (w0 < 0) own = w0 > -32 ? 0xffffffffu << -w0 : 0u;
+    if (w0 + 32 > ti.len) own &= w0 < ti.len ? 0xffffffffu >> (w0 + 32 - ti.len) : 0u;
+    uint32_t drawn = own && q < words ? b.map[q] & own : 0u;
+    if (drawn) {
+        if (own == 0xffffffffu) b.map[q] = 0u;
+        else atomicAnd(b.map + q, ~own);  // shared with the neighbouring block or row
+    }
+    // the coordinates meet at most two server buckets: T and, from `edge` on, the next
+    const int64_t j0 = ti.o + (rw < 0 ? 0 : rw);
+    const uint32_t T = (uint32_t)(j0 / kBucketSpan);
+    const int64_t edge = (int64_t)(T + 1) * kBucketSpan - (ti.o + w0);  // bits of this lane's word from here on are in the next
+    const uint32_t late = edge <= 0 ? drawn : edge < 32 ? drawn & (0xffffffffu << (int)edge) : 0u;
+    // counts of at most 1024 each: both sums in one word
+    uint32_t sums;
+    uint32_t rank = warp_exclusive_sum((uint32_t)__popc(drawn) | (uint32_t)__popc(late) << 16, lane, &sums);
+    const uint32_t rank_late = rank >> 16, total = sums & 0xffffu, total_late = sums >> 16;
+    rank &= 0xffffu;
+    uint32_t base = 0;
+    if (lane == 1 && deliver && total - total_late) base = atomicAdd(b.bcount + T, total - total_late);
+    if (lane == 2 && deliver && total_late) base = atomicAdd(b.bcount + T + 1, total_late);
+    // the segment's counter is one word for all of a worker's warps: one atomic per CTA (one per warp made the step twice as long)
+    if (lane == 0) sh_count[warp] = total;
+    __syncthreads();
+    uint32_t pos = rank;
+    {
+        uint32_t of_cta = 0;
+#pragma unroll
+        for (int w = 0; w < kWarps; ++w) {
+            if (w < warp) pos += sh_count[w];
+            of_cta += sh_count[w];
+        }
+        if (threadIdx.x == 0 && of_cta) sh_base = atomicAdd(b.slots + (size_t)i * t.nseg + ti.seg, of_cta);
+    }
+
+    bool wide = false;
+    if constexpr (sizeof(GT) == 2)
+        wide = whole && ((reinterpret_cast<uintptr_t>(g + rw) | reinterpret_cast<uintptr_t>(e + rw)) & 15u) == 0;
+    const Drawing<kRoom> dr{drawn, rank, sh_x[warp]};
+    if (wide) {
+        if constexpr (sizeof(GT) == 2) randk_sweep_span_bf16x8(g, e, rw, lane, dr);
+    } else if (whole) {
+        randk_sweep_span<true>(g, e, ti.len, rw, lane, dr);
+    } else if (rw < ti.len) {
+        randk_sweep_span<false>(g, e, ti.len, rw, lane, dr);
+    }
+
+    uint32_t early = __shfl_sync(0xffffffffu, base, 1) + rank - rank_late, next = __shfl_sync(0xffffffffu, base, 2) + rank_late;
+    __syncthreads();  // the drawn x and the CTA's first slot are there
+    pos += sh_base;
+    const SegInfo* si = t.segs + ti.seg;
+    const size_t slot0 = (size_t)i * (size_t)b.K + (size_t)si->slot0;
+    const uint32_t kb = si->kb;
+    while (drawn) {
+        const int k = __ffs(drawn) - 1;
+        drawn &= drawn - 1;
+        const int32_t j = (int32_t)(ti.o + w0 + k);
+        const float x = rank < (uint32_t)kRoom ? sh_x[warp][rank] : atomicExch(e + w0 + k, 0.0f);
+        ++rank;
+        if (pos < kb) {
+            b.idx[slot0 + pos] = j;
+            b.val[slot0 + pos] = x;
+        } else {
+            atomicOr(b.status, 1u);
+        }
+        ++pos;
+        if (deliver) {
+            const bool l = (late >> k) & 1u;
+            deliver_pair(b, T + (l ? 1u : 0u), l ? next : early, j, __float_as_uint(x));
+            if (l) ++next;
+            else ++early;
+        }
+    }
+}
+
+template <typename GT>
+static cudaError_t launch_randk_typed(compams_context* c, const GT* grads, bool deliver) {
+    TopkBuffers b = c->tk;  // the kernels see this handle's own rows of the message buffers
+    b.idx += (size_t)c->row0 * (size_t)c->K;
+    b.val += (size_t)c->row0 * (size_t)c->K;
     const int64_t per_worker = (c->K + kThreads - 1) / kThreads;
-    const unsigned grid = (unsigned)(per_worker * c->n);
-    randk_emit_kernel<<<grid, kThreads, 0, c->stream>>>(c->tab, c->tk, c->row0, c->seed, c->iter, deliver ? 1 : 0);
-    return counted(c, cudaGetLastError());
+    cudaError_t e = cudaSuccess;
+    for (int32_t i0 = 0; i0 < c->n && e == cudaSuccess; i0 += c->randk_group) {
+        const int32_t rows = c->n - i0 < c->randk_group ? c->n - i0 : c->randk_group;
+        const int64_t origin = (int64_t)i0 * c->d & ~(int64_t)31;
+        e = counted(c, launch_after(randk_mark_kernel, dim3((unsigned)(per_worker * rows)), dim3(kThreads), c->stream, c->tab, b, c->row0,
+                                    i0, origin, c->seed, c->iter));
+        if (e != cudaSuccess) break;
+        void (*kernel)(const Tables, const TopkBuffers, const GT*, int32_t, int64_t, int64_t, int, const SegParams) =
+            c->K * 32 > c->d ? randk_sweep_kernel<GT, 256> : randk_sweep_kernel<GT, 128>;  // mean of a warp: K / d x 1024
+        e = counted(c, launch_after(kernel, dim3((unsigned)c->tab.ntiles, (unsigned)rows), dim3(kThreads), c->stream,
+                                    c->tab, b, grads, i0, origin, c->randk_words, deliver ? 1 : 0, c->segp));
+    }
+    return e;
+}
+
+cudaError_t launch_randk(compams_context* c, const void* grads, bool deliver) {
+    return c->grad_bf16 ? launch_randk_typed(c, (const bf16_bits*)grads, deliver) : launch_randk_typed(c, (const float*)grads, deliver);
 }
 
 }  // namespace compams
