@@ -212,11 +212,8 @@ __device__ __forceinline__ void topk_sweep_tile_bf16x8(const bf16_bits* __restri
 // Tiles are shifted down by (i d + o) mod 32, the position of the block's first element within a
 // 128-byte line of G and E, so that every warp access covers whole lines (with rows that start
 // mid-line a warp's 512 bytes straddle five lines instead of four: measured 7 % slower).
-#ifndef COMPAMS_BF16_TOPK_SWEEP_CTAS
-#define COMPAMS_BF16_TOPK_SWEEP_CTAS 5
-#endif
 template <typename GT, bool MANY>
-__global__ void __launch_bounds__(kThreads, sizeof(GT) == 2 || MANY ? COMPAMS_BF16_TOPK_SWEEP_CTAS : 6) topk_sweep_kernel(Tables t, TopkBuffers b, const GT* __restrict__ G,
+__global__ void __launch_bounds__(kThreads, sizeof(GT) == 2 ? 5 : 4) topk_sweep_kernel(Tables t, TopkBuffers b, const GT* __restrict__ G,
                                                                  const __grid_constant__ SegParams sp_) {
     dependency_wait();   // launched as a programmatic dependent while n d <= kChainMaxElems: the kernel before must be done
     allow_dependents();  // ... and the next one may move in behind this one's last wave
@@ -242,6 +239,13 @@ __global__ void __launch_bounds__(kThreads, sizeof(GT) == 2 || MANY ? COMPAMS_BF
     const int r0s = ti.r0 - (int)(row0 & 31);
     const float kept_from = __uint_as_float(b.use_thr ? b.thr[sg] : kNothingKept);
     const bool whole = r0s >= 0 && r0s + kTile <= ti.len;
+    // The tile's lines are asked into the L2 first: four CTAs per SM with registers to spare then do better than six that
+    // spill (ResNet-18 shapes whole, n = 16, 0.1 %: step 395.9 -> 388.5 us; the prefetch with six CTAs 401.5, three 389.1;
+    // with bfloat16 gradients 386 -> 392, so not there).
+    if (sizeof(GT) == 4 && whole) {
+        asm volatile("prefetch.global.L2 [%0];" ::"l"(e + r0s + warp * kWarpSpan + lane * 32));
+        asm volatile("prefetch.global.L2 [%0];" ::"l"(g + r0s + warp * kWarpSpan + lane * 32));
+    }
     bool wide = false;
     if constexpr (sizeof(GT) == 2)
         wide = whole && ((reinterpret_cast<uintptr_t>(g + r0s) | reinterpret_cast<uintptr_t>(e + r0s)) & 15u) == 0;
@@ -277,13 +281,10 @@ __global__ void __launch_bounds__(kThreads, sizeof(GT) == 2 || MANY ? COMPAMS_BF
 // segment. A list that cannot decide: the cluster goes through the block itself, or, where the block is too long for
 // its few CTAs, leaves it to the dense passes of the whole GPU. Lists come longest first, every worker's copy of one
 // block side by side: the clusters that take longest start first and the last wave holds the shortest.
-#ifndef SEL_NT
-#define SEL_NT 512
-#endif
-#ifndef SEL_CTAS
-#define SEL_CTAS 2
-#endif
-constexpr int kSelThreads = SEL_NT;
+// Two CTAs of 512 threads per SM, 64 registers: CTAs of 1024 threads were slower wherever more than one list is worked on
+// (ResNet-50 shapes layer-wise, n = 32: step 1760 -> 1800 us; n = 8, d = 2^20: 42 -> 54), three CTAs of 512 at 40 registers faster
+// layer-wise (1744) and slower for single lists (n = 4, d = 65,536: 17.5 -> 19.1).
+constexpr int kSelThreads = 512;
 
 template <int NT>
 __device__ __forceinline__ void start_select(SelectShared<NT>& sh) {
@@ -367,7 +368,7 @@ __device__ __forceinline__ void select_segment(Group grp, SelectShared<NT>& sh, 
 // seg_list: `nlong` blocks that a cluster selects from, then `nshort` that one CTA does; a cluster's CTAs take as many
 // of the latter as they are. `defer`: the long lists' entries are emitted by topk_emit.
 template <int NT>
-__global__ void __launch_bounds__(NT, SEL_CTAS) topk_select_kernel(const __grid_constant__ Tables t,
+__global__ void __launch_bounds__(NT, 2) topk_select_kernel(const __grid_constant__ Tables t,
                                                                    const __grid_constant__ TopkBuffers b,
                                                                    const int32_t* __restrict__ seg_list, int nlong, int nshort,
                                                                    int deliver, int defer) {
@@ -464,7 +465,7 @@ __device__ __forceinline__ void fused_span(const GT* __restrict__ g, float* __re
 }
 
 template <typename GT>
-__global__ void __launch_bounds__(kSelThreads, SEL_CTAS) topk_fused_kernel(const __grid_constant__ Tables t,
+__global__ void __launch_bounds__(kSelThreads, 2) topk_fused_kernel(const __grid_constant__ Tables t,
                                                                            const __grid_constant__ TopkBuffers b,
                                                                            const GT* __restrict__ G,
                                                                            const int32_t* __restrict__ seg_list, int nlong, int nshort,

@@ -1,0 +1,75 @@
+"""The ways a Top-k selection can be carried out (one kernel with the sweep, a CTA or a cluster per candidate list, a
+separate emission, passes over the block) at the sizes where one takes over from another, and Block-Sign at the edges of
+its own dispatch: against the oracle, index sets and sign bits exact, floats within the parity tolerance."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2205_05632_b200 import BLOCKSIGN, RANDK, TOPK
+from parity import Pair
+
+pytestmark = pytest.mark.gpu
+
+
+def run(n, offs, comp, ratio, draw, steps=5, seed=None):
+    d = int(offs[-1])
+    gen = torch.Generator(device="cuda").manual_seed(n * 1000003 + d)
+    p = Pair(n, d, offs, comp, ratio, seed=seed)
+    try:
+        p.start(0.1 * torch.randn(d, generator=gen, device="cuda"))
+        for t in range(steps):
+            p.step(draw(gen, n, d), check_e=t in (1, steps - 1))
+        return p.gpu.buffer("status").cpu().tolist()
+    finally:
+        p.close()
+
+
+def normal(gen, n, d):
+    return torch.randn(n, d, generator=gen, device="cuda")
+
+
+def levels(gen, n, d):  # few distinct magnitudes: thresholds shared by many entries
+    return torch.randint(-400, 401, (n, d), generator=gen, device="cuda").float()
+
+
+@pytest.mark.parametrize("n,offs", [
+    (1, [0, 8192]), (2, [0, 8193]), (4, [0, 65536]), (1, [0, 131072]), (9, [0, 131072]), (10, [0, 131072]), (1, [0, 131073]),
+    (3, [0, 1, 3, 2051, 2100, 4150, 12343, 12350, 30001]), (2, [0, 2048, 4097, 8193 + 4097]),
+    (5, list(np.cumsum([0] + [700 + 97 * k for k in range(40)]))),
+])
+@pytest.mark.parametrize("ratio", [0.01, 0.1, 0.3])
+@pytest.mark.parametrize("draw", [normal, levels])
+def test_sweep_and_selection_in_one_kernel(n, offs, ratio, draw):
+    run(n, offs, TOPK, ratio, draw, steps=4)
+
+
+@pytest.mark.parametrize("n,d,ratio", [
+    (1, (1 << 21) + 5, 0.1),    # list emitted by a kernel of its own, 16 CTAs
+    (2, 3000001, 0.111),        # the densest selection with a candidate list ...
+    (2, 3000001, 0.112),        # ... and one without: always the dense passes
+    (3, 1500003, 0.02), (16, 400001, 0.02), (1, 262144, 0.002), (7, 150001, 0.05),
+])
+@pytest.mark.parametrize("draw", [normal, levels])
+def test_long_lists(n, d, ratio, draw):
+    run(n, [0, d], TOPK, ratio, draw, steps=5)
+
+
+def test_long_and_short_lists_side_by_side():
+    sizes = [900001, 37, 4096, 4097, 600003, 20000, 1, 70001, 250007, 9000]
+    st = run(3, list(np.cumsum([0] + sizes)), TOPK, 0.04, normal, steps=6)
+    assert st[2] > st[1]  # most selections inside their lists
+
+
+@pytest.mark.parametrize("n,offs", [
+    (16, [0, 64 * 8192 - 31]), (17, [0, 64 * 8192 - 31]), (1, [0, 256 * 8192]), (1, [0, 256 * 8192 + 1]), (4, [0, 1, 2050, 6150, 10249]),
+    (25, [0, 3, 2049, 20001]), (2, [0, 5, 8197, 16391, 24601, 24603]),
+])
+def test_blocksign_scales_added_up_by_either_kernel(n, offs):
+    run(n, offs, BLOCKSIGN, 1.0, normal, steps=4)
+
+
+@pytest.mark.parametrize("n,offs,ratio", [
+    (3, [0, 31, 1055, 1056, 9300, 30011], 0.02), (2, [0, 20001], 0.25), (2, [0, 20001], 0.95), (4, [0, 1024, 2048, 10240], 0.125),
+])
+def test_randk_spans_that_share_words_and_overflow_their_room(n, offs, ratio):
+    run(n, offs, RANDK, ratio, normal, steps=4, seed=11)
