@@ -373,16 +373,11 @@ __global__ void __launch_bounds__(kThreads, 4) bs_apply_kernel(const __grid_cons
     const uint32_t bar = (uint32_t)__cvta_generic_to_shared(&sh.arrived);
     if (threadIdx.x == 0) {
         const uint32_t bytes = hi > lo ? (uint32_t)(hi - lo) * 4u : 0u;
-        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar) : "memory");
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(4u * bytes) : "memory");
+        mbar_init(bar);
+        mbar_expect(bar, 4u * bytes);
         if (bytes) {
 #pragma unroll
-            for (int q = 0; q < 4; ++q)
-                asm volatile("cp.async.bulk.shared::cta.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-                                 (uint32_t)__cvta_generic_to_shared(&sh.state[q][lo])),
-                             "l"(vec[q] + g0 + lo), "r"(bytes), "r"(bar)
-                             : "memory");
+            for (int q = 0; q < 4; ++q) bulk_load(&sh.state[q][lo], vec[q] + g0 + lo, bytes, bar);
         }
     }
     dependency_wait();  // the state was last written a step ago; sign words and scales are this step's
@@ -472,13 +467,7 @@ __global__ void __launch_bounds__(kThreads, 4) bs_apply_kernel(const __grid_cons
         }
     }
     __syncthreads();
-    uint32_t there = 0;
-    for (int tries = 0; tries < (1 << 16) && !there; ++tries)
-        asm volatile("{\n.reg .pred p;\nmbarrier.try_wait.parity.shared::cta.b64 p, [%1], 0;\nselp.u32 %0, 1, 0, p;\n}"
-                     : "=r"(there)
-                     : "r"(bar)
-                     : "memory");
-    if (!there) {  // cannot happen: the copies are this CTA's own
+    if (!mbar_wait(bar)) {  // cannot happen: the copies are this CTA's own
         atomicOr(b.status, 4u);
         return;
     }
