@@ -494,6 +494,7 @@ int step_device(compams_context* c, const void* grads, float* theta) {
         ++c->iter;
         return run_kernel(c, COMPAMS_K_DENSE_MEAN_AMSGRAD, [&] { return launch_dense_mean_amsgrad(c, grads, theta); });
     }
+    c->whole_step = true;
     RC(compress_device(c, grads));
     return apply_device(c, theta);
 }
@@ -593,6 +594,7 @@ static int compress_any(compams_handle c, const void* grads, bool bf16) {
     if (c->compressed) return COMPAMS_ERR_INVALID_ARG;  // the previous compress has not been applied yet
     RC(on_handle_device(c));
     c->grad_bf16 = bf16;
+    c->whole_step = false;
     int rc;
     try {
         rc = compress_device(c, grads);

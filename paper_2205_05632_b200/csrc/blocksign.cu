@@ -530,11 +530,11 @@ cudaError_t launch_bs_sweep(compams_context* c, const void* grads) {
 }
 
 // Whether bs_apply adds up the tile sums itself, and bs_scales is not launched: n = 4, d = 65,536 10.8 -> 9.7 us, n = 8,
-// d = 2^20 29.3 -> 27.5. Not before an exchange (the messages have to be complete), not for larger blocks, of which every
+// d = 2^20 29.3 -> 27.5. Not between compams_compress and compams_apply (the messages have to be complete), not for larger blocks, of which every
 // CTA would read more sums than its share of the rest, nor for many workers (n = 24, d = 3.3 M in 90 blocks: 194.4 us
 // with bs_scales, 198.3 without: a warp adds up one worker after the other).
 bool bs_apply_adds_up(const compams_context* c) {
-    return c->n == c->n_total && c->n <= 2 * kWarps && c->bs_max_tiles <= kWarpTiles && (int64_t)c->bs_max_tiles * c->n <= 1024;
+    return c->whole_step && c->n <= 2 * kWarps && c->bs_max_tiles <= kWarpTiles && (int64_t)c->bs_max_tiles * c->n <= 1024;
 }
 
 cudaError_t launch_bs_scales(compams_context* c) {

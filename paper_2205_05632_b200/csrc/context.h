@@ -162,6 +162,7 @@ struct compams_context {
     int scales_cur = 0;
     int bs_max_tiles = 0;     // Block-Sign: tiles of the longest block
     bool e_is_x = false;  // Block-Sign: E holds the corrected gradient x of the last step, not e
+    bool whole_step = false;  // the call being enqueued is a whole step: nobody looks at the messages before its server side
     bool compressed = false;  // compams_compress has run and its compams_apply has not: the step is half done
 
 

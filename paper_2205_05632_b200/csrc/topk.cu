@@ -4,30 +4,30 @@
 // Keys are the fp32 bit patterns of x = g + e with the sign cleared (31 bits); selection is a
 // most-significant-digit radix select over them.
 //
-//   Blocks of at most kSmallMax coordinates: topk_small - one CTA holds the block in shared
-//   memory and does every radix pass there; E is written once.
+//   Small problems: topk_fused - sweep and selection of one (worker, block) by one cluster, or one CTA.
+//
+//   Otherwise blocks of at most kSmallMax coordinates: topk_small - one CTA holds the block in shared
+//   memory and does every radix pass there; E is written once. It runs beside the tail of the sweep.
 //
 //   Larger blocks, cut into tiles of kTile coordinates.
-//   Candidate path (one pass over [n, d]):
+//   Candidate path (one pass over [n, d]), for blocks that keep at most 1/9 of their coordinates:
 //     topk_sweep    x = g + e written over E (Algorithm 2, the corrected-gradient step); every key >= tau_hat, a threshold
 //                   predicted from the previous step, is appended to the segment's candidate list
 //     topk_select   if the list holds at least k_b and at most its capacity, the exact Top-k is inside it.
 //                   A histogram of the key offsets above tau_hat (bins sized from the last step) finds
 //                   the threshold bin; winners above it are emitted, the bin's few candidates are
-//                   ordered by (key, lower index first), the best kept, and the next tau_hat predicted.
-//                   Otherwise the segment is marked for the dense passes. Short lists: one 1024-thread
-//                   CTA per list (topk_select). A few long lists (whole-vector selection): every list
-//                   is cut into slices handled by two kernels of ordinary CTAs (topk_selhist, topk_selemit)
-//                   that meet through a global histogram and last-slice-finishes tickets.
-//   Dense passes (only for marked segments; exact for any input, e.g. all-equal values), one
+//                   ordered by (key, lower index first), the best kept, and the next tau_hat predicted. One CTA or one
+//                   thread-block cluster per list (select.cuh).
+//     topk_emit     writes out the winners of lists so long that their clusters would take many rounds
+//   A list that cannot decide: its cluster goes through the block itself (select.cuh), or the segment is marked for the
+//   dense passes (exact for any input, e.g. all-equal values), one
 //   cooperative kernel topk_dense whose stages are separated by grid-wide barriers:
 //     hist<1..3> / find<1..3>  three histogram passes over x, 11 + 10 + 10 key bits
 //     collect       keys above the threshold are emitted; threshold ties too unless only some fit,
 //                   in which case they are counted per tile
 //     ties          takes the lowest-index threshold ties, tile by tile in index order
-//   topk_scatter    closes the step per segment (count check, counters reset) and walks the
-//                   (index, value) messages: each pair is appended to the bucket of its coordinate range
-//                   for the server kernel (the server's average)
+//   Whoever emits an (index, value) pair also appends it to the bucket of its coordinate range for the server kernel (the
+//   server's average); topk_scatter does that for the messages of a sharded job and of always dense selections.
 //   The residual update at a kept coordinate (e = x - x = 0) is deferred: E keeps x there, and every selection
 //   leaves one magnitude per segment such that the kept elements are exactly those with |x| at or above it;
 //   whoever reads E next - the next sweep, or topk_materialize - treats them as 0. Where a selection cuts through

@@ -5,7 +5,7 @@ import numpy as np
 import pytest
 import torch
 
-from paper_2205_05632_b200 import BLOCKSIGN, RANDK, TOPK
+from paper_2205_05632_b200 import BLOCKSIGN, RANDK, TOPK, CompAMS
 from parity import Pair
 
 pytestmark = pytest.mark.gpu
@@ -73,3 +73,28 @@ def test_blocksign_scales_added_up_by_either_kernel(n, offs):
 ])
 def test_randk_spans_that_share_words_and_overflow_their_room(n, offs, ratio):
     run(n, offs, RANDK, ratio, normal, steps=4, seed=11)
+
+
+@pytest.mark.parametrize("comp", [TOPK, BLOCKSIGN, RANDK])
+def test_messages_are_complete_between_the_two_halves_of_a_step(comp):
+    # whatever a whole step leaves to its server side, compress() alone leaves what the step would have sent
+    n, offs = 3, [0, 5, 8197, 24601]
+    d = offs[-1]
+    gen = torch.Generator(device="cuda").manual_seed(5)
+    a, b = CompAMS(n, d, offs, comp, 0.02), CompAMS(n, d, offs, comp, 0.02)
+    ta, tb = torch.zeros(d, device="cuda"), torch.zeros(d, device="cuda")
+    for _ in range(3):
+        G = torch.randn(n, d, generator=gen, device="cuda")
+        a.step(G, ta)
+        b.compress(G)
+        first, second = (m.clone() for m in b.message_buffers())
+        b.apply(tb)
+        want, want2 = a.message_buffers()
+        if comp != BLOCKSIGN:  # the pairs of a segment come in any order
+            order, order_w = torch.argsort(first, 1), torch.argsort(want, 1)
+            first, second = first.gather(1, order), second.gather(1, order)
+            want, want2 = want.gather(1, order_w), want2.gather(1, order_w)
+        assert torch.equal(first, want) and torch.equal(second, want2)
+        assert torch.equal(ta, tb)
+    a.close()
+    b.close()
