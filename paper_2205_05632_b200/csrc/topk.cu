@@ -368,7 +368,7 @@ __device__ __forceinline__ void select_segment(Group grp, SelectShared<NT>& sh, 
 // seg_list: `nlong` blocks that a cluster selects from, then `nshort` that one CTA does; a cluster's CTAs take as many
 // of the latter as they are. `defer`: the long lists' entries are emitted by topk_emit.
 template <int NT>
-__global__ void __launch_bounds__(NT, 2) topk_select_kernel(const __grid_constant__ Tables t,
+__global__ void __launch_bounds__(NT, 1024 / NT) topk_select_kernel(const __grid_constant__ Tables t,
                                                                    const __grid_constant__ TopkBuffers b,
                                                                    const int32_t* __restrict__ seg_list, int nlong, int nshort,
                                                                    int deliver, int defer) {
@@ -1120,9 +1120,15 @@ static cudaError_t allow_large_cluster(K* kernel, int cluster) {
 
 cudaError_t launch_topk_select(compams_context* c) {
     const int64_t clusters = (int64_t)c->n * c->sel_long + ((int64_t)c->n * c->sel_short + c->sel_cluster - 1) / c->sel_cluster;
-    cudaError_t e = allow_large_cluster(topk_select_kernel<kSelThreads>, c->sel_cluster);
+    // A handful of long lists that are only counted here: twice the threads per CTA (n = 1, d = 28.5 M, 1 %: 241.2 -> 236.2 us;
+    // n = 2, d = 4.4 M, 7.85 %: 91.6 -> 89.0; n = 5, d = 9.3 M, 2 %: 179.2 -> 177.2; but eight lists, n = 8, d = 4.2 M, 10 %: 163.9 ->
+    // 172.0)
+    const bool wide = c->sel_parts && c->sel_cluster == 16 && (int64_t)c->n * c->sel_long <= 5;
+    void (*kernel)(const Tables, const TopkBuffers, const int32_t*, int, int, int, int) =
+        wide ? topk_select_kernel<2 * kSelThreads> : topk_select_kernel<kSelThreads>;
+    cudaError_t e = allow_large_cluster(kernel, c->sel_cluster);
     if (e != cudaSuccess) return e;
-    e = counted(c, launch_cluster(topk_select_kernel<kSelThreads>, dim3((unsigned)(clusters * c->sel_cluster)), dim3(kSelThreads),
+    e = counted(c, launch_cluster(kernel, dim3((unsigned)(clusters * c->sel_cluster)), dim3(wide ? 2 * kSelThreads : kSelThreads),
                                   c->sel_cluster, c->chain, c->stream, c->tab, own_rows(c), (const int32_t*)c->sel_segs, c->sel_long,
                                   c->sel_short, c->deliver ? 1 : 0, c->sel_parts ? 1 : 0));
     if (e != cudaSuccess || !c->sel_parts) return e;
