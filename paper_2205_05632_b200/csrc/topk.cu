@@ -523,6 +523,7 @@ __global__ void __launch_bounds__(kThreads) topk_emit_kernel(const __grid_consta
                                                              int deliver) {
     __shared__ uint2 surv[kSurvCap], few[kSurvCap];
     __shared__ uint32_t hist[kThreads], scratch[kWarps], sh_bin[2], sh_above, sh_in;
+    __shared__ uint32_t sh_wins, sh_first, sh_taken;
     __shared__ int is_last;
     // all lists' first parts first: the workers' entries of one coordinate range then reach its bucket close in time
     const unsigned lists = (unsigned)(t.n * nlong), item = blockIdx.x % lists, part = blockIdx.x / lists;
@@ -546,9 +547,25 @@ __global__ void __launch_bounds__(kThreads) topk_emit_kernel(const __grid_consta
     for (uint32_t p0 = part * (ListSlice::kU * kThreads); p0 < c; p0 += (uint32_t)parts * (ListSlice::kU * kThreads)) {
         uint2 cv[ListSlice::kU];
         sl.load<kThreads>(p0, cv);
+        // a round's winners are counted first and get their slots with one atomic on the list's counter (one per warp: n = 3,
+        // d = 117 M, 3.95 % 1573 us against 1496; n = 8, d = 4.2 M, 10 % 163.9 against 162.5)
+        if (threadIdx.x == 0) sh_wins = 0u;
+        __syncthreads();
+        uint32_t wins = 0;
+#pragma unroll
+        for (int u = 0; u < ListSlice::kU; ++u) wins += cv[u].y != kNoCandidate && (cv[u].y & 0x7fffffffu) >= win_from ? 1u : 0u;
+        wins = __reduce_add_sync(0xffffffffu, wins);
+        if ((threadIdx.x & 31) == 0 && wins) atomicAdd(&sh_wins, wins);
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            sh_first = atomicAdd(&st->emit_count, sh_wins);
+            sh_taken = 0u;
+        }
+        __syncthreads();
 #pragma unroll
         for (int h = 0; h < ListSlice::kU; h += 4)
-            emit<4>(b, job, 0u, &st->emit_count, gsurv, nsurv, cv + h, win_from, bin_from);
+            emit<4>(b, job, sh_first, &sh_taken, gsurv, nsurv, cv + h, win_from, bin_from);
+        __syncthreads();
     }
     __threadfence();
     __syncthreads();
