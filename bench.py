@@ -68,8 +68,8 @@ def measured_peak_gbs():
 # None is reported. The kernel's code is the stretch of its file between the two markers (the kernel with the
 # device functions it alone uses) plus the shared helper header.
 TRAFFIC_PER_ELEM = {
-    "topk_sweep": (1599850752 / 134217728, "topk.cu", ("constexpr uint32_t kNothingKept", "void predict_next("),
-                   "b1b2c4af58fd5755"),
+    "topk_sweep": (1576586752 / 134217728, "topk.cu", ("constexpr uint32_t kNothingKept", "// select: exact Top-k inside the candidate list"),
+                   "e86d5d79e9d70373"),
 }
 
 
