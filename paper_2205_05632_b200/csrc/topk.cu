@@ -918,7 +918,7 @@ __device__ __forceinline__ void close_segment(const TopkBuffers& b, const SegInf
 
 // All dense passes in one cooperative launch: the grid is resident as a whole and the passes are
 // separated by grid-wide barriers. When no segment is marked every CTA returns at once, so in the
-// steady state the dense path costs one empty launch per step.
+// steady state the dense path costs one empty launch per step, where it is launched at all.
 __global__ void __launch_bounds__(kThreads) topk_dense_kernel(Tables t, TopkBuffers b, int deliver) {
     __shared__ uint32_t sh[kBins1];
     __shared__ uint32_t scratch[kWarps];
