@@ -89,10 +89,11 @@ enum compams_kernel {
     COMPAMS_K_TOPK_MATERIALIZE = 6,   /* Top-k: zero e at the coordinates kept in the last step when E is read   */
     COMPAMS_K_RANDK_EMIT = 7,         /* Random-k: marks the drawn coordinates, then the sweep that takes their x */
     /* 8: reserved (never returned, never timed) */
-    COMPAMS_K_TOPK_SCATTER = 9,       /* Top-k: closes the step per segment; sparse scatter-accumulate         */
+    COMPAMS_K_TOPK_SCATTER = 9,       /* sharded jobs, always dense selections: messages to the server's buckets */
     COMPAMS_K_AMSGRAD = 10,           /* Top-k: AMSGrad update from the accumulated average                   */
     COMPAMS_K_TOPK_SMALL = 11,        /* Top-k: whole small blocks selected inside shared memory              */
-    COMPAMS_K_TOPK_SELECT = 12,       /* Top-k: exact selection inside the candidate lists                    */
+    COMPAMS_K_TOPK_SELECT = 12,       /* Top-k: exact selection inside the candidate lists, the emission of long
+                                         ones included; small problems: sweep and selection in one kernel     */
     COMPAMS_K_BS_SCALES = 13,         /* Block-Sign: scale of every (worker, block) from the tile sums        */
     COMPAMS_K_COUNT = 14
 };
@@ -345,7 +346,8 @@ int compams_get_buffer(compams_handle h, int32_t which, void** dev_ptr, int64_t*
 
 /* compams_check_status - synchronise the handle's stream, read the device status word and any
  * pending CUDA error. Returns OK, ERR_CUDA or ERR_DEVICE_STATUS; *status_word (host, may be null)
- * receives the raw word (bit 0: a Top-k segment emitted a wrong number of entries). */
+ * receives the raw word (bit 0: a segment emitted a wrong number of entries,
+ * bit 2: a server kernel gave up waiting for its own copies). */
 int compams_check_status(compams_handle h, uint32_t* status_word);
 
 /*
