@@ -380,8 +380,10 @@ __device__ __forceinline__ bool select_slices(const Group& grp, const TopkBuffer
         locate_bins<NT>(grp, sh, edge_need, 0u);
         out.edge += sh.bin[0] << s;
     }
-    const unsigned long long beyond = (unsigned long long)from + (1ull << S);
-    const uint32_t win_from = take_all ? from : beyond < 0x7f800000ull ? (uint32_t)beyond : 0x7f800000u;
+    // Keys have 31 bits, the bin holds one of them and S <= 21: the sum fits. Nothing may be cut off at the key of infinity:
+    // when the bin lies at or above it (k_b gradients and more that are infinite or NaN) its entries would be emitted as
+    // winners, and the ranking would read survivors that nobody has written.
+    const uint32_t win_from = take_all ? from : from + (1u << S);
     if (job.defer) {
         out.kept_from = win_from;
         out.tau = from;

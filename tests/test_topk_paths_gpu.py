@@ -98,3 +98,41 @@ def test_messages_are_complete_between_the_two_halves_of_a_step(comp):
         assert torch.equal(ta, tb)
     a.close()
     b.close()
+
+
+@pytest.mark.parametrize("n,offs,ratio", [
+    (2, [0, 1500], 0.02), (2, [0, 300, 40300], 0.02),                # one kernel: blocks without and with a list
+    (16, [0, 400001], 0.02), (1, [0, (1 << 21) + 5], 0.1),           # clusters; a list emitted by a kernel of its own
+    (3, [0, 600003, 604099, 1504100], 0.01),                         # clusters, one CTA per list, a block in shared memory
+])
+@pytest.mark.parametrize("bad", [float("inf"), float("nan")])
+@pytest.mark.parametrize("share", [1.2, 3.0, 1e9])  # of k_b: coordinates that are not finite (1e9: all of them)
+def test_gradients_that_are_not_finite_select_by_key_and_index(n, offs, ratio, bad, share):
+    # an overflow in a mixed-precision step: more such values in a block than it keeps, in the step after the first (whose
+    # selection has a list) and in the first one. Which are kept is unspecified for the caller; here: the lowest indices
+    d = offs[-1]
+    gen = torch.Generator(device="cuda").manual_seed(d)
+    for good_steps in (0, 3):
+        opt = CompAMS(n, d, offs, TOPK, ratio)
+        theta = torch.zeros(d, device="cuda")
+        for _ in range(good_steps):
+            opt.step(torch.randn(n, d, generator=gen, device="cuda"), theta)
+        G = torch.randn(n, d, generator=gen, device="cuda")
+        want = torch.zeros(n, d, dtype=torch.bool, device="cuda")
+        for lo, hi in zip(offs, offs[1:]):
+            k = max(1, int(ratio * (hi - lo)))
+            count = min(hi - lo, int(share * k) + 1)
+            for i in range(n):
+                where = lo + torch.randperm(hi - lo, generator=gen, device="cuda")[:count].sort().values
+                G[i, where] = bad
+                want[i, where[:k]] = True
+        opt.step(G, theta)
+        assert opt.check_status() == 0
+        idx = opt.buffer("topk_idx").long()
+        got = torch.zeros(n, d, dtype=torch.int32, device="cuda")
+        got.scatter_add_(1, idx, torch.ones_like(idx, dtype=torch.int32))
+        assert torch.equal(got, want.int())
+        for _ in range(2):  # the handle goes on
+            opt.step(torch.randn(n, d, generator=gen, device="cuda"), theta)
+            assert opt.check_status() == 0
+        opt.close()
