@@ -324,10 +324,11 @@ __device__ __forceinline__ SelectJob select_job(const Tables& t, const TopkBuffe
     return job;
 }
 
-// Called by all threads of the group; CTAs that have nothing to do return early.
+// Called by all threads of the group. `state_read`: a barrier of the group lies between its CTAs' reads of `s` and this call.
 template <int NT>
 __device__ __forceinline__ void select_segment(Group grp, SelectShared<NT>& sh, const Tables& t, const TopkBuffers& b,
-                                               const SegInfo& si, int i, int seg, const SelectState& s, bool deliver, bool defer) {
+                                               const SegInfo& si, int i, int seg, const SelectState& s, bool state_read, bool deliver,
+                                               bool defer) {
     const size_t sg = (size_t)i * t.nseg + seg;
     SegState* st = b.seg + sg;
     const unsigned ctas = grp.size;
@@ -337,7 +338,11 @@ __device__ __forceinline__ void select_segment(Group grp, SelectShared<NT>& sh, 
     int why = s.c < si.kb ? 3 : 4;
     if (s.tau_hat != kNoPrediction && s.c >= si.kb && s.c <= si.cap) {
         if (s.c <= (uint32_t)(ListSlice::kU * NT) && ctas > 1) {  // a short list: barriers of the cluster would cost more
-            if (grp.rank) return;                                  // than the other CTAs save
+            // than the other CTAs save. The first, alone from here on, will leave the next step's state in the words that
+            // they decide by: all must have read them (a CTA that came late would take the list for one that cannot decide,
+            // and meet the others in shared memory they have given up)
+            if (!state_read) grp.sync();
+            if (grp.rank) return;
             grp.size = 1;
         } else {
             job.defer = defer;
@@ -393,7 +398,7 @@ __global__ void __launch_bounds__(NT, 1024 / NT) topk_select_kernel(const __grid
     allow_dependents();  // ... and the next one may move in behind this one's last wave
     if (idle) return;
     const SelectState s = load_state(b.seg + (size_t)i * t.nseg + seg);
-    select_segment<NT>(grp, sh, t, b, si, i, seg, s, deliver != 0, defer != 0 && !alone);
+    select_segment<NT>(grp, sh, t, b, si, i, seg, s, false, deliver != 0, defer != 0 && !alone);
 }
 
 // Sweep and selection in one kernel, for problems so small that launches and latency are what a step costs: a cluster, or one CTA, takes one (worker, block), forms x = g + e, lists the candidates and selects
@@ -512,7 +517,7 @@ __global__ void __launch_bounds__(kSelThreads, 2) topk_fused_kernel(const __grid
     }
     grp.sync();  // the list and x are complete
     s.c = *listed;
-    select_segment<NT>(grp, sh, t, b, si, i, seg, s, deliver != 0, false);
+    select_segment<NT>(grp, sh, t, b, si, i, seg, s, true, deliver != 0, false);
 }
 
 // Emission of long lists that topk_select has found the threshold of: `parts` CTAs stream through each list, the winners
