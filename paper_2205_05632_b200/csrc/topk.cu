@@ -337,23 +337,23 @@ __device__ __forceinline__ void select_segment(Group grp, SelectShared<NT>& sh, 
     // the same decision in every CTA of the group: nobody writes these words before all have read them
     int why = s.c < si.kb ? 3 : 4;
     if (s.tau_hat != kNoPrediction && s.c >= si.kb && s.c <= si.cap) {
-        if (s.c <= (uint32_t)(ListSlice::kU * NT) && ctas > 1) {  // a short list: barriers of the cluster would cost more
-            // than the other CTAs save. The first, alone from here on, will leave the next step's state in the words that
-            // they decide by: all must have read them (a CTA that came late would take the list for one that cannot decide,
-            // and meet the others in shared memory they have given up)
-            if (!state_read) grp.sync();
-            if (grp.rank) return;
-            grp.size = 1;
-        } else {
-            job.defer = defer;
+        // a short list: barriers of the cluster would cost more than the other CTAs save, the first takes it alone. They
+        // wait for its verdict: a list that cannot decide needs all of them for the block.
+        const bool by_first = ctas > 1 && s.c <= (uint32_t)(ListSlice::kU * NT);
+        // the first will leave the next step's state in the words that they decide by: all must have read them
+        if (by_first && !state_read) grp.sync();
+        bool decided = false;
+        if (!by_first || grp.rank == 0) {
+            job.defer = defer && !by_first;
+            const uint2* list = b.cand + (size_t)i * (size_t)b.cand_total + (size_t)si.cand_off;
+            decided = select_from_list<NT>(by_first ? Group{1u, 0u} : grp, b, job, sh, st, b.thr + sg, list, s.c, s.tau_hat, s.S, s.boost,
+                                           &why);
+            job.defer = false;
+            if (by_first && threadIdx.x < ctas) *grp.of(&sh.decided, threadIdx.x) = decided ? 1u : 0u;
         }
-        const uint2* list = b.cand + (size_t)i * (size_t)b.cand_total + (size_t)si.cand_off;
-        if (select_from_list<NT>(grp, b, job, sh, st, b.thr + sg, list, s.c, s.tau_hat, s.S, s.boost, &why)) {
-            // the first CTA's shared memory stays until all have read from it (CTAs that have returned count as arrived)
-            if (ctas > 1) cg::this_cluster().sync();
-            return;
-        }
-        job.defer = false;
+        // the first CTA's shared memory stays until all have read from it
+        if (ctas > 1 && (by_first || decided)) cg::this_cluster().sync();
+        if (by_first ? sh.decided != 0u : decided) return;
     }
     if (first && s.tau_hat != kNoPrediction && si.cap) atomicAdd(b.status + why, 1u);
     if ((int64_t)si.len <= (int64_t)b.cluster_max * ctas) {

@@ -5,6 +5,7 @@ import numpy as np
 import pytest
 import torch
 
+import oracle
 from paper_2205_05632_b200 import BLOCKSIGN, RANDK, TOPK, CompAMS
 from parity import Pair
 
@@ -136,3 +137,30 @@ def test_gradients_that_are_not_finite_select_by_key_and_index(n, offs, ratio, b
             opt.step(torch.randn(n, d, generator=gen, device="cuda"), theta)
             assert opt.check_status() == 0
         opt.close()
+
+
+@pytest.mark.parametrize("n,d,ratio,count", [(1, 131072, 0.02, 2800), (4, 65536, 0.02, 1500), (1, 400001, 0.009, 3700)])
+def test_a_short_list_that_cannot_decide_leaves_the_block_to_its_whole_cluster(n, d, ratio, count):
+    # a list of at most 4096 entries, which the first CTA of a cluster takes alone, whose k_b-th largest key lies beyond its
+    # histogram: `count` nearly all equal magnitudes far above the last threshold. The lowest indices win
+    gen = torch.Generator(device="cuda").manual_seed(d)
+    opt = CompAMS(n, d, [0, d], TOPK, ratio)
+    theta = torch.zeros(d, device="cuda")
+    k = int(ratio * d)
+    assert k < count <= 4096
+    for _ in range(12):
+        opt.step(torch.randn(n, d, generator=gen, device="cuda"), theta)
+    before = opt.buffer("status").cpu().tolist()
+    e = opt.buffer("E").clone()
+    G = -e
+    for i in range(n):
+        where = torch.randperm(d, generator=gen, device="cuda")[:count]
+        G[i, where] += 1024.0  # x = (1024 - e) + e is 1024 but for the rounding of the difference, elsewhere it is 0
+    x = (G + e).cpu().numpy()
+    opt.step(G, theta)
+    after = opt.buffer("status").cpu().tolist()
+    assert after[0] == 0 and after[1] - before[1] == n and after[5] - before[5] == n
+    idx = np.sort(opt.buffer("topk_idx").cpu().numpy(), axis=1)
+    for i in range(n):
+        assert np.array_equal(idx[i], np.flatnonzero(oracle.topk_keep_mask(x[i], k)))
+    opt.close()
