@@ -338,7 +338,7 @@ int init_context(compams_context* c, const int64_t* block_offsets) {
             RC(dev_upload(c, &t.seg, seg0));
             c->seg_init_host = seg0;
             c->dense_count_init = never;
-            c->deliver = !c->randk && n == c->n_total && never == 0;
+            c->deliver = n == c->n_total && never == 0;
             std::vector<uint32_t> dc(1, never);
             RC(dev_upload(c, &t.dense_count, dc));
         }
@@ -456,9 +456,8 @@ int compress_device(compams_context* c, const void* grads) {
     // when E is next read (by the next sweep, or by topk_materialize when the caller asks for E)
     c->tk.use_thr = c->e_mask_pending ? 1 : 0;
     if (c->randk) {
-        // no selection: the drawn coordinates are marked, and the sweep takes them; with all workers in this handle the
-        // pairs go to the server in the same kernel, otherwise compams_apply delivers the exchanged messages
-        RC(run_kernel(c, COMPAMS_K_RANDK_EMIT, [&] { return launch_randk(c, grads, c->n == c->n_total); }));
+        // no selection: the drawn coordinates are marked, and the sweep takes them
+        RC(run_kernel(c, COMPAMS_K_RANDK_EMIT, [&] { return launch_randk(c, grads); }));
         return COMPAMS_OK;
     }
     if (c->fused) {
@@ -481,9 +480,8 @@ int apply_device(compams_context* c, float* theta) {
     if (c->compressor == COMPAMS_BLOCKSIGN) {
         return run_kernel(c, COMPAMS_K_BS_APPLY, [&] { return launch_bs_apply(c, theta); });
     }
-    // (with every worker in this handle Random-k and most selections have delivered their messages already)
-    if (!(c->deliver || (c->randk && c->n == c->n_total)))
-        RC(run_kernel(c, COMPAMS_K_TOPK_SCATTER, [&] { return launch_topk_scatter(c); }));
+    // (in a whole step Random-k and most selections have delivered their messages already)
+    if (!delivers(c)) RC(run_kernel(c, COMPAMS_K_TOPK_SCATTER, [&] { return launch_topk_scatter(c); }));
     RC(run_kernel(c, COMPAMS_K_AMSGRAD, [&] { return launch_amsgrad(c, theta); }));
     return COMPAMS_OK;
 }

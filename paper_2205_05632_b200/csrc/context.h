@@ -152,7 +152,7 @@ struct compams_context {
     int64_t randk_words = 0;       // ... its words
     bool many_candidates = false;  // Top-k: the lists hold more than 1/32 of the coordinates
     bool dense_kernel = false;  // some blocks are too long for a cluster to go through: the dense passes are launched every step
-    bool deliver = false;       // the selection hands the kept entries to the server itself (no topk_scatter)
+    bool deliver = false;       // in a whole step the worker side hands the kept entries to the server itself (no topk_scatter)
     std::vector<compams::SegState> seg_init_host;  // Top-k: the segments' state before the first step (set_state restores it)
     uint32_t dense_count_init = 0;
     uint64_t steps_done = 0;
@@ -198,6 +198,10 @@ inline cudaError_t counted(compams_context* c, cudaError_t e) {
     return e;
 }
 
+// Whether the worker side of the call being enqueued hands the kept entries to the server's buckets. Not between
+// compams_compress and compams_apply: the server then averages what it finds in the message buffers.
+inline bool delivers(const compams_context* c) { return c->deliver && c->whole_step; }
+
 // Each launcher enqueues its kernel(s) on ctx->stream and returns the launch status.
 cudaError_t launch_dense_mean_amsgrad(compams_context* c, const void* grads, float* theta);
 cudaError_t launch_bs_sweep(compams_context* c, const void* grads);
@@ -212,7 +216,7 @@ cudaError_t launch_topk_fused(compams_context* c, const void* grads);
 cudaError_t launch_topk_dense(compams_context* c);
 cudaError_t launch_topk_materialize(compams_context* c);
 cudaError_t launch_topk_scatter(compams_context* c);
-cudaError_t launch_randk(compams_context* c, const void* grads, bool deliver);
+cudaError_t launch_randk(compams_context* c, const void* grads);
 cudaError_t launch_amsgrad(compams_context* c, float* theta);
 
 }  // namespace compams

@@ -370,7 +370,7 @@ __global__ void __launch_bounds__(kThreads, 4) randk_sweep_kernel(
 }
 
 template <typename GT>
-static cudaError_t launch_randk_typed(compams_context* c, const GT* grads, bool deliver) {
+static cudaError_t launch_randk_typed(compams_context* c, const GT* grads) {
     TopkBuffers b = c->tk;  // the kernels see this handle's own rows of the message buffers
     b.idx += (size_t)c->row0 * (size_t)c->K;
     b.val += (size_t)c->row0 * (size_t)c->K;
@@ -385,13 +385,13 @@ static cudaError_t launch_randk_typed(compams_context* c, const GT* grads, bool 
         void (*kernel)(const Tables, const TopkBuffers, const GT*, int32_t, int64_t, int64_t, int, const SegParams) =
             c->K * 32 > c->d ? randk_sweep_kernel<GT, 256> : randk_sweep_kernel<GT, 128>;  // mean of a warp: K / d x 1024
         e = counted(c, launch_after(kernel, dim3((unsigned)c->tab.ntiles, (unsigned)rows), dim3(kThreads), c->stream,
-                                    c->tab, b, grads, i0, origin, c->randk_words, deliver ? 1 : 0, c->segp));
+                                    c->tab, b, grads, i0, origin, c->randk_words, delivers(c) ? 1 : 0, c->segp));
     }
     return e;
 }
 
-cudaError_t launch_randk(compams_context* c, const void* grads, bool deliver) {
-    return c->grad_bf16 ? launch_randk_typed(c, (const bf16_bits*)grads, deliver) : launch_randk_typed(c, (const float*)grads, deliver);
+cudaError_t launch_randk(compams_context* c, const void* grads) {
+    return c->grad_bf16 ? launch_randk_typed(c, (const bf16_bits*)grads) : launch_randk_typed(c, (const float*)grads);
 }
 
 }  // namespace compams

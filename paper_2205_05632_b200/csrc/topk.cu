@@ -1109,7 +1109,7 @@ template <typename GT>
 static cudaError_t launch_small_typed(compams_context* c, const GT* grads) {
     const dim3 grid((unsigned)c->tk.nsmall, (unsigned)c->n);
     return counted(c, launch_after(topk_small_kernel<GT>, grid, dim3(kThreads), c->stream, c->tab, own_rows(c), grads,
-                                   c->deliver ? 1 : 0, c->tab.ntiles > 0 ? 1 : 0));
+                                   delivers(c) ? 1 : 0, c->tab.ntiles > 0 ? 1 : 0));
 }
 
 cudaError_t launch_topk_small(compams_context* c, const void* grads) {
@@ -1152,13 +1152,13 @@ cudaError_t launch_topk_select(compams_context* c) {
     if (e != cudaSuccess) return e;
     e = counted(c, launch_cluster(kernel, dim3((unsigned)(clusters * c->sel_cluster)), dim3(wide ? 2 * kSelThreads : kSelThreads),
                                   c->sel_cluster, c->chain, c->stream, c->tab, own_rows(c), (const int32_t*)c->sel_segs, c->sel_long,
-                                  c->sel_short, c->deliver ? 1 : 0, c->sel_parts ? 1 : 0));
+                                  c->sel_short, delivers(c) ? 1 : 0, c->sel_parts ? 1 : 0));
     if (e != cudaSuccess || !c->sel_parts) return e;
     const dim3 grid((unsigned)((int64_t)c->n * c->sel_long * c->sel_parts));
     if (c->chain)
         return counted(c, launch_after(topk_emit_kernel, grid, dim3(kThreads), c->stream, c->tab, own_rows(c),
-                                       (const int32_t*)c->sel_segs, c->sel_long, c->sel_parts, c->deliver ? 1 : 0));
-    topk_emit_kernel<<<grid, kThreads, 0, c->stream>>>(c->tab, own_rows(c), c->sel_segs, c->sel_long, c->sel_parts, c->deliver ? 1 : 0);
+                                       (const int32_t*)c->sel_segs, c->sel_long, c->sel_parts, delivers(c) ? 1 : 0));
+    topk_emit_kernel<<<grid, kThreads, 0, c->stream>>>(c->tab, own_rows(c), c->sel_segs, c->sel_long, c->sel_parts, delivers(c) ? 1 : 0);
     return counted(c, cudaGetLastError());
 }
 
@@ -1169,7 +1169,7 @@ static cudaError_t launch_fused_typed(compams_context* c, const GT* grads) {
     if (e != cudaSuccess) return e;
     return counted(c, launch_cluster(topk_fused_kernel<GT>, dim3((unsigned)(clusters * c->sel_cluster)), dim3(kSelThreads), c->sel_cluster,
                                      true, c->stream, c->tab, own_rows(c), grads, (const int32_t*)c->sel_segs, c->sel_long, c->sel_short,
-                                     c->deliver ? 1 : 0));
+                                     delivers(c) ? 1 : 0));
 }
 
 cudaError_t launch_topk_fused(compams_context* c, const void* grads) {
@@ -1185,7 +1185,7 @@ cudaError_t launch_topk_dense(compams_context* c) {
         c->dense_grid = per_sm * c->num_sms;  // every CTA resident at once, as a cooperative launch requires
     }
     TopkBuffers b = own_rows(c);
-    int deliver = c->deliver ? 1 : 0;
+    int deliver = delivers(c) ? 1 : 0;
     void* args[] = {(void*)&c->tab, (void*)&b, (void*)&deliver};
     return counted(c, cudaLaunchCooperativeKernel((const void*)topk_dense_kernel, dim3((unsigned)c->dense_grid),
                                                   dim3(kThreads), args, 0, c->stream));

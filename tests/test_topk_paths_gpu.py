@@ -7,7 +7,7 @@ import torch
 
 import oracle
 from paper_2205_05632_b200 import BLOCKSIGN, RANDK, TOPK, CompAMS
-from parity import Pair
+from parity import Pair, close, unpack_sign_bits
 
 pytestmark = pytest.mark.gpu
 
@@ -163,4 +163,35 @@ def test_a_short_list_that_cannot_decide_leaves_the_block_to_its_whole_cluster(n
     idx = np.sort(opt.buffer("topk_idx").cpu().numpy(), axis=1)
     for i in range(n):
         assert np.array_equal(idx[i], np.flatnonzero(oracle.topk_keep_mask(x[i], k)))
+    opt.close()
+
+
+@pytest.mark.parametrize("n,offs,ratio", [(3, [0, 5, 8197, 24601], 0.02), (2, [0, 900001], 0.01), (2, [0, 3000, 900001], 0.3)])
+@pytest.mark.parametrize("comp", [TOPK, BLOCKSIGN, RANDK])
+def test_apply_averages_what_the_message_buffers_hold(n, offs, ratio, comp):
+    # the caller works on the messages between the two halves: one worker dropped, another's values halved
+    d = offs[-1]
+    gen = torch.Generator(device="cuda").manual_seed(9)
+    opt = CompAMS(n, d, offs, comp, ratio, record_average=True)
+    theta = 0.1 * torch.randn(d, generator=gen, device="cuda")
+    want = {"theta": theta.cpu().numpy().copy(), **{k: np.zeros(d, dtype=np.float32) for k in ("m", "v", "vhat")}}
+    for t in range(4):
+        opt.compress(torch.randn(n, d, generator=gen, device="cuda"))
+        first, second = opt.message_buffers()
+        second[0] *= 0.5
+        second[n - 1] = 0.0
+        C = np.zeros((n, d), dtype=np.float64)
+        if comp == BLOCKSIGN:
+            signs = unpack_sign_bits(first.cpu().numpy(), opt.buffer("sign_word_offsets").cpu().numpy(), np.asarray(offs))
+            C[:] = np.where(signs, -1.0, 1.0) * np.repeat(second.cpu().numpy(), np.diff(offs), axis=1)
+        else:
+            np.put_along_axis(C, first.cpu().numpy().astype(np.int64), second.cpu().numpy().astype(np.float64), 1)
+        opt.apply(theta)
+        gbar = C.sum(0).astype(np.float32) / np.float32(n)
+        oracle.amsgrad(gbar, want["m"], want["v"], want["vhat"], want["theta"], 1e-3, 0.9, 0.999, 1e-8)
+        close(opt.buffer("gbar"), gbar, "gbar", t)
+        close(theta, want["theta"], "theta", t)
+        for name in ("m", "v", "vhat"):
+            close(opt.buffer(name), want[name], name, t)
+        assert opt.check_status() == 0
     opt.close()
