@@ -555,9 +555,9 @@ cudaError_t launch_bs_apply(compams_context* c, float* theta) {
     void (*kernel)(const Tables, const BsBuffers, float*, const HyperParams, const SegParams) =
         own ? (b.gbar ? bs_apply_kernel<true, true> : bs_apply_kernel<false, true>)
             : (b.gbar ? bs_apply_kernel<true, false> : bs_apply_kernel<false, false>);
-    if (c->n == c->n_total) return counted(c, launch_after(kernel, grid, dim3(kThreads), c->stream, t, b, theta, c->hp, c->segp));
-    // sharded workers: the other workers' messages were written by the caller's exchange, which is
-    // ordered on the stream like any kernel; a plain launch waits for it
+    if (c->whole_step) return counted(c, launch_after(kernel, grid, dim3(kThreads), c->stream, t, b, theta, c->hp, c->segp));
+    // between compams_compress and compams_apply the caller may have put work on the stream that writes the messages, theta
+    // or both, and the kernel reads theta ahead of its wait: a plain launch comes after that work
     kernel<<<grid, dim3(kThreads), 0, c->stream>>>(t, b, theta, c->hp, c->segp);
     return counted(c, cudaGetLastError());
 }

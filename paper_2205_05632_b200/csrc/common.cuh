@@ -195,7 +195,8 @@ __device__ __forceinline__ TileInfo find_tile(const SegParams& sp, int tile) {
 // Programmatic dependent launch: a kernel launched with launch_after() may start while the kernel
 // before it on the stream is still draining. It may touch nothing that kernel (or any earlier one it
 // has not been ordered after) writes until dependency_wait() has returned; what it reads before that
-// - here: optimizer state that only the previous step wrote - overlaps the predecessor's tail.
+// - here: optimizer state that only the previous step wrote - overlaps the predecessor's tail. A kernel that reads ahead of
+// its wait therefore never comes first in a call of the library: what is in front of it then is the caller's.
 // allow_dependents() in the predecessor lets the successor's CTAs in as soon as all of its own have
 // started. Both are no-ops in a plainly launched kernel.
 __device__ __forceinline__ void dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }

@@ -195,3 +195,24 @@ def test_apply_averages_what_the_message_buffers_hold(n, offs, ratio, comp):
             close(opt.buffer(name), want[name], name, t)
         assert opt.check_status() == 0
     opt.close()
+
+
+@pytest.mark.parametrize("n,offs,ratio", [(3, [0, 5, 8197, 24601], 0.02), (2, [0, 900001], 0.01), (2, [0, 3000, 900001], 0.3)])
+@pytest.mark.parametrize("comp", [TOPK, BLOCKSIGN, RANDK])
+def test_apply_sees_what_the_stream_did_to_theta_since_compress(n, offs, ratio, comp):
+    # decoupled weight decay in front of the server's update, with the worker side done before or after it
+    d = offs[-1]
+    gen = torch.Generator(device="cuda").manual_seed(10)
+    a, b = CompAMS(n, d, offs, comp, ratio), CompAMS(n, d, offs, comp, ratio)
+    ta = 0.1 * torch.randn(d, generator=gen, device="cuda")
+    tb = ta.clone()
+    for _ in range(6):
+        G = torch.randn(n, d, generator=gen, device="cuda")
+        ta *= 0.9
+        a.step(G, ta)
+        b.compress(G)
+        tb *= 0.9
+        b.apply(tb)
+        assert torch.equal(ta, tb)
+    a.close()
+    b.close()
