@@ -44,9 +44,11 @@ class CompAMSOptimizer:
             self.theta[lo:hi].copy_(p.data.reshape(-1))
             p.data = self.theta[lo:hi].view(p.shape)
         self.G = torch.zeros(self.n, self.d, dtype=torch.float32, device=dev)
-        # collect(): the tensors' places in a row, and room for their gradients' addresses
-        self._places = (ctypes.c_int64 * len(self.offsets))(*self.offsets.tolist())
-        self._addresses = (ctypes.c_void_p * len(self.params))()
+        # collect(): the tensors that have elements, their places in a row, and room for their gradients' addresses
+        self._pieces = [p for p, size in zip(self.params, sizes) if size]
+        places = [int(o) for o, size in zip(self.offsets, sizes) if size] + [self.d]
+        self._places = (ctypes.c_int64 * len(places))(*places)
+        self._addresses = (ctypes.c_void_p * len(self._pieces))()
         blocks = np.array([0, self.d], dtype=np.int64) if whole_vector else self.offsets
         with torch.cuda.device(dev):
             self.opt = CompAMS(self.n, self.d, blocks, compressor, k_ratio, lr, beta1, beta2, eps)
@@ -58,7 +60,7 @@ class CompAMSOptimizer:
         if not 0 <= worker < self.n:
             raise CompAMSError("worker %d outside [0, %d)" % (worker, self.n))
         # one kernel for all tensors; a gradient that is not packed (channels-last, an expanded view) is packed first
-        grads = [p.grad for p in self.params]
+        grads = [p.grad for p in self._pieces]
         grads = [g if g is None or g.is_contiguous() else g.contiguous() for g in grads]
         self._addresses[:] = [None if g is None else g.data_ptr() for g in grads]
         dev = self.G.device

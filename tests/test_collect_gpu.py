@@ -37,3 +37,20 @@ def test_collected_rows_are_the_gradients_bit_for_bit(sizes, layout):
         assert all(p.grad is None for p in params)
     assert torch.equal(opt.G.view(torch.int32), want.view(torch.int32))
     opt.close()
+
+
+@pytest.mark.parametrize("sizes", [[0, 3], [5, 0], [0, 0, TILE + 1, 0, 2, 0], [7] * 80 + [0] + [7] * 80])
+def test_parameters_without_elements_are_passed_over(sizes):
+    # with the whole vector as one block they are no block of their own
+    params = [torch.nn.Parameter(torch.zeros(s, device="cuda")) for s in sizes]
+    opt = CompAMSOptimizer(params, 2, BLOCKSIGN, whole_vector=True)
+    opt.G.fill_(float("nan"))
+    want = torch.arange(2 * sum(sizes), device="cuda").float().view(2, -1)
+    for worker in range(2):
+        for p, g in zip(params, torch.split(want[worker], sizes)):
+            p.grad = g.clone()
+        opt.collect(worker)
+        assert all(p.grad is None for p in params)
+    assert torch.equal(opt.G, want)
+    opt.step()
+    opt.close()
