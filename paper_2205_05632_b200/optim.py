@@ -45,7 +45,7 @@ class CompAMSOptimizer:
             p.data = self.theta[lo:hi].view(p.shape)
         self.G = torch.zeros(self.n, self.d, dtype=torch.float32, device=dev)
         # collect(): the tensors that have elements, their places in a row, and room for their gradients' addresses
-        self._pieces = [p for p, size in zip(self.params, sizes) if size]
+        self._pieces = [(p, 4 * size) for p, size in zip(self.params, sizes) if size]
         places = [int(o) for o, size in zip(self.offsets, sizes) if size] + [self.d]
         self._places = (ctypes.c_int64 * len(places))(*places)
         self._addresses = (ctypes.c_void_p * len(self._pieces))()
@@ -59,15 +59,26 @@ class CompAMSOptimizer:
         """Row `worker` of G <- the gradients accumulated since the last collect(); they are cleared."""
         if not 0 <= worker < self.n:
             raise CompAMSError("worker %d outside [0, %d)" % (worker, self.n))
-        # one kernel for all tensors; a gradient that is not packed (channels-last, an expanded view) is packed first
-        grads = [p.grad for p in self._pieces]
-        grads = [g if g is None or g.is_contiguous() else g.contiguous() for g in grads]
-        self._addresses[:] = [None if g is None else g.data_ptr() for g in grads]
+        # one kernel for all tensors, which reads them by their addresses
         dev = self.G.device
+        index = dev.index
+        grads, addresses = [], []  # (the former keeps the packed copies until the kernel is enqueued)
+        for p, nbytes in self._pieces:
+            g = p.grad
+            if g is not None:
+                # not as the kernel reads it, after a model.half() or .cpu() for instance, channels-last, an expanded view; the
+                # negative of what lies in memory (the imaginary part of a conjugate), which only one element can be and be packed
+                if g.nbytes != nbytes or g.get_device() != index or not g.is_contiguous() or (nbytes == 4 and g.is_neg()):
+                    if 4 * g.numel() != nbytes:
+                        raise CompAMSError("a gradient of %d elements for a parameter of %d" % (g.numel(), nbytes // 4))
+                    g = g.to(dev, torch.float32).resolve_neg().contiguous()
+                grads.append(g)
+            addresses.append(None if g is None else g.data_ptr())
+        self._addresses[:] = addresses
         with torch.cuda.device(dev):
             stream = torch.cuda.current_stream(dev).cuda_stream
             _check(load_library().compams_collect(self.G.data_ptr() + 4 * self.d * worker, self._addresses, self._places,
-                                                  len(grads), stream), "compams_collect")
+                                                  len(addresses), stream), "compams_collect")
         for p in self.params:
             p.grad = None
 

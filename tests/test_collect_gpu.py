@@ -3,7 +3,7 @@ for bit, whatever the tensors' sizes, the row's 16-byte phase and the gradients'
 import pytest
 import torch
 
-from paper_2205_05632_b200 import BLOCKSIGN
+from paper_2205_05632_b200 import BLOCKSIGN, CompAMSError
 from paper_2205_05632_b200.optim import CompAMSOptimizer
 
 pytestmark = pytest.mark.gpu
@@ -53,4 +53,31 @@ def test_parameters_without_elements_are_passed_over(sizes):
         assert all(p.grad is None for p in params)
     assert torch.equal(opt.G, want)
     opt.step()
+    opt.close()
+
+
+def test_gradients_that_are_not_packed_float32_on_the_device_are_made_so():
+    # what the copy of one tensor after the other took: other types and devices, lazily negated values
+    params = [torch.nn.Parameter(torch.zeros(s, device="cuda")) for s in ([70], [1], [8, 9], [33])]
+    opt = CompAMSOptimizer(params, 1, BLOCKSIGN)
+    gen = torch.Generator(device="cuda").manual_seed(3)
+    for change in (lambda t: t.half(), lambda t: t.bfloat16(), lambda t: t.double(), lambda t: t.cpu()):
+        for p in params:
+            p.data = change(p.data)
+            p.grad = torch.randn(p.shape, generator=gen, device="cuda").to(p.device, p.dtype)
+        want = torch.cat([p.grad.reshape(-1).float().cuda() for p in params])
+        opt.collect(0)
+        assert torch.equal(opt.G[0], want)
+    for p in params:
+        p.data = torch.zeros(p.shape, device="cuda")
+        z = torch.view_as_complex(torch.randn(*p.shape, 2, generator=gen, device="cuda"))
+        p.grad = z.conj().imag
+        assert p.grad.is_neg()
+    want = torch.cat([p.grad.reshape(-1) for p in params]).resolve_neg()
+    opt.collect(0)
+    assert torch.equal(opt.G[0], want)
+    params[2].data = torch.zeros(5, device="cuda")
+    params[2].grad = torch.ones(5, device="cuda")
+    with pytest.raises(CompAMSError):
+        opt.collect(0)
     opt.close()
