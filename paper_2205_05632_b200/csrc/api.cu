@@ -312,6 +312,7 @@ int init_context(compams_context* c, const int64_t* block_offsets) {
         for (int32_t b = 0; b < M; ++b)
             ((!c->randk && !c->fused && c->off[b + 1] - c->off[b] <= kSmallMax) ? small : large).push_back(b);
         RC(build_tiles(c, large, true));
+        if (!c->plan_only) CU(fit_topk_cluster(c));
         TopkBuffers& t = c->tk;
         t.E = c->E;
         t.K = c->K;

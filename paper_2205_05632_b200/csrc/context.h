@@ -146,6 +146,7 @@ struct compams_context {
     int32_t* sel_segs = nullptr;  // Top-k: the tiled blocks with a selection kernel: sel_long, then sel_short of them
     int sel_long = 0, sel_short = 0;
     int sel_cluster = 1;          // CTAs per (worker, long block)
+    bool sel_wide = false;        // CTAs of 1024 threads
     bool fused = false;           // Top-k: every block is swept and selected from by one kernel (small n d)
     int sel_parts = 0;            // CTAs that emit a long list in a kernel of its own (0: the cluster emits it)
     int32_t randk_group = 1;       // Random-k: workers whose elements share the map at a time
@@ -211,6 +212,7 @@ cudaError_t launch_bs_apply(compams_context* c, float* theta);
 cudaError_t launch_bs_materialize(compams_context* c);
 cudaError_t launch_topk_small(compams_context* c, const void* grads);
 cudaError_t launch_topk_sweep(compams_context* c, const void* grads);
+cudaError_t fit_topk_cluster(compams_context* c);
 cudaError_t launch_topk_select(compams_context* c);
 cudaError_t launch_topk_fused(compams_context* c, const void* grads);
 cudaError_t launch_topk_dense(compams_context* c);

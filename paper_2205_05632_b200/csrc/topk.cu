@@ -1134,25 +1134,72 @@ cudaError_t launch_topk_sweep(compams_context* c, const void* grads) {
 // waits for its predecessor before its first global access): the launch latency and the prologue of a
 // kernel then overlap the tail of the one before, which is most of what such a step costs.
 
-// Clusters of more than 8 CTAs have to be asked for, once per kernel and device.
-template <typename K>
-static cudaError_t allow_large_cluster(K* kernel, int cluster) {
-    return cluster > 8 ? cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) : cudaSuccess;
+typedef void (*SelectKernel)(const Tables, const TopkBuffers, const int32_t*, int, int, int, int);
+
+// Whether the device can hold a cluster of `cluster` CTAs of a kernel (more than 8 have to be asked for, once per kernel and
+// device).
+template <typename... KArgs>
+static cudaError_t cluster_fits(void (*kernel)(KArgs...), int threads, int cluster, bool* fits) {
+    if (cluster > 8) {
+        const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+        if (e != cudaSuccess) return e;
+    }
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)cluster);
+    cfg.blockDim = dim3((unsigned)threads);
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = (unsigned)cluster;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    int clusters = 0;
+    *fits = cudaOccupancyMaxActiveClusters(&clusters, kernel, &cfg) == cudaSuccess && clusters > 0;
+    if (!*fits) cudaGetLastError();
+    return cudaSuccess;
+}
+
+// The clusters were planned without a device, for 148 SMs in GPCs of at least 16. Where SMs are shared out (another process, a
+// partition) and none of that size can be resident, smaller ones take over, each CTA with a larger share of the same blocks.
+cudaError_t fit_topk_cluster(compams_context* c) {
+    // A handful of long lists that are only counted by topk_select: twice the threads per CTA (n = 1, d = 28.5 M, 1 %: 241.2 ->
+    // 236.2 us; n = 2, d = 4.4 M, 7.85 %: 91.6 -> 89.0; n = 5, d = 9.3 M, 2 %: 179.2 -> 177.2; but eight lists, n = 8, d = 4.2 M,
+    // 10 %: 163.9 -> 172.0)
+    c->sel_wide = c->sel_parts && c->sel_cluster == 16 && (int64_t)c->n * c->sel_long <= 5;
+    const int planned = c->sel_cluster;
+    bool fits = planned == 1;
+    for (; !fits && c->sel_cluster > 1; c->sel_cluster /= fits ? 1 : 2) {
+        cudaError_t e;
+        if (c->fused) {
+            bool bf16 = false;
+            e = cluster_fits(topk_fused_kernel<float>, kSelThreads, c->sel_cluster, &fits);
+            if (e == cudaSuccess) e = cluster_fits(topk_fused_kernel<bf16_bits>, kSelThreads, c->sel_cluster, &bf16);
+            fits = fits && bf16;
+        } else {
+            e = cluster_fits(topk_select_kernel<kSelThreads>, kSelThreads, c->sel_cluster, &fits);
+        }
+        if (e != cudaSuccess) return e;
+    }
+    if (c->sel_wide && c->sel_cluster == planned) {
+        const cudaError_t e = cluster_fits(topk_select_kernel<2 * kSelThreads>, 2 * kSelThreads, c->sel_cluster, &fits);
+        if (e != cudaSuccess) return e;
+        c->sel_wide = fits;
+    } else {
+        c->sel_wide = false;
+    }
+    const int64_t most = (int64_t)c->tk.cluster_max * (planned / c->sel_cluster);
+    c->tk.cluster_max = most < INT32_MAX ? (int32_t)most : INT32_MAX;
+    return cudaSuccess;
 }
 
 cudaError_t launch_topk_select(compams_context* c) {
     const int64_t clusters = (int64_t)c->n * c->sel_long + ((int64_t)c->n * c->sel_short + c->sel_cluster - 1) / c->sel_cluster;
-    // A handful of long lists that are only counted here: twice the threads per CTA (n = 1, d = 28.5 M, 1 %: 241.2 -> 236.2 us;
-    // n = 2, d = 4.4 M, 7.85 %: 91.6 -> 89.0; n = 5, d = 9.3 M, 2 %: 179.2 -> 177.2; but eight lists, n = 8, d = 4.2 M, 10 %: 163.9 ->
-    // 172.0)
-    const bool wide = c->sel_parts && c->sel_cluster == 16 && (int64_t)c->n * c->sel_long <= 5;
-    void (*kernel)(const Tables, const TopkBuffers, const int32_t*, int, int, int, int) =
-        wide ? topk_select_kernel<2 * kSelThreads> : topk_select_kernel<kSelThreads>;
-    cudaError_t e = allow_large_cluster(kernel, c->sel_cluster);
-    if (e != cudaSuccess) return e;
-    e = counted(c, launch_cluster(kernel, dim3((unsigned)(clusters * c->sel_cluster)), dim3(wide ? 2 * kSelThreads : kSelThreads),
-                                  c->sel_cluster, c->chain, c->stream, c->tab, own_rows(c), (const int32_t*)c->sel_segs, c->sel_long,
-                                  c->sel_short, delivers(c) ? 1 : 0, c->sel_parts ? 1 : 0));
+    const SelectKernel kernel = c->sel_wide ? topk_select_kernel<2 * kSelThreads> : topk_select_kernel<kSelThreads>;
+    const cudaError_t e = counted(c, launch_cluster(kernel, dim3((unsigned)(clusters * c->sel_cluster)),
+                                                    dim3(c->sel_wide ? 2 * kSelThreads : kSelThreads), c->sel_cluster, c->chain, c->stream,
+                                                    c->tab, own_rows(c), (const int32_t*)c->sel_segs, c->sel_long, c->sel_short,
+                                                    delivers(c) ? 1 : 0, c->sel_parts ? 1 : 0));
     if (e != cudaSuccess || !c->sel_parts) return e;
     const dim3 grid((unsigned)((int64_t)c->n * c->sel_long * c->sel_parts));
     if (c->chain)
@@ -1165,8 +1212,6 @@ cudaError_t launch_topk_select(compams_context* c) {
 template <typename GT>
 static cudaError_t launch_fused_typed(compams_context* c, const GT* grads) {
     const int64_t clusters = (int64_t)c->n * c->sel_long + ((int64_t)c->n * c->sel_short + c->sel_cluster - 1) / c->sel_cluster;
-    const cudaError_t e = allow_large_cluster(topk_fused_kernel<GT>, c->sel_cluster);
-    if (e != cudaSuccess) return e;
     return counted(c, launch_cluster(topk_fused_kernel<GT>, dim3((unsigned)(clusters * c->sel_cluster)), dim3(kSelThreads), c->sel_cluster,
                                      true, c->stream, c->tab, own_rows(c), grads, (const int32_t*)c->sel_segs, c->sel_long, c->sel_short,
                                      delivers(c) ? 1 : 0));
