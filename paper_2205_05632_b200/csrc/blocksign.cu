@@ -12,6 +12,8 @@
 // done when E is next read: by the next step's sweep (with the scale of the step that produced
 // x) or by bs_materialize when the caller asks for E. Both evaluate the same single fp32
 // subtraction, so the values are those of the residual update bit for bit.
+#include <algorithm>
+
 #include "context.h"
 
 namespace compams {
@@ -500,6 +502,163 @@ __global__ void __launch_bounds__(kThreads, 4) bs_apply_kernel(const __grid_cons
     }
 }
 
+constexpr int kShortChunk = 32;  // workers whose sign words are staged (and transposed) at a time: one per lane
+
+// Transposes four 32 x 32 bit matrices held across a warp: on entry lane i holds x[q] = row i of matrix q
+// (bit c = element (i, c)); on return lane c holds column c (bit i = element (i, c)). Five rounds of the
+// usual block swap: in round j a lane exchanges with lane ^ j the half of its bits whose position differs
+// from its own index in bit j. Shifting the partner's word by +-j and keeping only the positions that
+// change is a rotation followed by a bitwise select.
+__device__ __forceinline__ void transpose32x4(uint32_t (&x)[4], int lane) {
+#pragma unroll
+    for (int j = 16; j >= 1; j >>= 1) {
+        const uint32_t m = j == 16 ? 0x0000ffffu : j == 8 ? 0x00ff00ffu : j == 4 ? 0x0f0f0f0fu : j == 2 ? 0x33333333u : 0x55555555u;
+        const bool up = (lane & j) != 0;
+        const uint32_t keep = up ? ~m : m;          // positions whose bit j equals the lane's stay
+        const uint32_t rot = up ? 32u - j : (uint32_t)j;  // the partner's bits move down (up) by j
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const uint32_t y = __shfl_xor_sync(0xffffffffu, x[q], j);
+            x[q] = (x[q] & keep) | (__funnelshift_l(y, y, rot) & ~keep);
+        }
+    }
+}
+
+// The same for few tiles: one CTA per 1024 coordinates, one float4 group per thread, so that a vector too short to give
+// bs_apply's CTAs of 2048 coordinates an SM each is spread twice as wide and a CTA has half the serial work.
+// TABLES = false: one predicated binary64 add per worker and coordinate. TABLES = true: 16-entry tables of 4 workers' scales,
+// the patterns from a transposition across the warp: lane i reads worker i's four words of the warp's 128 coordinates,
+// transpose32x4 turns them into one word per coordinate, and 16 shuffles hand every lane the patterns of its own 4 coordinates.
+// Bound by latency: the words and scales of up to 32 workers come in one round of loads (see launch_bs_apply for the figures).
+template <bool TABLES, bool RECORD>
+__global__ void __launch_bounds__(kThreads, 5) bs_apply_short_kernel(const __grid_constant__ Tables t, const __grid_constant__ BsBuffers b,
+                                                                     float* __restrict__ theta, const __grid_constant__ HyperParams hp,
+                                                                     const __grid_constant__ SegParams sp_) {
+    __shared__ uint32_t sh_bits[kShortChunk][33];        // [worker][word], rows padded against bank conflicts
+    __shared__ double sh_tab[kShortChunk / 4][16];       // TABLES: [group of 4 workers][subset] sum of the subset's
+                                                         // scales; else: the workers' scales
+    const int tile = blockIdx.x >> 3;
+    const TileInfo ti = sp_.nseg ? find_tile(sp_, tile) : load_tile(t.tiles, tile);
+    const int blk = ti.blk;
+    const int len = ti.len;
+    const int rs = ti.r0 + (int)(blockIdx.x & 7) * kWarpSpan;  // first coordinate of this CTA, relative to the block
+    if (rs >= len) return;
+    const int r = rs + (int)threadIdx.x * 4;
+    const int64_t o = ti.o;
+    float* gbar = b.gbar + o;
+    float* m = b.m + o;
+    float* v = b.v + o;
+    float* vh = b.vhat + o;
+    float* th = theta + o;
+    const int cls = align_class(m);  // all five vectors are 16-byte aligned at coordinate 0
+    const bool full = r + 3 < len;
+    float4 mm = make_float4(0.f, 0.f, 0.f, 0.f), vv = mm, hh = mm, tt = mm;
+    if (full) {
+        mm = load4(m + r, cls);
+        vv = load4(v + r, cls);
+        hh = load4(vh + r, cls);
+        tt = load4(th + r, cls);
+    }
+    dependency_wait();  // the state above was last written a step ago; sign words and scales are this step's
+    const size_t wbase = (size_t)(sp_.nseg ? (int64_t)sp_.wofs[ti.seg] : b.word_off[blk]) + (size_t)(rs >> 5);
+    const int lane = threadIdx.x & 31, wr = threadIdx.x >> 5;  // warp wr owns coordinates 128 wr ... of the CTA's 1024
+    const bool word_live = rs + lane * 32 < len;
+    double a0 = 0.0, a1 = 0.0, a2 = 0.0, a3 = 0.0, all = 0.0;
+    for (int i0 = 0; i0 < t.n; i0 += kShortChunk) {
+        const int nc = (t.n - i0 < kShortChunk) ? t.n - i0 : kShortChunk;
+        __syncthreads();
+        // warp wr stages the words of workers wr, wr + 8, ...: 32 consecutive words each, one per lane
+        for (int c = wr; c < nc; c += kWarps)
+            sh_bits[c][lane] = word_live ? __ldg(b.bits + (size_t)(i0 + c) * (size_t)b.W + wbase + lane) : 0u;
+        if constexpr (TABLES) {
+            const int ng = (nc + 3) >> 2;  // groups of 4 workers in this round
+            if (threadIdx.x < ng * 16) {   // one table entry per thread: the scales of the subset's members
+                const int gq = threadIdx.x >> 4, sub = threadIdx.x & 15;
+                double e = 0.0;
+#pragma unroll
+                for (int j = 0; j < 4; ++j)
+                    if (((sub >> j) & 1) && gq * 4 + j < nc)
+                        e += (double)b.scales_cur[(size_t)(i0 + gq * 4 + j) * t.M + blk];
+                sh_tab[gq][sub] = e;
+            }
+            __syncthreads();
+            // lane i: worker i's words of this warp's coordinates -> lane c: the workers' bits of coordinate 32 q + c
+            uint32_t x[4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) x[q] = lane < nc ? sh_bits[lane][wr * 4 + q] : 0u;
+            transpose32x4(x, lane);
+            // this thread's coordinates 4 lane + k lie in word q = lane / 8 at bit 4 (lane % 8) + k: their patterns
+            // sit in lane 4 (lane % 8) + k, matrix lane / 8 (a trip through shared memory instead of these 16
+            // shuffles was slower)
+            uint4 pat = make_uint4(0u, 0u, 0u, 0u);
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const uint32_t y0 = __shfl_sync(0xffffffffu, x[q], (lane & 7) * 4 + 0);
+                const uint32_t y1 = __shfl_sync(0xffffffffu, x[q], (lane & 7) * 4 + 1);
+                const uint32_t y2 = __shfl_sync(0xffffffffu, x[q], (lane & 7) * 4 + 2);
+                const uint32_t y3 = __shfl_sync(0xffffffffu, x[q], (lane & 7) * 4 + 3);
+                if ((lane >> 3) == q) pat = make_uint4(y0, y1, y2, y3);
+            }
+#pragma unroll
+            for (int gq = 0; gq < kShortChunk / 4; ++gq) {
+                if (gq < ng) {  // the same for every thread of the CTA
+                    all += sh_tab[gq][15];
+                    a0 += sh_tab[gq][(pat.x >> (4 * gq)) & 15u];
+                    a1 += sh_tab[gq][(pat.y >> (4 * gq)) & 15u];
+                    a2 += sh_tab[gq][(pat.z >> (4 * gq)) & 15u];
+                    a3 += sh_tab[gq][(pat.w >> (4 * gq)) & 15u];
+                }
+            }
+        } else {
+            double* sh_s = &sh_tab[0][0];
+            if (threadIdx.x < nc) sh_s[threadIdx.x] = (double)b.scales_cur[(size_t)(i0 + threadIdx.x) * t.M + blk];
+            __syncthreads();
+            const int wsel = threadIdx.x >> 3, nsh = (threadIdx.x & 7) * 4;  // this thread's word and its nibble in it
+#pragma unroll 4
+            for (int c = 0; c < nc; ++c) {
+                const double sc = sh_s[c];
+                const uint32_t nib = sh_bits[c][wsel] >> nsh;
+                all += sc;
+                if (nib & 1u) a0 += sc;
+                if (nib & 2u) a1 += sc;
+                if (nib & 4u) a2 += sc;
+                if (nib & 8u) a3 += sc;
+            }
+        }
+    }
+    a0 = all - (a0 + a0);
+    a1 = all - (a1 + a1);
+    a2 = all - (a2 + a2);
+    a3 = all - (a3 + a3);
+    if (r >= len) return;
+    const float gb[4] = {mean_from_acc(a0, hp), mean_from_acc(a1, hp), mean_from_acc(a2, hp),
+                         mean_from_acc(a3, hp)};
+    if (full) {
+        amsgrad_update(gb[0], mm.x, vv.x, hh.x, tt.x, hp);
+        amsgrad_update(gb[1], mm.y, vv.y, hh.y, tt.y, hp);
+        amsgrad_update(gb[2], mm.z, vv.z, hh.z, tt.z, hp);
+        amsgrad_update(gb[3], mm.w, vv.w, hh.w, tt.w, hp);
+        if constexpr (RECORD) store4(gbar + r, cls, make_float4(gb[0], gb[1], gb[2], gb[3]));
+        store4(m + r, cls, mm);
+        store4(v + r, cls, vv);
+        store4(vh + r, cls, hh);
+        store4(th + r, cls, tt);
+    } else {
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            if (r + k < len) {
+                float m1 = m[r + k], v1 = v[r + k], h1 = vh[r + k], t1 = th[r + k];
+                amsgrad_update(gb[k], m1, v1, h1, t1, hp);
+                if constexpr (RECORD) gbar[r + k] = gb[k];
+                m[r + k] = m1;
+                v[r + k] = v1;
+                vh[r + k] = h1;
+                th[r + k] = t1;
+            }
+        }
+    }
+}
+
 // The worker-side kernels see this handle's own rows of the message buffers (sign words, scales);
 // the server kernel sees the rows of all n_total workers.
 static BsBuffers own_rows(const compams_context* c) {
@@ -529,12 +688,26 @@ cudaError_t launch_bs_sweep(compams_context* c, const void* grads) {
     return counted(c, cudaGetLastError());
 }
 
-// Whether bs_apply adds up the tile sums itself, and bs_scales is not launched: n = 4, d = 65,536 10.8 -> 9.7 us, n = 8,
-// d = 2^20 29.3 -> 27.5. Not between compams_compress and compams_apply (the messages have to be complete), not for larger blocks, of which every
-// CTA would read more sums than its share of the rest, nor for many workers (n = 24, d = 3.3 M in 90 blocks: 194.4 us
-// with bs_scales, 198.3 without: a warp adds up one worker after the other).
+// Whether the server kernel is bs_apply_short: few tiles for the number of workers. us per step (whole vector, bs_apply with the tile
+// sums its own business or with bs_scales, whichever is faster, against bs_scales and bs_apply_short): n = 32, d = 65,536 (9 tiles)
+// 17.6 / 12.7, n = 16, d = 162,400 (20) 15.3 / 13.3, n = 16, d = 370,001 (46) 18.6 / 18.3, n = 24, d = 524,288 (65) 35.2 / 33.9; beyond the
+// line n = 16, d = 750,007 (92) 32.1 / 33.9, n = 32, d = 2^20 (129) 79.7 / 81.8. With few workers and very few tiles the
+// launch that is saved is worth more: n = 8, d = 100,003 (13) 10.8 / 11.5, but d = 162,400 (20) 12.3 / 11.9.
+static bool bs_apply_is_short(const compams_context* c) {
+    return c->tab.ntiles < std::min(4 * c->n_total, 96) && (c->n_total > 8 || c->tab.ntiles >= 16);
+}
+
+// Whether bs_apply adds up the tile sums itself, and bs_scales is not launched. Not between compams_compress and compams_apply (the
+// messages have to be complete), and not where every CTA would read more sums than its share of the rest, one worker after the other
+// by its eight warps. us per step without / with bs_scales: n = 8, d = 2^20 + 1 (129 tiles) 20.6 / 22.3, d = 1.5 M (184) 38.9 / 40.4, d = 2^21
+// + 3 (257) 50.9 / 50.9; n = 16, d = 2^20 44.1 / 45.2, d = 1.5 M 66.4 / 65.5; more workers gain only where all blocks are small: n = 32,
+// d = 750,007 in 150 blocks (6 tiles at most) 94.2 / 98.5, n = 17 in 40 blocks (21) 42.1 / 42.8, d = 1.5 M in 40 or 150 (34) 77.0 / 75.8
+// and 88.0 / 87.9.
 bool bs_apply_adds_up(const compams_context* c) {
-    return c->whole_step && c->n <= 2 * kWarps && c->bs_max_tiles <= kWarpTiles && (int64_t)c->bs_max_tiles * c->n <= 1024;
+    if (!c->whole_step || bs_apply_is_short(c)) return false;
+    if (c->n <= 8) return c->bs_max_tiles <= kWarpTiles;
+    if (c->n <= 2 * kWarps) return c->bs_max_tiles <= 160;
+    return (int64_t)c->bs_max_tiles * c->n <= 512;
 }
 
 cudaError_t launch_bs_scales(compams_context* c) {
@@ -549,12 +722,15 @@ cudaError_t launch_bs_apply(compams_context* c, float* theta) {
     b.scales_cur = c->scales[c->scales_cur];
     Tables t = c->tab;
     t.n = c->n_total;  // the average runs over every worker's message
-    const bool own = bs_apply_adds_up(c);
-    const dim3 grid((unsigned)(c->tab.ntiles * (kTile / kApplySpan)));
+    const bool own = bs_apply_adds_up(c), is_short = bs_apply_is_short(c);
+    const dim3 grid((unsigned)(c->tab.ntiles * (is_short ? kWarps : kTile / kApplySpan)));
     // (gbar stored or not is a template parameter: a run-time branch around the store slowed the kernel by a tenth)
     void (*kernel)(const Tables, const BsBuffers, float*, const HyperParams, const SegParams) =
         own ? (b.gbar ? bs_apply_kernel<true, true> : bs_apply_kernel<false, true>)
             : (b.gbar ? bs_apply_kernel<true, false> : bs_apply_kernel<false, false>);
+    if (is_short)  // tables from 20 workers up: n = 16, d = 162,400 13.6 us with, 13.3 without, n = 32, d = 524,288 43.9 with, 45.8 without
+        kernel = c->n_total >= 20 ? (b.gbar ? bs_apply_short_kernel<true, true> : bs_apply_short_kernel<true, false>)
+                                  : (b.gbar ? bs_apply_short_kernel<false, true> : bs_apply_short_kernel<false, false>);
     if (c->whole_step) return counted(c, launch_after(kernel, grid, dim3(kThreads), c->stream, t, b, theta, c->hp, c->segp));
     // between compams_compress and compams_apply the caller may have put work on the stream that writes the messages, theta
     // or both, and the kernel reads theta ahead of its wait: a plain launch comes after that work

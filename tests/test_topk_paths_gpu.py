@@ -63,9 +63,12 @@ def test_long_and_short_lists_side_by_side():
 
 @pytest.mark.parametrize("n,offs", [
     (16, [0, 64 * 8192 - 31]), (17, [0, 64 * 8192 - 31]), (1, [0, 256 * 8192]), (1, [0, 256 * 8192 + 1]), (4, [0, 1, 2050, 6150, 10249]),
-    (25, [0, 3, 2049, 20001]), (2, [0, 5, 8197, 16391, 24601, 24603]),
+    (25, [0, 3, 2049, 20001]), (2, [0, 5, 8197, 16391, 24601, 24603]), (16, [0, 160 * 8192]), (16, [0, 160 * 8192 + 1]),
+    (17, list(np.cumsum([0] + [611 + 37 * k for k in range(80)]))), (4, [0, 15 * 8192]), (5, [0, 19 * 8192]), (5, [0, 20 * 8192]),
+    (9, [0, 36 * 8192 - 32]), (9, [0, 36 * 8192]), (19, [0, 37, 20003]), (20, [0, 37, 20003]), (40, [0, 1000, 1003, 30001]),
+    (24, [0, 95 * 8192 - 40]), (24, [0, 96 * 8192 - 40]),
 ])
-def test_blocksign_scales_added_up_by_either_kernel(n, offs):
+def test_blocksign_server_kernels_and_who_adds_up_the_scales(n, offs):
     run(n, offs, BLOCKSIGN, 1.0, normal, steps=4)
 
 
