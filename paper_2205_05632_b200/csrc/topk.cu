@@ -972,13 +972,13 @@ __global__ void __launch_bounds__(kThreads) topk_small_kernel(Tables t, TopkBuff
     __shared__ uint32_t xs[kSmallMax];
     __shared__ uint32_t hist[256];
     __shared__ uint32_t scratch[kWarps];
-    __shared__ uint32_t sh_prefix, sh_krem, sh_cnt, sh_rlast;
+    __shared__ uint32_t sh_prefix, sh_krem, sh_cnt, sh_rlast, sh_taken;
     // Shares no block with the sweep before it: its CTAs move in behind the sweep's last wave, which has ordered itself
     // after everything earlier on the stream, and wait for the sweep only at their end, for the sake of the kernel after.
     if (!after_sweep) dependency_wait();
     allow_dependents();
     const int blk = b.small_blk[blockIdx.x];
-    const int i = blockIdx.y;
+    const int i = blockIdx.y, lane = threadIdx.x & 31;
     const int64_t o = t.off[blk];
     const int len = (int)(t.off[blk + 1] - o);
     const uint32_t kb = (uint32_t)(b.seg_off[blk + 1] - b.seg_off[blk]);
@@ -1021,7 +1021,10 @@ __global__ void __launch_bounds__(kThreads) topk_small_kernel(Tables t, TopkBuff
     const int chunk = (len + kThreads - 1) / kThreads;
     const int lo = (int)threadIdx.x * chunk;
     const int hi = (lo + chunk < len) ? lo + chunk : len;
-    if (threadIdx.x == 0) sh_rlast = take_all ? 0x7fffffffu : 0u;
+    if (threadIdx.x == 0) {
+        sh_rlast = take_all ? 0x7fffffffu : 0u;
+        sh_taken = 0u;
+    }
     __syncthreads();
     if (!take_all) {
         uint32_t mine = 0;
@@ -1041,24 +1044,42 @@ __global__ void __launch_bounds__(kThreads) topk_small_kernel(Tables t, TopkBuff
         const uint32_t top = (xs[r] & 0x7fffffffu) >> shift;
         return top > prefix || (top == prefix && (uint32_t)r <= rlast);
     };
-    uint32_t mine = 0;
-    for (int r = lo; r < hi; ++r) mine += kept(r) ? 1u : 0u;
-    uint32_t total;
-    uint32_t pos = block_inclusive_scan(mine, scratch, &total) - mine;
+    // Emission and residual in one pass, a warp taking 32 consecutive coordinates at a time: its kept entries share an atomic
+    // for their message slots and one per server bucket they meet, and e = x - g~ is 0 where kept, x elsewhere (Algorithm 2,
+    // the residual update). (With a stretch of coordinates and one atomic per kept entry per thread, n = 32, d = 65,536 in 70
+    // blocks took 27 us at 0.1 % and 90 at 10 %.)
     const size_t slot0 = (size_t)i * (size_t)b.K + (size_t)b.seg_off[blk];
-    for (int r = lo; r < hi; ++r) {
-        if (kept(r)) {
-            if (pos < kb) {
-                b.idx[slot0 + pos] = (int32_t)(o + r);
-                b.val[slot0 + pos] = __uint_as_float(xs[r]);
-                if (deliver) scatter_one(b, (int32_t)(o + r), xs[r]);
-            }
-            ++pos;
+    constexpr int U = 4;
+    for (int r0 = 0; r0 < len; r0 += U * kThreads) {
+        bool take[U];
+        uint2 cv[U];
+        uint32_t rel[U], wins = 0;
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int r = r0 + u * kThreads + (int)threadIdx.x;
+            const bool live = r < len;
+            take[u] = live && kept(r);
+            cv[u] = make_uint2((uint32_t)(o + (live ? r : len - 1)), live ? xs[r] : 0u);
+            if (live) e[r] = take[u] ? 0.0f : __uint_as_float(xs[r]);
+            const unsigned m = __ballot_sync(0xffffffffu, take[u]);
+            rel[u] = wins + (uint32_t)__popc(m & ((1u << lane) - 1u));
+            wins += (uint32_t)__popc(m);
         }
+        if (wins == 0u) continue;
+        uint32_t pos = 0;
+        if (lane == 0) pos = atomicAdd(&sh_taken, wins);
+        pos = __shfl_sync(0xffffffffu, pos, 0);
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            if (take[u] && pos + rel[u] < kb) {
+                b.idx[slot0 + pos + rel[u]] = (int32_t)cv[u].x;
+                b.val[slot0 + pos + rel[u]] = __uint_as_float(cv[u].y);
+            }
+        }
+        if (deliver) scatter_runs<U>(b, take, cv);
     }
-    if (threadIdx.x == 0 && total != kb) atomicOr(b.status, 1u);
-    // Algorithm 2, the residual update: e = x - g~ (0 where kept, x elsewhere)
-    for (int r = threadIdx.x; r < len; r += kThreads) e[r] = kept(r) ? 0.0f : __uint_as_float(xs[r]);
+    __syncthreads();
+    if (threadIdx.x == 0 && sh_taken != kb) atomicOr(b.status, 1u);
     if (after_sweep) dependency_wait();
 }
 
