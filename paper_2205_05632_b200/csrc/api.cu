@@ -85,24 +85,37 @@ int64_t kept_per_block(double k_ratio, int64_t d_b) {
 constexpr int64_t kPlanSms = 148;              // SMs that the choices below count on (a plan is made without a device)
 constexpr int64_t kFusedRound = 8192;          // coordinates one CTA of the fused sweep and selection has in flight
 constexpr int64_t kListlessFused = 2048;       // blocks up to this size are always selected from directly there
+constexpr int64_t kListlessFusedMax = 3 << 18; // n d up to which longer ones are, too
 // Coordinates per CTA up to which a cluster goes through a block itself when the list cannot decide. Beyond, the dense
 // passes of the whole GPU are launched every step to stand by: about 4 us, which only matters to short steps (a CTA gets through
 // about 2^16 coordinates in 30 us per pass, and needs five).
 constexpr int64_t kClusterMax = (int64_t)1 << 21, kClusterMaxLongStep = (int64_t)1 << 17;
-constexpr int64_t kListless = (int64_t)1 << 18;    // ... of a block that never has a list
+// ... of a block that never has a list, where its cluster goes through it on every step. Five passes by a few CTAs: the dense passes of
+// the whole GPU are faster from about there on (us per step, clusters / dense passes, 20 % kept: n = 4, d = 162,400 39 / 43, d = 262,144
+// 45 / 47, n = 8, d = 262,144 57 / 52 but 64 / 72 with 50 %, n = 1, d = 524,288 59 / 41, d = 2^21 + 3 177 / 56; 70 blocks, n = 8,
+// d = 65,536 49 / 57, d = 262,144 72 / 67).
+constexpr int64_t kListless = 1 << 14;
+
+// The candidate path pays off for sparse selections only: at most 1/9 of the block kept.
+bool has_list(int64_t kb, int64_t len) { return kb * 9 <= len; }
 
 // CTAs per long block when sweep and selection are one kernel, 0 when they are not. It pays where no CTA needs more than
 // one round of loads for its share and no two share an SM: n = 4, d = 65,536 15.9 -> 15.3 us, n = 3, d = 111,947 in 78
-// blocks 24.2 -> 18.4; but n = 1, d = 2^20 (16 CTAs, eight rounds) 25.7 -> 38.7, n = 32, d = 65,536 (256 CTAs) 17.8 -> 21.3.
+// blocks 24.2 -> 18.4; but n = 1, d = 2^20 (16 CTAs, eight rounds) 25.7 -> 38.7, n = 32, d = 65,536 (256 CTAs) 17.8 -> 21.3. Blocks
+// without a list take five passes by their clusters, which lose to the dense passes of the whole GPU from some problem size on (20 % kept:
+// n = 8, d = 65,536 43 against 45 us, n = 4, d = 162,400 in 70 blocks 36 against 62, n = 16, d = 65,536 67 against 55).
 int fused_cluster(const compams_context* c) {
     int64_t longest = 0, longs = 0, shorts = 0;
+    bool listless = false;
     for (int32_t b = 0; b < c->M; ++b) {
         const int64_t len = c->off[(size_t)b + 1] - c->off[(size_t)b];
         longest = std::max(longest, len);
         (len > kFusedRound ? longs : shorts) += c->n;
+        listless = listless || (len > kFusedRound && !has_list(c->seg_off[(size_t)b + 1] - c->seg_off[(size_t)b], len));
     }
     int64_t cluster = 1;
     while (cluster * kFusedRound < longest) cluster *= 2;
+    if (listless && c->n * c->d > kListlessFusedMax) return 0;
     return cluster <= 16 && longs * cluster <= kPlanSms && shorts <= 2 * kPlanSms ? (int)cluster : 0;
 }
 
@@ -158,12 +171,17 @@ int group_segments(compams_context* c, const std::vector<SegInfo>& segs) {
     std::vector<int32_t> few, many;  // blocks for one CTA, for a cluster of them
     for (size_t s = 0; s < segs.size(); ++s) (expected(segs[s]) < from ? few : many).push_back((int32_t)s);
     int64_t entries = 0;
+    // blocks without a list go to their clusters where those are short and all at work at once, one per GPC (n = 16, d = 65,536, 16
+    // clusters of 8, 20 % kept: 67 us, by the dense passes 55)
+    bool walk = (int64_t)many.size() * c->n <= 8 && ((int64_t)many.size() * cluster + (int64_t)few.size()) * c->n <= kPlanSms;
+    for (const std::vector<int32_t>* l : {&few, &many})
+        for (int32_t s : *l) walk = walk && (segs[(size_t)s].cap || segs[(size_t)s].len <= kListless * (l == &few ? 1 : cluster));
     for (std::vector<int32_t>* l : {&few, &many}) {
         const int64_t ctas = l == &few ? 1 : cluster;
         std::vector<int32_t> listed;
         for (int32_t s : *l) {
             if (segs[(size_t)s].len > cluster_max * ctas) c->dense_kernel = true;
-            if (segs[(size_t)s].cap || segs[(size_t)s].len <= std::min(kListless, cluster_max) * ctas) {
+            if (segs[(size_t)s].cap || walk) {
                 listed.push_back(s);
                 if (l == &many && segs[(size_t)s].cap) entries = std::max(entries, expected(segs[(size_t)s]));
             } else {  // always the dense passes
@@ -219,8 +237,7 @@ int build_tiles(compams_context* c, const std::vector<int32_t>& blocks, bool top
             const int64_t kb = c->seg_off[(size_t)b + 1] - c->seg_off[(size_t)b];
             si.slot0 = c->seg_off[(size_t)b];
             si.kb = (uint32_t)kb;
-            // the candidate path pays off for sparse selections only: at most 1/9 of the block kept
-            int64_t cap = (!c->randk && kb * 9 <= len) ? 8 * kb + 1024 : 0;
+            int64_t cap = !c->randk && has_list(kb, len) ? 8 * kb + 1024 : 0;
             if (c->fused && len <= kListlessFused) cap = 0;
             if (cap) cap = std::min(cap, len <= 65536 ? len : len / 4 + kb);
             cap = (cap + 1) & ~(int64_t)1;  // lists are read in 128-bit pairs
