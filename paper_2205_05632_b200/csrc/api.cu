@@ -86,10 +86,16 @@ constexpr int64_t kPlanSms = 148;              // SMs that the choices below cou
 constexpr int64_t kFusedRound = 8192;          // coordinates one CTA of the fused sweep and selection has in flight
 constexpr int64_t kListlessFused = 2048;       // blocks up to this size are always selected from directly there
 constexpr int64_t kListlessFusedMax = 3 << 18; // n d up to which longer ones are, too
-// Coordinates per CTA up to which a cluster goes through a block itself when the list cannot decide. Beyond, the dense
-// passes of the whole GPU are launched every step to stand by: about 4 us, which only matters to short steps (a CTA gets through
-// about 2^16 coordinates in 30 us per pass, and needs five).
+// Coordinates per CTA up to which a cluster goes through a block itself when the list cannot decide: about 0.75 ns each for
+// all its passes. Beyond, the dense passes of the whole GPU are launched every step to stand by: about 4 us when they have
+// nothing to do, which only matters to short steps.
 constexpr int64_t kClusterMax = (int64_t)1 << 21, kClusterMaxLongStep = (int64_t)1 << 17;
+// The first steps of a handle, and those after its accumulators have been replaced, are the ones whose lists do fail (none has a
+// prediction in the first; later ones fail when the gradient scale drops, or under a cycle of few batches). In these the dense passes
+// stand by wherever the clusters would take more than about twice their time, which is 5 ps per worker-element and 30 us
+// (first step / later ones, us: n = 1, d = 28.5 M, 1 % 451 / 232, by clusters alone 1329; n = 1, d = 4.2 M 104 / 58, 305; n = 4,
+// ResNet-18 shapes whole 498 / 172, 899).
+constexpr int kFirstSteps = 32;
 // ... of a block that never has a list, where its cluster goes through it on every step. Five passes by a few CTAs: the dense passes of
 // the whole GPU are faster from about there on (us per step, clusters / dense passes, 20 % kept: n = 4, d = 162,400 39 / 43, d = 262,144
 // 45 / 47, n = 8, d = 262,144 57 / 52 but 64 / 72 with 50 %, n = 1, d = 524,288 59 / 41, d = 2^21 + 3 177 / 56; 70 blocks, n = 8,
@@ -121,11 +127,13 @@ int fused_cluster(const compams_context* c) {
 
 // Decides which kernels select from which blocks, and with how many CTAs.
 int group_segments(compams_context* c, const std::vector<SegInfo>& segs) {
-    const int64_t cluster_max = (int64_t)c->n * c->tab.d <= kChainMaxElems ? kClusterMax : kClusterMaxLongStep;
-    c->tk.cluster_max = (int32_t)cluster_max;
+    const int64_t elems = (int64_t)c->n * c->d;
+    const int64_t cluster_max = elems <= kChainMaxElems ? kClusterMax : kClusterMaxLongStep;
+    c->cluster_max = (int32_t)cluster_max;
+    c->cluster_max_first = (int32_t)std::min(cluster_max, 80000 + elems / 75);
     c->sel_long = c->sel_short = c->sel_parts = 0;
     c->sel_cluster = 1;
-    c->dense_kernel = false;
+    c->dense_kernel = c->dense_first = false;
     c->seg_always_dense.assign(segs.size(), false);
     if (c->randk) return COMPAMS_OK;
     if (c->fused) {
@@ -133,7 +141,7 @@ int group_segments(compams_context* c, const std::vector<SegInfo>& segs) {
         for (size_t s = 0; s < segs.size(); ++s) (segs[s].len <= kFusedRound ? one : several).push_back((int32_t)s);
         c->sel_cluster = fused_cluster(c);
         std::stable_sort(several.begin(), several.end(), [&](int32_t a, int32_t b) { return segs[(size_t)a].len > segs[(size_t)b].len; });
-        c->tk.cluster_max = INT32_MAX;  // the dense passes are never launched
+        c->cluster_max = c->cluster_max_first = INT32_MAX;  // the dense passes are never launched
         c->sel_long = (int)several.size();
         c->sel_short = (int)one.size();
         several.insert(several.end(), one.begin(), one.end());
@@ -168,8 +176,25 @@ int group_segments(compams_context* c, const std::vector<SegInfo>& segs) {
             }
         }
     }
+    // A block too long for one CTA to go through gets a cluster however short its list (the first CTA takes that alone), where
+    // all CTAs of the kernel are at work at once: the dense passes need not stand by (n = 4, d = 2^21 + 3, 0.1 %: 51.0 -> 46.2 us).
+    int64_t lists = 0, by_length = 0, longest = 0;
+    for (const SegInfo& si : segs) {
+        lists += expected(si) >= from;
+        by_length += elems <= kChainMaxElems && expected(si) < from && si.cap && si.len > cluster_max;
+        longest = std::max<int64_t>(longest, si.len);
+    }
+    int lift = 0;
+    for (int c16 = cluster > 1 ? cluster : 16; by_length && !lift && c16 > 1; c16 = cluster > 1 ? 1 : c16 / 2) {
+        const int64_t ctas = c->n * ((lists + by_length) * c16 + (int64_t)segs.size() - lists - by_length);
+        if (ctas <= (c16 == 16 ? 1 : 2) * kPlanSms && longest <= cluster_max * c16) lift = c16;
+    }
+    if (lift) cluster = lift;
     std::vector<int32_t> few, many;  // blocks for one CTA, for a cluster of them
-    for (size_t s = 0; s < segs.size(); ++s) (expected(segs[s]) < from ? few : many).push_back((int32_t)s);
+    for (size_t s = 0; s < segs.size(); ++s) {
+        const bool is_many = expected(segs[s]) >= from || (lift && segs[s].cap && segs[s].len > cluster_max);
+        (is_many ? many : few).push_back((int32_t)s);
+    }
     int64_t entries = 0;
     // blocks without a list go to their clusters where those are short and all at work at once, one per GPC (n = 16, d = 65,536, 16
     // clusters of 8, 20 % kept: 67 us, by the dense passes 55)
@@ -181,6 +206,7 @@ int group_segments(compams_context* c, const std::vector<SegInfo>& segs) {
         std::vector<int32_t> listed;
         for (int32_t s : *l) {
             if (segs[(size_t)s].len > cluster_max * ctas) c->dense_kernel = true;
+            if (segs[(size_t)s].len > c->cluster_max_first * ctas) c->dense_first = true;
             if (segs[(size_t)s].cap || walk) {
                 listed.push_back(s);
                 if (l == &many && segs[(size_t)s].cap) entries = std::max(entries, expected(segs[(size_t)s]));
@@ -479,15 +505,19 @@ int compress_device(compams_context* c, const void* grads) {
         return COMPAMS_OK;
     }
     if (c->fused) {
+        c->tk.cluster_max = c->cluster_max;
         RC(run_kernel(c, COMPAMS_K_TOPK_SELECT, [&] { return launch_topk_fused(c, grads); }));
         c->e_mask_pending = true;
         return COMPAMS_OK;
     }
+    const bool first = c->first_steps > 0;
+    if (first) --c->first_steps;
+    c->tk.cluster_max = first ? c->cluster_max_first : c->cluster_max;
     if (c->tab.ntiles > 0) RC(run_kernel(c, COMPAMS_K_TOPK_SWEEP, [&] { return launch_topk_sweep(c, grads); }));
     if (c->tk.nsmall > 0) RC(run_kernel(c, COMPAMS_K_TOPK_SMALL, [&] { return launch_topk_small(c, grads); }));
     if (c->tab.ntiles > 0) {
         if (c->sel_long + c->sel_short > 0) RC(run_kernel(c, COMPAMS_K_TOPK_SELECT, [&] { return launch_topk_select(c); }));
-        if (c->dense_kernel) RC(run_kernel(c, COMPAMS_K_TOPK_DENSE, [&] { return launch_topk_dense(c); }));
+        if (c->dense_kernel || (first && c->dense_first)) RC(run_kernel(c, COMPAMS_K_TOPK_DENSE, [&] { return launch_topk_dense(c); }));
         c->e_mask_pending = true;
     }
     return COMPAMS_OK;
@@ -550,6 +580,7 @@ int create_handle(compams_handle* out, int32_t n, int32_t n_total, int32_t row0,
     c->hp.omb2 = 1.0f - beta2;
     c->hp.eps = eps;
     c->chain = (int64_t)n * d <= kChainMaxElems;
+    c->first_steps = kFirstSteps;
     c->hp.nf = (float)n_total;
     c->hp.inv_nf = ((n_total & (n_total - 1)) == 0) ? 1.0f / (float)n_total : 0.0f;
     c->plan_only = plan != nullptr;
@@ -763,6 +794,7 @@ int compams_set_state(compams_handle c, const float* e, const float* m, const fl
         // E now holds e itself; predictions made from the replaced accumulators are dropped
         c->e_is_x = false;
         c->e_mask_pending = false;
+        c->first_steps = kFirstSteps;
         if (c->tk.seg && !c->seg_init_host.empty()) {
             CU(cudaMemcpyAsync(c->tk.seg, c->seg_init_host.data(), c->seg_init_host.size() * sizeof(SegState),
                                cudaMemcpyHostToDevice, c->stream));

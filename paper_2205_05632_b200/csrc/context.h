@@ -152,7 +152,10 @@ struct compams_context {
     int32_t randk_group = 1;       // Random-k: workers whose elements share the map at a time
     int64_t randk_words = 0;       // ... its words
     bool many_candidates = false;  // Top-k: the lists hold more than 1/32 of the coordinates
+    int32_t cluster_max = 0, cluster_max_first = 0;  // TopkBuffers::cluster_max, and in the first steps
+    int first_steps = 0;        // of those still to come
     bool dense_kernel = false;  // some blocks are too long for a cluster to go through: the dense passes are launched every step
+    bool dense_first = false;   // ... in the first steps
     bool deliver = false;       // in a whole step the worker side hands the kept entries to the server itself (no topk_scatter)
     std::vector<compams::SegState> seg_init_host;  // Top-k: the segments' state before the first step (set_state restores it)
     uint32_t dense_count_init = 0;

@@ -1209,8 +1209,10 @@ cudaError_t fit_topk_cluster(compams_context* c) {
     } else {
         c->sel_wide = false;
     }
-    const int64_t most = (int64_t)c->tk.cluster_max * (planned / c->sel_cluster);
-    c->tk.cluster_max = most < INT32_MAX ? (int32_t)most : INT32_MAX;
+    for (int32_t* most : {&c->cluster_max, &c->cluster_max_first}) {
+        const int64_t m = (int64_t)*most * (planned / c->sel_cluster);
+        *most = m < INT32_MAX ? (int32_t)m : INT32_MAX;
+    }
     return cudaSuccess;
 }
 

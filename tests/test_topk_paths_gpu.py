@@ -48,7 +48,8 @@ def test_sweep_and_selection_in_one_kernel(n, offs, ratio, draw):
     (1, (1 << 21) + 5, 0.1),    # list emitted by a kernel of its own, 16 CTAs
     (2, 3000001, 0.111),        # the densest selection with a candidate list ...
     (2, 3000001, 0.112),        # ... and one without: always the dense passes
-    (3, 1500003, 0.02), (16, 400001, 0.02), (1, 262144, 0.002), (7, 150001, 0.05),
+    (3, 1500003, 0.02), (16, 400001, 0.02), (1, 262144, 0.002), (7, 150001, 0.05), (2, (1 << 21) + 3, 0.001),
+    (4, 262144, 0.2), (9, 20001, 0.2), (1, 262145, 0.2),  # no list: by its cluster, by the dense passes
 ])
 @pytest.mark.parametrize("draw", [normal, levels])
 def test_long_lists(n, d, ratio, draw):
@@ -219,3 +220,28 @@ def test_apply_sees_what_the_stream_did_to_theta_since_compress(n, offs, ratio, 
         assert torch.equal(ta, tb)
     a.close()
     b.close()
+
+
+def test_dense_passes_stand_by_in_the_first_steps_only():
+    # one worker's long block: a list that fails is left to the dense passes of the whole GPU while a handle is new, to its
+    # cluster afterwards
+    n, d = 1, (1 << 21) + 5
+    gen = torch.Generator(device="cuda").manual_seed(13)
+    p = Pair(n, d, [0, d], TOPK, 0.05)
+    try:
+        p.start(torch.zeros(d, device="cuda"))
+        launches, walks = [], []
+        for t in range(38):
+            before = p.gpu.buffer("status").cpu().tolist()[1], p.gpu.launch_count()
+            p.step((0.2 if t in (20, 36) else 1.0) * torch.randn(n, d, generator=gen, device="cuda"), check_e=t in (0, 20, 21, 36, 37))
+            launches.append(p.gpu.launch_count() - before[1])
+            walks.append(p.gpu.buffer("status").cpu().tolist()[1] - before[0])
+        assert walks[20] == 1 and walks[36] == 1  # the lists did fail
+        assert launches[30] == launches[34] + 1
+        # a replaced accumulator starts over
+        p.gpu.set_state(p.gpu.get_state())
+        theta, at = p.theta_gpu.clone(), p.gpu.launch_count()
+        p.gpu.step(torch.randn(n, d, generator=gen, device="cuda"), theta)
+        assert p.gpu.launch_count() - at == launches[30]
+    finally:
+        p.close()
