@@ -5,15 +5,15 @@ One benchmark "step" is one optimizer step (Algorithm 2: every worker's x = g + 
 the server's average and AMSGrad update) of ONE compressor on one batch of synthetic gradients. The
 headline workload is the largest single-GPU point of the scaling sweep: one block, d = 2^27 parameters,
 n = 32 workers, gradients N(0,1), Top-k with k = 1 % of d. The metric is gradient elements consumed per
-second (n d per step). Beside the headline the line carries, under "configs", one timed entry per
-workload and compressor: C1 (n=4, d=65,536), C2 / C3 (ResNet-18 shapes, n=16: Block-Sign per tensor,
+second (n d per step). Beside the headline one entry per workload and compressor is timed (a JSON line each on
+stderr, their step times under "configs_ms" in the headline's line): C1 (n=4, d=65,536), C2 / C3 (ResNet-18 shapes, n=16: Block-Sign per tensor,
 whole-vector Top-k at 0.1 % and 1 %), C4 (ResNet-50 shapes, n=32: layer-wise Top-k and Block-Sign) and the
 scaling sweep C5 (d = 2^20 .. 2^27, n = 1, 8, 32, Top-k / Block-Sign / k = d), each with its step time,
 its compulsory HBM bytes and the fraction of the HBM roofline that makes.
 
   python bench.py [--gpus N] [--steps K] [--warmup W] [--impl reference] [--only NAME ...]
 
-Prints ONE JSON line. With --gpus N > 1 (under torch.distributed.run) every rank runs an independent
+Prints ONE JSON line on stdout, short enough (LINE_MAX characters) for a record that keeps the end of the output. With --gpus N > 1 (under torch.distributed.run) every rank runs an independent
 replica of the headline on its own GPU ("replicas only": the path has no inter-GPU exchange) and the line
 reports the aggregate over the max time across ranks. --impl reference times the CPU oracle on the host
 cores, on a bounded sample of the headline workload, instead of the CUDA library.
@@ -40,6 +40,7 @@ from paper_2205_05632_b200 import workloads as W
 
 METRIC = "COMP-AMS step: gradient elems/s"
 UNIT = "elem/s"
+LINE_MAX = 2600
 L2_BYTES = 126 * 1024 * 1024
 NOMINAL_HBM_GBS = 8000.0  # the nominal HBM3e figure the target fraction is quoted against
 
@@ -166,6 +167,27 @@ class ClockSampler:
         if sm:
             out.update(sm_mhz=statistics.median(sm), sm_max_mhz=max(mx), reasons=sorted(reasons), samples=len(sm))
         return out
+
+
+def rounded(x):
+    """Floats to six significant digits, in nested lists and dicts."""
+    if isinstance(x, float):
+        return float("%.6g" % x)
+    if isinstance(x, dict):
+        return {k: rounded(v) for k, v in x.items()}
+    return [rounded(v) for v in x] if isinstance(x, (list, tuple)) else x
+
+
+def one_line(line):
+    """The line as printed: as many of the entries' times as fit LINE_MAX, in their order."""
+    line, times = rounded(line), rounded(line.get("configs_ms", {}))
+    while True:
+        if times:
+            line["configs_ms"] = times
+        text = json.dumps(line, separators=(",", ":"))
+        if len(text) <= LINE_MAX or not times:
+            return text
+        times.popitem()
 
 
 # ------------------------------------------------------------------------------------------------------
@@ -399,7 +421,7 @@ def run_reference(args):
         "cpu_baseline": {"value": value, "unit": UNIT, "cores": cores, "kind": "oracle", "sample": what},
         "e2e": {"value": value, "unit": UNIT, "h2d_bytes_per_step": 0, "d2h_bytes_per_step": 0},
     }
-    print(json.dumps(line))
+    print(one_line(line))
 
 
 # ------------------------------------------------------------------------------------------------------
@@ -554,13 +576,14 @@ def main():
                 continue
             entries.append(time_entry(name, build, mode, bf16, args.config_steps, args.config_warmup, peak, peak_kind,
                                       cache))
+            print(json.dumps(rounded(entries[-1])), file=sys.stderr, flush=True)
         cache.clear()
-        line["configs"] = entries
-        line["configs_protocol"] = ("per entry: %d steps between two CUDA events after %d warm-up steps, a different "
-                                    "gradient batch every step (each entry's `gradients`); min_bytes = (12 n + 32) d with error feedback ((10 n + 32) d with bfloat16 "
-                                    "gradients), (4 n + 32) d for k = d" % (args.config_steps, args.config_warmup))
+        # per entry: args.config_steps steps between two CUDA events after args.config_warmup warm-up steps, a different
+        # gradient batch every step (the entry's `gradients`); min_bytes = (12 n + 32) d with error feedback ((10 n + 32) d
+        # with bfloat16 gradients), (4 n + 32) d for k = d
+        line["configs_ms"] = {e["name"]: e["ms"] for e in entries}
     if rank == 0:
-        print(json.dumps(line))
+        print(one_line(line))
     if dist is not None:
         dist.barrier()
         dist.destroy_process_group()
