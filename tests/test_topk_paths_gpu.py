@@ -56,6 +56,12 @@ def test_long_lists(n, d, ratio, draw):
     run(n, [0, d], TOPK, ratio, draw, steps=5)
 
 
+def test_lists_of_several_rounds_that_one_cta_each_takes():
+    # more lists than clusters would fit: 5500 entries per list, a round is 4096
+    st = run(16, [40000 * b for b in range(21)], TOPK, 0.11, normal, steps=6)
+    assert st[2] > st[1]
+
+
 def test_long_and_short_lists_side_by_side():
     sizes = [900001, 37, 4096, 4097, 600003, 20000, 1, 70001, 250007, 9000]
     st = run(3, list(np.cumsum([0] + sizes)), TOPK, 0.04, normal, steps=6)
