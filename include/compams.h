@@ -70,7 +70,8 @@ enum compams_buffer {
     COMPAMS_BUF_SIGN_WORD_OFFSETS = 9, /* int64 [M+1] first word of block b inside a row of SIGN_BITS            */
     COMPAMS_BUF_SCALES = 10,      /* float  [n, M]   Block-Sign scales ||x_B||_1 / d_B                           */
     COMPAMS_BUF_STATUS = 11       /* uint32 [8]      [0] status word (0 = clean); Top-k counters since creation:
-                                                    [1] (worker, block) selections done by the dense passes,
+                                                    [1] (worker, block) selections decided by passes over the
+                                                    block, by the dense passes or by the block's own cluster,
                                                     [2] selections done inside the candidate list; why a list
                                                     was given up: [3] fewer candidates than k_b, [4] more than
                                                     its capacity, [5] threshold beyond the histogram's range,
@@ -89,7 +90,7 @@ enum compams_kernel {
     COMPAMS_K_TOPK_MATERIALIZE = 6,   /* Top-k: zero e at the coordinates kept in the last step when E is read   */
     COMPAMS_K_RANDK_EMIT = 7,         /* Random-k: marks the drawn coordinates, then the sweep that takes their x */
     /* 8: reserved (never returned, never timed) */
-    COMPAMS_K_TOPK_SCATTER = 9,       /* sharded jobs, always dense selections: messages to the server's buckets */
+    COMPAMS_K_TOPK_SCATTER = 9,       /* compams_apply, always dense selections: messages to the server's buckets */
     COMPAMS_K_AMSGRAD = 10,           /* Top-k: AMSGrad update from the accumulated average                   */
     COMPAMS_K_TOPK_SMALL = 11,        /* Top-k: whole small blocks selected inside shared memory              */
     COMPAMS_K_TOPK_SELECT = 12,       /* Top-k: exact selection inside the candidate lists, the emission of long
@@ -346,8 +347,8 @@ int compams_get_buffer(compams_handle h, int32_t which, void** dev_ptr, int64_t*
 
 /* compams_check_status - synchronise the handle's stream, read the device status word and any
  * pending CUDA error. Returns OK, ERR_CUDA or ERR_DEVICE_STATUS; *status_word (host, may be null)
- * receives the raw word (bit 0: a segment emitted a wrong number of entries,
- * bit 2: a server kernel gave up waiting for its own copies). */
+ * receives the raw word (bit 0: a segment emitted a wrong number of entries, bit 1: the dense passes
+ * counted fewer entries in a block than it keeps, bit 2: a server kernel gave up waiting for its own copies). */
 int compams_check_status(compams_handle h, uint32_t* status_word);
 
 /*

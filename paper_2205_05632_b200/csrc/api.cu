@@ -223,8 +223,9 @@ int group_segments(compams_context* c, const std::vector<SegInfo>& segs) {
     c->sel_short = (int)few.size();
     c->sel_cluster = cluster;
     // Lists that their clusters would have to go through in many rounds are emitted by a kernel of its own: from three
-    // rounds on where the clusters leave SMs idle (n = 2, d = 4.4 M, 7.85 % kept: 119 us by the cluster, 95 by topk_emit), from eight
-    // where they do not (ResNet-18 shapes whole, n = 16, 1 %: 4.3 rounds, 386 against 398 us)
+    // rounds on where the clusters leave SMs idle (by the cluster / by topk_emit, us per step: d = 2^22, n = 1, 1.6 rounds 58.2 / 59.7, 3.2
+    // 74.1 / 66.2, 8 91.6 / 67.9; n = 8, 2.4 rounds 117 / 122, 4 131.9 / 130.7, 8 170 / 160), from eight where they do not (d = 9 M, n = 16,
+    // 3.4 rounds 333 / 334, 6.9 364 / 360, 13.7 429 / 409; d = 4 M, n = 32, 6.1 rounds 329 / 344, 12.2 404 / 423)
     if (c->sel_long && entries >= (cluster == 16 ? 3 : 8) * (int64_t)cluster * 4096) {
         const int64_t lists = (int64_t)c->n * c->sel_long;
         c->sel_parts = (int)((entries + 2047) / 2048);
@@ -266,7 +267,6 @@ int build_tiles(compams_context* c, const std::vector<int32_t>& blocks, bool top
             int64_t cap = !c->randk && has_list(kb, len) ? 8 * kb + 1024 : 0;
             if (c->fused && len <= kListlessFused) cap = 0;
             if (cap) cap = std::min(cap, len <= 65536 ? len : len / 4 + kb);
-            cap = (cap + 1) & ~(int64_t)1;  // lists are read in 128-bit pairs
             si.cap = (uint32_t)cap;
             si.cand_off = cand_total;
             cand_total += cap;

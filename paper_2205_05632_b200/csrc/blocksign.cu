@@ -162,12 +162,9 @@ __device__ __forceinline__ void bs_sweep_tile_bf16x8(const bf16_bits* __restrict
 // mid-line a warp's 512 bytes straddle five lines instead of four: measured 7 % slower). The
 // sign words stay indexed by coordinate: word q of the block takes its low 32 - s bits from the
 // q-th group of 32 shifted coordinates and its high s bits from the next group. The word a tile
-// shares with the next tile is put together by bs_scales from the two shares left in `edge`.
-#ifndef COMPAMS_BF16_SWEEP_CTAS
-#define COMPAMS_BF16_SWEEP_CTAS 5
-#endif
+// shares with the next tile is put together by bs_scales, or by bs_apply, from the two shares left in `edge`.
 template <typename GT>
-__global__ void __launch_bounds__(kThreads, sizeof(GT) == 2 ? COMPAMS_BF16_SWEEP_CTAS : 8) bs_sweep_kernel(Tables t, BsBuffers b, const GT* __restrict__ G,
+__global__ void __launch_bounds__(kThreads, sizeof(GT) == 2 ? 5 : 8) bs_sweep_kernel(Tables t, BsBuffers b, const GT* __restrict__ G,
                                                                int deferred, const __grid_constant__ SegParams sp_) {
     __shared__ double red[kWarps];
     __shared__ uint32_t sh_first[kWarps];
@@ -349,9 +346,10 @@ struct ApplyShared {
 // Bound by memory from here on (32 B per coordinate and the sign bits); before, with one predicated binary64 add per worker
 // and coordinate, or 16-entry tables and a transposition across the warp, by instruction issue (786 instructions per 4
 // coordinates at n = 16, half of them the sum), and with blocks off the 16-byte grid by 32-bit accesses: steps of ResNet-18
-// shapes, n = 16 427 -> 404 us; d = 6.6 M in 7 ragged blocks, n = 4 105 -> 96; 8 of 32 workers, ResNet-50 shapes 649 -> 623.
+// shapes, n = 16 429 -> 406 us; d = 6.6 M in 7 ragged blocks, n = 4 105 -> 96; 8 of 32 workers, ResNet-50 shapes 652 -> 627.
 // Tried: 8 consecutive coordinates per thread in the update too, by 256-bit accesses from registers (417 us on the first,
-// 142 on the second), three and five CTAs per SM, CTAs of 64 and 128 threads for small vectors (slower than 256).
+// 142 on the second), three and five CTAs per SM, CTAs of 64 and 128 threads for small vectors (slower than 256; those have
+// bs_apply_short).
 // OWN: the tile sums have not been added up by bs_scales (small blocks, all workers in this handle): every CTA adds up
 // its block's, and completes the sign words that its tile has in common with the next.
 template <bool RECORD, bool OWN>

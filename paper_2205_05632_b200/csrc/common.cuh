@@ -204,7 +204,7 @@ __device__ __forceinline__ void allow_dependents() { asm volatile("griddepcontro
 
 // Bulk copies of a CTA's own: an mbarrier in shared memory (its address) that one thread initialises, told how many bytes to
 // expect, and waited for by all (after a __syncthreads that follows the initialisation). Addresses and sizes are
-// multiples of 16. The wait gives up, false, after some seconds.
+// multiples of 16. The wait gives up, false, after 65,536 tries, each of which the hardware may hold for a while.
 __device__ __forceinline__ void mbar_init(uint32_t bar) {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar) : "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");

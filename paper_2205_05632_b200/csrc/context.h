@@ -9,10 +9,6 @@
 #include "../../include/compams.h"
 #include "common.cuh"
 
-#ifndef COMPAMS_CHAIN_MAX
-#define COMPAMS_CHAIN_MAX ((int64_t)1 << 28)
-#endif
-
 namespace compams {
 
 constexpr int kSmallMax = 4096;    // Top-k blocks up to this size are selected inside one CTA's shared memory
@@ -27,7 +23,7 @@ constexpr int kWarpCand = 128;           // candidates a warp of the sweep can s
 constexpr int kWarpCandMany = 256;       // ... where more than 1/32 of the coordinates are kept
 constexpr int kSurvCap = 2048;           // threshold-bin entries a select can rank in shared memory
 constexpr int kSelBins = 4096;           // bins of the candidate select's first histogram
-constexpr int64_t kChainMaxElems = COMPAMS_CHAIN_MAX;  // n d up to which a step's kernels are chained
+constexpr int64_t kChainMaxElems = (int64_t)1 << 28;  // n d up to which a step's kernels are chained
 
 // Per (worker, large block) Top-k selection state.
 struct SegState {
@@ -90,7 +86,7 @@ struct TopkBuffers {
     SegState* seg;             // [n * nseg]
     uint32_t* tile_ties;       // [n, ntiles]
     uint2* cand;               // [n, cand_total] (coordinate, bits of x) pairs collected by the sweep
-    int64_t cand_total;        // candidate slots per worker (even: lists are read in 128-bit pairs)
+    int64_t cand_total;        // candidate slots per worker
     int32_t cluster_max;       // coordinates per CTA up to which a select's cluster goes through the block itself
     uint32_t* dense_count;     // [1] segments currently marked for the dense passes
     uint32_t* sel_ticket;      // [n * long lists, 2] threshold-bin entries collected; parts of the emission done

@@ -5,8 +5,8 @@
 // four state vectors: (4n + 32) bytes per coordinate, plus 4 for gbar while the caller has asked for it to be recorded
 // (a null gbar: not written).
 //
-// amsgrad_bucket: the server update of the Top-k path. The scatter kernel has grouped the kept
-// (coordinate, value) entries of all workers by coordinate range; one CTA per range sums them in
+// amsgrad_bucket: the server update of the Top-k and Random-k paths. Whoever emitted the kept (coordinate, value)
+// entries, or topk_scatter, has grouped those of all workers by coordinate range; one CTA per range sums them in
 // binary64 in shared memory, rounds, divides by n and applies the moment, maximum and parameter updates.
 #include "context.h"
 
@@ -76,7 +76,7 @@ __global__ void __launch_bounds__(kThreads, CTAS_PER_SM) dense_mean_amsgrad_kern
 // the terms' exponents) + log2 n <= 53, i.e. the magnitudes kept at one coordinate lie within 2^24 of one
 // another at n = 32. Wider spreads (one worker keeps 1e-12 where another keeps 1) can round differently from
 // run to run in the last bit of gbar, which stays inside the tolerance the step is specified to. Entries
-// that did not fit their bucket were added to acc[] by the scatter kernel and are folded in (and acc
+// that did not fit their bucket were added to acc[] when they were delivered and are folded in (and acc
 // cleared) here. Bound by memory (32 B per coordinate, 8 per entry). With the state requested into registers instead of
 // shared memory the step took 388.2 instead of 385.3 us (ResNet-18 shapes whole, n = 16, 0.1 %), 243.7 instead of 241.2 (n = 1,
 // d = 28.5 M, 1 %); six CTAs per SM are no better, seven lose 5 %.

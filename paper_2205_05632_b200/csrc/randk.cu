@@ -15,7 +15,7 @@
 // The map is what makes the drawn coordinates meet their x in index order: it is small enough for the L2 (64 MB: hence the
 // groups), where setting a bit costs a fraction of a visit to DRAM. (A sweep that left x in E, and one atomic exchange per
 // slot that fetched it from there and zeroed it, was bound by the rate of scattered accesses, 16 to 18 G per second: step on
-// ResNet-18 shapes, n = 16, 1 % 481 -> 415 us, n = 8, d = 2^26, 10 % 4086 -> 2397.)
+// ResNet-18 shapes, n = 16, 1 % 486 -> 429 us, n = 8, d = 2^26, 10 % 4086 -> 2397.)
 #include "context.h"
 #include "scatter.cuh"
 

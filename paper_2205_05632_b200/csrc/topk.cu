@@ -26,8 +26,8 @@
 //     collect       keys above the threshold are emitted; threshold ties too unless only some fit,
 //                   in which case they are counted per tile
 //     ties          takes the lowest-index threshold ties, tile by tile in index order
-//   Whoever emits an (index, value) pair also appends it to the bucket of its coordinate range for the server kernel (the
-//   server's average); topk_scatter does that for the messages of a sharded job and of always dense selections.
+//   In a whole step whoever emits an (index, value) pair also appends it to the bucket of its coordinate range for the server
+//   kernel (the server's average); topk_scatter does that from the messages in compams_apply and after always dense selections.
 //   The residual update at a kept coordinate (e = x - x = 0) is deferred: E keeps x there, and every selection
 //   leaves one magnitude per segment such that the kept elements are exactly those with |x| at or above it;
 //   whoever reads E next - the next sweep, or topk_materialize - treats them as 0. Where a selection cuts through
@@ -281,9 +281,9 @@ __global__ void __launch_bounds__(kThreads, sizeof(GT) == 2 ? 5 : 4) topk_sweep_
 // segment. A list that cannot decide: the cluster goes through the block itself, or, where the block is too long for
 // its few CTAs, leaves it to the dense passes of the whole GPU. Lists come longest first, every worker's copy of one
 // block side by side: the clusters that take longest start first and the last wave holds the shortest.
-// Two CTAs of 512 threads per SM, 64 registers: CTAs of 1024 threads were slower wherever more than one list is worked on
-// (ResNet-50 shapes layer-wise, n = 32: step 1760 -> 1800 us; n = 8, d = 2^20: 42 -> 54), three CTAs of 512 at 40 registers faster
-// layer-wise (1744) and slower for single lists (n = 4, d = 65,536: 17.5 -> 19.1).
+// Two CTAs of 512 threads per SM, 64 registers: CTAs of 1024 threads were slower for many lists (ResNet-50 shapes layer-wise,
+// n = 32: step 1760 -> 1800 us; n = 8, d = 2^20: 42 -> 54; a few that are only counted take them, see fit_topk_cluster), three CTAs
+// of 512 at 40 registers faster layer-wise (1744) and slower for single lists (n = 4, d = 65,536: 17.5 -> 19.1).
 constexpr int kSelThreads = 512;
 
 template <int NT>
@@ -1087,7 +1087,7 @@ __global__ void __launch_bounds__(kThreads) topk_small_kernel(Tables t, TopkBuff
 // scatter: the kept (index, value) pairs of the messages are handed to the server grouped by coordinate range.
 
 // All messages at once: `count` pairs of every worker the server averages over. For the messages that the selection did
-// not deliver itself: those of a sharded job, and of handles whose blocks keep so many entries that the dense passes
+// not deliver itself: those that compams_apply finds, and of handles whose blocks keep so many entries that the dense passes
 // select them (their CTAs append entry by entry; here the lanes of a warp that meet in a bucket share one atomic).
 __global__ void __launch_bounds__(kThreads) topk_scatter_kernel(TopkBuffers b, int64_t count) {
     dependency_wait();
@@ -1184,10 +1184,10 @@ static cudaError_t cluster_fits(void (*kernel)(KArgs...), int threads, int clust
 // The clusters were planned without a device, for 148 SMs in GPCs of at least 16. Where SMs are shared out (another process, a
 // partition) and none of that size can be resident, smaller ones take over, each CTA with a larger share of the same blocks.
 cudaError_t fit_topk_cluster(compams_context* c) {
-    // A handful of long lists that are only counted by topk_select: twice the threads per CTA (n = 1, d = 28.5 M, 1 %: 241.2 ->
-    // 236.2 us; n = 2, d = 4.4 M, 7.85 %: 91.6 -> 89.0; n = 5, d = 9.3 M, 2 %: 179.2 -> 177.2; but eight lists, n = 8, d = 4.2 M,
-    // 10 %: 163.9 -> 172.0)
-    c->sel_wide = c->sel_parts && c->sel_cluster == 16 && (int64_t)c->n * c->sel_long <= 5;
+    // As many long lists as there are GPCs for them, less one, that are only counted by topk_select: twice the threads per CTA
+    // (512 / 1024 threads, us per step: d = 2^22, 10 %, n = 1 70.3 / 68.0, n = 5 122.5 / 119.7, n = 7 147.1 / 144.7, n = 8 160.7 / 168.7;
+    // d = 9 M, 2 %, n = 1 100.0 / 98.7, n = 7 200.8 / 200.5, n = 8 217.3 / 225.1)
+    c->sel_wide = c->sel_parts && c->sel_cluster == 16 && (int64_t)c->n * c->sel_long <= 7;
     const int planned = c->sel_cluster;
     bool fits = planned == 1;
     for (; !fits && c->sel_cluster > 1; c->sel_cluster /= fits ? 1 : 2) {
