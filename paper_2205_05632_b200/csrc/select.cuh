@@ -38,7 +38,7 @@ struct SelectShared {
     uint32_t winners, base;       // winners of this CTA: counted, then written so far; its first message slot
     uint32_t slots, nsurv;        // the first CTA's: message slots handed out, entries collected
     uint32_t listed;              // the first CTA's: candidates listed by a sweep of the same kernel
-    uint32_t decided;             // the first CTA's verdict on a list that it has taken alone
+    uint32_t undecided;           // 1: the first CTA has taken the list alone and could not decide
 };
 
 // The CTAs that select together: those of the cluster, or the first of them alone.

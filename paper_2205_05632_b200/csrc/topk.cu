@@ -294,6 +294,7 @@ __device__ __forceinline__ void start_select(SelectShared<NT>& sh) {
         sh.slots = 0u;
         sh.nsurv = 0u;
         sh.listed = 0u;
+        sh.undecided = 0u;
     }
     __syncthreads();
 }
@@ -324,50 +325,61 @@ __device__ __forceinline__ SelectJob select_job(const Tables& t, const TopkBuffe
     return job;
 }
 
+// A block whose list of c candidates has not decided, for the reason `why`: by its group, or left to the dense passes. Not
+// inlined, and the block's description and state are fetched again, so that a list that decides need not keep them in registers.
+template <int NT>
+__device__ __noinline__ void select_without_list(Group grp, SelectShared<NT>& sh, const Tables& t, const TopkBuffers& b, int i, int seg,
+                                                 uint32_t c, int why, bool deliver) {
+    const SegInfo si = t.segs[seg];
+    const size_t sg = (size_t)i * t.nseg + seg;
+    SegState* st = b.seg + sg;
+    const bool first = grp.rank == 0 && threadIdx.x == 0;
+    const bool predicted = st->tau_hat != kNoPrediction;
+    const uint32_t boost = st->boost;
+    if (first && predicted && si.cap) atomicAdd(b.status + why, 1u);
+    if ((int64_t)si.len <= (int64_t)b.cluster_max * grp.size) {
+        grp.sync();  // the state has been read by all
+        if (first && predicted && c < si.kb) margin_came_up_short(st);
+        const SelectJob job = select_job(t, b, si, i, deliver);
+        select_from_block<NT>(grp, b, job, sh, st, b.thr + sg, job.erow + si.o, (uint32_t)si.len, (uint32_t)si.o, si.cap != 0u, boost);
+        if (grp.size > 1) cg::this_cluster().sync();
+        return;
+    }
+    if (first) {
+        st->fallback = 1u;
+        atomicAdd(b.dense_count, 1u);
+        if (predicted && c < si.kb) margin_came_up_short(st);
+    }
+}
+
 // Called by all threads of the group. `state_read`: a barrier of the group lies between its CTAs' reads of `s` and this call.
 template <int NT>
 __device__ __forceinline__ void select_segment(Group grp, SelectShared<NT>& sh, const Tables& t, const TopkBuffers& b,
                                                const SegInfo& si, int i, int seg, const SelectState& s, bool state_read, bool deliver,
                                                bool defer) {
     const size_t sg = (size_t)i * t.nseg + seg;
-    SegState* st = b.seg + sg;
-    const unsigned ctas = grp.size;
-    const bool first = grp.rank == 0 && threadIdx.x == 0;
-    SelectJob job = select_job(t, b, si, i, deliver);
     // the same decision in every CTA of the group: nobody writes these words before all have read them
     int why = s.c < si.kb ? 3 : 4;
     if (s.tau_hat != kNoPrediction && s.c >= si.kb && s.c <= si.cap) {
         // a short list: barriers of the cluster would cost more than the other CTAs save, the first takes it alone. They
         // wait for its verdict: a list that cannot decide needs all of them for the block.
-        const bool by_first = ctas > 1 && s.c <= (uint32_t)(ListSlice::kU * NT);
+        const bool by_first = grp.size > 1 && s.c <= (uint32_t)(ListSlice::kU * NT);
         // the first will leave the next step's state in the words that they decide by: all must have read them
         if (by_first && !state_read) grp.sync();
         bool decided = false;
         if (!by_first || grp.rank == 0) {
+            SelectJob job = select_job(t, b, si, i, deliver);
             job.defer = defer && !by_first;
             const uint2* list = b.cand + (size_t)i * (size_t)b.cand_total + (size_t)si.cand_off;
-            decided = select_from_list<NT>(by_first ? Group{1u, 0u} : grp, b, job, sh, st, b.thr + sg, list, s.c, s.tau_hat, s.S, s.boost,
-                                           &why);
-            job.defer = false;
-            if (by_first && threadIdx.x < ctas) *grp.of(&sh.decided, threadIdx.x) = decided ? 1u : 0u;
+            decided = select_from_list<NT>(by_first ? Group{1u, 0u} : grp, b, job, sh, b.seg + sg, b.thr + sg, list, s.c, s.tau_hat, s.S,
+                                           s.boost, &why);
+            if (by_first && !decided && threadIdx.x < grp.size) *grp.of(&sh.undecided, threadIdx.x) = 1u;
         }
         // the first CTA's shared memory stays until all have read from it
-        if (ctas > 1 && (by_first || decided)) cg::this_cluster().sync();
-        if (by_first ? sh.decided != 0u : decided) return;
+        if (grp.size > 1 && (by_first || decided)) cg::this_cluster().sync();
+        if (by_first ? sh.undecided == 0u : decided) return;
     }
-    if (first && s.tau_hat != kNoPrediction && si.cap) atomicAdd(b.status + why, 1u);
-    if ((int64_t)si.len <= (int64_t)b.cluster_max * ctas) {
-        grp.sync();  // the state has been read by all
-        if (first && s.tau_hat != kNoPrediction && s.c < si.kb) margin_came_up_short(st);
-        select_from_block<NT>(grp, b, job, sh, st, b.thr + sg, job.erow + si.o, (uint32_t)si.len, (uint32_t)si.o, si.cap != 0u, s.boost);
-        if (ctas > 1) cg::this_cluster().sync();
-        return;
-    }
-    if (first) {
-        st->fallback = 1u;
-        atomicAdd(b.dense_count, 1u);
-        if (s.tau_hat != kNoPrediction && s.c < si.kb) margin_came_up_short(st);
-    }
+    select_without_list<NT>(grp, sh, t, b, i, seg, s.c, why, deliver);
 }
 
 // seg_list: `nlong` blocks that a cluster selects from, then `nshort` that one CTA does; a cluster's CTAs take as many
