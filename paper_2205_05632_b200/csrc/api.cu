@@ -270,6 +270,7 @@ int build_tiles(compams_context* c, const std::vector<int32_t>& blocks, bool top
             int64_t cap = !c->randk && has_list(kb, len) ? 8 * kb + 1024 : 0;
             if (c->fused && len <= kListlessFused) cap = 0;
             if (cap) cap = std::min(cap, len <= 65536 ? len : len / 4 + kb);
+            cap = (cap + 15) & ~(int64_t)15;  // lists start on 128-byte lines
             si.cap = (uint32_t)cap;
             si.cand_off = cand_total;
             cand_total += cap;
