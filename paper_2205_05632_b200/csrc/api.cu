@@ -232,7 +232,7 @@ int group_segments(compams_context* c, const std::vector<SegInfo>& segs) {
     if (c->sel_long && entries >= (cluster == 16 ? 3 : 8) * (int64_t)cluster * 4096) {
         const int64_t lists = (int64_t)c->n * c->sel_long;
         c->sel_parts = (int)((entries + 2047) / 2048);
-        RC(dev_alloc(c, &c->tk.sel_ticket, (size_t)lists * 2));
+        RC(dev_alloc(c, &c->tk.sel_ticket, (size_t)lists * 4));
         RC(dev_alloc(c, &c->tk.sel_surv, (size_t)lists * kSurvCap, false));
     }
     many.insert(many.end(), few.begin(), few.end());

@@ -36,34 +36,44 @@ __device__ __forceinline__ void scatter_warp(const TopkBuffers& b, bool valid, i
     deliver_pair(b, T, base + (uint32_t)__popc(peers & ((1u << lane) - 1u)), j, xbits);
 }
 
-// U entries (coordinate, bits) per thread, the whole warp together, of which the `take`n ones are delivered: neighbouring
-// lanes whose entries fall into the same bucket (taken or not) get their slots with one atomic, and all U rounds of
-// atomics are in flight before the first is waited for. The lists that Top-k emits from are grouped by coordinate
+// U entries (coordinate, bits) per thread, the whole warp together, of which the `take`n ones are delivered (`wins`: their
+// ballots): neighbouring lanes whose entries fall into the same bucket (taken or not) get their slots with one atomic, and all U
+// rounds of atomics are in flight between ask() and put(). The lists that Top-k emits from are grouped by coordinate
 // range, so the runs are long; entries in random order cost one atomic each. (Finding all equal buckets of the warp
 // with __match_any_sync instead took most of the emission's instructions.)
 template <int U>
-__device__ __forceinline__ void scatter_runs(const TopkBuffers& b, const bool (&take)[U], const uint2 (&cv)[U]) {
-    const int lane = threadIdx.x & 31;
-    const unsigned below = (1u << lane) - 1u, upto = below | (1u << lane);
+struct RunSlots {
     uint32_t base[U], head[U], rank[U];
+    __device__ __forceinline__ void ask(const TopkBuffers& b, const unsigned (&wins)[U], const uint2 (&cv)[U]) {
+        const int lane = threadIdx.x & 31;
+        const unsigned below = (1u << lane) - 1u, upto = below | (1u << lane);
 #pragma unroll
-    for (int u = 0; u < U; ++u) {
-        const uint32_t T = cv[u].x / (uint32_t)kBucketSpan;
-        const uint32_t left = __shfl_up_sync(0xffffffffu, T, 1);
-        const unsigned heads = __ballot_sync(0xffffffffu, lane == 0 || left != T);
-        const unsigned wins = __ballot_sync(0xffffffffu, take[u]);
-        head[u] = 31u - (uint32_t)__clz(heads & upto);  // first lane of this lane's run
-        const unsigned later = heads & ~upto;           // heads of the runs after it
-        const unsigned run = (later ? (later & (0u - later)) - 1u : 0xffffffffu) & ~((1u << head[u]) - 1u);
-        rank[u] = (uint32_t)__popc(wins & run & below);
-        base[u] = 0;
-        if (head[u] == (uint32_t)lane && (wins & run)) base[u] = atomicAdd(b.bcount + T, (uint32_t)__popc(wins & run));
+        for (int u = 0; u < U; ++u) {
+            const uint32_t T = cv[u].x / (uint32_t)kBucketSpan;
+            const uint32_t left = __shfl_up_sync(0xffffffffu, T, 1);
+            const unsigned heads = __ballot_sync(0xffffffffu, lane == 0 || left != T);
+            head[u] = 31u - (uint32_t)__clz(heads & upto);  // first lane of this lane's run
+            const unsigned later = heads & ~upto;           // heads of the runs after it
+            const unsigned run = (later ? (later & (0u - later)) - 1u : 0xffffffffu) & ~((1u << head[u]) - 1u);
+            rank[u] = (uint32_t)__popc(wins[u] & run & below);
+            base[u] = 0;
+            if (head[u] == (uint32_t)lane && (wins[u] & run)) base[u] = atomicAdd(b.bcount + T, (uint32_t)__popc(wins[u] & run));
+        }
     }
+    __device__ __forceinline__ void put(const TopkBuffers& b, const unsigned (&wins)[U], const uint2 (&cv)[U]) const {
+        const int lane = threadIdx.x & 31;
 #pragma unroll
-    for (int u = 0; u < U; ++u) {
-        const uint32_t first = __shfl_sync(0xffffffffu, base[u], head[u]);
-        if (take[u]) deliver_pair(b, cv[u].x / (uint32_t)kBucketSpan, first + rank[u], (int32_t)cv[u].x, cv[u].y);
+        for (int u = 0; u < U; ++u) {
+            const uint32_t first = __shfl_sync(0xffffffffu, base[u], head[u]);
+            if ((wins[u] >> lane) & 1u) deliver_pair(b, cv[u].x / (uint32_t)kBucketSpan, first + rank[u], (int32_t)cv[u].x, cv[u].y);
+        }
     }
+};
+template <int U>
+__device__ __forceinline__ void scatter_runs(const TopkBuffers& b, const unsigned (&wins)[U], const uint2 (&cv)[U]) {
+    RunSlots<U> slots;
+    slots.ask(b, wins, cv);
+    slots.put(b, wins, cv);
 }
 
 }  // namespace compams
