@@ -296,7 +296,8 @@ __global__ void __launch_bounds__(kThreads) bs_materialize_kernel(Tables t, floa
     }
 }
 
-constexpr int kApplyChunk = 16;         // workers whose sign words and scales are staged at a time
+// Workers whose sign words and scales are staged at a time: with tables of 8 workers' scales, of 4 workers'.
+constexpr int kApplyEights = 16, kApplyFours = 32;
 
 // Transposes an 8 x 8 bit matrix whose rows are the bytes of lo (rows 0-3) and hi (rows 4-7): afterwards bit i of byte k
 // is what bit k of byte i was. Three rounds of the usual block swap.
@@ -318,14 +319,16 @@ __device__ __forceinline__ void transpose8(uint32_t& lo, uint32_t& hi) {
 constexpr int kApplySpan = 8 * kThreads;  // coordinates per CTA of bs_apply
 
 // Shared memory of one bs_apply CTA.
+template <bool FOURS>
 struct ApplyShared {
+    static constexpr int kChunk = FOURS ? kApplyFours : kApplyEights;
     float state[4][kApplySpan + 4];  // m, v, vhat, theta of the CTA's coordinates, from a 16-byte boundary on
     union {
         struct {
-            uint32_t bits[kApplyChunk][kApplySpan / 32];  // [worker][word]
-            double eight[kApplyChunk / 8][256];           // subset sums of 8 workers' scales
-            double four[kApplyChunk / 4][16];             // ... of 4 workers'
-            double scale[kApplyChunk];
+            uint32_t bits[kChunk][kApplySpan / 32];   // [worker][word]
+            double four[kChunk / 4][16];              // subset sums of 4 workers' scales
+            double eight[FOURS ? 1 : kChunk / 8][256];  // ... of 8 workers'
+            double scale[kChunk];
         } sum;
         float gbar[kApplySpan + 4];
     };
@@ -347,16 +350,21 @@ struct ApplyShared {
 // and coordinate, or 16-entry tables and a transposition across the warp, by instruction issue (786 instructions per 4
 // coordinates at n = 16, half of them the sum), and with blocks off the 16-byte grid by 32-bit accesses: steps of ResNet-18
 // shapes, n = 16 429 -> 406 us; d = 6.6 M in 7 ragged blocks, n = 4 105 -> 96; 8 of 32 workers, ResNet-50 shapes 652 -> 627.
+// FOURS, from 17 workers on: the words and scales of up to 32 workers come in one round of loads, and a coordinate adds two entries of
+// 16-entry tables per 8 workers: all 16 entries of one lie in different banks, where the lanes' lookups in 256 entries met in
+// three on average, which is what two rounds of 16 workers were bound by (the shared-memory pipe 73 % busy at n = 32; 8 of 32
+// workers, ResNet-50 shapes, this kernel 192 -> 155 us and the step 628 -> 599; n = 32, d = 4.2 M 288 -> 282).
 // Tried: 8 consecutive coordinates per thread in the update too, by 256-bit accesses from registers (417 us on the first,
 // 142 on the second), three and five CTAs per SM, CTAs of 64 and 128 threads for small vectors (slower than 256; those have
 // bs_apply_short).
 // OWN: the tile sums have not been added up by bs_scales (small blocks, all workers in this handle): every CTA adds up
 // its block's, and completes the sign words that its tile has in common with the next.
-template <bool RECORD, bool OWN>
+template <bool RECORD, bool OWN, bool FOURS>
 __global__ void __launch_bounds__(kThreads, 4) bs_apply_kernel(const __grid_constant__ Tables t, const __grid_constant__ BsBuffers b,
                                                                float* __restrict__ theta, const __grid_constant__ HyperParams hp,
                                                                const __grid_constant__ SegParams sp_) {
-    __shared__ __align__(128) ApplyShared sh;
+    constexpr int kApplyChunk = ApplyShared<FOURS>::kChunk;
+    __shared__ __align__(128) ApplyShared<FOURS> sh;
     const int tile = blockIdx.x / (kTile / kApplySpan);
     const TileInfo ti = sp_.nseg ? find_tile(sp_, tile) : load_tile(t.tiles, tile);
     const int blk = ti.blk;
@@ -421,6 +429,7 @@ __global__ void __launch_bounds__(kThreads, 4) bs_apply_kernel(const __grid_cons
             sh.sum.scale[threadIdx.x] = (double)b.scales_cur[(size_t)(i0 + threadIdx.x) * t.M + blk];
         }
         __syncthreads();
+        static_assert(kApplyChunk * 4 <= kThreads, "one table entry per thread");
         if (threadIdx.x < kApplyChunk * 4) {  // one table entry per thread: the scales of the subset's members
             const int q = threadIdx.x >> 4, sub = threadIdx.x & 15;
             double e = 0.0;
@@ -430,10 +439,12 @@ __global__ void __launch_bounds__(kThreads, 4) bs_apply_kernel(const __grid_cons
             sh.sum.four[q][sub] = e;
         }
         __syncthreads();
+        if constexpr (!FOURS) {
 #pragma unroll
-        for (int g = 0; g < kApplyChunk / 8; ++g)
-            if (g < ng) sh.sum.eight[g][threadIdx.x] = sh.sum.four[2 * g][threadIdx.x & 15] + sh.sum.four[2 * g + 1][threadIdx.x >> 4];
-        __syncthreads();
+            for (int g = 0; g < kApplyChunk / 8; ++g)
+                if (g < ng) sh.sum.eight[g][threadIdx.x] = sh.sum.four[2 * g][threadIdx.x & 15] + sh.sum.four[2 * g + 1][threadIdx.x >> 4];
+            __syncthreads();
+        }
 #pragma unroll
         for (int g = 0; g < kApplyChunk / 8; ++g) {
             if (g < ng) {  // the same for every thread of the CTA
@@ -443,11 +454,20 @@ __global__ void __launch_bounds__(kThreads, 4) bs_apply_kernel(const __grid_cons
                 uint32_t p0 = __byte_perm(__byte_perm(x[0], x[1], 0x0040), __byte_perm(x[2], x[3], 0x0040), 0x5410);
                 uint32_t p1 = __byte_perm(__byte_perm(x[4], x[5], 0x0040), __byte_perm(x[6], x[7], 0x0040), 0x5410);
                 transpose8(p0, p1);
-                all += sh.sum.eight[g][255];
+                if constexpr (FOURS) {
+                    all += sh.sum.four[2 * g][15] + sh.sum.four[2 * g + 1][15];
 #pragma unroll
-                for (int k = 0; k < 4; ++k) {
-                    a[k] += sh.sum.eight[g][(p0 >> (8 * k)) & 255u];
-                    a[4 + k] += sh.sum.eight[g][(p1 >> (8 * k)) & 255u];
+                    for (int k = 0; k < 4; ++k) {
+                        a[k] += sh.sum.four[2 * g][(p0 >> (8 * k)) & 15u] + sh.sum.four[2 * g + 1][(p0 >> (8 * k + 4)) & 15u];
+                        a[4 + k] += sh.sum.four[2 * g][(p1 >> (8 * k)) & 15u] + sh.sum.four[2 * g + 1][(p1 >> (8 * k + 4)) & 15u];
+                    }
+                } else {
+                    all += sh.sum.eight[g][255];
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) {
+                        a[k] += sh.sum.eight[g][(p0 >> (8 * k)) & 255u];
+                        a[4 + k] += sh.sum.eight[g][(p1 >> (8 * k)) & 255u];
+                    }
                 }
             }
         }
@@ -724,8 +744,13 @@ cudaError_t launch_bs_apply(compams_context* c, float* theta) {
     const dim3 grid((unsigned)(c->tab.ntiles * (is_short ? kWarps : kTile / kApplySpan)));
     // (gbar stored or not is a template parameter: a run-time branch around the store slowed the kernel by a tenth)
     void (*kernel)(const Tables, const BsBuffers, float*, const HyperParams, const SegParams) =
-        own ? (b.gbar ? bs_apply_kernel<true, true> : bs_apply_kernel<false, true>)
-            : (b.gbar ? bs_apply_kernel<true, false> : bs_apply_kernel<false, false>);
+        own ? (b.gbar ? bs_apply_kernel<true, true, false> : bs_apply_kernel<false, true, false>)
+            : (b.gbar ? bs_apply_kernel<true, false, false> : bs_apply_kernel<false, false, false>);
+    // more than 16 workers: one round for up to 32, and lookups without bank conflicts (9 to 16 workers: n = 16, ResNet-18 shapes
+    // 406.5 without, 405.5 with, n = 12, d = 9 M 260.2 / 260.4)
+    if (c->n_total > kApplyEights)
+        kernel = own ? (b.gbar ? bs_apply_kernel<true, true, true> : bs_apply_kernel<false, true, true>)
+                     : (b.gbar ? bs_apply_kernel<true, false, true> : bs_apply_kernel<false, false, true>);
     if (is_short)  // tables from 20 workers up: n = 16, d = 162,400 13.6 us with, 13.3 without, n = 32, d = 524,288 43.9 with, 45.8 without
         kernel = c->n_total >= 20 ? (b.gbar ? bs_apply_short_kernel<true, true> : bs_apply_short_kernel<true, false>)
                                   : (b.gbar ? bs_apply_short_kernel<false, true> : bs_apply_short_kernel<false, false>);

@@ -74,6 +74,9 @@ def test_long_and_short_lists_side_by_side():
     (17, list(np.cumsum([0] + [611 + 37 * k for k in range(80)]))), (4, [0, 15 * 8192]), (5, [0, 19 * 8192]), (5, [0, 20 * 8192]),
     (9, [0, 36 * 8192 - 32]), (9, [0, 36 * 8192]), (19, [0, 37, 20003]), (20, [0, 37, 20003]), (40, [0, 1000, 1003, 30001]),
     (24, [0, 95 * 8192 - 40]), (24, [0, 96 * 8192 - 40]),
+    # 17 workers and more: tables of 4 workers, 32 per round
+    (17, [0, 3, 70 * 8192 + 5]), (32, [0, 97 * 8192]), (33, [0, 5, 2054, 97 * 8192 + 3]), (40, list(np.cumsum([0] + [9001] * 90))),
+    (65, [0, 4101, 97 * 8192 + 4101]),
 ])
 def test_blocksign_server_kernels_and_who_adds_up_the_scales(n, offs):
     run(n, offs, BLOCKSIGN, 1.0, normal, steps=4)
