@@ -62,90 +62,121 @@ __device__ __forceinline__ uint32_t fmix32(uint32_t h) {
     return h;
 }
 
-// Image of r under the permutation of {0, ..., m - 1} with the given round keys; m < 2^32.
-__device__ __forceinline__ uint32_t randk_permute(uint32_t m, uint32_t r, const uint32_t* keys) {
+// One application of the network to x, whose domain has 2 w bits.
+__device__ __forceinline__ uint32_t randk_network(uint32_t x, int w, const uint32_t (&k)[6]) {
+    const uint32_t mask = (1u << w) - 1u;
+    uint32_t L = x >> w, R = x & mask;
+#pragma unroll
+    for (int round = 0; round < 6; ++round) {
+        const uint32_t nR = L ^ (fmix32(R ^ k[round]) & mask);
+        L = R;
+        R = nR;
+    }
+    return (L << w) | R;
+}
+__device__ __forceinline__ int randk_half_bits(uint32_t m) {
     int bits = 2;
     while (bits < 32 && (1u << bits) < m) bits += 2;
-    const int w = bits >> 1;
-    const uint32_t mask = (1u << w) - 1u;
-    uint32_t k[6];
-#pragma unroll
-    for (int i = 0; i < 6; ++i) k[i] = keys[i];
-    uint32_t x = r;
-    do {
-        uint32_t L = x >> w, R = x & mask;
-#pragma unroll
-        for (int round = 0; round < 6; ++round) {
-            const uint32_t nR = L ^ (fmix32(R ^ k[round]) & mask);
-            L = R;
-            R = nR;
-        }
-        x = (L << w) | R;
-    } while (x >= m);  // at most a few rounds on average: the domain is less than four times m
-    return x;
+    return bits >> 1;
 }
 
-struct Drawn {
-    bool valid;
-    int32_t il;  // worker within the handle
-    int64_t q;   // slot within the worker's message row
-    int32_t j;   // the drawn coordinate
-    int32_t blk; // its block
-    uint32_t r;  // the slot within the block's
-};
-
-// A CTA covers kThreads consecutive message slots of one worker; every thread computes the coordinate of its
-// slot. The slots of one block are consecutive, so the thread holding a block's first slot (or thread 0, for a
-// block begun in the CTA before) derives the round keys once and the others read them from shared memory.
-// Called by all threads of the CTA.
-__device__ __forceinline__ Drawn randk_draw(const Tables& t, const TopkBuffers& b, int32_t row0, uint64_t seed,
-                                            uint64_t step, uint32_t (*keys)[6]) {
-    const uint32_t per_worker = (uint32_t)((b.K + kThreads - 1) / kThreads);
-    const int tid = threadIdx.x;
-    Drawn dr;
-    dr.il = (int32_t)(blockIdx.x / per_worker);
-    dr.q = (int64_t)(blockIdx.x % per_worker) * kThreads + tid;
-    dr.valid = dr.q < b.K;
-    dr.j = dr.blk = 0;
-    dr.r = 0;
-    int64_t o = 0;
-    uint32_t len = 1, r = 0;
-    if (dr.valid) {
-        int lo = 0, hi = t.M - 1;  // the slot's block, by bisection of the slot offsets
-        while (lo < hi) {
-            const int mid = (lo + hi + 1) >> 1;
-            if (__ldg(b.seg_off + mid) <= dr.q) lo = mid; else hi = mid - 1;
-        }
-        dr.blk = lo;
-        o = __ldg(t.off + lo);
-        len = (uint32_t)(__ldg(t.off + lo + 1) - o);
-        dr.r = r = (uint32_t)(dr.q - __ldg(b.seg_off + lo));
-        if (tid == 0 || r == 0) {
-            const RoundKeys rk = randk_round_keys(seed, step, (uint64_t)(row0 + dr.il), (uint64_t)lo);
-#pragma unroll
-            for (int i = 0; i < 6; ++i) keys[tid][i] = rk.k[i];
-        }
+// The block of a message slot, by bisection of the slot offsets.
+__device__ __forceinline__ int block_of_slot(const Tables& t, const TopkBuffers& b, int64_t q) {
+    int lo = 0, hi = t.M - 1;
+    while (lo < hi) {
+        const int mid = (lo + hi + 1) >> 1;
+        if (__ldg(b.seg_off + mid) <= q) lo = mid; else hi = mid - 1;
     }
-    __syncthreads();
-    if (dr.valid) {
-        const int leader = r < (uint32_t)tid ? tid - (int)r : 0;
-        dr.j = (int32_t)(o + randk_permute(len, r, keys[leader]));
-    }
-    return dr;
+    return lo;
 }
 
-// Bit f - origin of the map stands for element f of the flat [n, d] buffers; origin is a multiple of 32, so that the map's
-// words are the 128-byte lines of E.
+// Sets the bits of the drawn coordinates. Bit f - origin of the map stands for element f of the flat [n, d] buffers; origin is a
+// multiple of 32, so that the map's words are the 128-byte lines of E. A CTA covers `per_thread` x kThreads consecutive message slots
+// of one worker; every thread computes the coordinates of its slots. Bound by the instructions of the network (a warp issues in two
+// cycles of three): a lane that is back inside the block goes on to its next slot while its neighbours still walk, so that a warp
+// waits for the longest sum of walks and not, slot for slot, for the longest walk, and the round keys serve that many more slots
+// (one slot per thread took 37 us for 1.8 M slots in blocks of 11.2 M coordinates, two thirds of the domain, this takes 25:
+// ResNet-18 shapes, n = 16, 430 -> 418 us per step).
 __global__ void __launch_bounds__(kThreads) randk_mark_kernel(const __grid_constant__ Tables t, const __grid_constant__ TopkBuffers b,
-                                                              int32_t row0, int32_t i0, int64_t origin, uint64_t seed, uint64_t step) {
+                                                              int32_t row0, int32_t i0, int64_t origin, uint64_t seed, uint64_t step,
+                                                              int per_thread) {
     __shared__ uint32_t keys[kThreads][6];
+    const int64_t span = (int64_t)per_thread * kThreads;
+    const uint32_t per_worker = (uint32_t)((b.K + span - 1) / span);
+    const int tid = threadIdx.x;
+    const int il = (int)(blockIdx.x / per_worker);
+    const int64_t first = (int64_t)(blockIdx.x % per_worker) * span, last = first + span < b.K ? first + span : b.K;
+    const uint64_t worker = (uint64_t)(row0 + i0 + il);
+    const int64_t row = (int64_t)(i0 + il) * t.d - origin;
+    auto mark = [&](int64_t j) {
+        const int64_t f = row + j;
+        atomicOr(b.map + (f >> 5), 1u << (f & 31));
+    };
+    const int blk0 = block_of_slot(t, b, first);
+    if (__ldg(b.seg_off + blk0 + 1) >= last) {  // one block
+        if (tid == 0) {
+            const RoundKeys rk = randk_round_keys(seed, step, worker, (uint64_t)blk0);
+#pragma unroll
+            for (int i = 0; i < 6; ++i) keys[0][i] = rk.k[i];
+        }
+        const int64_t o = __ldg(t.off + blk0);
+        const uint32_t len = (uint32_t)(__ldg(t.off + blk0 + 1) - o);
+        const int w = randk_half_bits(len);
+        const int64_t slot0 = __ldg(b.seg_off + blk0);
+        __syncthreads();
+        uint32_t k[6];
+#pragma unroll
+        for (int i = 0; i < 6; ++i) k[i] = keys[0][i];
+        dependency_wait();
+        allow_dependents();
+        if (tid == 0 && first == slot0) b.slots[(size_t)(i0 + il) * t.nseg + blk0] = 0u;  // every block is tiled: segment = block
+        int64_t q = first + tid;
+        uint32_t x = (uint32_t)(q - slot0);
+        while (q < last) {
+            x = randk_network(x, w, k);
+            if (x < len) {
+                mark(o + x);
+                q += kThreads;
+                x = (uint32_t)(q - slot0);
+            }
+        }
+        return;
+    }
     dependency_wait();
     allow_dependents();
-    const Drawn dr = randk_draw(t, b, row0 + i0, seed, step, keys);
-    if (!dr.valid) return;
-    if (dr.r == 0u) b.slots[(size_t)(i0 + dr.il) * t.nseg + dr.blk] = 0u;  // every block is tiled: segment = block
-    const int64_t f = (int64_t)(i0 + dr.il) * t.d + dr.j - origin;
-    atomicOr(b.map + (f >> 5), 1u << (f & 31));
+    // several blocks: the slots of one block are consecutive, so the thread holding a block's first slot (or thread 0, for a
+    // block begun before) derives the round keys once and the others read them from shared memory
+    for (int64_t q0 = first; q0 < last; q0 += kThreads) {
+        const int64_t q = q0 + tid;
+        const bool valid = q < last;
+        int64_t o = 0;
+        uint32_t len = 1, r = 0;
+        if (valid) {
+            const int blk = block_of_slot(t, b, q);
+            o = __ldg(t.off + blk);
+            len = (uint32_t)(__ldg(t.off + blk + 1) - o);
+            r = (uint32_t)(q - __ldg(b.seg_off + blk));
+            if (tid == 0 || r == 0) {
+                const RoundKeys rk = randk_round_keys(seed, step, worker, (uint64_t)blk);
+#pragma unroll
+                for (int i = 0; i < 6; ++i) keys[tid][i] = rk.k[i];
+            }
+            if (r == 0) b.slots[(size_t)(i0 + il) * t.nseg + blk] = 0u;
+        }
+        __syncthreads();
+        if (valid) {
+            const uint32_t* mine = keys[r < (uint32_t)tid ? tid - (int)r : 0];
+            const int w = randk_half_bits(len);
+            uint32_t k[6];
+#pragma unroll
+            for (int i = 0; i < 6; ++i) k[i] = mine[i];
+            uint32_t x = r;
+            do x = randk_network(x, w, k);
+            while (x >= len);  // at most a few rounds on average: the domain is less than four times the block
+            mark(o + x);
+        }
+        __syncthreads();  // the keys have been read
+    }
 }
 
 // A warp's drawn coordinates while it streams: lane l's word of the map for the warp's l-th 32 coordinates, the number of
@@ -405,13 +436,17 @@ static cudaError_t launch_randk_typed(compams_context* c, const GT* grads) {
     TopkBuffers b = c->tk;  // the kernels see this handle's own rows of the message buffers
     b.idx += (size_t)c->row0 * (size_t)c->K;
     b.val += (size_t)c->row0 * (size_t)c->K;
-    const int64_t per_worker = (c->K + kThreads - 1) / kThreads;
     cudaError_t e = cudaSuccess;
     for (int32_t i0 = 0; i0 < c->n && e == cudaSuccess; i0 += c->randk_group) {
         const int32_t rows = c->n - i0 < c->randk_group ? c->n - i0 : c->randk_group;
         const int64_t origin = (int64_t)i0 * c->d & ~(int64_t)31;
+        // as many slots per thread as leave two CTAs per SM, eight at most (n = 3, d = 25 M in 100 blocks, 5 %: four and eight 381 us per
+        // step, sixteen 410, one 416)
+        const int64_t most = c->K * rows / (2 * 148 * kThreads);
+        const int per_thread = (int)(most < 1 ? 1 : most > 8 ? 8 : most);
+        const int64_t per_worker = (c->K + per_thread * kThreads - 1) / (per_thread * kThreads);
         e = counted(c, launch_after(randk_mark_kernel, dim3((unsigned)(per_worker * rows)), dim3(kThreads), c->stream, c->tab, b, c->row0,
-                                    i0, origin, c->seed, c->iter));
+                                    i0, origin, c->seed, c->iter, per_thread));
         if (e != cudaSuccess) break;
         void (*kernel)(const Tables, const TopkBuffers, const GT*, int32_t, int64_t, int64_t, int, const SegParams) =
             c->K * 32 > c->d ? randk_sweep_kernel<GT, 256> : randk_sweep_kernel<GT, 128>;  // mean of a warp: K / d x 1024

@@ -89,6 +89,15 @@ def test_randk_spans_that_share_words_and_overflow_their_room(n, offs, ratio):
     run(n, offs, RANDK, ratio, normal, steps=4, seed=11)
 
 
+@pytest.mark.parametrize("n,offs,ratio", [
+    # several slots per thread: one block per CTA, blocks that begin inside one, a row whose last CTA is short
+    (1, [0, 4 * 757761], 0.05), (2, [0, 1048575], 0.1), (3, [0, 1, 40, 500009, 500010, 520000, 1500001], 0.1),
+    (2, list(np.cumsum([0] + [1500 + 7 * k for k in range(700)])), 0.06),
+])
+def test_randk_several_slots_per_thread(n, offs, ratio):
+    run(n, offs, RANDK, ratio, normal, steps=3, seed=5)
+
+
 @pytest.mark.parametrize("comp", [TOPK, BLOCKSIGN, RANDK])
 def test_messages_are_complete_between_the_two_halves_of_a_step(comp):
     # whatever a whole step leaves to its server side, compress() alone leaves what the step would have sent
