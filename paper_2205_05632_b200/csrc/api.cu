@@ -518,9 +518,11 @@ int compress_device(compams_context* c, const void* grads) {
     if (first) --c->first_steps;
     c->tk.cluster_max = first ? c->cluster_max_first : c->cluster_max;
     if (c->tab.ntiles > 0) RC(run_kernel(c, COMPAMS_K_TOPK_SWEEP, [&] { return launch_topk_sweep(c, grads); }));
-    if (c->tk.nsmall > 0) RC(run_kernel(c, COMPAMS_K_TOPK_SMALL, [&] { return launch_topk_small(c, grads); }));
+    const bool selects = c->tab.ntiles > 0 && c->sel_long + c->sel_short > 0, small_last = selects && small_beside_select(c);
+    if (c->tk.nsmall > 0 && !small_last) RC(run_kernel(c, COMPAMS_K_TOPK_SMALL, [&] { return launch_topk_small(c, grads); }));
     if (c->tab.ntiles > 0) {
-        if (c->sel_long + c->sel_short > 0) RC(run_kernel(c, COMPAMS_K_TOPK_SELECT, [&] { return launch_topk_select(c); }));
+        if (selects) RC(run_kernel(c, COMPAMS_K_TOPK_SELECT, [&] { return launch_topk_select(c); }));
+        if (c->tk.nsmall > 0 && small_last) RC(run_kernel(c, COMPAMS_K_TOPK_SMALL, [&] { return launch_topk_small(c, grads); }));
         if (c->dense_kernel || (first && c->dense_first)) RC(run_kernel(c, COMPAMS_K_TOPK_DENSE, [&] { return launch_topk_dense(c); }));
         c->e_mask_pending = true;
     }

@@ -7,7 +7,7 @@
 //   Small problems: topk_fused - sweep and selection of one (worker, block) by one cluster, or one CTA.
 //
 //   Otherwise blocks of at most kSmallMax coordinates: topk_small - one CTA holds the block in shared
-//   memory and does every radix pass there; E is written once. It runs beside the tail of the sweep.
+//   memory and does every radix pass there; E is written once. It runs beside the selection of the larger blocks.
 //
 //   Larger blocks, cut into tiles of kTile coordinates.
 //   Candidate path (one pass over [n, d]), for blocks that keep at most 1/9 of their coordinates:
@@ -385,12 +385,12 @@ __device__ __forceinline__ void select_segment(Group grp, SelectShared<NT>& sh, 
 }
 
 // seg_list: `nlong` blocks that a cluster selects from, then `nshort` that one CTA does; a cluster's CTAs take as many
-// of the latter as they are. `defer`: the long lists' entries are emitted by topk_emit.
+// of the latter as they are. `defer`: the long lists' entries are emitted by topk_emit. `early`: the next kernel is topk_small.
 template <int NT>
 __global__ void __launch_bounds__(NT, 1024 / NT) topk_select_kernel(const __grid_constant__ Tables t,
                                                                    const __grid_constant__ TopkBuffers b,
                                                                    const int32_t* __restrict__ seg_list, int nlong, int nshort,
-                                                                   int deliver, int defer) {
+                                                                   int deliver, int defer, int early) {
     __shared__ SelectShared<NT> sh;
     Group grp{cg::this_cluster().num_blocks(), cg::this_cluster().block_rank()};
     unsigned item = blockIdx.x / grp.size;
@@ -408,8 +408,9 @@ __global__ void __launch_bounds__(NT, 1024 / NT) topk_select_kernel(const __grid
     const int seg = segs[idle ? 0u : q];  // the block tables are never written by a kernel
     const SegInfo si = t.segs[seg];
     start_select<NT>(sh);
+    if (early) allow_dependents();  // topk_small needs nothing of the sweep's either (which has waited for everything before it)
     dependency_wait();   // launched as a programmatic dependent while n d <= kChainMaxElems: the kernel before must be done
-    allow_dependents();  // ... and the next one may move in behind this one's last wave
+    if (!early) allow_dependents();  // ... and the next one may move in behind this one's last wave
     if (idle) return;
     const SelectState s = load_state(b.seg + (size_t)i * t.nseg + seg);
     select_segment<NT>(grp, sh, t, b, si, i, seg, s, false, deliver != 0, defer != 0 && !alone);
@@ -1025,8 +1026,9 @@ __global__ void __launch_bounds__(kThreads) topk_small_kernel(Tables t, TopkBuff
     __shared__ uint32_t hist[256];
     __shared__ uint32_t scratch[kWarps];
     __shared__ uint32_t sh_prefix, sh_krem, sh_cnt, sh_rlast, sh_taken;
-    // Shares no block with the sweep before it: its CTAs move in behind the sweep's last wave, which has ordered itself
-    // after everything earlier on the stream, and wait for the sweep only at their end, for the sake of the kernel after.
+    // Shares no block with the sweep and the selection: its CTAs move in behind the last wave of the kernel before it, which comes
+    // after a sweep that has ordered itself after everything earlier on the stream, and wait for that kernel only at their end, for
+    // the sake of the kernel after.
     if (!after_sweep) dependency_wait();
     allow_dependents();
     const int blk = b.small_blk[blockIdx.x];
@@ -1207,7 +1209,7 @@ cudaError_t launch_topk_sweep(compams_context* c, const void* grads) {
 // waits for its predecessor before its first global access): the launch latency and the prologue of a
 // kernel then overlap the tail of the one before, which is most of what such a step costs.
 
-typedef void (*SelectKernel)(const Tables, const TopkBuffers, const int32_t*, int, int, int, int);
+typedef void (*SelectKernel)(const Tables, const TopkBuffers, const int32_t*, int, int, int, int, int);
 
 // Whether the device can hold a cluster of `cluster` CTAs of a kernel (more than 8 have to be asked for, once per kernel and
 // device).
@@ -1274,7 +1276,7 @@ cudaError_t launch_topk_select(compams_context* c) {
     const cudaError_t e = counted(c, launch_cluster(kernel, dim3((unsigned)(clusters * c->sel_cluster)),
                                                     dim3(c->sel_wide ? 2 * kSelThreads : kSelThreads), c->sel_cluster, c->chain, c->stream,
                                                     c->tab, own_rows(c), (const int32_t*)c->sel_segs, c->sel_long, c->sel_short,
-                                                    delivers(c) ? 1 : 0, c->sel_parts ? 1 : 0));
+                                                    delivers(c) ? 1 : 0, c->sel_parts ? 1 : 0, small_beside_select(c) ? 1 : 0));
     if (e != cudaSuccess || !c->sel_parts) return e;
     const dim3 grid((unsigned)((int64_t)c->n * c->sel_long * c->sel_parts));
     if (c->chain)
