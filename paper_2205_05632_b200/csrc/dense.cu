@@ -80,7 +80,10 @@ __global__ void __launch_bounds__(kThreads, CTAS_PER_SM) dense_mean_amsgrad_kern
 // cleared) here. Bound by memory (32 B per coordinate, 8 per entry). With the state requested into registers instead of
 // shared memory the step took 388.2 instead of 385.3 us (ResNet-18 shapes whole, n = 16, 0.1 %), 243.7 instead of 241.2 (n = 1,
 // d = 28.5 M, 1 %); six CTAs per SM are no better, seven lose 5 %.
-template <bool RECORD>
+// EARLY: the kernel of the next step may move in before this one is done (it waits before it touches anything), where a step is two
+// kernels of a few CTAs each: n = 4, d = 65,536 15.2 -> 14.8 us, n = 8, d = 95,648 17.6 -> 17.0; larger steps get slower (ResNet-18 shapes by
+// layers, n = 4 237.5 -> 242.9, d = 2^20, n = 8 Block-Sign 27.4 -> 28.2), and as a run-time branch it cost them 1 %.
+template <bool RECORD, bool EARLY>
 __global__ void __launch_bounds__(kThreads, 5) amsgrad_bucket_kernel(int64_t d, const __grid_constant__ TopkBuffers b, float* __restrict__ theta,
                                                                      const __grid_constant__ HyperParams hp) {
     static_assert(kBucketSpan == 4 * kThreads, "one float4 group per thread");
@@ -102,6 +105,7 @@ __global__ void __launch_bounds__(kThreads, 5) amsgrad_bucket_kernel(int64_t d, 
         for (int q = 0; q < 4; ++q) bulk_load(state[q], vec[q] + (int64_t)T * kBucketSpan, bytes, bar);
     }
     dependency_wait();  // everything below is this step's: the buckets
+    if constexpr (EARLY) allow_dependents();
     // the bucket's first round of entries is requested before its fill count is known (the slots
     // exist whatever they hold; an entry is used only if the count covers it)
     const uint2* ent = b.bucket + (size_t)T * (size_t)b.bucket_cap;
@@ -187,8 +191,10 @@ cudaError_t launch_dense_mean_amsgrad(compams_context* c, const void* grads, flo
 
 cudaError_t launch_amsgrad(compams_context* c, float* theta) {
     const dim3 grid((unsigned)c->tk.nbucket);
-    return counted(c, c->tk.gbar ? launch_after(amsgrad_bucket_kernel<true>, grid, dim3(kThreads), c->stream, c->d, c->tk, theta, c->hp)
-                                 : launch_after(amsgrad_bucket_kernel<false>, grid, dim3(kThreads), c->stream, c->d, c->tk, theta, c->hp));
+    void (*kernel)(int64_t, const TopkBuffers, float*, const HyperParams) =
+        c->fused ? (c->tk.gbar ? amsgrad_bucket_kernel<true, true> : amsgrad_bucket_kernel<false, true>)
+                 : (c->tk.gbar ? amsgrad_bucket_kernel<true, false> : amsgrad_bucket_kernel<false, false>);
+    return counted(c, launch_after(kernel, grid, dim3(kThreads), c->stream, c->d, c->tk, theta, c->hp));
 }
 
 }  // namespace compams
