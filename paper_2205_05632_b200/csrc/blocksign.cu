@@ -18,15 +18,6 @@
 
 namespace compams {
 
-// Sign bits of the 4 values of this lane -> the 32-bit word of its 8-lane group (all 8 lanes get it).
-__device__ __forceinline__ uint32_t pack_group_word(uint32_t nibble, int lane) {
-    uint32_t w = nibble << ((lane & 7) * 4);
-    w |= __shfl_xor_sync(0xffffffffu, w, 1);
-    w |= __shfl_xor_sync(0xffffffffu, w, 2);
-    w |= __shfl_xor_sync(0xffffffffu, w, 4);
-    return w;
-}
-
 // |x| as a binary64 number without a conversion instruction: for a normal fp32 value the
 // binary64 pattern is the same fraction shifted left by 29 bits under an exponent rebiased by 896.
 __device__ __forceinline__ double abs_as_double(float x) {
@@ -35,8 +26,27 @@ __device__ __forceinline__ double abs_as_double(float x) {
     return __hiloint2double((int)((b >> 3) + 0x38000000u), (int)(b << 29));
 }
 
+// Four of them added one after the other, with one test for the rare ones.
+__device__ __forceinline__ void add_abs4(const float (&x)[4], double& acc) {
+    uint32_t key[4], least = 0xffffffffu;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        key[k] = __float_as_uint(x[k]) & 0x7fffffffu;
+        least = least < key[k] ? least : key[k];
+    }
+    if (least >= 0x00800000u) {
+#pragma unroll
+        for (int k = 0; k < 4; ++k) acc += __hiloint2double((int)((key[k] >> 3) + 0x38000000u), (int)(key[k] << 29));
+    } else {
+#pragma unroll
+        for (int k = 0; k < 4; ++k) acc += (double)__uint_as_float(key[k]);
+    }
+}
+
 // One warp's 1024 consecutive coordinates starting at rw (relative to the block; rw may be negative
-// or reach past the block in a tile at either end of it: such coordinates are skipped).
+// or reach past the block in a tile at either end of it: such coordinates are skipped). The signs come by ballots and are put in
+// coordinate order once, at the end (with nibbles that four shuffles per iteration joined into words, and a test per element for
+// the values that abs_as_double has to convert: n = 2, d = 1 M 16.4 us per step, now 15.8; ResNet-18 shapes, n = 16 405.7 / 402.5).
 template <bool FULL, typename GT>
 __device__ __forceinline__ void bs_sweep_tile(const GT* __restrict__ g, float* __restrict__ e, int len, int rw,
                                               int lane, bool deferred, float sp, double& acc, uint32_t& mymask) {
@@ -68,6 +78,7 @@ __device__ __forceinline__ void bs_sweep_tile(const GT* __restrict__ g, float* _
             }
         }
     };
+    uint32_t sg[4] = {0u, 0u, 0u, 0u};
     load_batch(0, gbuf[0], ebuf[0]);
 #pragma unroll
     for (int bt = 0; bt < NBT; ++bt) {
@@ -79,7 +90,6 @@ __device__ __forceinline__ void bs_sweep_tile(const GT* __restrict__ g, float* _
             const int it = bt * NB + u;
             const int r = rw + it * 128 + lane * 4;
             float xs[4];
-            uint32_t nib = 0;
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
                 float xo = lane_elem(ev[u], k);
@@ -89,10 +99,10 @@ __device__ __forceinline__ void bs_sweep_tile(const GT* __restrict__ g, float* _
                 xs[k] = x;
                 const bool live = FULL || ((unsigned)(r + k) < (unsigned)len);
                 if (live) {
-                    acc += abs_as_double(x);
-                    nib |= (__float_as_uint(x) >> 31) << k;
+                    if (!(FULL)) acc += abs_as_double(x);
                 }
             }
+            if (FULL) add_abs4(xs, acc);
             if (FULL || (r >= 0 && r + 3 < len)) {
                 store4(e + r, ce, make_float4(xs[0], xs[1], xs[2], xs[3]));
             } else {
@@ -100,10 +110,23 @@ __device__ __forceinline__ void bs_sweep_tile(const GT* __restrict__ g, float* _
                 for (int k = 0; k < 4; ++k)
                     if ((unsigned)(r + k) < (unsigned)len) e[r + k] = xs[k];
             }
-            uint32_t w = pack_group_word(nib, lane);
-            uint32_t wv = __shfl_sync(0xffffffffu, w, (lane & 3) * 8);
-            if ((lane >> 2) == it) mymask = wv;  // lane l ends up holding the sign mask of the warp's l-th 32 coordinates
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const uint32_t m = __ballot_sync(0xffffffffu, (int)__float_as_uint(xs[k]) < 0 && (FULL || (unsigned)(r + k) < (unsigned)len));
+                if ((lane >> 2) == it) sg[k] = m;
+            }
         }
+    }
+    // lane l holds the sign ballots of the iteration with the warp's l-th 32 coordinates: bit p of sg[k] is coordinate 4 p + k, and the
+    // lane's own 32 are bits 8 (l % 4) ... of each
+    mymask = 0u;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        uint32_t y = (sg[k] >> ((lane & 3) * 8)) & 0xffu;  // eight bits to every fourth position
+        y = (y | (y << 12)) & 0x000f000fu;
+        y = (y | (y << 6)) & 0x03030303u;
+        y = (y | (y << 3)) & 0x11111111u;
+        mymask |= y << k;
     }
 }
 
@@ -163,8 +186,9 @@ __device__ __forceinline__ void bs_sweep_tile_bf16x8(const bf16_bits* __restrict
 // sign words stay indexed by coordinate: word q of the block takes its low 32 - s bits from the
 // q-th group of 32 shifted coordinates and its high s bits from the next group. The word a tile
 // shares with the next tile is put together by bs_scales, or by bs_apply, from the two shares left in `edge`.
-template <typename GT>
-__global__ void __launch_bounds__(kThreads, sizeof(GT) == 2 ? 5 : 8) bs_sweep_kernel(Tables t, BsBuffers b, const GT* __restrict__ G,
+// AHEAD: the tile's lines are asked into the L2 first, with five CTAs per SM: see launch_bs_sweep.
+template <typename GT, bool AHEAD>
+__global__ void __launch_bounds__(kThreads, sizeof(GT) == 2 || AHEAD ? 5 : 8) bs_sweep_kernel(Tables t, BsBuffers b, const GT* __restrict__ G,
                                                                int deferred, const __grid_constant__ SegParams sp_) {
     __shared__ double red[kWarps];
     __shared__ uint32_t sh_first[kWarps];
@@ -187,6 +211,10 @@ __global__ void __launch_bounds__(kThreads, sizeof(GT) == 2 ? 5 : 8) bs_sweep_ke
     double acc = 0.0;
     uint32_t mymask = 0;
     const bool whole = r0s >= 0 && r0s + kTile <= ti.len;
+    if (AHEAD && whole) {
+        asm volatile("prefetch.global.L2 [%0];" ::"l"(e + rw + lane * 32));
+        asm volatile("prefetch.global.L2 [%0];" ::"l"(g + rw + lane * 32));
+    }
     bool wide = false;
     if constexpr (sizeof(GT) == 2)
         wide = whole && ((reinterpret_cast<uintptr_t>(g + rw) | reinterpret_cast<uintptr_t>(e + rw)) & 15u) == 0;
@@ -688,22 +716,25 @@ static BsBuffers own_rows(const compams_context* c) {
     return b;
 }
 
-cudaError_t launch_bs_sweep(compams_context* c, const void* grads) {
-    dim3 grid((unsigned)c->tab.ntiles, (unsigned)c->n);
-    if (c->chain) {  // n d <= kChainMaxElems: the launch overlaps the tail of whatever kernel precedes it on the stream
-        if (c->grad_bf16)
-            return counted(c, launch_after(bs_sweep_kernel<bf16_bits>, grid, dim3(kThreads), c->stream, c->tab, own_rows(c),
-                                (const bf16_bits*)grads, c->e_is_x ? 1 : 0, c->segp));
-        return counted(c, launch_after(bs_sweep_kernel<float>, grid, dim3(kThreads), c->stream, c->tab, own_rows(c),
-                            (const float*)grads, c->e_is_x ? 1 : 0, c->segp));
-    }
-    if (c->grad_bf16)
-        bs_sweep_kernel<bf16_bits><<<grid, kThreads, 0, c->stream>>>(c->tab, own_rows(c), (const bf16_bits*)grads,
-                                                                     c->e_is_x ? 1 : 0, c->segp);
-    else
-        bs_sweep_kernel<float><<<grid, kThreads, 0, c->stream>>>(c->tab, own_rows(c), (const float*)grads,
-                                                                 c->e_is_x ? 1 : 0, c->segp);
+template <typename GT>
+static cudaError_t launch_sweep_typed(compams_context* c, void (*kernel)(Tables, BsBuffers, const GT*, int, const SegParams), const GT* grads) {
+    const dim3 grid((unsigned)c->tab.ntiles, (unsigned)c->n);
+    const int deferred = c->e_is_x ? 1 : 0;
+    if (c->chain)  // n d <= kChainMaxElems: the launch overlaps the tail of whatever kernel precedes it on the stream
+        return counted(c, launch_after(kernel, grid, dim3(kThreads), c->stream, c->tab, own_rows(c), grads, deferred, c->segp));
+    kernel<<<grid, kThreads, 0, c->stream>>>(c->tab, own_rows(c), grads, deferred, c->segp);
     return counted(c, cudaGetLastError());
+}
+
+// The build that asks ahead takes over where the sweep is many waves long (us per step without / with: 8 of 32 workers, ResNet-50 shapes
+// 594 / 587; n = 4, d = 20 M in 60 blocks 279 / 278; n = 16, d = 2^23 299 / 297; n = 2, d = 90 M 768 / 763; but n = 16, d = 4 M 150 / 152,
+// n = 9, d = 2.9 M 74 / 78, n = 8, d = 2^20 27.5 / 29.8).
+constexpr int64_t kAheadElems = (int64_t)1 << 26;
+
+cudaError_t launch_bs_sweep(compams_context* c, const void* grads) {
+    if (c->grad_bf16) return launch_sweep_typed(c, bs_sweep_kernel<bf16_bits, false>, (const bf16_bits*)grads);
+    const bool ahead = (int64_t)c->n * c->d >= kAheadElems;
+    return launch_sweep_typed(c, ahead ? bs_sweep_kernel<float, true> : bs_sweep_kernel<float, false>, (const float*)grads);
 }
 
 // Whether the server kernel is bs_apply_short: few tiles for the number of workers. us per step (whole vector, bs_apply with the tile

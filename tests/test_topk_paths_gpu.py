@@ -82,6 +82,20 @@ def test_blocksign_server_kernels_and_who_adds_up_the_scales(n, offs):
     run(n, offs, BLOCKSIGN, 1.0, normal, steps=4)
 
 
+def test_blocksign_sweep_that_asks_ahead():
+    run(3, [0, 31, 9001, 9001 + 3 * 8192, 22369623], BLOCKSIGN, 1.0, normal, steps=2)  # n d just above 2^26
+
+
+def test_blocksign_whole_tiles_with_zeros_and_subnormals():
+    def draw(gen, n, d):
+        g = torch.randn(n, d, generator=gen, device="cuda")
+        g[:, ::7] = 0.0
+        g[:, 3::11] = -0.0
+        g[:, 5::13] *= 2.0 ** -130
+        return g
+    run(3, [0, 2 * 8192, 5 * 8192 + 70], BLOCKSIGN, 1.0, draw, steps=3)
+
+
 @pytest.mark.parametrize("n,offs,ratio", [
     (3, [0, 31, 1055, 1056, 9300, 30011], 0.02), (2, [0, 20001], 0.25), (2, [0, 20001], 0.95), (4, [0, 1024, 2048, 10240], 0.125),
 ])
