@@ -26,20 +26,22 @@ __device__ __forceinline__ double abs_as_double(float x) {
     return __hiloint2double((int)((b >> 3) + 0x38000000u), (int)(b << 29));
 }
 
-// Four of them added one after the other, with one test for the rare ones.
+// Four of them added one after the other, with one test for the rare ones: the patterns without sign, counted from the smallest normal
+// one up, reach 0xfe000000 where a value is infinite or NaN and, wrapped, where it is zero or subnormal. Those four go by the rule above
+// each, so that what a value adds does not depend on its neighbours.
 __device__ __forceinline__ void add_abs4(const float (&x)[4], double& acc) {
-    uint32_t key[4], least = 0xffffffffu;
+    uint32_t p[4], most = 0u;
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
-        key[k] = __float_as_uint(x[k]) & 0x7fffffffu;
-        least = least < key[k] ? least : key[k];
+        p[k] = 2u * __float_as_uint(x[k]) - 0x01000000u;
+        most = most > p[k] ? most : p[k];
     }
-    if (least >= 0x00800000u) {
+    if (most < 0xfe000000u) {
 #pragma unroll
-        for (int k = 0; k < 4; ++k) acc += __hiloint2double((int)((key[k] >> 3) + 0x38000000u), (int)(key[k] << 29));
+        for (int k = 0; k < 4; ++k) acc += __hiloint2double((int)((p[k] >> 4) + 0x38100000u), (int)(p[k] << 28));
     } else {
 #pragma unroll
-        for (int k = 0; k < 4; ++k) acc += (double)__uint_as_float(key[k]);
+        for (int k = 0; k < 4; ++k) acc += abs_as_double(x[k]);
     }
 }
 

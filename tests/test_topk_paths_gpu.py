@@ -96,6 +96,22 @@ def test_blocksign_whole_tiles_with_zeros_and_subnormals():
     run(3, [0, 2 * 8192, 5 * 8192 + 70], BLOCKSIGN, 1.0, draw, steps=3)
 
 
+@pytest.mark.parametrize("d", [8192, 8192 + 5])  # a whole tile; tiles that are not
+@pytest.mark.parametrize("beside", [1.0, 0.0, 2.0 ** -130])
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+def test_blocksign_an_infinity_adds_the_same_beside_any_values(d, beside, dtype):
+    # its pattern read as a number, 2^128, whose quotient by d is the scale: the other values, at most 1 each, are below half an ulp
+    opt = CompAMS(1, d, [0, d], BLOCKSIGN)
+    g = torch.ones(1, d, device="cuda", dtype=dtype)
+    g[0, 4000:4008] = beside
+    g[0, 4002] = float("inf")
+    opt.compress(g)
+    bits, scales = opt.message_buffers()
+    assert scales.item() == float(np.float32(2.0 ** 128 / d))
+    opt.apply(torch.zeros(d, device="cuda"))
+    opt.close()
+
+
 @pytest.mark.parametrize("n,offs,ratio", [
     (3, [0, 31, 1055, 1056, 9300, 30011], 0.02), (2, [0, 20001], 0.25), (2, [0, 20001], 0.95), (4, [0, 1024, 2048, 10240], 0.125),
 ])
