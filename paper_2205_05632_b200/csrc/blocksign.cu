@@ -48,8 +48,11 @@ __device__ __forceinline__ void add_abs4(const float (&x)[4], double& acc) {
 // One warp's 1024 consecutive coordinates starting at rw (relative to the block; rw may be negative
 // or reach past the block in a tile at either end of it: such coordinates are skipped). The signs come by ballots and are put in
 // coordinate order once, at the end (with nibbles that four shuffles per iteration joined into words, and a test per element for
-// the values that abs_as_double has to convert: n = 2, d = 1 M 16.4 us per step, now 15.8; ResNet-18 shapes, n = 16 405.7 / 402.5).
-template <bool FULL, typename GT>
+// the values that abs_as_double has to convert: n = 2, d = 1 M 16.4 us per step, now 15.5). A lane keeps its own byte of every ballot,
+// one register: with all of the four ballots the build of eight CTAs per SM spilled 52 bytes (n = 2, d = 1 M 15.9 us, n = 8, d = 1.3 M 38.6,
+// now 38.1, d = 2^20 27.5 / 27.4). WORDS keeps the four, for the builds of five CTAs per SM, which have registers to spare (n = 16,
+// d = 2^23 300 against 306; bfloat16, 80 blocks in d = 3 M, n = 32 210.7 against 213.3).
+template <bool FULL, bool WORDS, typename GT>
 __device__ __forceinline__ void bs_sweep_tile(const GT* __restrict__ g, float* __restrict__ e, int len, int rw,
                                               int lane, bool deferred, float sp, double& acc, uint32_t& mymask) {
     const int cg = align_class(g + rw), ce = align_class(e + rw);
@@ -80,7 +83,7 @@ __device__ __forceinline__ void bs_sweep_tile(const GT* __restrict__ g, float* _
             }
         }
     };
-    uint32_t sg[4] = {0u, 0u, 0u, 0u};
+    uint32_t sg[WORDS ? 4 : 1] = {};
     load_batch(0, gbuf[0], ebuf[0]);
 #pragma unroll
     for (int bt = 0; bt < NBT; ++bt) {
@@ -99,10 +102,7 @@ __device__ __forceinline__ void bs_sweep_tile(const GT* __restrict__ g, float* _
                 float ee = deferred ? __fsub_rn(xo, copysignf(sp, xo)) : xo;
                 float x = __fadd_rn(lane_elem(gv[u], k), ee);  // the corrected-gradient step: x = g + e
                 xs[k] = x;
-                const bool live = FULL || ((unsigned)(r + k) < (unsigned)len);
-                if (live) {
-                    if (!(FULL)) acc += abs_as_double(x);
-                }
+                if (!FULL && (unsigned)(r + k) < (unsigned)len) acc += abs_as_double(x);
             }
             if (FULL) add_abs4(xs, acc);
             if (FULL || (r >= 0 && r + 3 < len)) {
@@ -115,7 +115,10 @@ __device__ __forceinline__ void bs_sweep_tile(const GT* __restrict__ g, float* _
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
                 const uint32_t m = __ballot_sync(0xffffffffu, (int)__float_as_uint(xs[k]) < 0 && (FULL || (unsigned)(r + k) < (unsigned)len));
-                if ((lane >> 2) == it) sg[k] = m;
+                if ((lane >> 2) == it) {
+                    if constexpr (WORDS) sg[k] = m;
+                    else sg[0] |= ((m >> ((lane & 3) * 8)) & 0xffu) << (8 * k);
+                }
             }
         }
     }
@@ -124,7 +127,7 @@ __device__ __forceinline__ void bs_sweep_tile(const GT* __restrict__ g, float* _
     mymask = 0u;
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
-        uint32_t y = (sg[k] >> ((lane & 3) * 8)) & 0xffu;  // eight bits to every fourth position
+        uint32_t y = (WORDS ? sg[WORDS ? k : 0] >> ((lane & 3) * 8) : sg[0] >> (8 * k)) & 0xffu;  // eight bits to every fourth position
         y = (y | (y << 12)) & 0x000f000fu;
         y = (y | (y << 6)) & 0x03030303u;
         y = (y | (y << 3)) & 0x11111111u;
@@ -210,6 +213,7 @@ __global__ void __launch_bounds__(kThreads, sizeof(GT) == 2 || AHEAD ? 5 : 8) bs
     const int r0s = ti.r0 - s;
     const int rw = r0s + warp * kWarpSpan;
 
+    constexpr bool kWords = sizeof(GT) == 2 || AHEAD;
     double acc = 0.0;
     uint32_t mymask = 0;
     const bool whole = r0s >= 0 && r0s + kTile <= ti.len;
@@ -223,9 +227,9 @@ __global__ void __launch_bounds__(kThreads, sizeof(GT) == 2 || AHEAD ? 5 : 8) bs
     if (wide) {
         if constexpr (sizeof(GT) == 2) bs_sweep_tile_bf16x8(g, e, rw, lane, deferred != 0, sp, acc, mymask);
     } else if (whole) {
-        bs_sweep_tile<true>(g, e, ti.len, rw, lane, deferred != 0, sp, acc, mymask);
+        bs_sweep_tile<true, kWords>(g, e, ti.len, rw, lane, deferred != 0, sp, acc, mymask);
     } else {
-        bs_sweep_tile<false>(g, e, ti.len, rw, lane, deferred != 0, sp, acc, mymask);
+        bs_sweep_tile<false, kWords>(g, e, ti.len, rw, lane, deferred != 0, sp, acc, mymask);
     }
 
     // tile sum in binary64 (fixed shuffle tree); bs_scales adds the tile sums of a block in a fixed order
