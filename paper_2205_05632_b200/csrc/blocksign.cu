@@ -52,7 +52,8 @@ __device__ __forceinline__ void add_abs4(const float (&x)[4], double& acc) {
 // one register: with all of the four ballots the build of eight CTAs per SM spilled 52 bytes (n = 2, d = 1 M 15.9 us, n = 8, d = 1.3 M 38.6,
 // now 38.1, d = 2^20 27.5 / 27.4). WORDS keeps the four, for the builds of five CTAs per SM, which have registers to spare (n = 16,
 // d = 2^23 300 against 306; bfloat16, 80 blocks in d = 3 M, n = 32 210.7 against 213.3).
-template <bool FULL, bool WORDS, typename GT>
+// CUT: a warp past the end of the block stops.
+template <bool FULL, bool WORDS, bool CUT, typename GT>
 __device__ __forceinline__ void bs_sweep_tile(const GT* __restrict__ g, float* __restrict__ e, int len, int rw,
                                               int lane, bool deferred, float sp, double& acc, uint32_t& mymask) {
     const int cg = align_class(g + rw), ce = align_class(e + rw);
@@ -87,6 +88,7 @@ __device__ __forceinline__ void bs_sweep_tile(const GT* __restrict__ g, float* _
     load_batch(0, gbuf[0], ebuf[0]);
 #pragma unroll
     for (int bt = 0; bt < NBT; ++bt) {
+        if (CUT && rw + bt * NB * 128 >= len) break;
         float4 (&gv)[NB] = gbuf[bt & 1];
         float4 (&ev)[NB] = ebuf[bt & 1];
         if (bt + 1 < NBT) load_batch(bt + 1, gbuf[(bt + 1) & 1], ebuf[(bt + 1) & 1]);
@@ -191,8 +193,9 @@ __device__ __forceinline__ void bs_sweep_tile_bf16x8(const bf16_bits* __restrict
 // sign words stay indexed by coordinate: word q of the block takes its low 32 - s bits from the
 // q-th group of 32 shifted coordinates and its high s bits from the next group. The word a tile
 // shares with the next tile is put together by bs_scales, or by bs_apply, from the two shares left in `edge`.
-// AHEAD: the tile's lines are asked into the L2 first, with five CTAs per SM: see launch_bs_sweep.
-template <typename GT, bool AHEAD>
+// AHEAD: the tile's lines are asked into the L2 first, with five CTAs per SM; CUT: for many tiles that are mostly empty: see
+// launch_bs_sweep.
+template <typename GT, bool AHEAD, bool CUT>
 __global__ void __launch_bounds__(kThreads, sizeof(GT) == 2 || AHEAD ? 5 : 8) bs_sweep_kernel(Tables t, BsBuffers b, const GT* __restrict__ G,
                                                                int deferred, const __grid_constant__ SegParams sp_) {
     __shared__ double red[kWarps];
@@ -227,9 +230,9 @@ __global__ void __launch_bounds__(kThreads, sizeof(GT) == 2 || AHEAD ? 5 : 8) bs
     if (wide) {
         if constexpr (sizeof(GT) == 2) bs_sweep_tile_bf16x8(g, e, rw, lane, deferred != 0, sp, acc, mymask);
     } else if (whole) {
-        bs_sweep_tile<true, kWords>(g, e, ti.len, rw, lane, deferred != 0, sp, acc, mymask);
+        bs_sweep_tile<true, kWords, false>(g, e, ti.len, rw, lane, deferred != 0, sp, acc, mymask);
     } else {
-        bs_sweep_tile<false, kWords>(g, e, ti.len, rw, lane, deferred != 0, sp, acc, mymask);
+        bs_sweep_tile<false, kWords, CUT>(g, e, ti.len, rw, lane, deferred != 0, sp, acc, mymask);
     }
 
     // tile sum in binary64 (fixed shuffle tree); bs_scales adds the tile sums of a block in a fixed order
@@ -737,10 +740,23 @@ static cudaError_t launch_sweep_typed(compams_context* c, void (*kernel)(Tables,
 // n = 9, d = 2.9 M 74 / 78, n = 8, d = 2^20 27.5 / 29.8).
 constexpr int64_t kAheadElems = (int64_t)1 << 26;
 
+// Where most of the tiles lies outside the blocks (many small ones) the sweep is bound by the instructions of warps that have nothing, or
+// little, to do, and the build that lets them stop takes over; one that does not test for it starts 0.5 us earlier, which is what
+// counts where the CTAs are few. us per step without / with: 152 blocks in d = 75,215 (17 times as much in tiles), n = 32 72 / 37, n = 4
+// 17.5 / 13.5, but n = 1 12.5 / 12.7; 150 in d = 750,007 (2.6 times), n = 8 35.8 / 29.0, bfloat16 39.4 / 37.2, but n = 1 16.3 / 16.9; one block,
+// n = 4, d = 100,003 9.2 / 9.8; 80 in d = 3 M (1.2 times), n = 8 75.9 / 76.5.
+static bool sweep_is_cut(const compams_context* c) {
+    return (int64_t)c->tab.ntiles * kTile >= 2 * c->d && (int64_t)c->n * c->tab.ntiles > 2 * c->num_sms;
+}
+
 cudaError_t launch_bs_sweep(compams_context* c, const void* grads) {
-    if (c->grad_bf16) return launch_sweep_typed(c, bs_sweep_kernel<bf16_bits, false>, (const bf16_bits*)grads);
+    const bool cut = sweep_is_cut(c);
+    if (c->grad_bf16)
+        return launch_sweep_typed(c, cut ? bs_sweep_kernel<bf16_bits, false, true> : bs_sweep_kernel<bf16_bits, false, false>, (const bf16_bits*)grads);
     const bool ahead = (int64_t)c->n * c->d >= kAheadElems;
-    return launch_sweep_typed(c, ahead ? bs_sweep_kernel<float, true> : bs_sweep_kernel<float, false>, (const float*)grads);
+    return launch_sweep_typed(c, cut     ? bs_sweep_kernel<float, false, true>
+                                 : ahead ? bs_sweep_kernel<float, true, false>
+                                         : bs_sweep_kernel<float, false, false>, (const float*)grads);
 }
 
 // Whether the server kernel is bs_apply_short: few tiles for the number of workers. us per step (whole vector, bs_apply with the tile

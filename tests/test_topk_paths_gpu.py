@@ -86,6 +86,15 @@ def test_blocksign_sweep_that_asks_ahead():
     run(3, [0, 31, 9001, 9001 + 3 * 8192, 22369623], BLOCKSIGN, 1.0, normal, steps=2)  # n d just above 2^26
 
 
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+@pytest.mark.parametrize("n,sizes", [
+    # mostly empty tiles: blocks that end inside a warp's first 128 coordinates, at its edges, at the next warp's, in the last one
+    (6, [1, 31, 32, 97, 127, 128, 129, 1023, 1024, 1025, 1151, 7168, 7169, 3] * 5), (2, [200] * 150), (33, [5, 130, 1500] * 4),
+])
+def test_blocksign_sweep_of_mostly_empty_tiles(n, sizes, dtype):
+    run(n, list(np.cumsum([0] + sizes)), BLOCKSIGN, 1.0, lambda gen, n, d: normal(gen, n, d).to(dtype), steps=3)
+
+
 def test_blocksign_whole_tiles_with_zeros_and_subnormals():
     def draw(gen, n, d):
         g = torch.randn(n, d, generator=gen, device="cuda")
