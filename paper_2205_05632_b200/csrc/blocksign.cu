@@ -735,10 +735,18 @@ static cudaError_t launch_sweep_typed(compams_context* c, void (*kernel)(Tables,
     return counted(c, cudaGetLastError());
 }
 
-// The build that asks ahead takes over where the sweep is many waves long (us per step without / with: 8 of 32 workers, ResNet-50 shapes
-// 594 / 587; n = 4, d = 20 M in 60 blocks 279 / 278; n = 16, d = 2^23 299 / 297; n = 2, d = 90 M 768 / 763; but n = 16, d = 4 M 150 / 152,
-// n = 9, d = 2.9 M 74 / 78, n = 8, d = 2^20 27.5 / 29.8).
+// The build that asks ahead takes over where the sweep is many waves long. What it gives depends on the GPU it runs on: us per step without /
+// with, on the boxes where most was gained and where least: ResNet-18 shapes, n = 16 395.0 / 389.8, 405.7 / 409.0; 8 of 32 workers, ResNet-50
+// shapes 578.3 / 575.2, 597.2 / 597.0; n = 16, d = 2^23 293.6 / 291.8, 300.1 / 302.0; n = 2, d = 90 M 762.1 / 760.0, 769.7 / 770.3; n = 6,
+// d = 30 M 479 / 478, 492 / 495. Below it loses everywhere: n = 16, d = 4 M 150 / 152, n = 9, d = 2.9 M 74 / 78, n = 8, d = 2^20 27.5 / 29.8. In
+// steps too long to be chained it loses with one block, or a few, more than it gives - n = 32, d = 2^24 1057 / 1064, 1082 / 1109, d = 2^25 2098 /
+// 2117, 2141 / 2194, n = 20, d = 40 M 1650 / 1669, 1689 / 1724, n = 16, d = 40 M in two blocks 1378 / 1387 - and gains with many: n = 32, d =
+// 25 M in 161 1646 / 1610, 1685 / 1693, n = 13, d = 21.6 M in 134 681 / 672, n = 8, d = 100 M in 21 2049 / 2032, n = 12, d = 50 M in 31 1439 / 1423,
+// ten blocks in d = 2^24, n = 32 1117 / 1114.
 constexpr int64_t kAheadElems = (int64_t)1 << 26;
+static bool sweep_asks_ahead(const compams_context* c) {
+    return (int64_t)c->n * c->d >= kAheadElems && (c->chain || c->M > 8);
+}
 
 // Where most of the tiles lies outside the blocks (many small ones) the sweep is bound by the instructions of warps that have nothing, or
 // little, to do, and the build that lets them stop takes over; one that does not test for it starts 0.5 us earlier, which is what
@@ -753,7 +761,7 @@ cudaError_t launch_bs_sweep(compams_context* c, const void* grads) {
     const bool cut = sweep_is_cut(c);
     if (c->grad_bf16)
         return launch_sweep_typed(c, cut ? bs_sweep_kernel<bf16_bits, false, true> : bs_sweep_kernel<bf16_bits, false, false>, (const bf16_bits*)grads);
-    const bool ahead = (int64_t)c->n * c->d >= kAheadElems;
+    const bool ahead = sweep_asks_ahead(c);
     return launch_sweep_typed(c, cut     ? bs_sweep_kernel<float, false, true>
                                  : ahead ? bs_sweep_kernel<float, true, false>
                                          : bs_sweep_kernel<float, false, false>, (const float*)grads);
