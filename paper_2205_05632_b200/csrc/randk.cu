@@ -96,7 +96,8 @@ __device__ __forceinline__ int block_of_slot(const Tables& t, const TopkBuffers&
 // cycles of three): a lane that is back inside the block goes on to its next slot while its neighbours still walk, so that a warp
 // waits for the longest sum of walks and not, slot for slot, for the longest walk, and the round keys serve that many more slots
 // (one slot per thread took 37 us for 1.8 M slots in blocks of 11.2 M coordinates, two thirds of the domain, this takes 25:
-// ResNet-18 shapes, n = 16, 430 -> 418 us per step).
+// ResNet-18 shapes, n = 16, 430 -> 418 us per step). With one slot per thread there is nothing to go on to, and the bit is set behind
+// the walk (inside it n = 2, d = 300,001, 5 % took 18.9 us per step, now 18.0; n = 16, 1 % 27.4 / 26.4).
 __global__ void __launch_bounds__(kThreads) randk_mark_kernel(const __grid_constant__ Tables t, const __grid_constant__ TopkBuffers b,
                                                               int32_t row0, int32_t i0, int64_t origin, uint64_t seed, uint64_t step,
                                                               int per_thread) {
@@ -132,6 +133,13 @@ __global__ void __launch_bounds__(kThreads) randk_mark_kernel(const __grid_const
         if (tid == 0 && first == slot0) b.slots[(size_t)(i0 + il) * t.nseg + blk0] = 0u;  // every block is tiled: segment = block
         int64_t q = first + tid;
         uint32_t x = (uint32_t)(q - slot0);
+        if (per_thread == 1) {  // nothing to go on to
+            if (q >= last) return;
+            do x = randk_network(x, w, k);
+            while (x >= len);
+            mark(o + x);
+            return;
+        }
         while (q < last) {
             x = randk_network(x, w, k);
             if (x < len) {
