@@ -464,9 +464,11 @@ static cudaError_t launch_randk_typed(compams_context* c, const GT* grads) {
     for (int32_t i0 = 0; i0 < c->n && e == cudaSuccess; i0 += c->randk_group) {
         const int32_t rows = c->n - i0 < c->randk_group ? c->n - i0 : c->randk_group;
         const int64_t origin = (int64_t)i0 * c->d & ~(int64_t)31;
-        // as many slots per thread as leave two CTAs per SM, eight at most (n = 3, d = 25 M in 100 blocks, 5 %: four and eight 381 us per
-        // step, sixteen 410, one 416)
-        const int64_t most = c->K * rows / (2 * 148 * kThreads);
+        // as many slots per thread as leave eight CTAs per SM, an SM full of them, eight at most. us per step with one slot, as many as
+        // leave two CTAs, four, eight: n = 8, d = 3 M in 20 blocks, 1 % 81.1, 85.3, 81.0, 81.0; n = 2, d = 2 M in 60, 5 % 38.4, 40.8, 38.3, 38.3;
+        // n = 16, d = 6 M in 150, 1 % 261, 273, 267, 262; n = 4, d = 9 M in 100, 5 % 198, 193, 193, 186; ResNet-18 shapes whole, n = 16 431, 420,
+        // 418, 420. (n = 3, d = 25 M in 100 blocks, 5 %, eight at most 382, sixteen 410.)
+        const int64_t most = c->K * rows / (8 * (int64_t)c->num_sms * kThreads);
         const int per_thread = (int)(most < 1 ? 1 : most > 8 ? 8 : most);
         const int64_t per_worker = (c->K + per_thread * kThreads - 1) / (per_thread * kThreads);
         e = counted(c, launch_after(randk_mark_kernel, dim3((unsigned)(per_worker * rows)), dim3(kThreads), c->stream, c->tab, b, c->row0,

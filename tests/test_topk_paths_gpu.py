@@ -132,6 +132,9 @@ def test_randk_spans_that_share_words_and_overflow_their_room(n, offs, ratio):
     # several slots per thread: one block per CTA, blocks that begin inside one, a row whose last CTA is short
     (1, [0, 4 * 757761], 0.05), (2, [0, 1048575], 0.1), (3, [0, 1, 40, 500009, 500010, 520000, 1500001], 0.1),
     (2, list(np.cumsum([0] + [1500 + 7 * k for k in range(700)])), 0.06),
+    # two, three, eight and four per thread on 148 SMs, blocks that begin inside a CTA's slots
+    (4, [0, 700001, 1600003], 0.1), (8, [0, 4099, 1200007], 0.1), (8, [0, 900001, 900002, 903000, 3300001], 0.1),
+    (4, list(np.cumsum([0] + [3000 + 11 * k for k in range(250)])), 0.3),
 ])
 def test_randk_several_slots_per_thread(n, offs, ratio):
     run(n, offs, RANDK, ratio, normal, steps=3, seed=5)
