@@ -239,6 +239,30 @@ int group_segments(compams_context* c, const std::vector<SegInfo>& segs) {
     return dev_upload(c, &c->sel_segs, many);
 }
 
+// Whether topk_small, whose longest block is `longest`, comes behind topk_select and runs beside it: nothing of either is the other's.
+// In front, where it stays with an emission kernel behind the selection, it runs beside the tail of the sweep and delays the selection by
+// what sticks out; behind, it starts when all of the selection's CTAs have and costs the step a microsecond or two of its own. us per
+// step in front / behind, of 290 layouts of n = 1 to 32, which the conditions divide with no loss above 1.5 % and give up 3 % at most:
+// - Blocks of 2500 to 4096 coordinates stick out of any sweep: n = 1, 3 x 600,000 with three of 2500 41.1 / 38.0, n = 8, 8 x 50,000 with
+//   eight 36.7 / 26.0, n = 2, d = 2 M in 100 blocks 47.4 / 40.2.
+// - Shorter ones only of a sweep of about one wave that has CTAs on all SMs: n = 4, 20 x 20,000 (240 tiles) with 20 of 30 26.6 / 24.0; but
+//   n = 4, 3 x 600,000 (888) 45.4 / 47.1, n = 2, d = 200,535 in 15 (58) 19.2 / 21.4; nor where more is kept or the server kernel has more CTAs
+//   than fit at once: n = 16, 3 x 50,000, 6 % 30.0 / 32.0, n = 1, 3 x 600,000 (222) 36.2 / 37.9.
+// - There is no room beside CTAs of the selection on every SM (n = 32, 8 x 50,000 with eight of 2500 58.8 / 61.9, n = 4, d = 1.7 M in 99
+//   50.4 / 51.4), and nothing to gain where both are more than a wave (n = 10, d = 855,151 in 108, bfloat16 62.5 / 66.6) or the small blocks
+//   are most of the step (n = 11, d = 135,392 in 128, 6.8 % 40.9 / 42.6, bfloat16 45.4 / 48.9).
+bool small_beside_select(const compams_context* c, int64_t longest) {
+    const int64_t n = c->n, tiles = n * c->tab.ntiles, small = n * c->tk.nsmall;
+    const int64_t ctas = n * ((int64_t)c->sel_long * c->sel_cluster + c->sel_short);
+    if (!small || !ctas || c->sel_parts) return false;
+    if (c->sel_cluster == 1 && ctas > kPlanSms && ctas <= 2 * kPlanSms) return false;
+    if (ctas > 2 * kPlanSms && small > 3 * kPlanSms) return false;
+    if (small > 7 * kPlanSms && tiles <= 2 * kPlanSms) return false;
+    if (longest >= (tiles > 4 * kPlanSms ? 700 : 1024)) return true;
+    return tiles > kPlanSms && tiles <= 4 * kPlanSms && !c->many_candidates &&
+           (tiles > 2 * kPlanSms || c->d <= 5 * kPlanSms * kBucketSpan);
+}
+
 // Cuts the listed blocks into tiles of kTile coordinates and uploads the tile and segment tables.
 // For Top-k (`topk` true) every listed block also gets its message slots and candidate capacity.
 int build_tiles(compams_context* c, const std::vector<int32_t>& blocks, bool topk) {
@@ -368,6 +392,9 @@ int init_context(compams_context* c, const int64_t* block_offsets) {
         RC(dev_upload(c, &d_small, small));
         t.small_blk = d_small;
         t.nsmall = (int32_t)small.size();
+        int64_t longest = 0;
+        for (int32_t b : small) longest = std::max(longest, c->off[b + 1] - c->off[b]);
+        c->small_last = small_beside_select(c, longest);
         // the messages of all n_total workers: this handle's selection fills its own rows, the other
         // rows are filled by the caller's exchange before compams_apply
         RC(dev_alloc(c, &t.idx, (size_t)c->n_total * (size_t)c->K));
@@ -518,11 +545,10 @@ int compress_device(compams_context* c, const void* grads) {
     if (first) --c->first_steps;
     c->tk.cluster_max = first ? c->cluster_max_first : c->cluster_max;
     if (c->tab.ntiles > 0) RC(run_kernel(c, COMPAMS_K_TOPK_SWEEP, [&] { return launch_topk_sweep(c, grads); }));
-    const bool selects = c->tab.ntiles > 0 && c->sel_long + c->sel_short > 0, small_last = selects && small_beside_select(c);
-    if (c->tk.nsmall > 0 && !small_last) RC(run_kernel(c, COMPAMS_K_TOPK_SMALL, [&] { return launch_topk_small(c, grads); }));
+    if (c->tk.nsmall > 0 && !c->small_last) RC(run_kernel(c, COMPAMS_K_TOPK_SMALL, [&] { return launch_topk_small(c, grads); }));
     if (c->tab.ntiles > 0) {
-        if (selects) RC(run_kernel(c, COMPAMS_K_TOPK_SELECT, [&] { return launch_topk_select(c); }));
-        if (c->tk.nsmall > 0 && small_last) RC(run_kernel(c, COMPAMS_K_TOPK_SMALL, [&] { return launch_topk_small(c, grads); }));
+        if (c->sel_long + c->sel_short > 0) RC(run_kernel(c, COMPAMS_K_TOPK_SELECT, [&] { return launch_topk_select(c); }));
+        if (c->small_last) RC(run_kernel(c, COMPAMS_K_TOPK_SMALL, [&] { return launch_topk_small(c, grads); }));
         if (c->dense_kernel || (first && c->dense_first)) RC(run_kernel(c, COMPAMS_K_TOPK_DENSE, [&] { return launch_topk_dense(c); }));
         c->e_mask_pending = true;
     }

@@ -144,6 +144,7 @@ struct compams_context {
     int sel_cluster = 1;          // CTAs per (worker, long block)
     bool sel_wide = false;        // CTAs of 1024 threads
     bool fused = false;           // Top-k: every block is swept and selected from by one kernel (small n d)
+    bool small_last = false;      // Top-k: topk_small comes behind topk_select and runs beside it
     int sel_parts = 0;            // CTAs that emit a long list in a kernel of its own (0: the cluster emits it)
     int32_t randk_group = 1;       // Random-k: workers whose elements share the map at a time
     int64_t randk_words = 0;       // ... its words
@@ -201,12 +202,6 @@ inline cudaError_t counted(compams_context* c, cudaError_t e) {
 // Whether the worker side of the call being enqueued hands the kept entries to the server's buckets. Not between
 // compams_compress and compams_apply: the server then averages what it finds in the message buffers.
 inline bool delivers(const compams_context* c) { return c->deliver && c->whole_step; }
-
-// Whether topk_small comes behind topk_select and runs beside it: nothing of either is the other's, and one after the other they were
-// a step's longest chain (us per step, topk_small in front of topk_select / behind it: n = 10, d = 113,851 in 18 blocks, 6.6 %,
-// bfloat16 35.1 / 30.4, n = 2, d = 2 M in 100 blocks 44.8 / 39.2, n = 3, d = 300,000 in 40 25.0 / 23.4). With an emission kernel behind the
-// selection it stays in front, beside the tail of the sweep.
-inline bool small_beside_select(const compams_context* c) { return c->tk.nsmall > 0 && !c->sel_parts; }
 
 // Each launcher enqueues its kernel(s) on ctx->stream and returns the launch status.
 cudaError_t launch_dense_mean_amsgrad(compams_context* c, const void* grads, float* theta);

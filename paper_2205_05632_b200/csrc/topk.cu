@@ -1276,7 +1276,7 @@ cudaError_t launch_topk_select(compams_context* c) {
     const cudaError_t e = counted(c, launch_cluster(kernel, dim3((unsigned)(clusters * c->sel_cluster)),
                                                     dim3(c->sel_wide ? 2 * kSelThreads : kSelThreads), c->sel_cluster, c->chain, c->stream,
                                                     c->tab, own_rows(c), (const int32_t*)c->sel_segs, c->sel_long, c->sel_short,
-                                                    delivers(c) ? 1 : 0, c->sel_parts ? 1 : 0, small_beside_select(c) ? 1 : 0));
+                                                    delivers(c) ? 1 : 0, c->sel_parts ? 1 : 0, c->small_last ? 1 : 0));
     if (e != cudaSuccess || !c->sel_parts) return e;
     const dim3 grid((unsigned)((int64_t)c->n * c->sel_long * c->sel_parts));
     if (c->chain)

@@ -44,6 +44,42 @@ def test_sweep_and_selection_in_one_kernel(n, offs, ratio, draw):
     run(n, offs, TOPK, ratio, draw, steps=4)
 
 
+@pytest.mark.parametrize("n,sizes,ratio", [
+    (4, [50000, 2500] * 8, 0.01),                 # topk_small behind topk_select
+    (8, [20000, 30] * 9, 0.02),                   # ... for the sake of a short sweep
+    (2, [90000, 900, 30, 7] * 3 + [20000] * 9, 0.02),  # in front of it: two orders of kernels, as for the following
+    (20, [20000, 2500] * 8, 0.02),                # a wave of selecting CTAs
+    (10, [20000] * 33 + [4000, 9] * 24, 0.03),    # more than a wave of both
+    (1, [(1 << 21) + 5, 4096, 30], 0.1),          # with an emission kernel
+    (3, [30000, 4096, 60000, 17], 0.2),           # without lists
+])
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+def test_steps_with_small_blocks_do_not_depend_on_what_is_waited_for(n, sizes, ratio, dtype):
+    # back to back, in between kernels that write what the step reads, and one at a time: the same bits
+    offs = list(np.cumsum([0] + sizes))
+    d, steps = int(offs[-1]), 8
+    gen = torch.Generator(device="cuda").manual_seed(d)
+    batches = [normal(gen, n, d).to(dtype) for _ in range(steps)]
+    results = []
+    for wait in (False, True):
+        opt, theta, G = CompAMS(n, d, offs, TOPK, ratio), torch.zeros(d, device="cuda"), torch.empty_like(batches[0])
+        for t in range(steps):
+            G.copy_(batches[t])
+            theta.add_(0.125)
+            if wait:
+                torch.cuda.synchronize()
+            opt.step(G, theta)
+            if t % 3 == 2:  # two steps without anything between them
+                opt.step(G, theta)
+            if wait:
+                torch.cuda.synchronize()
+        assert opt.check_status() == 0
+        results.append([theta] + [opt.buffer(name).clone() for name in ("E", "m", "v", "vhat")])
+        opt.close()
+    for name, a, b in zip(("theta", "E", "m", "v", "vhat"), *results):
+        assert torch.equal(a, b), name
+
+
 @pytest.mark.parametrize("n,d,ratio", [
     (1, (1 << 21) + 5, 0.1),    # list emitted by a kernel of its own, 16 CTAs
     (2, 3000001, 0.111),        # the densest selection with a candidate list ...
