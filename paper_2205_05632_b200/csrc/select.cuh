@@ -447,14 +447,17 @@ __device__ __forceinline__ bool select_slices(const Group& grp, const TopkBuffer
         }
     }
     if (!take_all && !by_index) {
-        // as many as the histogram has counted; never more than have been written
-        const uint32_t got = *grp.of(&sh.nsurv, 0), count = got < c0 ? got : c0;
-        if (got != c0 && rank == 0 && threadIdx.x == 0) atomicOr(b.status, 1u);
+        // As many as the histogram has counted, which the arrays have room for; no more than have been collected are ranked. The two
+        // counts agree on every path: a slice of one round is the same registers in both passes, and nothing writes a list or a block
+        // in between. Should they not, the status word says so and no entry that nobody wrote reaches a message.
+        const uint32_t got = *grp.of(&sh.nsurv, 0);  // travels with the entries
         if (rank) {
             const uint2* src = grp.of(sh.surv, 0);
-            for (uint32_t q = threadIdx.x; q < count; q += NT) sh.surv[q] = src[q];
+            for (uint32_t q = threadIdx.x; q < c0; q += NT) sh.surv[q] = src[q];
             __syncthreads();
         }
+        const uint32_t count = got < c0 ? got : c0;
+        if (got != c0 && rank == 0 && threadIdx.x == 0) atomicOr(b.status, 1u);
         out.closer = rank_survivors(b, job, sh.surv, count, k_rem, (threadIdx.x >> 5) * C + rank, C * (NT / 32), &out.tau);
     }
     // with the whole bin kept, everything from its lower edge on; otherwise the kept entries of the bin have been zeroed
