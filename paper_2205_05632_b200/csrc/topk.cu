@@ -630,7 +630,10 @@ __global__ void __launch_bounds__(kThreads, 4) topk_emit_kernel(const __grid_con
     }
     if (!is_last) return;
     __threadfence();
-    uint32_t k_rem = st->k_rem, count = k_rem ? __ldcg(nsurv) : 0u;
+    // put_survivors counts past kSurvCap but stores no more (topk_select defers no list with more in its threshold bin)
+    const uint32_t in_bin = __ldcg(nsurv);
+    uint32_t k_rem = st->k_rem, count = k_rem ? (in_bin < (uint32_t)kSurvCap ? in_bin : (uint32_t)kSurvCap) : 0u;
+    if (in_bin > (uint32_t)kSurvCap && threadIdx.x == 0) atomicOr(b.status, 1u);
     const uint32_t wins = job.kb - k_rem, taken = sh_above;
     __syncthreads();
     for (uint32_t q = threadIdx.x; q < count; q += kThreads) surv[q] = __ldcg(gsurv + q);
