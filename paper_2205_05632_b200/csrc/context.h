@@ -89,7 +89,7 @@ struct TopkBuffers {
     int64_t cand_total;        // candidate slots per worker
     int32_t cluster_max;       // coordinates per CTA up to which a select's cluster goes through the block itself
     uint32_t* dense_count;     // [1] segments currently marked for the dense passes
-    uint32_t* sel_ticket;      // [n * long lists, 4] threshold-bin entries collected, -, message slots taken, parts of the emission done
+    uint32_t* sel_ticket;      // [n * long lists, 4] threshold-bin entries collected, unused, one 64-bit word: message slots taken, parts done
     uint2* sel_surv;           // [n * long lists, kSurvCap] threshold-bin entries of a long list
     uint32_t* map;             // Random-k: a bit per element of a group of workers, set where it is drawn
     uint32_t* slots;           // Random-k: [n * nseg] message slots handed out this step

@@ -8,8 +8,8 @@
 // halves of the first three words of one Philox4x64-10 block (Salmon, Moraes, Dror, Shaw, SC 2011) at counter
 // (0, 0, b, i) under key (seed, t); the round function is the 32-bit finalizer of MurmurHash3 applied to
 // (right half xor round key). Being the image of k_b distinct inputs under a bijection, the set has exactly k_b
-// members and needs no selection. Two kernels per group of workers: randk_mark, one thread per message slot, computes the
-// slot's coordinate and sets its bit in a map of the group's elements; randk_sweep forms x = g + e, and where the bit is
+// members and needs no selection. Two kernels per group of workers: randk_mark, one to eight message slots per thread, computes
+// each slot's coordinate and sets its bit in a map of the group's elements; randk_sweep forms x = g + e, and where the bit is
 // set x goes to the message and to the server and 0 to E (the residual of a kept coordinate), x to E elsewhere.
 //
 // The map is what makes the drawn coordinates meet their x in index order: it is small enough for the L2 (64 MB: hence the

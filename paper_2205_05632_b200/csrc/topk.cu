@@ -535,8 +535,8 @@ __global__ void __launch_bounds__(kSelThreads, 2) topk_fused_kernel(const __grid
     select_segment<NT>(grp, sh, t, b, si, i, seg, s, true, deliver != 0, false);
 }
 
-// Emission of long lists that topk_select has found the threshold of: `parts` CTAs stream through each list, the winners
-// take message slots warp by warp, the threshold bin's entries are collected, and the CTA that comes last ranks them
+// Emission of long lists that topk_select has found the threshold of: `parts` CTAs stream through each list, a round's winners
+// take their message slots with one atomic, the threshold bin's entries are collected, and the CTA that comes last ranks them
 // and closes the segment. A CTA is bound by its chain of dependent accesses - list, slots, stores - and a list by the few CTAs an
 // SM holds: the first round's entries do not wait for the list's length, bucket slots and message slots are asked for together,
 // and the counter that hands out the message slots counts the parts, too, so that no fence stands behind the stores (n = 8, d =
@@ -562,7 +562,11 @@ __global__ void __launch_bounds__(kThreads, 4) topk_emit_kernel(const __grid_con
     ListSlice sl;
     sl.list = b.cand + (size_t)i * (size_t)b.cand_total + (size_t)si.cand_off;
     sl.lo = 0u;
-    sl.hi = si.cap;  // the first round's loads do not wait for the count
+    // The first round's loads do not wait for the count. Parts are as many as the longest list has: those of a shorter list read past
+    // its end, within its room, which costs nothing that shows (us per step without any early load / so / up to the expected length:
+    // n = 8, 10 % of 6 M and 12 x 250,000 320.5 / 310.2 / 310.2; n = 4, 5 % of 20 M and 12 x 1.2 M 545 / 535 / 535; n = 2, 3 % of 16, 8, 4, 2, 1
+    // and 0.5 M 366 / 358 / 362).
+    sl.hi = si.cap;
     uint2 cv[U];
     uint32_t p0 = part * (U * kThreads);
     sl.load<kThreads>(p0, cv);
@@ -1208,8 +1212,10 @@ cudaError_t launch_topk_sweep(compams_context* c, const void* grads) {
     return c->grad_bf16 ? launch_sweep_typed(c, (const bf16_bits*)grads) : launch_sweep_typed(c, (const float*)grads);
 }
 
-// While n d <= kChainMaxElems the kernels of a step are launched as programmatic dependents of one another (each
-// waits for its predecessor before its first global access): the launch latency and the prologue of a
+// While n d <= kChainMaxElems the kernels of a step are launched as programmatic dependents of one another (each waits for its
+// predecessor before it touches anything that a kernel of this step, or of the one before, may still write; topk_small, which
+// shares no block with topk_sweep and topk_select, starts beside them and waits at its end, which is safe because the sweep's CTAs let
+// the next kernel in only behind their own wait): the launch latency and the prologue of a
 // kernel then overlap the tail of the one before, which is most of what such a step costs.
 
 typedef void (*SelectKernel)(const Tables, const TopkBuffers, const int32_t*, int, int, int, int, int);
