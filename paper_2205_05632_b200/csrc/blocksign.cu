@@ -364,7 +364,7 @@ struct ApplyShared {
         struct {
             uint32_t bits[kChunk][kApplySpan / 32];   // [worker][word]
             double four[kChunk / 4][16];              // subset sums of 4 workers' scales
-            double eight[FOURS ? 1 : kChunk / 8][256];  // ... of 8 workers'
+            double eight[FOURS ? 1 : kChunk / 8][FOURS ? 1 : 256];  // ... of 8 workers', not with FOURS
             double scale[kChunk];
         } sum;
         float gbar[kApplySpan + 4];
